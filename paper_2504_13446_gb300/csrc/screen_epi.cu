@@ -973,6 +973,7 @@ struct EpiTheta {
     float xsb, pxs;          // skip pairs with screened score <= xsb
     bool have_pf;
   };
+  static constexpr bool kReloads = true;   // chunk() reads accumulator columns again
   static constexpr size_t kSmem = sizeof(int16_t) * 2 * 128 * kJS +
                                   sizeof(int) * (2 * kThetaBN * 32 + 3 * kThetaBN) +
                                   sizeof(tc::RowBound) * kThetaBN;

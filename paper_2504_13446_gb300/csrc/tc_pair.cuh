@@ -121,24 +121,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       prefetch_map(&mAh); prefetch_map(&mBh);
       if (op.split) { prefetch_map(&mAl); prefetch_map(&mBl); }
       uint32_t it = 0;
+      Ring<STAGES> ring;
       for (int p = pair0; p < npairs && !failed; p += npair_ctas) {
         const int rb = 2 * p + rank;    // may be one past the last row block
-        for (int ct = 0; ct < sch.nct && !failed; ++ct)
+        for (int ct = 0; ct < sch.nct && !failed; ++ct) {
+          ChunkWalk w;
           for (int kc = 0; kc < nk; ++kc, ++it) {
-            const int s = it % STAGES;
-            const uint32_t ph = (it / STAGES) & 1;
-            if (!mbar_wait(&empty[s], ph ^ 1, kWaitLimit, true)) { failed = true; break; }
+            const uint32_t s = ring.s;
+            if (!mbar_wait(&empty[s], ring.ph ^ 1, kWaitLimit, true)) { failed = true; break; }
             unsigned char *sa = stages + (size_t)s * L::kStage;
             unsigned char *sb = sa + L::kA;
-            const int g = kc / op.kchunks, c = kc - g * op.kchunks;
             mbar_expect_tx(&full[s], L::kStage);
             // split order: hi.lo, lo.hi, then hi.hi (small terms first)
-            const bool alo = op.split && g == 1, blo = op.split && g == 0;
-            const int kx = c * KCH;
+            const bool alo = op.split && w.g == 1, blo = op.split && w.g == 0;
+            const int kx = w.c * KCH;
             tma_load_2d(sa, alo ? &mAl : &mAh, kx, rb * BM, &full[s]);
             tma_load_2d_mc(sb + (size_t)rank * kHalfB, blo ? &mBl : &mBh, kx,
                            ct * BN + rank * (BN / 2), &full[s], (uint16_t)0x3);
+            w.next(op.kchunks);
+            ring.next();
           }
+        }
       }
       issued = it;
       if (failed) {
@@ -150,33 +153,27 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(BM, BN);
-      uint32_t it = 0, t = 0;
-      for (int p = pair0; p < npairs && !failed; p += npair_ctas)
-        for (int ct = 0; ct < sch.nct && !failed; ++ct, ++t) {
-          const int b = t & 1;
-          const uint32_t aph = (t >> 1) & 1;
-          if (!mbar_wait(&acc_empty[b], aph ^ 1, kWaitLimit, true)) { failed = true; break; }
-          tc_fence_after();
-          const uint32_t dt = tmem + (uint32_t)(b * BN);
-          for (int kc = 0; kc < nk; ++kc, ++it) {
-            const int s = it % STAGES;
-            const uint32_t ph = (it / STAGES) & 1;
-            if (!mbar_wait(&full[s], ph)) { failed = true; break; }
-            tc_fence_after();
-            const uint32_t sa = smem_u32(stages + (size_t)s * L::kStage);
-            const uint32_t sb = sa + L::kA;
-            const int c = kc % op.kchunks;
-            const int steps = min(4, op.ksteps - c * 4);
-            for (int k = 0; k < steps; ++k)
-              umma_bf16(dt, sw128_desc(sa + k * 32), sw128_desc(sb + k * 32), idesc,
-                        (kc > 0 || k > 0) ? 1u : 0u);
-            umma_commit_mc(&empty[s], (uint16_t)0x3);
-          }
-          if (failed) break;
-          umma_commit(&acc_full[b]);
-        }
+    const uint32_t idesc = idesc_bf16(BM, BN);
+    const uint64_t desc0 = sw128_desc(smem_u32(stages));
+    Ring<STAGES> ring;
+    bool ready = false;
+    uint32_t t = 0;
+    for (int p = pair0; p < npairs && !failed; p += npair_ctas)
+      for (int ct = 0; ct < sch.nct && !failed; ++ct, ++t) {
+        const int b = t & 1;
+        const uint32_t aph = (t >> 1) & 1;
+        if (!mbar_wait_warp(&acc_empty[b], aph ^ 1, kWaitLimit, true)) { failed = true; break; }
+        tc_fence_after();
+        const uint32_t dt = tmem + (uint32_t)(b * BN);
+        failed = !mma_tile<STAGES, L::kStage, L::kA>(
+            op, nk, full, desc0, ring, ready,
+            [&](uint64_t da, uint64_t db, uint32_t acc) { umma_bf16(dt, da, db, idesc, acc); },
+            [&](uint32_t s, bool last) {
+              umma_commit_mc(&empty[s], (uint16_t)0x3);
+              if (last) umma_commit(&acc_full[b]);
+            });
+      }
+    if (elect_one()) {
       if (failed) {
         atomicExch(err, 2);
         *s_failed = 1;
@@ -184,6 +181,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       umma_commit(drain);
       mbar_wait(drain, 0);
     }
+    __syncwarp();
   } else {
     // ----------------------------------------------------------- epilogue
     const int e = warp - 2;
@@ -200,23 +198,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       u.rb0 = rb; u.rb1 = rb + 1; u.ct0 = 0; u.ct1 = sch.nct;
       if (real) epi.unit_begin(escratch, u, et, ts);
       epi_sync();
-      for (int ct = 0; ct < sch.nct && !failed; ++ct, ++t) {
+      for (int ct = 0; ct < sch.nct; ++ct, ++t) {
         const int b = t & 1;
         const uint32_t aph = (t >> 1) & 1;
-        const bool ok = mbar_wait(&acc_full[b], aph, op.epi_wait);
-        if (epi_vote_any(!ok)) { failed = true; break; }
+        if (!failed && !mbar_wait_warp(&acc_full[b], aph, op.epi_wait)) failed = true;
         tc_fence_after();
+        auto release = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[b]);
+        };
         if (real) {
           epi.tile_begin(escratch, rb, ct, r, half, ts);
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN);
-          epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts);
+          if (!failed)
+            epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts, release);
           epi.tile_end(escratch, rb, ct, r, half, ts);
+        } else if (!failed) {
+          release();
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[b]);
       }
-      epi_sync();
+      failed = epi_vote_any(failed);
       if (!failed && real) epi.unit_end(escratch, u, et, ts);
       epi_sync();
     }
@@ -393,24 +395,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (op.split) { prefetch_map(&mAl); prefetch_map(&mBl); }
       const uint32_t full0 = map_to_rank(smem_u32(full), 0);
       uint32_t it = 0;
+      Ring<STAGES> ring;
       for (int p = pair0; p < npairs && !failed; p += npair_ctas) {
         const int rb = 2 * p + rank;    // may be one past the last row block
-        for (int ct = 0; ct < sch.nct && !failed; ++ct)
+        for (int ct = 0; ct < sch.nct && !failed; ++ct) {
+          ChunkWalk w;
           for (int kc = 0; kc < nk; ++kc, ++it) {
-            const int s = it % STAGES;
-            const uint32_t ph = (it / STAGES) & 1;
-            if (!mbar_wait(&empty[s], ph ^ 1, kWaitLimit, true)) { failed = true; break; }
+            const uint32_t s = ring.s;
+            if (!mbar_wait(&empty[s], ring.ph ^ 1, kWaitLimit, true)) { failed = true; break; }
             unsigned char *sa = stages + (size_t)s * L::kStage;
             unsigned char *sb = sa + L::kA;
-            const int g = kc / op.kchunks, c = kc - g * op.kchunks;
             if (rank == 0) mbar_expect_tx(&full[s], 2 * L::kStage);
             // split order: hi.lo, lo.hi, then hi.hi (small terms first)
-            const bool alo = op.split && g == 1, blo = op.split && g == 0;
-            const int kx = c * KCH;
+            const bool alo = op.split && w.g == 1, blo = op.split && w.g == 0;
+            const int kx = w.c * KCH;
             const uint32_t fb = full0 + (uint32_t)(s * sizeof(uint64_t));
             tma_load_2d_peerbar(sa, alo ? &mAl : &mAh, kx, rb * BM, fb);
             tma_load_2d_peerbar(sb, blo ? &mBl : &mBh, kx, ct * BN + rank * (BN / 2), fb);
+            w.next(op.kchunks);
+            ring.next();
           }
+        }
       }
       issued = it;
       if (failed) {
@@ -420,39 +425,38 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       const uint32_t idesc = idesc_bf16(2 * BM, BN);
-      uint32_t it = 0, t = 0;
+      const uint64_t desc0 = sw128_desc(smem_u32(stages));
+      Ring<STAGES> ring;
+      bool ready = false;
+      uint32_t t = 0;
       for (int p = pair0; p < npairs && !failed; p += npair_ctas)
         for (int ct = 0; ct < sch.nct && !failed; ++ct, ++t) {
           const int b = t & 1;
           const uint32_t aph = (t >> 1) & 1;
-          if (!mbar_wait(&acc_empty[b], aph ^ 1, kWaitLimit, true)) { failed = true; break; }
+          if (!mbar_wait_warp(&acc_empty[b], aph ^ 1, kWaitLimit, true)) { failed = true; break; }
           tc_fence_after();
           const uint32_t dt = tmem + (uint32_t)(b * BN);
-          for (int kc = 0; kc < nk; ++kc, ++it) {
-            const int s = it % STAGES;
-            const uint32_t ph = (it / STAGES) & 1;
-            if (!mbar_wait(&full[s], ph)) { failed = true; break; }
-            tc_fence_after();
-            const uint32_t sa = smem_u32(stages + (size_t)s * L::kStage);
-            const uint32_t sb = sa + L::kA;
-            const int c = kc % op.kchunks;
-            const int steps = min(4, op.ksteps - c * 4);
-            for (int k = 0; k < steps; ++k)
-              umma_bf16_pair(dt, sw128_desc(sa + k * 32), sw128_desc(sb + k * 32), idesc,
-                             (kc > 0 || k > 0) ? 1u : 0u);
-            umma_commit_pair(&empty[s], (uint16_t)0x3);
-          }
-          if (failed) break;
-          umma_commit_pair(&acc_full[b], (uint16_t)0x3);
+          failed = !mma_tile<STAGES, L::kStage, L::kA>(
+              op, nk, full, desc0, ring, ready,
+              [&](uint64_t da, uint64_t db, uint32_t acc) {
+                umma_bf16_pair(dt, da, db, idesc, acc);
+              },
+              [&](uint32_t s, bool last) {
+                umma_commit_pair(&empty[s], (uint16_t)0x3);
+                if (last) umma_commit_pair(&acc_full[b], (uint16_t)0x3);
+              });
         }
-      if (failed) {
-        atomicExch(err, 2);
-        *s_failed = 1;
+      if (elect_one()) {
+        if (failed) {
+          atomicExch(err, 2);
+          *s_failed = 1;
+        }
+        // the drain barriers of both CTAs complete once every MMA above has
+        umma_commit_pair(drain, (uint16_t)0x3);
       }
-      // the drain barriers of both CTAs complete once every MMA above has
-      umma_commit_pair(drain, (uint16_t)0x3);
+      __syncwarp();
     }
   } else {
     // ----------------------------------------------------------- epilogue
@@ -471,23 +475,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       u.rb0 = rb; u.rb1 = rb + 1; u.ct0 = 0; u.ct1 = sch.nct;
       if (real) epi.unit_begin(escratch, u, et, ts);
       epi_sync();
-      for (int ct = 0; ct < sch.nct && !failed; ++ct, ++t) {
+      for (int ct = 0; ct < sch.nct; ++ct, ++t) {
         const int b = t & 1;
         const uint32_t aph = (t >> 1) & 1;
-        const bool ok = mbar_wait(&acc_full[b], aph, op.epi_wait);
-        if (epi_vote_any(!ok)) { failed = true; break; }
+        if (!failed && !mbar_wait_warp(&acc_full[b], aph, op.epi_wait)) failed = true;
         tc_fence_after();
+        auto release = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(ae0 + (uint32_t)(b * sizeof(uint64_t)));
+        };
         if (real) {
           epi.tile_begin(escratch, rb, ct, r, half, ts);
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN);
-          epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts);
+          if (!failed)
+            epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts, release);
           epi.tile_end(escratch, rb, ct, r, half, ts);
+        } else if (!failed) {
+          release();
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(ae0 + (uint32_t)(b * sizeof(uint64_t)));
       }
-      epi_sync();
+      failed = epi_vote_any(failed);
       if (!failed && real) epi.unit_end(escratch, u, et, ts);
       epi_sync();
     }

@@ -53,9 +53,9 @@ __device__ __forceinline__ Unit unit_of(const Schedule &s, int i) {
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // Barrier of the 256 epilogue threads that also ORs a predicate over them, so
-// that every epilogue warp takes the same decision after a bounded wait (a
-// warp that gave up and one that did not would otherwise disagree on the
-// number of barriers still to come).
+// that every epilogue warp takes the same decision at the end of a unit (a warp
+// that gave up a bounded wait and one that did not would otherwise disagree on
+// the number of barriers still to come).
 __device__ __forceinline__ bool epi_vote_any(bool p) {
   uint32_t r;
   asm volatile(
@@ -67,22 +67,95 @@ __device__ __forceinline__ bool epi_vote_any(bool p) {
   return r != 0;
 }
 
+// K chunks of a tile in the order they are multiplied: a counter over the chunks
+// of `nseg` segments (no division: the issue loops run once per chunk and are on
+// the critical path of the MMAs).
+struct ChunkWalk {
+  int c = 0, g = 0;   // chunk within the segment, segment
+  __device__ __forceinline__ void next(int kchunks) {
+    if (++c == kchunks) {
+      c = 0;
+      ++g;
+    }
+  }
+};
+
+// Position in a ring of STAGES pipeline stages and the phase parity of its pass.
+template <int STAGES>
+struct Ring {
+  uint32_t s = 0, ph = 0;
+  __device__ __forceinline__ void next() {
+    if (++s == (uint32_t)STAGES) {
+      s = 0;
+      ph ^= 1;
+    }
+  }
+};
+
+// MMA issue for one accumulator tile (whole warp, converged).  The warp walks the
+// chunk loop together and one elected lane issues, so that descriptors and
+// addresses live in uniform registers; the next stage's barrier is looked at
+// before this stage's MMAs are issued, which hides its latency.  Measured per
+// 64-wide chunk of a 128 x 256 tile (four MMAs, 516 cycles of tensor pipe): one
+// lane in a divergent branch with a division per chunk 920 cycles, this form 570.
+// Returns false when a bounded wait gave up.
+template <int STAGES, uint32_t kStageBytes, uint32_t kABytes, class Issue, class Free>
+__device__ __forceinline__ bool mma_tile(const Operands &op, int nk, uint64_t *full,
+                                         uint64_t desc0, Ring<STAGES> &ring, bool &ready,
+                                         Issue &&issue, Free &&release) {
+  const int last = op.ksteps - (op.kchunks - 1) * 4;   // MMA steps of a segment's last chunk
+  int c = 0;
+  for (int kc = 0; kc < nk; ++kc) {
+    if (!ready && !mbar_wait_warp(&full[ring.s], ring.ph)) return false;
+    const uint32_t s = ring.s;
+    ring.next();
+    ready = mbar_test_warp(&full[ring.s], ring.ph);
+    tc_fence_after();
+    const uint64_t da = desc0 + (uint64_t)(s * (kStageBytes >> 4));
+    const uint64_t db = da + (kABytes >> 4);
+    const int steps = ++c == op.kchunks ? last : 4;
+    if (c == op.kchunks) c = 0;
+    if (elect_one()) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k < steps) issue(da + 2 * k, db + 2 * k, (kc | k) != 0 ? 1u : 0u);
+      release(s, kc == nk - 1);
+    }
+    __syncwarp();
+  }
+  return true;
+}
+
+// Whether the epilogue's chunk() reads TMEM again (then a tile's accumulator is
+// released only after its last chunk; otherwise right after its last load).
+template <class Epi, class = void>
+struct EpiReloads {
+  static constexpr bool value = false;
+};
+template <class Epi>
+struct EpiReloads<Epi, decltype((void)Epi::kReloads)> {
+  static constexpr bool value = Epi::kReloads;
+};
+
 // This thread's half row of an accumulator tile (TMEM row address trow): 64
 // columns per TMEM load (one wait), handed to the epilogue as chunks of 32.
-template <int BN, class Epi>
+// `release` frees the accumulator once nothing will read it again.
+template <int BN, class Epi, class Free>
 __device__ __forceinline__ void epi_tile_columns(const Epi &epi, char *S, int rb, int ct, int r,
                                                  int half, uint32_t trow,
-                                                 typename Epi::Thread &ts) {
+                                                 typename Epi::Thread &ts, Free &&release) {
 #pragma unroll 1
   for (int cc = 0; cc < BN / 64; cc += 2) {
     const int col = half * (BN / 2) + cc * 32;
     float v[64];
     tmem_ld64(trow + col, v);
+    if (!EpiReloads<Epi>::value && cc + 2 >= BN / 64) release();
     epi.chunk(S, rb, ct, r, col, trow + (uint32_t)col,
               *reinterpret_cast<const float(*)[32]>(v), ts);
     epi.chunk(S, rb, ct, r, col + 32, trow + (uint32_t)(col + 32),
               *reinterpret_cast<const float(*)[32]>(v + 32), ts);
   }
+  if (EpiReloads<Epi>::value) release();
 }
 
 template <int BN>
@@ -141,24 +214,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       prefetch_map(&mAh); prefetch_map(&mBh);
       if (op.split) { prefetch_map(&mAl); prefetch_map(&mBl); }
       uint32_t it = 0;
+      Ring<STAGES> ring;
+      const int kstep = op.fp8 ? 2 * KCH : KCH;  // elements of 128 bytes
       for (int ui = blockIdx.x; ui < sch.nunits && !failed; ui += gridDim.x) {
         Unit u = unit_of(sch, ui);
         for (int rb = u.rb0; rb < u.rb1 && !failed; ++rb)
-          for (int ct = u.ct0; ct < u.ct1 && !failed; ++ct)
+          for (int ct = u.ct0; ct < u.ct1 && !failed; ++ct) {
+            ChunkWalk w;
             for (int kc = 0; kc < nk; ++kc, ++it) {
-              const int s = it % STAGES;
-              const uint32_t ph = (it / STAGES) & 1;
-              if (!mbar_wait(&empty[s], ph ^ 1, kWaitLimit, true)) { failed = true; break; }
+              const uint32_t s = ring.s;
+              if (!mbar_wait(&empty[s], ring.ph ^ 1, kWaitLimit, true)) { failed = true; break; }
               unsigned char *sa = stages + (size_t)s * L::kStage;
               unsigned char *sb = sa + L::kA;
-              const int g = kc / op.kchunks, c = kc - g * op.kchunks;
               mbar_expect_tx(&full[s], L::kStage);
               // split order: hi.lo, lo.hi, then hi.hi (small terms first)
-              const bool alo = op.split && g == 1, blo = op.split && g == 0;
-              const int kx = c * (op.fp8 ? 2 * KCH : KCH);  // elements of 128 bytes
+              const bool alo = op.split && w.g == 1, blo = op.split && w.g == 0;
+              const int kx = w.c * kstep;
               tma_load_2d(sa, alo ? &mAl : &mAh, kx, rb * BM, &full[s]);
               tma_load_2d(sb, blo ? &mBl : &mBh, kx, ct * BN, &full[s]);
+              w.next(op.kchunks);
+              ring.next();
             }
+          }
       }
       if (failed) {
         atomicExch(err, 1);
@@ -169,46 +246,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA
-    if (lane == 0) {
-      const uint32_t idesc = op.fp8 ? idesc_e4m3(BM, BN) : idesc_bf16(BM, BN);
-      uint32_t it = 0, t = 0;
-      for (int ui = blockIdx.x; ui < sch.nunits && !failed; ui += gridDim.x) {
-        Unit u = unit_of(sch, ui);
-        for (int rb = u.rb0; rb < u.rb1 && !failed; ++rb)
-          for (int ct = u.ct0; ct < u.ct1 && !failed; ++ct, ++t) {
-            const int b = t & 1;
-            const uint32_t aph = (t >> 1) & 1;
-            if (!mbar_wait(&acc_empty[b], aph ^ 1, kWaitLimit, true)) { failed = true; break; }
-            tc_fence_after();
-            const uint32_t dt = tmem + (uint32_t)(b * BN);
-            for (int kc = 0; kc < nk; ++kc, ++it) {
-              const int s = it % STAGES;
-              const uint32_t ph = (it / STAGES) & 1;
-              if (!mbar_wait(&full[s], ph)) { failed = true; break; }
-              tc_fence_after();
-              const uint32_t sa = smem_u32(stages + (size_t)s * L::kStage);
-              const uint32_t sb = sa + L::kA;
-              const int c = kc % op.kchunks;
-              const int steps = min(4, op.ksteps - c * 4);
-              for (int k = 0; k < steps; ++k) {
-                if (op.fp8)
-                  umma_e4m3(dt, sw128_desc(sa + k * 32), sw128_desc(sb + k * 32), idesc,
-                            (kc > 0 || k > 0) ? 1u : 0u);
-                else
-                  umma_bf16(dt, sw128_desc(sa + k * 32), sw128_desc(sb + k * 32), idesc,
-                            (kc > 0 || k > 0) ? 1u : 0u);
-              }
-              umma_commit(&empty[s]);
-            }
-            if (failed) break;
-            umma_commit(&acc_full[b]);
-          }
-      }
+    const uint32_t idesc = op.fp8 ? idesc_e4m3(BM, BN) : idesc_bf16(BM, BN);
+    const uint64_t desc0 = sw128_desc(smem_u32(stages));
+    Ring<STAGES> ring;
+    bool ready = false;
+    uint32_t t = 0;
+    for (int ui = blockIdx.x; ui < sch.nunits && !failed; ui += gridDim.x) {
+      Unit u = unit_of(sch, ui);
+      for (int rb = u.rb0; rb < u.rb1 && !failed; ++rb)
+        for (int ct = u.ct0; ct < u.ct1 && !failed; ++ct, ++t) {
+          const int b = t & 1;
+          const uint32_t aph = (t >> 1) & 1;
+          if (!mbar_wait_warp(&acc_empty[b], aph ^ 1, kWaitLimit, true)) { failed = true; break; }
+          tc_fence_after();
+          const uint32_t dt = tmem + (uint32_t)(b * BN);
+          failed = !mma_tile<STAGES, L::kStage, L::kA>(
+              op, nk, full, desc0, ring, ready,
+              [&](uint64_t da, uint64_t db, uint32_t acc) {
+                if (op.fp8) umma_e4m3(dt, da, db, idesc, acc);
+                else umma_bf16(dt, da, db, idesc, acc);
+              },
+              [&](uint32_t s, bool last) {
+                umma_commit(&empty[s]);
+                if (last) umma_commit(&acc_full[b]);
+              });
+        }
+    }
+    if (elect_one()) {
       if (failed) atomicExch(err, 2);
-      // all MMAs issued by this thread complete before the CTA releases TMEM
+      // all MMAs issued by this warp complete before the CTA releases TMEM
       umma_commit(drain);
       mbar_wait(drain, 0);
     }
+    __syncwarp();
   } else {
     // ----------------------------------------------------------- epilogue
     const int e = warp - 2;                 // 0..7
@@ -222,22 +292,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       Unit u = unit_of(sch, ui);
       epi.unit_begin(escratch, u, et, ts);
       epi_sync();
-      for (int rb = u.rb0; rb < u.rb1 && !failed; ++rb)
-        for (int ct = u.ct0; ct < u.ct1 && !failed; ++ct, ++t) {
+      for (int rb = u.rb0; rb < u.rb1; ++rb)
+        for (int ct = u.ct0; ct < u.ct1; ++ct, ++t) {
           const int b = t & 1;
           const uint32_t aph = (t >> 1) & 1;
-          const bool ok = mbar_wait(&acc_full[b], aph, op.epi_wait);
-          if (epi_vote_any(!ok)) { failed = true; break; }
+          // a warp that gave up goes through the rest of the unit without waiting or
+          // reading, so that every warp passes the same barriers (the vote below)
+          if (!failed && !mbar_wait_warp(&acc_full[b], aph, op.epi_wait)) failed = true;
           tc_fence_after();
           epi.tile_begin(escratch, rb, ct, r, half, ts);
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN);
-          epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts);
+          if (!failed)
+            epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts, [&]() {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&acc_empty[b]);
+            });
           epi.tile_end(escratch, rb, ct, r, half, ts);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&acc_empty[b]);
         }
-      epi_sync();
+      failed = epi_vote_any(failed);
       if (!failed) epi.unit_end(escratch, u, et, ts);
       epi_sync();
     }
