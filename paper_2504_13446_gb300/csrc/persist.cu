@@ -69,16 +69,34 @@ struct Header {
   double build_ms[8];
 };
 
+// A device array as it stands in the file: `bytes` contiguous bytes.  An array of
+// rows with a wider pitch on the device (row > 0: row bytes kept of every ld
+// bytes) is written and read without its padding.
 struct Arr {
   uint32_t id;
   void **ptr;
   uint64_t bytes;
+  uint64_t row = 0, ld = 0;
+  uint64_t device_bytes() const { return row ? bytes / row * ld : bytes; }
+  // whole rows per staging chunk
+  uint64_t chunk() const { return row ? std::max<uint64_t>(kChunk / row, 1) * row : kChunk; }
 };
+
+// Bytes [off, off + b) of the file form of `a`, to or from the host buffer.
+cudaError_t copy_part(const Arr &a, uint64_t off, size_t b, void *host, bool to_host) {
+  char *dev = (char *)*a.ptr + (a.row ? off / a.row * a.ld : off);
+  const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+  if (!a.row || a.row == a.ld)
+    return to_host ? cudaMemcpy(host, dev, b, kind) : cudaMemcpy(dev, host, b, kind);
+  return to_host ? cudaMemcpy2D(host, a.row, dev, a.ld, a.row, b / a.row, kind)
+                 : cudaMemcpy2D(dev, a.ld, host, a.row, a.row, b / a.row, kind);
+}
 
 // Every device array of an index with its size; list_entries = xloff[n].
 std::vector<Arr> arrays(rkr_index *x, int64_t list_entries) {
   const uint64_t n = (uint64_t)x->n, m = (uint64_t)x->m, d = (uint64_t)x->d;
   const uint64_t ns = (uint64_t)x->nsamp, kp = (uint64_t)x->Ut.kp, rb = sizeof(tc::RowBound);
+  const uint64_t ul = (uint64_t)x->Ut.ld() * 2, pl = (uint64_t)x->Pt.ld() * 2;
   std::vector<Arr> a = {
       {1, (void **)&x->U, n * d * 4},          {2, (void **)&x->Ps, m * d * 4},
       {3, (void **)&x->perm, m * 4},           {4, (void **)&x->pnorm, m * 8},
@@ -90,9 +108,11 @@ std::vector<Arr> arrays(rkr_index *x, int64_t list_entries) {
       {14, (void **)&x->S, ns * d * 4},        {15, (void **)&x->snrm, ns * 4},
       {16, (void **)&x->sw, ns * 4},           {17, (void **)&x->samp_items, ns * 4},
       {18, (void **)&x->phk, (uint64_t)x->phn * 8}, {19, (void **)&x->phv, (uint64_t)x->phn * 4},
-      {20, (void **)&x->Ut.hi, n * kp * 2},    {21, (void **)&x->Ut.lo, n * kp * 2},
+      {20, (void **)&x->Ut.hi, n * kp * 2, kp * 2, ul},
+      {21, (void **)&x->Ut.lo, n * kp * 2, kp * 2, ul},
       {22, (void **)&x->Ut.rb1, n * rb},       {23, (void **)&x->Ut.rb3, n * rb},
-      {24, (void **)&x->Pt.hi, m * kp * 2},    {25, (void **)&x->Pt.lo, m * kp * 2},
+      {24, (void **)&x->Pt.hi, m * kp * 2, kp * 2, pl},
+      {25, (void **)&x->Pt.lo, m * kp * 2, kp * 2, pl},
       {26, (void **)&x->Pt.rb1, m * rb},       {27, (void **)&x->Pt.rb3, m * rb},
   };
   if (x->has_exact) {
@@ -163,10 +183,10 @@ extern "C" rkr_status rkr_index_device_bytes(const rkr_index *idx_c, int64_t *ou
     RKR_CUDA(cudaMemcpy(&list_entries, idx->xloff + idx->n, sizeof(int64_t),
                         cudaMemcpyDeviceToHost));
   int64_t tot = 0;
-  for (const Arr &a : arrays(idx, list_entries)) tot += (int64_t)a.bytes;
+  for (const Arr &a : arrays(idx, list_entries)) tot += (int64_t)a.device_bytes();
   // the concatenated split operands (derived, not saved)
   for (const TcSide *t : {&idx->Ut, &idx->Pt})
-    if (t->cat) tot += (int64_t)t->rows * 3 * t->kp * 2;
+    if (t->cat) tot += (int64_t)t->rows * tc_pitch(3 * t->kp) * 2;
   *out = tot;
   return RKR_OK;
 }
@@ -210,9 +230,9 @@ extern "C" rkr_status rkr_index_save(const rkr_index *idx_c, const char *path) {
     RKR_TRY(put(fh.f, h, &a.id, 4));
     RKR_TRY(put(fh.f, h, &zero, 4));
     RKR_TRY(put(fh.f, h, &a.bytes, 8));
-    for (uint64_t off = 0; off < a.bytes; off += kChunk) {
-      const size_t b = (size_t)std::min<uint64_t>(kChunk, a.bytes - off);
-      RKR_CUDA(cudaMemcpy(buf.p, (const char *)*a.ptr + off, b, cudaMemcpyDeviceToHost));
+    for (uint64_t off = 0; off < a.bytes; off += a.chunk()) {
+      const size_t b = (size_t)std::min<uint64_t>(a.chunk(), a.bytes - off);
+      RKR_CUDA(copy_part(a, off, b, buf.p, true));
       RKR_TRY(put(fh.f, h, buf.p, b));
     }
   }
@@ -276,6 +296,7 @@ extern "C" rkr_status rkr_index_load(const char *path, rkr_index **out) {
   for (TcSide *t : {&idx->Ut, &idx->Pt}) {
     t->d = (int)hd.d;
     t->kp = (int)hd.kp;
+    t->pitch = tc_pitch(t->kp);
     t->owned = true;
   }
   idx->Ut.rows = hd.n;
@@ -296,17 +317,17 @@ extern "C" rkr_status rkr_index_load(const char *path, rkr_index **out) {
     if (id != a.id || bytes != a.bytes)
       return fail(RKR_EINVAL, "index file array %u (%llu bytes) where %u (%llu bytes) belongs",
                   id, (unsigned long long)bytes, a.id, (unsigned long long)a.bytes);
-    if (pool_malloc_async(a.ptr, a.bytes, (cudaStream_t)0) != cudaSuccess) {
+    if (pool_malloc_async(a.ptr, a.device_bytes(), (cudaStream_t)0) != cudaSuccess) {
       cudaGetLastError();
       *a.ptr = nullptr;
       return fail(RKR_ENOMEM, "device allocation of %llu bytes failed",
-                  (unsigned long long)a.bytes);
+                  (unsigned long long)a.device_bytes());
     }
     RKR_CUDA(cudaStreamSynchronize((cudaStream_t)0));
-    for (uint64_t off = 0; off < a.bytes; off += kChunk) {
-      const size_t b = (size_t)std::min<uint64_t>(kChunk, a.bytes - off);
+    for (uint64_t off = 0; off < a.bytes; off += a.chunk()) {
+      const size_t b = (size_t)std::min<uint64_t>(a.chunk(), a.bytes - off);
       RKR_TRY(get(fh.f, h, buf.p, b));
-      RKR_CUDA(cudaMemcpy((char *)*a.ptr + off, buf.p, b, cudaMemcpyHostToDevice));
+      RKR_CUDA(copy_part(a, off, b, buf.p, false));
     }
   }
   const uint64_t want = h.done();

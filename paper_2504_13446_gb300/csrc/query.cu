@@ -89,7 +89,7 @@ __global__ void k_skip_scores(int64_t n, const BinFP *__restrict__ bf,
 }
 
 // Rows of the deep queries, gathered for their own screening launches.
-__global__ void k_gather_qrows(int nd, const int32_t *__restrict__ rows, int kp,
+__global__ void k_gather_qrows(int nd, const int32_t *__restrict__ rows, int kp, int ld,
                                const __nv_bfloat16 *__restrict__ hi,
                                const __nv_bfloat16 *__restrict__ lo,
                                const tc::RowBound *__restrict__ rb1,
@@ -101,8 +101,8 @@ __global__ void k_gather_qrows(int nd, const int32_t *__restrict__ rows, int kp,
   if (i >= nd) return;
   const int64_t r = rows[i];
   for (int k = threadIdx.x; k < kp; k += blockDim.x) {
-    ohi[(int64_t)i * kp + k] = hi[r * kp + k];
-    olo[(int64_t)i * kp + k] = lo[r * kp + k];
+    ohi[(int64_t)i * ld + k] = hi[r * ld + k];
+    olo[(int64_t)i * ld + k] = lo[r * ld + k];
   }
   if (threadIdx.x < 32) {  // the histograms of the skipping pass are incomplete
     hist[r * 32 + threadIdx.x] = 0;
@@ -1117,22 +1117,23 @@ static rkr_status screen_plan(const rkr_index *idx, const QueryCommon &qc, int n
   }
   const int nd = (int)plan.deep.size();
   if (nd > 0) {
-    const int kp = qc.Qt.kp;
+    const int kp = qc.Qt.kp, ld = qc.Qt.ld();
     TcSide &D = plan.dside;
     RKR_TRY(tmp_alloc(plan.bdeep, &plan.deep_d, nd, st));
-    RKR_TRY(tmp_alloc(plan.bdhi, &D.hi, (size_t)nd * kp, st));
-    RKR_TRY(tmp_alloc(plan.bdlo, &D.lo, (size_t)nd * kp, st));
+    RKR_TRY(tmp_alloc(plan.bdhi, &D.hi, (size_t)nd * ld, st));
+    RKR_TRY(tmp_alloc(plan.bdlo, &D.lo, (size_t)nd * ld, st));
     RKR_TRY(tmp_alloc(plan.bdr1, &D.rb1, nd, st));
     RKR_TRY(tmp_alloc(plan.bdr3, &D.rb3, nd, st));
     D.rows = nd;
     D.d = qc.Qt.d;
     D.kp = kp;
+    D.pitch = qc.Qt.pitch;
     D.owned = false;
     RKR_CUDA(cudaMemcpyAsync(plan.deep_d, plan.deep.data(), sizeof(int32_t) * nd,
                              cudaMemcpyHostToDevice, st));
     {
       const int prof_slot = prof_begin("k_gather_qrows", st);
-      k_gather_qrows<<<nd, 128, 0, st>>>(nd, plan.deep_d, kp, qc.Qt.hi, qc.Qt.lo, qc.Qt.rb1,
+      k_gather_qrows<<<nd, 128, 0, st>>>(nd, plan.deep_d, kp, ld, qc.Qt.hi, qc.Qt.lo, qc.Qt.rb1,
                                          qc.Qt.rb3, D.hi, D.lo, D.rb1, D.rb3, hist, nq);
       prof_end(prof_slot, st, 0.0);
     }
@@ -1193,8 +1194,8 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
   TcSide sub = qc.Qt;
   sub.owned = false;
   sub.rows = qb - qa;
-  sub.hi = qc.Qt.hi + (size_t)qa * qc.Qt.kp;
-  sub.lo = qc.Qt.lo + (size_t)qa * qc.Qt.kp;
+  sub.hi = qc.Qt.hi + (size_t)qa * qc.Qt.ld();
+  sub.lo = qc.Qt.lo + (size_t)qa * qc.Qt.ld();
   sub.rb1 = qc.Qt.rb1 + qa;
   sub.rb3 = qc.Qt.rb3 + qa;
   DevBuf bf;
@@ -1234,8 +1235,8 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
     TcSide ds = plan.dside;
     ds.owned = false;
     ds.rows = db - da;
-    ds.hi = plan.dside.hi + (size_t)da * ds.kp;
-    ds.lo = plan.dside.lo + (size_t)da * ds.kp;
+    ds.hi = plan.dside.hi + (size_t)da * ds.ld();
+    ds.lo = plan.dside.lo + (size_t)da * ds.ld();
     ds.rb1 = plan.dside.rb1 + da;
     ds.rb3 = plan.dside.rb3 + da;
     ThetaArgs ad = a;

@@ -17,7 +17,7 @@ namespace rkr {
 // hi = bf16(x), lo = bf16(x - hi) (x - hi and x - hi - lo are exact in FP32),
 // zero padding up to kp, and the bound terms of single and split products
 // (FP64 sums, square roots rounded up to FP32).
-__global__ void k_stage_bf16(const float *__restrict__ X, int64_t rows, int d, int kp,
+__global__ void k_stage_bf16(const float *__restrict__ X, int64_t rows, int d, int kp, int ld,
                              __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
                              tc::RowBound *__restrict__ rb1, tc::RowBound *__restrict__ rb3) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -32,8 +32,8 @@ __global__ void k_stage_bf16(const float *__restrict__ X, int64_t rows, int d, i
     __nv_bfloat16 l = __float2bfloat16_rn(r1);
     float lf = __bfloat162float(l);
     float r3 = r1 - lf;
-    hi[i * kp + k] = h;
-    lo[i * kp + k] = l;
+    hi[i * ld + k] = h;
+    lo[i * ld + k] = l;
     sx += (double)v * v;
     sh += (double)hf * hf;
     sl += (double)lf * lf;
@@ -54,7 +54,8 @@ rkr_status tc_stage(const float *X, int64_t rows, int d, TcSide &out, cudaStream
   out.rows = rows;
   out.d = d;
   out.kp = (d + 15) / 16 * 16;
-  size_t cnt = (size_t)std::max<int64_t>(rows, 1) * out.kp;
+  out.pitch = tc_pitch(out.kp);
+  size_t cnt = (size_t)std::max<int64_t>(rows, 1) * out.ld();
   auto alloc = [&](void **p, size_t bytes) -> rkr_status {
     cudaError_t e = pool_malloc_async(p, bytes, st);
     if (e != cudaSuccess) {
@@ -69,8 +70,8 @@ rkr_status tc_stage(const float *X, int64_t rows, int d, TcSide &out, cudaStream
   RKR_TRY(alloc((void **)&out.rb3, sizeof(tc::RowBound) * std::max<int64_t>(rows, 1)));
   out.owned = true;
   if (rows > 0) {
-    k_stage_bf16<<<(unsigned)((rows + 127) / 128), 128, 0, st>>>(X, rows, d, out.kp, out.hi,
-                                                                 out.lo, out.rb1, out.rb3);
+    k_stage_bf16<<<(unsigned)((rows + 127) / 128), 128, 0, st>>>(X, rows, d, out.kp, out.ld(),
+                                                                 out.hi, out.lo, out.rb1, out.rb3);
     note_launch();
     RKR_CUDA(cudaGetLastError());
   }
@@ -80,8 +81,8 @@ rkr_status tc_stage(const float *X, int64_t rows, int d, TcSide &out, cudaStream
 // cat row = three kp-wide segments: role 1 (A) [hi | lo | hi], role 2 (B) [lo | hi | hi],
 // so that segment g of A times segment g of B is the split's g-th product.
 __global__ void k_make_cat(const __nv_bfloat16 *__restrict__ hi,
-                           const __nv_bfloat16 *__restrict__ lo, int64_t rows, int kp, int role,
-                           __nv_bfloat16 *__restrict__ cat) {
+                           const __nv_bfloat16 *__restrict__ lo, int64_t rows, int kp, int ld,
+                           int ldc, int role, __nv_bfloat16 *__restrict__ cat) {
   const int64_t words = (int64_t)kp / 8;   // 16-byte words per segment
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= rows * 3 * words) return;
@@ -89,14 +90,15 @@ __global__ void k_make_cat(const __nv_bfloat16 *__restrict__ hi,
   const int g = (int)(w / words);
   const int64_t c = w - (int64_t)g * words;
   const bool from_lo = role == 1 ? g == 1 : g == 0;
-  const uint4 *src = (const uint4 *)((from_lo ? lo : hi) + r * kp) + c;
-  ((uint4 *)(cat + r * 3 * kp))[w] = *src;
+  const uint4 *src = (const uint4 *)((from_lo ? lo : hi) + r * ld) + c;
+  ((uint4 *)(cat + r * ldc))[w] = *src;
 }
 
 rkr_status tc_make_cat(TcSide &s, int role, cudaStream_t st) {
   if (s.cat || s.rows <= 0 || split_chunks_cat(s.kp) >= split_chunks_segmented(s.kp))
     return RKR_OK;
-  const size_t bytes = (size_t)s.rows * 3 * s.kp * 2;
+  const int ldc = tc_pitch(3 * s.kp);
+  const size_t bytes = (size_t)s.rows * ldc * 2;
   cudaError_t e = pool_malloc_async((void **)&s.cat, bytes, st);
   if (e != cudaSuccess) {   // the segmented form still works: go on without
     cudaGetLastError();
@@ -105,8 +107,8 @@ rkr_status tc_make_cat(TcSide &s, int role, cudaStream_t st) {
   }
   s.cat_role = role;
   const int64_t total = s.rows * 3 * (s.kp / 8);
-  k_make_cat<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(s.hi, s.lo, s.rows, s.kp, role,
-                                                              s.cat);
+  k_make_cat<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(s.hi, s.lo, s.rows, s.kp, s.ld(),
+                                                              ldc, role, s.cat);
   note_launch();
   RKR_CUDA(cudaGetLastError());
   return RKR_OK;
@@ -187,14 +189,14 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-rkr_status make_map(CUtensorMap *map, const __nv_bfloat16 *base, int64_t rows, int kp,
+rkr_status make_map(CUtensorMap *map, const __nv_bfloat16 *base, int64_t rows, int kp, int ld,
                     int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return fail(RKR_ECUDA, "cuTensorMapEncodeTiled is not available");
-  if (((uintptr_t)base & 15) != 0 || (kp * 2) % 16 != 0)
+  if (((uintptr_t)base & 15) != 0 || (ld * 2) % 16 != 0)
     return fail(RKR_EINTERNAL, "tensor map base or pitch not 16-byte aligned");
   cuuint64_t dims[2] = {(cuuint64_t)kp, (cuuint64_t)std::max<int64_t>(rows, 1)};
-  cuuint64_t strides[1] = {(cuuint64_t)kp * 2};
+  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
   cuuint32_t box[2] = {(cuuint32_t)tc::KCH, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)base, dims, strides, box,
@@ -538,10 +540,10 @@ extern "C" rkr_status rkr_screen_scores_static(const float *U, int64_t n, const 
   // the error word is the only scratch that must start at zero; everything else
   // is written in full before it is read
   RKR_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-  k_stage_bf16<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(U, n, d, kp, A.hi, A.lo, A.rb1,
+  k_stage_bf16<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(U, n, d, kp, kp, A.hi, A.lo, A.rb1,
                                                             A.rb3);
   note_launch();
-  k_stage_bf16<<<(unsigned)((mx + 127) / 128), 128, 0, st>>>(X, mx, d, kp, B.hi, B.lo, B.rb1,
+  k_stage_bf16<<<(unsigned)((mx + 127) / 128), 128, 0, st>>>(X, mx, d, kp, kp, B.hi, B.lo, B.rb1,
                                                              B.rb3);
   note_launch();
   k_tile_bounds<<<(unsigned)((ntiles + 127) / 128), 128, 0, st>>>(split ? B.rb3 : B.rb1, mx, BN,

@@ -1920,7 +1920,7 @@ __global__ void k_rc_refine(const int2 *__restrict__ items, const unsigned long 
 __global__ void k_gather_side(const __nv_bfloat16 *__restrict__ hi,
                               const __nv_bfloat16 *__restrict__ lo,
                               const tc::RowBound *__restrict__ rb1,
-                              const tc::RowBound *__restrict__ rb3, int kp,
+                              const tc::RowBound *__restrict__ rb3, int kp, int ld,
                               const int32_t *__restrict__ rows, int64_t count,
                               __nv_bfloat16 *__restrict__ ohi, __nv_bfloat16 *__restrict__ olo,
                               tc::RowBound *__restrict__ orb1, tc::RowBound *__restrict__ orb3) {
@@ -1928,8 +1928,8 @@ __global__ void k_gather_side(const __nv_bfloat16 *__restrict__ hi,
   if (i >= count) return;
   int64_t src = rows[i];
   for (int k = threadIdx.x; k < kp; k += blockDim.x) {
-    ohi[i * kp + k] = hi[src * kp + k];
-    olo[i * kp + k] = lo[src * kp + k];
+    ohi[i * ld + k] = hi[src * ld + k];
+    olo[i * ld + k] = lo[src * ld + k];
   }
   if (threadIdx.x == 0) {
     orb1[i] = rb1[src];
@@ -1994,8 +1994,9 @@ static rkr_status tc_recount_bn(const rkr_index *idx, const TcSide &Ut, const Tc
   A.rows = nseg;
   A.d = Ut.d;
   A.kp = Ut.kp;
+  A.pitch = Ut.pitch;
   A.owned = false;
-  size_t cnt = (size_t)nseg * A.kp;
+  size_t cnt = (size_t)nseg * A.ld();
   RKR_CUDA(pool_malloc_async((void **)&A.hi, cnt * 2, st));
   RKR_CUDA(pool_malloc_async((void **)&A.lo, cnt * 2, st));
   RKR_CUDA(pool_malloc_async((void **)&A.rb1, sizeof(tc::RowBound) * nseg, st));
@@ -2003,7 +2004,7 @@ static rkr_status tc_recount_bn(const rkr_index *idx, const TcSide &Ut, const Tc
   dim3 blk(32, 8);
   {
     const int prof_slot = prof_begin("k_gather_side", st);
-    k_gather_side<<<(unsigned)((nseg + 7) / 8), blk, 0, st>>>(Ut.hi, Ut.lo, Ut.rb1, Ut.rb3, A.kp,
+    k_gather_side<<<(unsigned)((nseg + 7) / 8), blk, 0, st>>>(Ut.hi, Ut.lo, Ut.rb1, Ut.rb3, A.kp, A.ld(),
                                                                seg_user, nseg, A.hi, A.lo, A.rb1,
                                                                A.rb3);
     prof_end(prof_slot, st, 0.0);

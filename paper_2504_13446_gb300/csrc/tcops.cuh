@@ -10,16 +10,25 @@
 
 namespace rkr {
 
-// One side of a screen: rows of bf16 hi and lo parts (row pitch kp, zero padded
-// beyond d), per-row bound terms for single and split products, and TMA maps.
+// Row pitch (elements) of a staged operand of `width` bf16 columns.  A TMA box
+// reads 128 bytes of each row: with a pitch that is no multiple of 128 bytes
+// almost every such piece straddles two cache lines.
+inline int tc_pitch(int width) {
+  return width == 16 || width == 32 ? width : (width + tc::KCH - 1) / tc::KCH * tc::KCH;
+}
+
+// One side of a screen: rows of bf16 hi and lo parts (kp columns, zero padded
+// beyond d, at row pitch ld()), per-row bound terms for single and split products.
 struct TcSide {
   int64_t rows = 0;
   int d = 0, kp = 0;
+  int pitch = 0;                 // row pitch of hi and lo in elements; 0 = kp
+  int ld() const { return pitch ? pitch : kp; }
   __nv_bfloat16 *hi = nullptr, *lo = nullptr;
   tc::RowBound *rb1 = nullptr;   // single product terms
   tc::RowBound *rb3 = nullptr;   // split product terms
-  // Split operand with the three products' K ranges side by side (row pitch
-  // 3 kp): [hi | lo | hi] for A (cat_role 1), [lo | hi | hi] for B (cat_role 2).
+  // Split operand with the three products' K ranges side by side (3 kp columns
+  // at row pitch tc_pitch(3 kp)): [hi | lo | hi] for A (cat_role 1), [lo | hi | hi] for B (cat_role 2).
   // One pass over K = 3 kp issues the split's MMAs in the same order on the same
   // slices, so the scores are bit-identical, in fewer pipeline stages when kp is
   // not a multiple of 64 (d = 200: 10 stages per tile instead of 12).
@@ -45,8 +54,9 @@ rkr_status tc_tile_bounds(const TcSide &b, int bn, int split, tc::RowBound **out
 // Number of SMs of the current device.
 int sm_count();
 
-// Encode a 2-D bf16 tensor map over rows x kp with boxes of 64 x box_rows.
-rkr_status make_map(CUtensorMap *map, const __nv_bfloat16 *base, int64_t rows, int kp,
+// Encode a 2-D bf16 tensor map over rows x kp (row pitch ld) with boxes of
+// 64 x box_rows.
+rkr_status make_map(CUtensorMap *map, const __nv_bfloat16 *base, int64_t rows, int kp, int ld,
                     int box_rows);
 
 // Rounds of the screens' epilogue accumulator wait before it gives up (a test
@@ -101,11 +111,12 @@ rkr_status launch_screen(const TcSide &A, const TcSide &B, int split, const tc::
   const __nv_bfloat16 *ah = cat ? A.cat : A.hi, *al = cat ? A.cat : A.lo;
   const __nv_bfloat16 *bh = cat ? B.cat : B.hi, *bl = cat ? B.cat : B.lo;
   const int kw = cat ? 3 * A.kp : A.kp;
+  const int lda = cat ? tc_pitch(kw) : A.ld(), ldb = cat ? tc_pitch(kw) : B.ld();
   CUtensorMap mAh, mAl, mBh, mBl;
-  RKR_TRY(make_map(&mAh, ah, A.rows, kw, tc::BM));
-  RKR_TRY(make_map(&mAl, al, A.rows, kw, tc::BM));
-  RKR_TRY(make_map(&mBh, bh, B.rows, kw, BN));
-  RKR_TRY(make_map(&mBl, bl, B.rows, kw, BN));
+  RKR_TRY(make_map(&mAh, ah, A.rows, kw, lda, tc::BM));
+  RKR_TRY(make_map(&mAl, al, A.rows, kw, lda, tc::BM));
+  RKR_TRY(make_map(&mBh, bh, B.rows, kw, ldb, BN));
+  RKR_TRY(make_map(&mBl, bl, B.rows, kw, ldb, BN));
   tc::Operands op;
   op.nrows = A.rows;
   op.ncols = B.rows;
@@ -128,8 +139,8 @@ rkr_status launch_screen(const TcSide &A, const TcSide &B, int split, const tc::
     auto pk = tc::k_screen_2sm<BN, S2, Epi>;
     RKR_CUDA(cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
     CUtensorMap mBh2, mBl2;
-    RKR_TRY(make_map(&mBh2, bh, B.rows, kw, BN / 2));
-    RKR_TRY(make_map(&mBl2, bl, B.rows, kw, BN / 2));
+    RKR_TRY(make_map(&mBh2, bh, B.rows, kw, ldb, BN / 2));
+    RKR_TRY(make_map(&mBl2, bl, B.rows, kw, ldb, BN / 2));
     if (launch_cluster_pairs(pk, smem2, sch, st, mAh, mAl, mBh2, mBl2, op, epi, err_dev))
       return RKR_OK;
     RKR_CUDA(cudaGetLastError());
@@ -139,8 +150,8 @@ rkr_status launch_screen(const TcSide &A, const TcSide &B, int split, const tc::
     auto pk = tc::k_screen_pair<BN, STAGES, Epi>;
     RKR_CUDA(cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     CUtensorMap mBh2, mBl2;
-    RKR_TRY(make_map(&mBh2, bh, B.rows, kw, BN / 2));
-    RKR_TRY(make_map(&mBl2, bl, B.rows, kw, BN / 2));
+    RKR_TRY(make_map(&mBh2, bh, B.rows, kw, ldb, BN / 2));
+    RKR_TRY(make_map(&mBl2, bl, B.rows, kw, ldb, BN / 2));
     if (launch_cluster_pairs(pk, smem, sch, st, mAh, mAl, mBh2, mBl2, op, epi, err_dev))
       return RKR_OK;
     RKR_CUDA(cudaGetLastError());
