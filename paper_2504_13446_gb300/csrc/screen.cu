@@ -421,7 +421,7 @@ rkr_status tc_scores_e4m3(const float *U, int64_t n, const float *X, int64_t mx,
     const int grid = std::min(sch.nunits, sm_count());
     if (s == RKR_OK && grid > 0) {
       ProfScope prof(EpiStore8::name(), st, 2.0 * (double)n * (double)mx * (double)kp);
-      kern<<<grid, tc::kThreads, smem, st>>>(mA, mA, mB, mB, op, sch, e, err);
+      kern<<<grid, tc::screen_threads<EpiStore8>(), smem, st>>>(mA, mA, mB, mB, op, sch, e, err);
       note_launch();
       ce = cudaGetLastError();
       if (ce != cudaSuccess) s = cuda_fail(ce, "FP8 screen launch");

@@ -107,6 +107,8 @@ struct PairQueue {
 // thread at near-final extremes, so few items are queued.
 struct EpiFb {
   static const char *name() { return "k_screen<EpiFb>"; }
+  static constexpr int kWarps = 8;   // 30.0 ms at 1M x 100k x 200 (16 warps: 31.2)
+  static constexpr int kGroups = kWarps / 4;   // threads of a row
   struct Thread {
     float b, mxlo, mnhi;
     int64_t row;
@@ -120,8 +122,9 @@ struct EpiFb {
   tc::Gacc gacc;
   float gcan;
   PairQueue q;
-  const float2 *seed;   // per row: (largest lower end, smallest upper end) to start from, or null
-  float2 *seed_out;     // seeding launch: per (row, column half) extremes, no queue
+  // per (row, column group): (largest lower end, smallest upper end) to start from, or null
+  const float2 *seed;
+  float2 *seed_out;     // seeding launch: these extremes are written, nothing is queued
   __device__ __forceinline__ void unit_begin(char *, const tc::Unit &u, int et,
                                              Thread &ts) const {
     ts.mxlo = -INFINITY;
@@ -132,9 +135,12 @@ struct EpiFb {
       const int w = (et >> 5) + 2, lane = et & 31;
       const int64_t row = (int64_t)u.rb0 * tc::BM + (w & 3) * 32 + lane;
       if (row < nrows) {
-        const float2 a = seed[2 * row], b = seed[2 * row + 1];
-        ts.mxlo = fmaxf(a.x, b.x);
-        ts.mnhi = fminf(a.y, b.y);
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) {
+          const float2 a = seed[kGroups * row + g];
+          ts.mxlo = fmaxf(ts.mxlo, a.x);
+          ts.mnhi = fminf(ts.mnhi, a.y);
+        }
       }
     }
   }
@@ -220,7 +226,7 @@ struct EpiFb {
     if (!seed_out) return;
     const int w = (et >> 5) + 2, lane = et & 31;
     const int64_t row = (int64_t)u.rb0 * tc::BM + (w & 3) * 32 + lane;
-    if (row < nrows) seed_out[2 * row + ((et >> 5) >> 2)] = make_float2(ts.mxlo, ts.mnhi);
+    if (row < nrows) seed_out[kGroups * row + (et >> 7)] = make_float2(ts.mxlo, ts.mnhi);
   }
 };
 
@@ -320,7 +326,7 @@ rkr_status tc_fbounds(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt, 
   a.q = PairQueue{qitems, qcount, cap, flags + 1};
   // seeding launch over the first columns (the largest norms), then the full pass
   float2 *seed;
-  RKR_CUDA(pool_malloc_async(&seed, sizeof(float2) * 2 * n, st));
+  RKR_CUDA(pool_malloc_async(&seed, sizeof(float2) * EpiFb::kGroups * n, st));
   TcSide head = Pt;
   head.owned = false;
   head.rows = std::min<int64_t>(m, 4 * BN);
@@ -391,6 +397,7 @@ __global__ void k_xgrid(int64_t n, const double *__restrict__ fmin,
 // more than 65535 items gets the trivial bounds 0 and m instead.
 struct EpiXT {
   static const char *name() { return "k_screen<EpiXT>"; }
+  static constexpr int kWarps = 8;   // 98 ms at 1M x 100k x 200 (16 warps: 102)
   struct Thread {
     float skip, b, g0;
     int64_t row;
@@ -402,7 +409,7 @@ struct EpiXT {
   // list cursors of the block's 128 rows, then a 32 x 32 staging tile per warp
   // stored [column][lane] (a lane's lookups hit its own bank)
   static constexpr size_t kStageOff = sizeof(uint32_t) * 128;
-  static constexpr size_t kSmem = kStageOff + sizeof(float) * 8 * 32 * 32;
+  static constexpr size_t kSmem = kStageOff + sizeof(float) * kWarps * 32 * 32;
   int64_t nrows, ncols;
   int bn;
   const tc::RowBound *rowb, *tileb;
@@ -463,7 +470,7 @@ struct EpiXT {
   }
   __device__ void tile_end(char *, int, int, int, int, Thread &) const {}
   __device__ void unit_end(char *S, const tc::Unit &u, int et, Thread &) const {
-    tc::epi_sync();
+    tc::epi_sync<kWarps>();
     if (et >= 128) return;
     const int64_t g = (int64_t)u.rb0 * tc::BM + et;
     if (g < nrows) lcnt[g] = lslot(S)[et];
@@ -806,6 +813,7 @@ rkr_status tc_exact_table(rkr_index *idx, const TcSide &Ut, const TcSide &Pt, cu
 // stored [bin][row] so that a warp's 32 rows never share a bank.
 struct EpiDeep {
   static const char *name() { return "k_screen<EpiDeep>"; }
+  static constexpr int kWarps = 16;
   static constexpr int kBins = kDGrid + 1;
   struct Thread {
     float b, top_lo;     // bound; lower ends above top_lo are above the whole grid
@@ -818,7 +826,7 @@ struct EpiDeep {
   };
   static constexpr size_t kHist = sizeof(uint32_t) * 128 * kBins;   // one of Hlo, Hhi
   static constexpr size_t kStageOff = 2 * kHist;
-  static constexpr size_t kSmem = kStageOff + sizeof(float) * 8 * 32 * 32;
+  static constexpr size_t kSmem = kStageOff + sizeof(float) * kWarps * 16 * 32;
   int64_t nrows, ncols;
   int bn;
   const tc::RowBound *rowb, *tileb;
@@ -832,7 +840,7 @@ struct EpiDeep {
   __device__ static uint32_t *hlo(char *S, int r) { return (uint32_t *)S + r; }
   __device__ static uint32_t *hhi(char *S, int r) { return (uint32_t *)(S + kHist) + r; }
   __device__ void unit_begin(char *S, const tc::Unit &u, int et, Thread &ts) const {
-    for (int i = et; i < 2 * 128 * kBins; i += 256) ((uint32_t *)S)[i] = 0u;
+    for (int i = et; i < 2 * 128 * kBins; i += 32 * kWarps) ((uint32_t *)S)[i] = 0u;
     ts.row = -1;
     ts.tp.start(tileb, u.ct0);
   }
@@ -854,18 +862,21 @@ struct EpiDeep {
     if (ts.row >= nrows) return;
     const int64_t c0 = (int64_t)ct * bn + col;
     const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) - 2;
-    float *tile = (float *)(S + kStageOff) + warp * 32 * 32 + lane;
+    float *tile = (float *)(S + kStageOff) + warp * 16 * 32 + lane;
     // scores whose upper end reaches the grid's first point (the others count nowhere)
-#pragma unroll
-    for (int j = 0; j < 32; ++j) tile[j * 32] = v[j];
     uint32_t mask = bitmask32([&](int j) { return __fadd_ru(v[j], ts.b) >= ts.bot_hi; });
     const int64_t left = ncols - c0;
     if (left < 32) mask &= left <= 0 ? 0u : (1u << left) - 1u;
     const BinFP &bf = ts.bf;
     const bool fast = bf.invd32 > 0.0f && bf.err <= 1e6f;   // the row's grid has a step
-    while (mask) {
-      const int j = __ffs(mask) - 1;
-      mask &= mask - 1;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) tile[j * 32] = v[16 * h + j];
+    uint32_t mine = h ? mask >> 16 : mask & 0xffffu;
+    while (mine) {
+      const int j = __ffs(mine) - 1;
+      mine &= mine - 1;
       const float x = tile[j * 32];
       const float lo = __fsub_rd(x, ts.b), hi = __fadd_ru(x, ts.b);
       int jl, jh;
@@ -888,13 +899,14 @@ struct EpiDeep {
       atomicAdd(&hlo(S, r)[jl * 128], 1u);
       atomicAdd(&hhi(S, r)[jh * 128], 1u);
     }
+    }
   }
   __device__ void tile_end(char *, int, int, int, int, Thread &) const {}
   __device__ void unit_end(char *S, const tc::Unit &u, int et, Thread &ts) const {
     const int w = (et >> 5) + 2, lane = et & 31;
     const int r = (w & 3) * 32 + lane, half = et >> 7;
     const int64_t row = (int64_t)u.rb0 * tc::BM + r;
-    tc::epi_sync();
+    tc::epi_sync<kWarps>();
     if (row >= nrows || half != 0) return;
     // DLO[c] = sum over bins above c
     uint32_t rl = 0, rh = 0;
@@ -974,6 +986,7 @@ struct EpiTheta {
     bool have_pf;
   };
   static constexpr bool kReloads = true;   // chunk() reads accumulator columns again
+  static constexpr int kWarps = 8;
   static constexpr size_t kSmem = sizeof(int16_t) * 2 * 128 * kJS +
                                   sizeof(int) * (2 * kThetaBN * 32 + 3 * kThetaBN) +
                                   sizeof(tc::RowBound) * kThetaBN;
@@ -1061,7 +1074,7 @@ struct EpiTheta {
       fetch(rb, et, ts);
       fetch_row(rb, r, ts);
     }
-    tc::epi_sync();  // readers of the previous tile are done with the level tables
+    tc::epi_sync<kWarps>();  // readers of the previous tile are done with the level tables
     // scatter the 32 words this thread holds into padded rows
     int16_t *J = jtab(S);
     for (int t2 = 0; t2 < 2; ++t2) {
@@ -1082,7 +1095,7 @@ struct EpiTheta {
       ts.fm = ts.pfm;
       ts.xsb = __fsub_rd(ts.pxs, ts.b);
     }
-    tc::epi_sync();
+    tc::epi_sync<kWarps>();
     // prefetch the next row block of this unit while this tile is processed
     ts.have_pf = rb + 1 < ts.rb1;
     if (ts.have_pf) {
@@ -1250,6 +1263,7 @@ rkr_status tc_theta_pass(int pass, const rkr_index *idx, const TcSide &Ut, const
 // pairs are queued for the canonical FP64 evaluation.
 struct EpiTable {
   static const char *name() { return "k_screen<EpiTable>"; }
+  static constexpr int kWarps = 16;
   struct Thread {
     int64_t u;
     tc::RowBound ru;
@@ -1309,7 +1323,7 @@ struct EpiTable {
 // and fewer than 2^16 sampled rows.
 struct EpiTableSm {
   static const char *name() { return "k_screen<EpiTable>"; }
-  static constexpr bool kResident = true;
+  static constexpr int kWarps = 16;
   static constexpr int kBinWords = 256;   // 512 16-bit counters per user
   struct Thread {
     int64_t u;
@@ -1330,7 +1344,7 @@ struct EpiTableSm {
   PairQueue q;
   __device__ void unit_begin(char *S, const tc::Unit &, int et, Thread &ts) const {
     uint32_t *H = (uint32_t *)S;
-    for (int i = et; i < tc::BM * kBinWords; i += 256) H[i] = 0u;
+    for (int i = et; i < tc::BM * kBinWords; i += 32 * kWarps) H[i] = 0u;
     ts.u = -1;
   }
   __device__ __forceinline__ void tile_begin(char *, int rb, int, int r, int, Thread &ts) const {
@@ -1364,7 +1378,7 @@ struct EpiTableSm {
     const uint32_t *H = (const uint32_t *)S;
     const int bins = tau + 1;
     const int64_t row0 = (int64_t)u.rb0 * tc::BM;
-    for (int i = et; i < tc::BM * bins; i += 256) {
+    for (int i = et; i < tc::BM * bins; i += 32 * kWarps) {
       const int r = i / bins, c = i - r * bins;
       if (row0 + r >= nrows) continue;
       const uint32_t cnt = (H[r * kBinWords + (c >> 1)] >> ((c & 1) * 16)) & 0xffffu;
@@ -1520,14 +1534,15 @@ constexpr int kSkimBN = 256;
 
 struct EpiSkim {
   static const char *name() { return "k_screen<EpiSkim>"; }
+  static constexpr int kWarps = 16;
   struct Thread {
     float b, xsb, pxs;
     int64_t u, fu;      // current row; row whose terms prb, pxs hold
     tc::RowBound prb;
   };
-  // a 32 x 32 staging tile per epilogue warp, stored [column][lane]: a lane reads
+  // a 16 x 32 staging tile per epilogue warp, stored [column][lane]: a lane reads
   // back its own emitted scores from shared memory, not from TMEM
-  static constexpr size_t kSmem = sizeof(float) * 8 * 32 * 32;
+  static constexpr size_t kSmem = sizeof(float) * kWarps * 16 * 32;
   int64_t nrows, ncols;
   const tc::RowBound *rowb, *tileb;
   tc::Gacc gacc;
@@ -1574,19 +1589,22 @@ struct EpiSkim {
     int64_t pos = (int64_t)base + incl - n;
     const int64_t rbase = (int64_t)blockIdx.x * L.rcap;
     // each lane walks its own emitted columns, in column order
-    float *tile = (float *)S + ((threadIdx.x >> 5) - 2) * 32 * 32 + lane;
+    float *tile = (float *)S + ((threadIdx.x >> 5) - 2) * 16 * 32 + lane;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) tile[j * 32] = v[j];
-    uint32_t mine = pm;
-    while (mine) {
-      const int j = __ffs(mine) - 1;
-      mine &= mine - 1u;
-      if (pos < L.rcap) {  // entries past the region are dropped; cnt records them
-        L.u[rbase + pos] = (int32_t)ts.u;
-        L.q[rbase + pos] = (int32_t)(c0 + j);
-        L.x[rbase + pos] = tile[j * 32];
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) tile[j * 32] = v[16 * h + j];
+      uint32_t mine = h ? pm >> 16 : pm & 0xffffu;
+      while (mine) {
+        const int j = __ffs(mine) - 1;
+        mine &= mine - 1u;
+        if (pos < L.rcap) {  // entries past the region are dropped; cnt records them
+          L.u[rbase + pos] = (int32_t)ts.u;
+          L.q[rbase + pos] = (int32_t)(c0 + 16 * h + j);
+          L.x[rbase + pos] = tile[j * 32];
+        }
+        ++pos;
       }
-      ++pos;
     }
   }
   __device__ void tile_end(char *, int, int, int, int, Thread &) const {}
@@ -1627,12 +1645,31 @@ rkr_status tc_skim(const rkr_index *idx, const TcSide &Ut, const TcSide &Qt, con
 
 // =============================================================== recount
 
+// Thresholds on a screened score v with bound b against u.q in [tdn, tup]
+// (consecutive floats or equal): for every float v,
+//   v >= thi  <=>  v - b rounded down > tup   (the score's lower end is above u.q)
+//   v >  tlo  <=>  v + b rounded up   > tdn   (its upper end is above u.q)
+// since a float exceeds tup exactly when it is at least the next float after tup,
+// and a rounding towards a float never passes it.  thi is NaN (never reached) when
+// no finite score's lower end can exceed tup.
+__host__ __device__ __forceinline__ float next_up(float x) { return nextafterf(x, INFINITY); }
+__device__ __forceinline__ void rc_thresholds(float tdn, float tup, float b, float &tlo,
+                                              float &thi) {
+  const float hi = __fadd_ru(next_up(tup), b);
+  thi = hi < INFINITY ? hi : __int_as_float(0x7fffffff);
+  tlo = __fsub_rd(tdn, b);
+}
+
 struct EpiRC {
   static const char *name() { return "k_screen<EpiRC>"; }
+  static constexpr int kWarps = 16;
   // One threshold per row (segments of one candidate): an item is certainly above
   // u.q when its lower end exceeds u.q, possibly above when its upper end does.
+  // Both ends are compared through the tile's thresholds on the screened score
+  // itself (tile_begin), one compare and one predicated add each.
   struct Thread {
-    float b, tdn, tup;           // bound; u.q rounded down / up to float
+    float tdn, tup;              // u.q rounded down / up to float
+    float tlo, thi;              // possibly above: score > tlo; certainly: score >= thi
     int64_t sg;
     int64_t self;                // item tying exactly with u.q (never above), or -1
     uint32_t *h, *hh;
@@ -1680,20 +1717,33 @@ struct EpiRC {
   }
   __device__ __forceinline__ void tile_begin(char *, int, int ct, int, int, Thread &ts) const {
     const tc::RowBound tb = ts.tp.take(tileb, ct, ncols, bn);
-    ts.b = ts.sg < nseg ? tc::screen_bound_tc(ts.ru, tb, gacc, gcan) : 0.0f;
+    const float b = ts.sg < nseg ? tc::screen_bound_tc(ts.ru, tb, gacc, gcan) : 0.0f;
+    rc_thresholds(ts.tdn, ts.tup, b, ts.tlo, ts.thi);
   }
   __device__ __forceinline__ void chunk(char *, int, int ct, int, int col, uint32_t,
                                         const float (&v)[32], Thread &ts) const {
     const int64_t c0 = (int64_t)ct * bn + col;
-    uint32_t mlo = bitmask32([&](int j) { return __fsub_rd(v[j], ts.b) > ts.tup; });
-    uint32_t mhi = bitmask32([&](int j) { return __fadd_ru(v[j], ts.b) > ts.tdn; });
     const int64_t left = ncols - c0;
+    const bool self = ts.self >= c0 && ts.self < c0 + 32;
+    if (hist_hi && left >= 32 && !self) {   // only the two counts are wanted
+      uint32_t lo[2] = {0, 0}, hi[2] = {0, 0};
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        lo[j & 1] += v[j] >= ts.thi;
+        hi[j & 1] += v[j] > ts.tlo;
+      }
+      ts.clo += lo[0] + lo[1];
+      ts.chi += hi[0] + hi[1];
+      return;
+    }
+    uint32_t mlo = bitmask32([&](int j) { return v[j] >= ts.thi; });
+    uint32_t mhi = bitmask32([&](int j) { return v[j] > ts.tlo; });
     if (left < 32) {
       const uint32_t keep = left <= 0 ? 0u : (1u << left) - 1u;
       mlo &= keep;
       mhi &= keep;
     }
-    if (ts.self >= c0 && ts.self < c0 + 32) mhi &= ~(1u << (int)(ts.self - c0));
+    if (self) mhi &= ~(1u << (int)(ts.self - c0));
     ts.clo += __popc(mlo);
     ts.chi += __popc(mhi);
     if (!hist_hi) {
@@ -1726,6 +1776,7 @@ struct EpiRC {
 // is that threshold) has a known position and is counted there.
 struct EpiRCm {
   static const char *name() { return "k_screen<EpiRCm>"; }
+  static constexpr int kWarps = 8;
   static constexpr int kL = kRecountSeg;
   struct Thread {
     float b, t0, tl;     // bound; lowest threshold rounded down, highest rounded up
@@ -1861,7 +1912,7 @@ struct EpiRCm {
       atomicAdd(&hlo(S, r)[ts.L * 128], ts.top);
       if (hist_hi) atomicAdd(&hhi(S, r)[ts.L * 128], ts.top);
     }
-    tc::epi_sync();
+    tc::epi_sync<kWarps>();
     if (ts.L == 0 || half != 0) return;
     // position 0 (above no threshold) is never read
     uint32_t *h = hist + 2 * ts.st0, *hh = hist_hi ? hist_hi + 2 * ts.st0 : nullptr;

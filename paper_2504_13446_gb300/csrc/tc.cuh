@@ -10,9 +10,9 @@
 // Warp roles (one CTA per SM, persistent):
 //   warp 0      TMA producer (one lane)
 //   warp 1      TMEM allocation and MMA issue (one lane)
-//   warps 2..9  epilogue: warp w reads TMEM lanes 32*(w%4) .. +31 and half
-//               (w-2)/4 of the columns, so each accumulator row (user) is
-//               handled by two threads
+//   warps 2..   epilogue, 8 or 16 warps (epi_warps): warp w reads TMEM lanes
+//               32*(w%4) .. +31 and column group (w-2)/4, so each accumulator
+//               row (user) is handled by two or four threads
 // All waits are bounded; a timeout sets an error word, drains what is in
 // flight and returns.
 #pragma once
@@ -29,8 +29,28 @@ namespace tc {
 
 constexpr int BM = 128;
 constexpr int KCH = 64;               // bf16 elements per K chunk (128 bytes)
-constexpr int kEpiWarps = 8;
-constexpr int kThreads = 32 * (2 + kEpiWarps);
+
+// Epilogue warps of a screen: Epi::kWarps, 8 unless the epilogue says 16.  An
+// epilogue whose time is latency (TMEM loads, shared and global round trips of the
+// scores it keeps) gains from four warps per scheduler; 16 warps leave 112
+// registers a thread, so one that needs more keeps 8.
+template <class Epi, class = void>
+struct EpiWarps {
+  static constexpr int value = 8;
+};
+template <class Epi>
+struct EpiWarps<Epi, decltype((void)Epi::kWarps)> {
+  static constexpr int value = Epi::kWarps;
+};
+template <class Epi>
+constexpr int epi_warps() {
+  static_assert(EpiWarps<Epi>::value == 8 || EpiWarps<Epi>::value == 16, "8 or 16 warps");
+  return EpiWarps<Epi>::value;
+}
+template <class Epi>
+constexpr int screen_threads() {
+  return 32 * (2 + epi_warps<Epi>());
+}
 constexpr uint32_t kWaitLimit = 1u << 22;   // try_wait rounds before giving up
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {

@@ -65,7 +65,7 @@ __device__ __forceinline__ void cluster_sync() {
 // (loads the peer issued just before it stopped included), and a second
 // cluster barrier keeps either CTA from leaving while the other still waits.
 template <int BN, int STAGES, class Epi>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(screen_threads<Epi>(), 1)
     k_screen_pair(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                   const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
                   Operands op, Schedule sch, Epi epi, int *err) {
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], kEpiWarps);
+      mbar_init(&acc_empty[b], epi_warps<Epi>());
     }
     mbar_init(drain, 1);
     fence_barrier_init();
@@ -184,10 +184,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else {
     // ----------------------------------------------------------- epilogue
+    constexpr int EW = epi_warps<Epi>();
     const int e = warp - 2;
     const int et = threadIdx.x - 64;
     const int quarter = warp & 3;
-    const int half = e >> 2;
+    const int group = e >> 2;   // column group
     const int r = quarter * 32 + lane;
     uint32_t t = 0;
     typename Epi::Thread ts;
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       Unit u;
       u.rb0 = rb; u.rb1 = rb + 1; u.ct0 = 0; u.ct1 = sch.nct;
       if (real) epi.unit_begin(escratch, u, et, ts);
-      epi_sync();
+      epi_sync<EW>();
       for (int ct = 0; ct < sch.nct; ++ct, ++t) {
         const int b = t & 1;
         const uint32_t aph = (t >> 1) & 1;
@@ -209,18 +210,18 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (lane == 0) mbar_arrive(&acc_empty[b]);
         };
         if (real) {
-          epi.tile_begin(escratch, rb, ct, r, half, ts);
+          epi.tile_begin(escratch, rb, ct, r, group, ts);
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN);
           if (!failed)
-            epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts, release);
-          epi.tile_end(escratch, rb, ct, r, half, ts);
+            epi_tile_columns<BN>(epi, escratch, rb, ct, r, group, trow, ts, release);
+          epi.tile_end(escratch, rb, ct, r, group, ts);
         } else if (!failed) {
           release();
         }
       }
-      failed = epi_vote_any(failed);
+      failed = epi_vote_any<EW>(failed);
       if (!failed && real) epi.unit_end(escratch, u, et, ts);
-      epi_sync();
+      epi_sync<EW>();
     }
     if (failed && lane == 0) {
       atomicExch(err, 3);
@@ -341,7 +342,7 @@ constexpr size_t screen2_smem_bytes() {
 // producer waits again for the stages still in flight, and a second cluster
 // barrier keeps either CTA from leaving while the other still waits.
 template <int BN, int STAGES, class Epi>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(screen_threads<Epi>(), 1)
     k_screen_2sm(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                  const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
                  Operands op, Schedule sch, Epi epi, int *err) {
@@ -374,7 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 2 * kEpiWarps);
+      mbar_init(&acc_empty[b], 2 * epi_warps<Epi>());
     }
     mbar_init(drain, 1);
     fence_barrier_init();
@@ -460,10 +461,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // ----------------------------------------------------------- epilogue
+    constexpr int EW = epi_warps<Epi>();
     const int e = warp - 2;
     const int et = threadIdx.x - 64;
     const int quarter = warp & 3;
-    const int half = e >> 2;
+    const int group = e >> 2;   // column group
     const int r = quarter * 32 + lane;
     const uint32_t ae0 = map_to_rank(smem_u32(acc_empty), 0);
     uint32_t t = 0;
@@ -474,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       Unit u;
       u.rb0 = rb; u.rb1 = rb + 1; u.ct0 = 0; u.ct1 = sch.nct;
       if (real) epi.unit_begin(escratch, u, et, ts);
-      epi_sync();
+      epi_sync<EW>();
       for (int ct = 0; ct < sch.nct; ++ct, ++t) {
         const int b = t & 1;
         const uint32_t aph = (t >> 1) & 1;
@@ -486,18 +488,18 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (lane == 0) mbar_arrive_cluster(ae0 + (uint32_t)(b * sizeof(uint64_t)));
         };
         if (real) {
-          epi.tile_begin(escratch, rb, ct, r, half, ts);
+          epi.tile_begin(escratch, rb, ct, r, group, ts);
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN);
           if (!failed)
-            epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts, release);
-          epi.tile_end(escratch, rb, ct, r, half, ts);
+            epi_tile_columns<BN>(epi, escratch, rb, ct, r, group, trow, ts, release);
+          epi.tile_end(escratch, rb, ct, r, group, ts);
         } else if (!failed) {
           release();
         }
       }
-      failed = epi_vote_any(failed);
+      failed = epi_vote_any<EW>(failed);
       if (!failed && real) epi.unit_end(escratch, u, et, ts);
-      epi_sync();
+      epi_sync<EW>();
     }
     if (failed && lane == 0) {
       atomicExch(err, 3);

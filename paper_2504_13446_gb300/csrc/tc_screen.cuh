@@ -6,17 +6,19 @@
 // epilogue state in the CTA; column-owned units (one column tile, a range of
 // row blocks) keep per-column state.
 //
-// Epi must provide (all called by the 256 epilogue threads, const members):
+// Epi must provide (all called by the epilogue threads, 32 * epi_warps<Epi>() of
+// them, const members):
 //   struct Thread;                                    per-thread state
 //   static constexpr size_t kSmem;                    bytes of epilogue scratch
-//   void unit_begin(char *S, const Unit &u, int et, Thread &)   et = 0..255
+//   void unit_begin(char *S, const Unit &u, int et, Thread &)   et = 0..threads-1
 //   void tile_begin(char *S, int rb, int ct, int r, int h, Thread &)
 //   void chunk(char *S, int rb, int ct, int r, int col, uint32_t tm, const float (&v)[32], Thread &)
 //   void tile_end(char *S, int rb, int ct, int r, int h, Thread &)
 //   void unit_end(char *S, const Unit &u, int et, Thread &)
-// r is the accumulator row (0..127), h the column half, col the first of the
-// 32 columns of the chunk within the tile.  Named barrier 1 (256 threads) is
-// available to unit_begin/unit_end and tile_begin/tile_end as tc::epi_sync().
+// r is the accumulator row (0..127), h the column group, col the first of the
+// 32 columns of the chunk within the tile.  Named barrier 1 (the epilogue threads)
+// is available to unit_begin/unit_end and tile_begin/tile_end as tc::epi_sync<W>(),
+// W the epilogue's warps.
 #pragma once
 
 #include "tc.cuh"
@@ -50,19 +52,23 @@ __device__ __forceinline__ Unit unit_of(const Schedule &s, int i) {
   return u;
 }
 
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+template <int WARPS>
+__device__ __forceinline__ void epi_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * WARPS) : "memory");
+}
 
-// Barrier of the 256 epilogue threads that also ORs a predicate over them, so
+// Barrier of the epilogue threads that also ORs a predicate over them, so
 // that every epilogue warp takes the same decision at the end of a unit (a warp
 // that gave up a bounded wait and one that did not would otherwise disagree on
 // the number of barriers still to come).
+template <int WARPS>
 __device__ __forceinline__ bool epi_vote_any(bool p) {
   uint32_t r;
   asm volatile(
       "{\n .reg .pred a, b;\n setp.ne.u32 a, %1, 0;\n"
-      " barrier.red.or.pred b, 1, 256, a;\n selp.u32 %0, 1, 0, b;\n}\n"
+      " barrier.red.or.pred b, 1, %2, a;\n selp.u32 %0, 1, 0, b;\n}\n"
       : "=r"(r)
-      : "r"((uint32_t)p)
+      : "r"((uint32_t)p), "n"(32 * WARPS)
       : "memory");
   return r != 0;
 }
@@ -137,23 +143,36 @@ struct EpiReloads<Epi, decltype((void)Epi::kReloads)> {
   static constexpr bool value = Epi::kReloads;
 };
 
-// This thread's half row of an accumulator tile (TMEM row address trow): 64
-// columns per TMEM load (one wait), handed to the epilogue as chunks of 32.
+// This thread's columns of an accumulator row (TMEM row address trow), handed to
+// the epilogue as chunks of 32.  With 8 warps a load brings 64 columns (one wait
+// for two chunks); with 16, registers allow 32 and other warps cover the wait.
 // `release` frees the accumulator once nothing will read it again.
 template <int BN, class Epi, class Free>
 __device__ __forceinline__ void epi_tile_columns(const Epi &epi, char *S, int rb, int ct, int r,
-                                                 int half, uint32_t trow,
+                                                 int group, uint32_t trow,
                                                  typename Epi::Thread &ts, Free &&release) {
+  constexpr int kCols = BN / (epi_warps<Epi>() / 4);   // columns of this thread
+  if constexpr (epi_warps<Epi>() == 8) {
 #pragma unroll 1
-  for (int cc = 0; cc < BN / 64; cc += 2) {
-    const int col = half * (BN / 2) + cc * 32;
-    float v[64];
-    tmem_ld64(trow + col, v);
-    if (!EpiReloads<Epi>::value && cc + 2 >= BN / 64) release();
-    epi.chunk(S, rb, ct, r, col, trow + (uint32_t)col,
-              *reinterpret_cast<const float(*)[32]>(v), ts);
-    epi.chunk(S, rb, ct, r, col + 32, trow + (uint32_t)(col + 32),
-              *reinterpret_cast<const float(*)[32]>(v + 32), ts);
+    for (int cc = 0; cc < kCols; cc += 64) {
+      const int col = group * kCols + cc;
+      float v[64];
+      tmem_ld64(trow + col, v);
+      if (!EpiReloads<Epi>::value && cc + 64 >= kCols) release();
+      epi.chunk(S, rb, ct, r, col, trow + (uint32_t)col,
+                *reinterpret_cast<const float(*)[32]>(v), ts);
+      epi.chunk(S, rb, ct, r, col + 32, trow + (uint32_t)(col + 32),
+                *reinterpret_cast<const float(*)[32]>(v + 32), ts);
+    }
+  } else {
+#pragma unroll 1
+    for (int cc = 0; cc < kCols; cc += 32) {
+      const int col = group * kCols + cc;
+      float v[32];
+      tmem_ld32(trow + col, v);
+      if (!EpiReloads<Epi>::value && cc + 32 >= kCols) release();
+      epi.chunk(S, rb, ct, r, col, trow + (uint32_t)col, v, ts);
+    }
   }
   if (EpiReloads<Epi>::value) release();
 }
@@ -167,7 +186,7 @@ struct Layout {
 };
 
 template <int BN, int STAGES, class Epi>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(screen_threads<Epi>(), 1)
     k_screen(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
              const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
              Operands op, Schedule sch, Epi epi, int *err) {
@@ -196,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], kEpiWarps);
+      mbar_init(&acc_empty[b], epi_warps<Epi>());
     }
     mbar_init(drain, 1);
     fence_barrier_init();
@@ -281,17 +300,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else {
     // ----------------------------------------------------------- epilogue
-    const int e = warp - 2;                 // 0..7
-    const int et = threadIdx.x - 64;        // 0..255
+    constexpr int EW = epi_warps<Epi>();
+    const int e = warp - 2;                 // 0 .. EW - 1
+    const int et = threadIdx.x - 64;        // 0 .. 32 EW - 1
     const int quarter = warp & 3;
-    const int half = e >> 2;
+    const int group = e >> 2;               // column group
     const int r = quarter * 32 + lane;      // accumulator row (user within the block)
     uint32_t t = 0;
     typename Epi::Thread ts;
     for (int ui = blockIdx.x; ui < sch.nunits && !failed; ui += gridDim.x) {
       Unit u = unit_of(sch, ui);
       epi.unit_begin(escratch, u, et, ts);
-      epi_sync();
+      epi_sync<EW>();
       for (int rb = u.rb0; rb < u.rb1; ++rb)
         for (int ct = u.ct0; ct < u.ct1; ++ct, ++t) {
           const int b = t & 1;
@@ -300,19 +320,19 @@ __global__ void __launch_bounds__(kThreads, 1)
           // reading, so that every warp passes the same barriers (the vote below)
           if (!failed && !mbar_wait_warp(&acc_full[b], aph, op.epi_wait)) failed = true;
           tc_fence_after();
-          epi.tile_begin(escratch, rb, ct, r, half, ts);
+          epi.tile_begin(escratch, rb, ct, r, group, ts);
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN);
           if (!failed)
-            epi_tile_columns<BN>(epi, escratch, rb, ct, r, half, trow, ts, [&]() {
+            epi_tile_columns<BN>(epi, escratch, rb, ct, r, group, trow, ts, [&]() {
               tc_fence_before();
               __syncwarp();
               if (lane == 0) mbar_arrive(&acc_empty[b]);
             });
-          epi.tile_end(escratch, rb, ct, r, half, ts);
+          epi.tile_end(escratch, rb, ct, r, group, ts);
         }
-      failed = epi_vote_any(failed);
+      failed = epi_vote_any<EW>(failed);
       if (!failed) epi.unit_end(escratch, u, et, ts);
-      epi_sync();
+      epi_sync<EW>();
     }
     if (failed && lane == 0) atomicExch(err, 3);
   }

@@ -77,7 +77,7 @@ bool launch_cluster_pairs(K kern, size_t smem, const tc::Schedule &sch, cudaStre
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(tc::kThreads);
+  cfg.blockDim = dim3(tc::screen_threads<Epi>());
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
@@ -159,7 +159,7 @@ rkr_status launch_screen(const TcSide &A, const TcSide &B, int split, const tc::
 #endif
   auto kern = tc::k_screen<BN, STAGES, Epi>;
   RKR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<grid, tc::kThreads, smem, st>>>(mAh, mAl, mBh, mBl, op, sch, epi, err_dev);
+  kern<<<grid, tc::screen_threads<Epi>(), smem, st>>>(mAh, mAl, mBh, mBl, op, sch, epi, err_dev);
   note_launch();
   RKR_CUDA(cudaGetLastError());
   return RKR_OK;
