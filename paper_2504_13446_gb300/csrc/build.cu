@@ -288,14 +288,19 @@ rkr_status make_binfp(const rkr_index *idx, float R, BinFP *out, cudaStream_t st
   return RKR_OK;
 }
 
-rkr_status make_binfp_grid(const rkr_index *idx, const double *g0, const double *gmax, int G,
-                           float R, double *delta_out, BinFP *out, cudaStream_t st) {
+rkr_status make_binfp_rows(int64_t rows, const float *nrm, const double *g0, const double *gmax,
+                           int G, float R, double *delta_out, BinFP *out, cudaStream_t st) {
   int bs = 256;
-  k_binfp<<<(unsigned)((idx->n + bs - 1) / bs), bs, 0, st>>>(idx->n, g0, gmax, G, idx->unrm, R,
-                                                              delta_out, out);
+  k_binfp<<<(unsigned)((rows + bs - 1) / bs), bs, 0, st>>>(rows, g0, gmax, G, nrm, R, delta_out,
+                                                           out);
   note_launch();
   RKR_CUDA(cudaGetLastError());
   return RKR_OK;
+}
+
+rkr_status make_binfp_grid(const rkr_index *idx, const double *g0, const double *gmax, int G,
+                           float R, double *delta_out, BinFP *out, cudaStream_t st) {
+  return make_binfp_rows(idx->n, idx->unrm, g0, gmax, G, R, delta_out, out, st);
 }
 
 // ------------------------------------------------------------ rank table

@@ -100,8 +100,11 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
 // Per-batch bin parameters for values bounded by ||u|| * R (paper grid).
 rkr_status make_binfp(const rkr_index *idx, float R, BinFP *out, cudaStream_t st);
 
-// Bin parameters of a grid g0 + j * (gmax - g0) / (G - 1), j < G; writes the
-// step to delta_out when it is not null.
+// Bin parameters of `rows` grids g0 + j * (gmax - g0) / (G - 1), j < G, for values
+// bounded by nrm * R; writes the steps to delta_out.
+rkr_status make_binfp_rows(int64_t rows, const float *nrm, const double *g0, const double *gmax,
+                           int G, float R, double *delta_out, BinFP *out, cudaStream_t st);
+// The same for every user of the index; delta_out may be null.
 rkr_status make_binfp_grid(const rkr_index *idx, const double *g0, const double *gmax, int G,
                            float R, double *delta_out, BinFP *out, cudaStream_t st);
 
@@ -132,6 +135,7 @@ struct ThetaArgs {
   const int64_t *qoff;          // pass 2
   uint32_t *qcursor;
   int32_t *cand_u, *cand_q;
+  float *cand_x;                // pass 2: screened score of each candidate
   int nq_all;                   // queries of the whole batch (pass 1 histogram pitch)
   const float *xs;              // per-user skip scores (null: every pair is screened)
   const int32_t *qmap;          // global query of each column (null: qa + column)
@@ -164,17 +168,35 @@ rkr_status tc_skim(const rkr_index *idx, const TcSide &Ut, const TcSide &Qt, con
 // With hist_hi (bounds mode) nothing is queued: undecided items give count intervals.
 // split = 0 screens with the single BF16 product (bounds mode only: wider count
 // intervals for a third of the tensor work); the exact mode always splits.
-// Segments of one threshold pass seg_self (the item equal to the query, or -1);
-// segments of several thresholds (up to kRecountSeg) pass self_col / self_pos
-// instead: per candidate slot of the segment, the columns of items equal to a
-// threshold's query in ascending order (-1 after the last) and the number of the
-// segment's thresholds below each such item's score.
+// Rows of one threshold pass thr (u.q rounded down / up to float, or an interval
+// holding it) and seg_self (the item equal to the query, or -1); with a null
+// seg_start row i's threshold is ths[i] (exact mode only) and its counts go to
+// hist[i] and hist_hi[i].  Segments of several thresholds (up to kRecountSeg) pass
+// self_col / self_pos instead: per candidate slot of the segment, the columns of
+// items equal to a threshold's query in ascending order (-1 after the last) and
+// the number of the segment's thresholds below each such item's score.
 rkr_status tc_recount(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt, int64_t nseg,
                       int64_t ncand, const int64_t *seg_start, const int32_t *seg_len,
-                      const int32_t *seg_user, const int32_t *seg_self, const double *ths,
-                      uint32_t *hist, uint32_t *hist_hi, cudaStream_t st, int64_t *refined,
-                      int split = 1, const int32_t *self_col = nullptr,
+                      const int32_t *seg_user, const int32_t *seg_self, const float2 *thr,
+                      const double *ths, uint32_t *hist, uint32_t *hist_hi, cudaStream_t st,
+                      int64_t *refined, int split = 1, const int32_t *self_col = nullptr,
                       const int32_t *self_pos = nullptr);
+// Rows `users` of a side as a side of their own (the caller frees A): hi, rb1 and,
+// with_lo, lo and rb3.
+rkr_status tc_gather_side(const TcSide &src, const int32_t *users, int64_t count, bool with_lo,
+                          TcSide &A, cudaStream_t st);
+void tc_gather_free(TcSide &A, cudaStream_t st);
+// Count intervals of `rows` users (side A, hi and rb1) on a grid of kDGrid points
+// per row: CLO[c] <= #{p : s(u,p) > y_c} <= CHI[c], one single-product screen.
+struct CountGrid {
+  const BinFP *ybin;      // bin parameters of the grid, per row
+  const double *yg0;      // its first point
+  const float *ytop;      // its last point rounded up to float
+  const float *ybot;      // its first point rounded down to float
+  uint32_t *CLO, *CHI;    // rows x kDGrid
+};
+rkr_status tc_count_grid(const rkr_index *idx, const TcSide &A, const TcSide &Pt,
+                         const CountGrid &g, cudaStream_t st);
 constexpr int kXGrid = 128;
 constexpr int kDGrid = RKR_DEEP_GRID;   // points of the deep count grid (exact_table = 2)
 constexpr int kRecountSeg = 32;     // thresholds per recount segment (one per screen row)

@@ -452,7 +452,8 @@ __global__ void k_seg_prep(int64_t nseg, const int64_t *__restrict__ seg_start,
                            const int32_t *__restrict__ order, const double *__restrict__ th,
                            const int32_t *__restrict__ cq, const int32_t *__restrict__ qself,
                            int32_t *__restrict__ seg_user, int32_t *__restrict__ seg_self,
-                           double *__restrict__ ths, uint32_t *__restrict__ hist,
+                           float2 *__restrict__ thr, double *__restrict__ ths,
+                           uint32_t *__restrict__ hist,
                            int32_t *__restrict__ self_col, int32_t *__restrict__ self_pos) {
   int64_t sg = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (sg >= nseg) return;
@@ -463,7 +464,10 @@ __global__ void k_seg_prep(int64_t nseg, const int64_t *__restrict__ seg_start,
   seg_self[sg] = L == 1 ? qself[cq[order[st0]]] : -1;
   for (int i = 0; i < L; ++i) ths[st0 + i] = th[order[st0 + i]];
   for (int i = 0; i <= L; ++i) hist[2 * st0 + i] = 0;
-  if (L == 1) return;
+  if (L == 1) {
+    thr[sg] = make_float2(__double2float_rd(ths[st0]), __double2float_ru(ths[st0]));
+    return;
+  }
   int32_t *sc = self_col + st0, *sp = self_pos + st0;
   int ns = 0;
   for (int i = 0; i < L; ++i) {
@@ -1211,6 +1215,7 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
   a.qcursor = cursor_d;
   a.cand_u = cand_u;
   a.cand_q = cand_q;
+  a.cand_x = cand_x;
   a.xs = plan.xs;
   a.lskip = plan.lskip;
   if (plan.listed) {
@@ -1292,19 +1297,73 @@ __global__ void k_scatter_back(int64_t n, const int32_t *__restrict__ oi,
   ccount[oi[i]] = c2[i];
 }
 
+// Rows of a recount with one threshold each: the row's threshold and the item tying
+// exactly with it.  With cx (the screened scores of all candidates, by their index
+// ci) and no_theta, a row whose candidate has a screened score takes the interval
+// [score - bound, score + bound] holding u.q as its threshold, so no row of U or Q
+// is read; the others take the canonical u.q rounded both ways (ths, when wanted,
+// gets the value itself).  ncanon counts the canonical products.
+__global__ void k_row_thresholds(int64_t count, const int32_t *__restrict__ cu,
+                                 const int32_t *__restrict__ cq, const int32_t *__restrict__ ci,
+                                 const float *__restrict__ cx, const tc::RowBound *__restrict__ urb,
+                                 const tc::RowBound *__restrict__ qrb, tc::Gacc gacc, float gcan,
+                                 const float *__restrict__ U, const float *__restrict__ Q, int d,
+                                 const int32_t *__restrict__ qself, float2 *__restrict__ thr,
+                                 double *__restrict__ ths, int32_t *__restrict__ rself,
+                                 unsigned long long *__restrict__ ncanon) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  bool canon = false;
+  if (i < count) {
+    const int64_t u = cu[i];
+    const int q = cq[i];
+    rself[i] = qself[q];
+    const float x = cx ? cx[ci[i]] : __int_as_float(0x7fffffff);
+    if (x == x) {
+      const float b = tc::screen_bound_tc(urb[u], qrb[q], gacc, gcan);
+      thr[i] = make_float2(__fsub_rd(x, b), __fadd_ru(x, b));
+    } else {
+      const double t = canon_dot(U + u * d, Q + (int64_t)q * d, d);
+      thr[i] = make_float2(__double2float_rd(t), __double2float_ru(t));
+      if (ths) ths[i] = t;
+      canon = true;
+    }
+  }
+  const int c = __popc(__ballot_sync(0xffffffffu, canon));
+  if (c && (threadIdx.x & 31) == 0) atomicAdd(ncanon, (unsigned long long)c);
+}
+
+// Distinct users among the rows: a bit per user, counted when first set.
+__global__ void k_distinct_users(int64_t count, const int32_t *__restrict__ cu,
+                                 uint32_t *__restrict__ bits,
+                                 unsigned long long *__restrict__ distinct) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  bool first = false;
+  if (i < count) {
+    const uint32_t u = (uint32_t)cu[i], b = 1u << (u & 31);
+    first = !(bits[u >> 5] & b) && !(atomicOr(&bits[u >> 5], b) & b);
+  }
+  const int c = __popc(__ballot_sync(0xffffffffu, first));
+  if (c && (threadIdx.x & 31) == 0) atomicAdd(distinct, (unsigned long long)c);
+}
+
 // Exact ranks of the candidates whose cu entry is valid (the others keep their
-// ccount): compact them, canonical u.q, sort by (user, u.q), one grouped
-// tensor-core pass over P per user.  ccount[i] = #{p : s(u_i, p) > u_i.q_i}.
+// ccount): compact them, canonical u.q, one tensor-core pass over P with a row per
+// candidate (or, with rc_seg_min, per segment of a user's sorted thresholds).
+// ccount[i] = #{p : s(u_i, p) > u_i.q_i}.
 // With clb_all (bounds mode) items the screen cannot place are not resolved:
-// ccount gets an upper and clb a lower bound of the count instead.
+// ccount gets an upper and clb a lower bound of the count instead.  The
+// single-product bounds pass takes a candidate's threshold from its screened score
+// cx_all where it has one: the item bounds are some 50 times wider.
 // With ncols > 0 only the first ncols items of the norm-sorted P are screened.
-static rkr_status recount_candidates(const rkr_index *idx, const float *Qd, int64_t total,
+static rkr_status recount_candidates(const rkr_index *idx, const QueryCommon &qc, int64_t total,
                                      const int32_t *cu_all, const int32_t *cq_all,
+                                     const float *cx_all,
                                      const int32_t *qself, uint32_t *ccount_all,
                                      uint32_t *clb_all, unsigned long long *ties_d,
                                      cudaStream_t st, int64_t *nusers = nullptr,
                                      int split = 1, int64_t ncols = 0,
                                      int64_t *ncanon = nullptr) {
+  const float *Qd = qc.Qd;
   TcSide Pv = idx->Pt;   // a view: the same rows, possibly fewer of them
   if (ncols > 0 && ncols < Pv.rows) Pv.rows = ncols;
   const int bs = 256;
@@ -1329,6 +1388,77 @@ static rkr_status recount_candidates(const rkr_index *idx, const float *Qd, int6
   RKR_CUDA(cudaStreamSynchronize(st));
   const int64_t cnt = (int64_t)hc;
   if (cnt == 0) return RKR_OK;
+  const char *span = ncols > 0   ? "span:recount(prefix)"
+                     : clb_all ? (split ? "span:recount(bounds,split)" : "span:recount(bounds,single)")
+                               : "span:recount(exact)";
+  auto add_ties = [&](const int64_t *refined) -> rkr_status {
+    if (!ties_d) return RKR_OK;
+    // accumulate over chunks: [0] undecided items, [1] canonical evaluations
+    unsigned long long t[2] = {0, 0};
+    RKR_CUDA(cudaMemcpyAsync(t, ties_d, sizeof(t), cudaMemcpyDeviceToHost, st));
+    RKR_CUDA(cudaStreamSynchronize(st));
+    t[0] += (unsigned long long)refined[0];
+    t[1] += (unsigned long long)refined[1];
+    RKR_CUDA(cudaMemcpyAsync(ties_d, t, sizeof(t), cudaMemcpyHostToDevice, st));
+    RKR_CUDA(cudaStreamSynchronize(st));
+    return RKR_OK;
+  };
+  const unsigned blocks = (unsigned)((cnt + bs - 1) / bs);
+  if (tuning().rc_seg_min == 0) {   // one row per candidate, in candidate order
+    DevBuf b1, b2, b3, b4, b5, b6, b7;
+    float2 *thr;
+    double *ths = nullptr;
+    int32_t *rself;
+    uint32_t *lo, *hi = nullptr, *bits;
+    unsigned long long *num;   // [0] canonical products, [1] distinct users
+    RKR_TRY(tmp_alloc(b1, &thr, cnt, st));
+    if (!clb_all) RKR_TRY(tmp_alloc(b2, &ths, cnt, st));
+    RKR_TRY(tmp_alloc(b3, &rself, cnt, st));
+    RKR_TRY(tmp_alloc(b4, &lo, cnt, st));
+    if (clb_all) RKR_TRY(tmp_alloc(b5, &hi, cnt, st));
+    RKR_TRY(tmp_alloc(b6, &num, 2, st));
+    RKR_CUDA(cudaMemsetAsync(num, 0, 2 * sizeof(unsigned long long), st));
+    RKR_CUDA(cudaMemsetAsync(lo, 0, sizeof(uint32_t) * cnt, st));
+    if (hi) RKR_CUDA(cudaMemsetAsync(hi, 0, sizeof(uint32_t) * cnt, st));
+    const float *cx = clb_all && !split ? cx_all : nullptr;
+    {
+      const int prof_slot = prof_begin("k_row_thresholds", st);
+      k_row_thresholds<<<blocks, bs, 0, st>>>(cnt, cu, cq, ci, cx, idx->Ut.rb3, qc.Qt.rb3,
+                                              tc_gacc(idx->Ut.kp, 1), tc_gcan(idx->d), idx->U, Qd,
+                                              idx->d, qself, thr, ths, rself, num);
+      prof_end(prof_slot, st, 0.0);
+    }
+    note_launch();
+    RKR_CUDA(cudaGetLastError());
+    if (nusers) {
+      const size_t words = (size_t)(idx->n + 31) / 32;
+      RKR_TRY(tmp_alloc(b7, &bits, words, st));
+      RKR_CUDA(cudaMemsetAsync(bits, 0, sizeof(uint32_t) * words, st));
+      k_distinct_users<<<blocks, bs, 0, st>>>(cnt, cu, bits, num + 1);
+      note_launch();
+      RKR_CUDA(cudaGetLastError());
+    }
+    int64_t refined[2] = {0, 0};
+    {
+      ProfScope prof(span, st, 0.0);
+      RKR_TRY(tc_recount(idx, idx->Ut, Pv, cnt, cnt, nullptr, nullptr, cu, rself, thr, ths, lo, hi,
+                         st, refined, split));
+    }
+    RKR_TRY(add_ties(refined));
+    unsigned long long hn[2] = {0, 0};
+    RKR_CUDA(cudaMemcpyAsync(hn, num, sizeof(hn), cudaMemcpyDeviceToHost, st));
+    k_scatter_back<<<blocks, bs, 0, st>>>(cnt, ci, clb_all ? hi : lo, ccount_all);
+    note_launch();
+    if (clb_all) {
+      k_scatter_back<<<blocks, bs, 0, st>>>(cnt, ci, lo, clb_all);
+      note_launch();
+    }
+    RKR_CUDA(cudaGetLastError());
+    RKR_CUDA(cudaStreamSynchronize(st));
+    if (ncanon) *ncanon += (int64_t)hn[0];
+    if (nusers) *nusers += (int64_t)hn[1];
+    return RKR_OK;
+  }
   if (ncanon) *ncanon += cnt;   // k_cand_theta forms each row's canonical u.q
   RKR_TRY(tmp_alloc(bcc, &ccount, cnt, st));
   int64_t Np2 = 1;
@@ -1370,14 +1500,16 @@ static rkr_status recount_candidates(const rkr_index *idx, const float *Qd, int6
   const int64_t n1 = (int64_t)segu[0], n2 = (int64_t)segu[2], off2 = cnt - n2;
   if (nusers) *nusers += (int64_t)segu[1];
   // per segment slot (front range: one threshold; back range: several)
-  DevBuf b10, b11, b12, b13;
+  DevBuf b10, b11, b12, b13, b14;
   int32_t *suser, *sself, *scol, *spos;
+  float2 *thr;
+  RKR_TRY(tmp_alloc(b14, &thr, cnt, st));
   RKR_TRY(tmp_alloc(b10, &suser, cnt, st));
   RKR_TRY(tmp_alloc(b11, &sself, cnt, st));
   RKR_TRY(tmp_alloc(b12, &scol, cnt, st));
   RKR_TRY(tmp_alloc(b13, &spos, cnt, st));
   k_seg_prep<<<(unsigned)((cnt + bs - 1) / bs), bs, 0, st>>>(
-      cnt, sstart, slen, khi, val, th, cq, qself, suser, sself, ths, hist, scol, spos);
+      cnt, sstart, slen, khi, val, th, cq, qself, suser, sself, thr, ths, hist, scol, spos);
   note_launch();
   RKR_CUDA(cudaGetLastError());
   int64_t refined[2] = {0, 0};
@@ -1388,18 +1520,15 @@ static rkr_status recount_candidates(const rkr_index *idx, const float *Qd, int6
     RKR_CUDA(cudaMemsetAsync(hist_hi, 0, sizeof(uint32_t) * 2 * cnt, st));
   }
   {
-    ProfScope prof(ncols > 0   ? "span:recount(prefix)"
-                   : clb_all ? (split ? "span:recount(bounds,split)" : "span:recount(bounds,single)")
-                             : "span:recount(exact)",
-                   st, 0.0);
+    ProfScope prof(span, st, 0.0);
     if (n1 > 0)
-      RKR_TRY(tc_recount(idx, idx->Ut, Pv, n1, cnt, sstart, slen, suser, sself, ths, hist,
+      RKR_TRY(tc_recount(idx, idx->Ut, Pv, n1, cnt, sstart, slen, suser, sself, thr, ths, hist,
                          hist_hi, st, refined, split));
     if (n2 > 0) {
       int64_t ref2[2] = {0, 0};
       RKR_TRY(tc_recount(idx, idx->Ut, Pv, n2, cnt, sstart + off2, slen + off2,
-                         suser + off2, sself + off2, ths, hist, hist_hi, st, ref2, split, scol,
-                         spos));
+                         suser + off2, sself + off2, thr, ths, hist, hist_hi, st, ref2, split,
+                         scol, spos));
       refined[0] += ref2[0];
       refined[1] += ref2[1];
     }
@@ -1413,15 +1542,7 @@ static rkr_status recount_candidates(const rkr_index *idx, const float *Qd, int6
   }
   note_launch();
   RKR_CUDA(cudaGetLastError());
-  if (ties_d) {  // accumulate over chunks: [0] undecided items, [1] canonical evaluations
-    unsigned long long r[2] = {0, 0};
-    RKR_CUDA(cudaMemcpyAsync(r, ties_d, sizeof(r), cudaMemcpyDeviceToHost, st));
-    RKR_CUDA(cudaStreamSynchronize(st));
-    r[0] += (unsigned long long)refined[0];
-    r[1] += (unsigned long long)refined[1];
-    RKR_CUDA(cudaMemcpyAsync(ties_d, r, sizeof(r), cudaMemcpyHostToDevice, st));
-    RKR_CUDA(cudaStreamSynchronize(st));
-  }
+  RKR_TRY(add_ties(refined));
   {
     const int prof_slot = prof_begin("k_scatter_counts", st);
     k_scatter_counts<<<(unsigned)((nseg + bs - 1) / bs), bs, 0, st>>>((int64_t)nseg, sstart, slen,
@@ -1465,6 +1586,206 @@ static rkr_status count_valid(const int32_t *v, int64_t n, unsigned long long *o
   return RKR_OK;
 }
 
+// Interval [lo, hi] of a candidate's u.q in float: from its screened score, or from
+// the compensated product of its rows.
+__device__ __forceinline__ void cand_interval(int64_t u, int q, float x,
+                                              const tc::RowBound *__restrict__ urb,
+                                              const tc::RowBound *__restrict__ qrb, tc::Gacc gacc,
+                                              float gcan, const float *__restrict__ U,
+                                              const float *__restrict__ Q, int d, float &lo,
+                                              float &hi) {
+  if (x == x) {
+    const float b = tc::screen_bound_tc(urb[u], qrb[q], gacc, gcan);
+    lo = __fsub_rd(x, b);
+    hi = __fadd_ru(x, b);
+  } else {
+    double l, h;
+    dot2_interval(U + u * d, Q + (int64_t)q * d, d, l, h);
+    lo = __double2float_rd(l);
+    hi = __double2float_ru(h);
+  }
+}
+
+// Order-preserving 32-bit key of a float, and its inverse.
+__device__ __forceinline__ uint32_t float_key(float x) {
+  const uint32_t b = __float_as_uint(x);
+  return (b >> 31) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float key_float(uint32_t k) {
+  return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k);
+}
+
+// Range of the open candidates' u.q per user, as keys (kmin starts at ~0, kmax at 0).
+__global__ void k_open_range(int64_t cnt, const int32_t *__restrict__ cu_fb,
+                             const int32_t *__restrict__ cq, const float *__restrict__ cx,
+                             const tc::RowBound *__restrict__ urb,
+                             const tc::RowBound *__restrict__ qrb, tc::Gacc gacc, float gcan,
+                             const float *__restrict__ U, const float *__restrict__ Q, int d,
+                             uint32_t *__restrict__ kmin, uint32_t *__restrict__ kmax) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= cnt) return;
+  const int64_t u = cu_fb[i];
+  if (u < 0) return;
+  float lo, hi;
+  cand_interval(u, cq[i], cx[i], urb, qrb, gacc, gcan, U, Q, d, lo, hi);
+  const uint32_t a = float_key(lo), b = float_key(hi);
+  if (a < kmin[u]) atomicMin(&kmin[u], a);
+  if (b > kmax[u]) atomicMax(&kmax[u], b);
+}
+
+// Users with open candidates, each with a grid from its smallest to its largest u.q.
+__global__ void k_grid_users(int64_t n, const uint32_t *__restrict__ kmin,
+                             const uint32_t *__restrict__ kmax, const float *__restrict__ unrm,
+                             unsigned long long *__restrict__ cursor, int32_t *__restrict__ ulist,
+                             int32_t *__restrict__ uslot, double *__restrict__ yg0,
+                             double *__restrict__ ymax, float *__restrict__ ytop,
+                             float *__restrict__ ybot, float *__restrict__ nrm) {
+  const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool has = u < n && kmin[u] != 0xffffffffu;
+  const unsigned act = __ballot_sync(0xffffffffu, has);
+  if (!has) return;
+  const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
+  unsigned long long base = 0;
+  if (lane == leader) base = atomicAdd(cursor, (unsigned long long)__popc(act));
+  base = __shfl_sync(act, base, leader);
+  const int64_t s = (int64_t)base + __popc(act & ((1u << lane) - 1u));
+  const float lo = key_float(kmin[u]), hi = key_float(kmax[u]);
+  ulist[s] = (int32_t)u;
+  uslot[u] = (int32_t)s;
+  yg0[s] = (double)lo;
+  ymax[s] = (double)hi;
+  ytop[s] = hi;
+  ybot[s] = lo;
+  nrm[s] = unrm[u];
+}
+
+// Count bounds of the open candidates from their user's grid: u.q >= y_{jl - 1} and
+// u.q < y_{jh} give CLO[jh] <= count <= CHI[jl - 1].
+__global__ void k_grid_bound(int64_t cnt, const int32_t *__restrict__ cu_fb,
+                             const int32_t *__restrict__ cq, const float *__restrict__ cx,
+                             const tc::RowBound *__restrict__ urb,
+                             const tc::RowBound *__restrict__ qrb, tc::Gacc gacc, float gcan,
+                             const float *__restrict__ U, const float *__restrict__ Q, int d,
+                             const int32_t *__restrict__ uslot, const double *__restrict__ yg0,
+                             const double *__restrict__ ydx, const uint32_t *__restrict__ CLO,
+                             const uint32_t *__restrict__ CHI, uint32_t *__restrict__ ccount,
+                             uint32_t *__restrict__ clb) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= cnt) return;
+  const int64_t u = cu_fb[i];
+  if (u < 0) return;
+  float lo, hi;
+  cand_interval(u, cq[i], cx[i], urb, qrb, gacc, gcan, U, Q, d, lo, hi);
+  const int64_t s = uslot[u];
+  const int jl = exact_j((double)lo, yg0[s], ydx[s], kDGrid);
+  const int jh = exact_j((double)hi, yg0[s], ydx[s], kDGrid);
+  if (jl >= 1) ccount[i] = min(ccount[i], CHI[s * kDGrid + jl - 1]);
+  if (jh < kDGrid) clb[i] = max(clb[i], CLO[s * kDGrid + jh]);
+}
+
+// When a chunk's open candidates (h of them) are many per user, their counts are
+// first bounded together: one single-product screen of the users concerned against
+// P counts each user's scores on a grid of kDGrid points spanning its candidates'
+// u.q, and the cap (k-th smallest count upper bound) then drops most of them.  A
+// grid row costs about six recount rows (every score inside the grid goes to two
+// histograms), so it is built from kGridPerUser candidates per user on, where it
+// can save a recount of each.  *h is the number still open on return.  Nothing
+// happens when the scratch cannot be had.
+constexpr int64_t kGridPerUser = 12;
+constexpr int64_t kGridMinRows = (int64_t)1 << 16;
+
+static rkr_status grid_prune(const rkr_index *idx, const QueryCommon &qc, int qa, int qb,
+                             int64_t cnt, const int64_t *qoff_rel, const uint32_t *cursor,
+                             const int32_t *cq, const float *cx, uint32_t *ccount, uint32_t *clb,
+                             int32_t *cu_fb, unsigned long long *h, cudaStream_t st) {
+  const int64_t n = idx->n;
+  const tc::Gacc gacc = tc_gacc(idx->Ut.kp, 1);
+  const float gcan = tc_gcan(idx->d);
+  DevBuf b[13];
+  bool ok = true;
+  auto get = [&](int i, auto **p, size_t count) {
+    if (!ok) return;
+    if (pool_malloc_async((void **)p, count * sizeof(**p), st) != cudaSuccess) {
+      cudaGetLastError();
+      ok = false;
+      return;
+    }
+    b[i].p = (void *)*p;
+    b[i].st = st;
+  };
+  uint32_t *kmin = nullptr, *kmax = nullptr;
+  int32_t *ulist = nullptr, *uslot = nullptr;
+  double *yg0 = nullptr, *ymax = nullptr, *ydx = nullptr;
+  float *ytop = nullptr, *ybot = nullptr, *nrm = nullptr;
+  unsigned long long *num = nullptr;
+  get(0, &kmin, n);
+  get(1, &kmax, n);
+  get(2, &num, 1);
+  if (!ok) return RKR_OK;
+  RKR_CUDA(cudaMemsetAsync(kmin, 0xff, sizeof(uint32_t) * n, st));
+  RKR_CUDA(cudaMemsetAsync(kmax, 0, sizeof(uint32_t) * n, st));
+  RKR_CUDA(cudaMemsetAsync(num, 0, sizeof(unsigned long long), st));
+  const unsigned cblocks = (unsigned)((cnt + 255) / 256), ublocks = (unsigned)((n + 255) / 256);
+  k_open_range<<<cblocks, 256, 0, st>>>(cnt, cu_fb, cq, cx, idx->Ut.rb3, qc.Qt.rb3, gacc, gcan,
+                                        idx->U, qc.Qd, idx->d, kmin, kmax);
+  note_launch();
+  get(3, &ulist, n);
+  get(4, &uslot, n);
+  get(5, &yg0, n);
+  get(6, &ymax, n);
+  get(7, &ytop, n);
+  get(8, &ybot, n);
+  get(9, &nrm, n);
+  if (!ok) return RKR_OK;
+  k_grid_users<<<ublocks, 256, 0, st>>>(n, kmin, kmax, idx->unrm, num, ulist, uslot, yg0, ymax,
+                                        ytop, ybot, nrm);
+  note_launch();
+  RKR_CUDA(cudaGetLastError());
+  unsigned long long users = 0;
+  RKR_CUDA(cudaMemcpyAsync(&users, num, sizeof(users), cudaMemcpyDeviceToHost, st));
+  RKR_CUDA(cudaStreamSynchronize(st));
+  if (users == 0 || *h < (unsigned long long)kGridPerUser * users) return RKR_OK;
+  const int64_t nu = (int64_t)users;
+  BinFP *ybin = nullptr;
+  uint32_t *CLO = nullptr, *CHI = nullptr;
+  DevBuf bb;
+  get(10, &ydx, nu);
+  get(11, &CLO, nu * kDGrid);
+  get(12, &CHI, nu * kDGrid);
+  if (ok && pool_malloc_async(&ybin, sizeof(BinFP) * nu, st) == cudaSuccess) {
+    bb.p = ybin;
+    bb.st = st;
+  } else {
+    cudaGetLastError();
+    return RKR_OK;
+  }
+  RKR_TRY(make_binfp_rows(nu, nrm, yg0, ymax, kDGrid, idx->pmax, ydx, ybin, st));
+  TcSide A;
+  if (tc_gather_side(idx->Ut, ulist, nu, false, A, st) != RKR_OK) {
+    set_error("%s", "");
+    return RKR_OK;
+  }
+  const rkr_status gs =
+      tc_count_grid(idx, A, idx->Pt, CountGrid{ybin, yg0, ytop, ybot, CLO, CHI}, st);
+  tc_gather_free(A, st);
+  RKR_TRY(gs);
+  k_grid_bound<<<cblocks, 256, 0, st>>>(cnt, cu_fb, cq, cx, idx->Ut.rb3, qc.Qt.rb3, gacc, gcan,
+                                        idx->U, qc.Qd, idx->d, uslot, yg0, ydx, CLO, CHI, ccount,
+                                        clb);
+  note_launch();
+  {
+    const int prof_slot = prof_begin("k_recount_filter", st);
+    k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount,
+                                                         clb, cu_fb);
+    prof_end(prof_slot, st, 0.0);
+  }
+  note_launch();
+  k_drop_decided<<<cblocks, 256, 0, st>>>(cnt, ccount, clb, cu_fb);
+  note_launch();
+  RKR_CUDA(cudaGetLastError());
+  return count_valid(cu_fb, cnt, h, st);
+}
+
 // Early termination over the norm-sorted items (tuning rc_prefix; Alg. 1 sorts P
 // by descending norm).  For the queries with many candidates still to recount,
 // every such candidate is first screened against the first m1 items only: its
@@ -1476,8 +1797,9 @@ static rkr_status count_valid(const int32_t *v, int64_t n, unsigned long long *o
 // to the recount.  On return *h2 is the number of candidates still to recount.
 static rkr_status prefix_prune(const rkr_index *idx, const QueryCommon &qc, int qa, int qb,
                                int64_t cnt, const int64_t *qoff_rel, const uint32_t *cursor,
-                               const int32_t *cq, const int32_t *qself, uint32_t *ccount,
-                               uint32_t *clb, int32_t *cu_fb, int64_t *recount_users,
+                               const int32_t *cq, const float *cx, const int32_t *qself,
+                               uint32_t *ccount, uint32_t *clb, int32_t *cu_fb,
+                               int64_t *recount_users,
                                unsigned long long *h2, int64_t *rows, int64_t *pruned,
                                int64_t *ncanon, cudaStream_t st) {
   const int64_t m1 = idx->m / tuning().rc_prefix / 256 * 256;
@@ -1504,7 +1826,7 @@ static rkr_status prefix_prune(const rkr_index *idx, const QueryCommon &qc, int 
   if (npre == 0) return RKR_OK;
   *rows += (int64_t)npre;
   // certain (lo1) and possible (hi1) counts over the prefix, single product
-  RKR_TRY(recount_candidates(idx, qc.Qd, cnt, cu_pre, cq, qself, hi1, lo1, nullptr, st, nullptr,
+  RKR_TRY(recount_candidates(idx, qc, cnt, cu_pre, cq, cx, qself, hi1, lo1, nullptr, st, nullptr,
                              0, m1, ncanon));
   k_prefix_pick<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, cu_pre, hi1, lo1, clb,
                                           cu_fb, cu_park);
@@ -1514,7 +1836,7 @@ static rkr_status prefix_prune(const rkr_index *idx, const QueryCommon &qc, int 
   RKR_TRY(count_valid(cu_park, cnt, &parked, st));
   RKR_TRY(count_valid(cu_fb, cnt, &h, st));
   if (h > 0)  // the promising rows and the other queries' rows, over all of P
-    RKR_TRY(recount_candidates(idx, qc.Qd, cnt, cu_fb, cq, qself, ccount, clb, nullptr, st,
+    RKR_TRY(recount_candidates(idx, qc, cnt, cu_fb, cq, cx, qself, ccount, clb, nullptr, st,
                                recount_users, tuning().rc_single_first ? 0 : 1, 0, ncanon));
   {
     const int prof_slot = prof_begin("k_recount_filter", st);
@@ -2080,7 +2402,7 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
         // undecided items of those that remain.
         for (int pass = tuning().rc_single_first ? 0 : 1; pass < 2 && h2 > 0; ++pass) {
           const bool first = pass == 0 || !tuning().rc_single_first;
-          RKR_TRY(recount_candidates(idx, qc.Qd, cnt, cu_fb, cq, qself, ccount, clb, nullptr,
+          RKR_TRY(recount_candidates(idx, qc, cnt, cu_fb, cq, cx, qself, ccount, clb, nullptr,
                                      st, first ? &recount_users : nullptr, pass == 0 ? 0 : 1, 0,
                                      &canon_rows));
           if (pass == 1) recount_split += (int64_t)h2;
@@ -2105,12 +2427,15 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
         }
         recount_open += (int64_t)h2;
         if (h2 > 0)
-          RKR_TRY(recount_candidates(idx, qc.Qd, cnt, cu_fb, cq, qself, ccount, nullptr, ties_d,
+          RKR_TRY(recount_candidates(idx, qc, cnt, cu_fb, cq, cx, qself, ccount, nullptr, ties_d,
                                      st, nullptr, 1, 0, &canon_rows));
         return RKR_OK;
       };
+      if (!lp && lstat_host_fb >= (unsigned long long)kGridMinRows)
+        RKR_TRY(grid_prune(idx, qc, qa, qb, cnt, qoff_rel, cursor, cq, cx, ccount, clb, cu_fb,
+                           &lstat_host_fb, st));
       if (!lp && tuning().rc_prefix > 0 && lstat_host_fb >= (unsigned long long)prefix_min_rows(1))
-        RKR_TRY(prefix_prune(idx, qc, qa, qb, cnt, qoff_rel, cursor, cq, qself, ccount, clb, cu_fb,
+        RKR_TRY(prefix_prune(idx, qc, qa, qb, cnt, qoff_rel, cursor, cq, cx, qself, ccount, clb, cu_fb,
                              &recount_users, &lstat_host_fb, &prefix_rows, &prefix_pruned,
                              &canon_rows, st));
       if (lstat_host_fb > 0) RKR_TRY(recount_open_candidates(lstat_host_fb));
@@ -2216,7 +2541,7 @@ rkr_status run_rank_pairs(const rkr_index *idx, const QueryCommon &qc, int nq, i
   RKR_CUDA(cudaMemcpyAsync(ls, lstat, sizeof(ls), cudaMemcpyDeviceToHost, st));
   RKR_CUDA(cudaStreamSynchronize(st));
   if (ls[0] > 0)  // pairs below their user's tail list: exact recount
-    RKR_TRY(recount_candidates(idx, qc.Qd, npairs, cu_fb, cq, qself, ccount, nullptr, ties, st));
+    RKR_TRY(recount_candidates(idx, qc, npairs, cu_fb, cq, nullptr, qself, ccount, nullptr, ties, st));
   k_count_to_rank<<<(unsigned)((npairs + 255) / 256), 256, 0, st>>>(npairs, ccount, out_rank);
   note_launch();
   RKR_CUDA(cudaGetLastError());

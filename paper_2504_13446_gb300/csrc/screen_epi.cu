@@ -919,31 +919,36 @@ struct EpiDeep {
   }
 };
 
-rkr_status tc_deep_table(rkr_index *idx, const TcSide &Ut, const TcSide &Pt, const float *ytop,
-                         const float *ybot, cudaStream_t st) {
-  // 128-column tiles: four 32 KB stages fit beside the histograms and the tile
+rkr_status tc_count_grid(const rkr_index *idx, const TcSide &A, const TcSide &Pt,
+                         const CountGrid &g, cudaStream_t st) {
   constexpr int BN = 128;
-  const int64_t n = idx->n, m = idx->m;
+  const int64_t n = A.rows, m = Pt.rows;
   int *flags;
   tc::RowBound *tb = nullptr;
   RKR_CUDA(pool_malloc_async(&flags, sizeof(int) * 2, st));
   RKR_CUDA(cudaMemsetAsync(flags, 0, sizeof(int) * 2, st));
   RKR_TRY(tc_tile_bounds(Pt, BN, 0, &tb, st));
   EpiDeep e;
-  e.nrows = n; e.ncols = m; e.bn = BN; e.rowb = Ut.rb1; e.tileb = tb;
-  e.gacc = tc_gacc(Ut.kp, 0); e.gcan = tc_gcan(idx->d);
-  e.ybin = idx->ybin; e.yg0 = idx->yg0; e.ytop = ytop; e.ybot = ybot;
-  e.DLO = idx->DLO; e.DHI = idx->DHI;
-  rkr_status s = launch_screen<BN, tc::stages1<BN, EpiDeep>()>(Ut, Pt, 0, row_schedule(n, m, BN),
+  e.nrows = n; e.ncols = m; e.bn = BN; e.rowb = A.rb1; e.tileb = tb;
+  e.gacc = tc_gacc(A.kp, 0); e.gcan = tc_gcan(idx->d);
+  e.ybin = g.ybin; e.yg0 = g.yg0; e.ytop = g.ytop; e.ybot = g.ybot;
+  e.DLO = g.CLO; e.DHI = g.CHI;
+  rkr_status s = launch_screen<BN, tc::stages1<BN, EpiDeep>()>(A, Pt, 0, row_schedule(n, m, BN),
                                                               e, flags, st);
   int hf[2] = {0, 0};
   cudaMemcpyAsync(hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, st);
   cudaError_t err = cudaStreamSynchronize(st);
   for (void *p : {(void *)tb, (void *)flags}) cudaFreeAsync(p, st);
-  if (err != cudaSuccess) return cuda_fail(err, "tc_deep_table");
+  if (err != cudaSuccess) return cuda_fail(err, "tc_count_grid");
   RKR_TRY(s);
-  if (hf[0]) return fail(RKR_ETIMEOUT, "deep-grid screen wait timed out (%d)", hf[0]);
+  if (hf[0]) return fail(RKR_ETIMEOUT, "count-grid screen wait timed out (%d)", hf[0]);
   return RKR_OK;
+}
+
+rkr_status tc_deep_table(rkr_index *idx, const TcSide &Ut, const TcSide &Pt, const float *ytop,
+                         const float *ybot, cudaStream_t st) {
+  return tc_count_grid(idx, Ut, Pt,
+                       CountGrid{idx->ybin, idx->yg0, ytop, ybot, idx->DLO, idx->DHI}, st);
 }
 
 // ================================================================= theta
@@ -1009,6 +1014,7 @@ struct EpiTheta {
   const int64_t *qoff;
   uint32_t *qcursor;
   int32_t *cand_u, *cand_q;
+  float *cand_x;                // PASS 2: the candidate's screened score
   int *ovf;                     // PASS 2: set when a query's segment would overflow
   const float *xs;              // per user: pairs scoring <= xs[u] - b are skipped (or null)
   const uint32_t *member;       // per-query user subsets (bitmaps), or null
@@ -1183,7 +1189,7 @@ struct EpiTheta {
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (on[i] && lb[i] <= caps(S)[cl[i]]) emit(qglob(S)[cl[i]], ts.u);
+          if (on[i] && lb[i] <= caps(S)[cl[i]]) emit(qglob(S)[cl[i]], ts.u, x[i]);
       }
     }
   }
@@ -1194,7 +1200,7 @@ struct EpiTheta {
     if (bkt >= kFine) bkt = kFine - 1;
     atomicAdd(&fine[(int64_t)q * kFine + bkt], 1u);
   }
-  __device__ void emit(int q, int64_t u) const {
+  __device__ void emit(int q, int64_t u, float x) const {
     uint32_t pos = atomicAdd(&qcursor[q], 1u);
     int64_t at = qoff[q] + pos;
     if (at >= qoff[q + 1]) {  // more than the pass-1 count: never written out of the segment
@@ -1203,6 +1209,7 @@ struct EpiTheta {
     }
     cand_u[at] = (int32_t)u;
     cand_q[at] = q;
+    cand_x[at] = x;
   }
   __device__ void tile_end(char *, int, int, int, int, Thread &) const {}
   __device__ void unit_end(char *S, const tc::Unit &u, int et, Thread &) const {
@@ -1241,6 +1248,7 @@ static rkr_status theta_launch(const rkr_index *idx, const TcSide &Ut, const TcS
   e.member = a.member; e.mwords = a.mwords;
   e.lstar = a.lstar; e.cap = a.cap; e.fine = a.fine;
   e.qoff = a.qoff; e.qcursor = a.qcursor; e.cand_u = a.cand_u; e.cand_q = a.cand_q;
+  e.cand_x = a.cand_x;
   static_assert(tc::screen_smem_bytes<kThetaBN, 4, EpiTheta<1>>() <= 232448, "theta smem");
   rkr_status s = launch_screen<kThetaBN, 4>(Ut, Qt, split, sch, e, err, st);
   cudaFreeAsync(tb, st);
@@ -1672,7 +1680,6 @@ struct EpiRC {
     float tlo, thi;              // possibly above: score > tlo; certainly: score >= thi
     int64_t sg;
     int64_t self;                // item tying exactly with u.q (never above), or -1
-    uint32_t *h, *hh;
     uint32_t clo, chi;           // items certainly / possibly above u.q
     tc::RowBound ru;             // the row's bound terms
     TilePrefetch tp;             // the bound terms of the next column tile
@@ -1683,9 +1690,10 @@ struct EpiRC {
   const tc::RowBound *rowb, *tileb;
   tc::Gacc gacc;
   float gcan;
-  const int64_t *seg_start;
+  const int64_t *seg_start;   // null: row i's counts go to hist[i] and hist_hi[i]
   const int32_t *seg_len;
   const double *ths;
+  const float2 *thr;          // per row: u.q rounded down / up
   const int32_t *seg_self;
   uint32_t *hist;
   // Bounds mode (hist_hi not null): the possibly-above count goes to hist_hi and
@@ -1702,12 +1710,9 @@ struct EpiRC {
     ts.tp.start(tileb, u.ct0);
     if (ts.sg < nseg) {
       ts.ru = rowb[ts.sg];
-      const int64_t st0 = seg_start[ts.sg];
-      const double t = ths[st0];
-      ts.h = hist + 2 * st0;
-      ts.hh = hist_hi ? hist_hi + 2 * st0 : nullptr;
-      ts.tdn = __double2float_rd(t);
-      ts.tup = __double2float_ru(t);
+      const float2 t = thr[ts.sg];
+      ts.tdn = t.x;
+      ts.tup = t.y;
       ts.self = seg_self[ts.sg];
     } else {
       ts.self = -1;
@@ -1758,8 +1763,10 @@ struct EpiRC {
   __device__ __forceinline__ void tile_end(char *, int, int, int, int, Thread &) const {}
   __device__ __forceinline__ void unit_end(char *, const tc::Unit &, int, Thread &ts) const {
     if (ts.sg >= nseg) return;
-    if (ts.clo) atomicAdd(&ts.h[1], ts.clo);      // position 1: above the one threshold
-    if (ts.hh && ts.chi) atomicAdd(&ts.hh[1], ts.chi);
+    // position 1 of a segment's histogram: above its one threshold
+    const int64_t at = seg_start ? 2 * seg_start[ts.sg] + 1 : ts.sg;
+    if (ts.clo) atomicAdd(&hist[at], ts.clo);
+    if (hist_hi && ts.chi) atomicAdd(&hist_hi[at], ts.chi);
   }
 };
 
@@ -1943,8 +1950,8 @@ __global__ void k_rc_refine(const int2 *__restrict__ items, const unsigned long 
   for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < c;
        i += (unsigned long long)gridDim.x * blockDim.x) {
     int2 it = items[i];
-    int64_t st0 = seg_start[it.x];
-    int L = seg_len[it.x];
+    const int64_t st0 = seg_start ? seg_start[it.x] : it.x;   // null: rows of one threshold
+    const int L = seg_start ? seg_len[it.x] : 1;
     const int64_t u = seg_user[it.x];
     const float *uu = U + u * d, *pp = Ps + (int64_t)it.y * d;
     float acc = 0.0f;
@@ -1963,11 +1970,13 @@ __global__ void k_rc_refine(const int2 *__restrict__ items, const unsigned long 
       double s = canon_dot(uu, pp, d);
       while (pos < a0 && t[pos] < s) ++pos;
     }
-    atomicAdd(&hist[2 * st0 + pos], 1u);
+    if (seg_start) atomicAdd(&hist[2 * st0 + pos], 1u);
+    else if (pos) atomicAdd(&hist[st0], 1u);
   }
 }
 
-// Gather rows of a side: out row i = side row idx[i].
+// Gather rows of a side: out row i = side row idx[i], 16 bytes a thread; olo and
+// orb3 may be null (single-product screens read hi and rb1 only).
 __global__ void k_gather_side(const __nv_bfloat16 *__restrict__ hi,
                               const __nv_bfloat16 *__restrict__ lo,
                               const tc::RowBound *__restrict__ rb1,
@@ -1975,59 +1984,105 @@ __global__ void k_gather_side(const __nv_bfloat16 *__restrict__ hi,
                               const int32_t *__restrict__ rows, int64_t count,
                               __nv_bfloat16 *__restrict__ ohi, __nv_bfloat16 *__restrict__ olo,
                               tc::RowBound *__restrict__ orb1, tc::RowBound *__restrict__ orb3) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.y + threadIdx.y;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.y + threadIdx.y;
   if (i >= count) return;
-  int64_t src = rows[i];
-  for (int k = threadIdx.x; k < kp; k += blockDim.x) {
-    ohi[i * ld + k] = hi[src * ld + k];
-    olo[i * ld + k] = lo[src * ld + k];
+  const int64_t src = rows[i];
+  const int words = kp >> 3;   // kp is a multiple of 16, rows start on 32-byte boundaries
+  for (int k = threadIdx.x; k < words; k += blockDim.x) {
+    ((uint4 *)(ohi + i * ld))[k] = ((const uint4 *)(hi + src * ld))[k];
+    if (olo) ((uint4 *)(olo + i * ld))[k] = ((const uint4 *)(lo + src * ld))[k];
   }
   if (threadIdx.x == 0) {
     orb1[i] = rb1[src];
-    orb3[i] = rb3[src];
+    if (orb3) orb3[i] = rb3[src];
   }
+}
+
+rkr_status tc_gather_side(const TcSide &src, const int32_t *users, int64_t count, bool with_lo,
+                          TcSide &A, cudaStream_t st) {
+  A.rows = count;
+  A.d = src.d;
+  A.kp = src.kp;
+  A.pitch = src.pitch;
+  A.owned = false;
+  const size_t cnt = (size_t)std::max<int64_t>(count, 1) * A.ld();
+  auto alloc = [&](auto **p, size_t bytes) {
+    if (pool_malloc_async((void **)p, bytes, st) == cudaSuccess) return true;
+    cudaGetLastError();
+    *p = nullptr;
+    return false;
+  };
+  bool ok = alloc(&A.hi, cnt * 2) &&
+            alloc(&A.rb1, sizeof(tc::RowBound) * std::max<int64_t>(count, 1));
+  if (ok && with_lo)
+    ok = alloc(&A.lo, cnt * 2) &&
+         alloc(&A.rb3, sizeof(tc::RowBound) * std::max<int64_t>(count, 1));
+  if (!ok) {
+    tc_gather_free(A, st);
+    return fail(RKR_ENOMEM, "device allocation of %zu bytes failed", cnt * 2);
+  }
+  if (count > 0) {
+    // 8 lanes of 16 bytes cover 128 bytes of a row
+    const int prof_slot = prof_begin("k_gather_side", st);
+    k_gather_side<<<(unsigned)((count + 31) / 32), dim3(8, 32), 0, st>>>(
+        src.hi, src.lo, src.rb1, src.rb3, A.kp, A.ld(), users, count, A.hi, A.lo, A.rb1, A.rb3);
+    prof_end(prof_slot, st, 0.0);
+    note_launch();
+    RKR_CUDA(cudaGetLastError());
+  }
+  return RKR_OK;
+}
+
+void tc_gather_free(TcSide &A, cudaStream_t st) {
+  for (void *p : {(void *)A.hi, (void *)A.lo, (void *)A.rb1, (void *)A.rb3})
+    if (p) cudaFreeAsync(p, st);
+  A.hi = A.lo = nullptr;
+  A.rb1 = A.rb3 = nullptr;
 }
 
 template <int BN, int STAGES, class Epi>
 static rkr_status tc_recount_bn(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt,
                                 int64_t nseg, int64_t ncand, const int64_t *seg_start,
                                 const int32_t *seg_len, const int32_t *seg_user,
-                                const int32_t *seg_self, const double *ths, uint32_t *hist,
-                                uint32_t *hist_hi, cudaStream_t st, int64_t *refined, int split,
+                                const int32_t *seg_self, const float2 *thr, const double *ths,
+                                uint32_t *hist, uint32_t *hist_hi, cudaStream_t st, int64_t *refined, int split,
                                 const int32_t *self_col, const int32_t *self_pos);
 
 rkr_status tc_recount(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt, int64_t nseg,
                       int64_t ncand, const int64_t *seg_start, const int32_t *seg_len,
-                      const int32_t *seg_user, const int32_t *seg_self, const double *ths,
-                      uint32_t *hist, uint32_t *hist_hi, cudaStream_t st, int64_t *refined,
-                      int split, const int32_t *self_col, const int32_t *self_pos) {
+                      const int32_t *seg_user, const int32_t *seg_self, const float2 *thr,
+                      const double *ths, uint32_t *hist, uint32_t *hist_hi, cudaStream_t st,
+                      int64_t *refined, int split, const int32_t *self_col,
+                      const int32_t *self_pos) {
   // the exact mode places every item, so it always runs the split product
   if (!hist_hi) split = 1;
   if (self_col) {   // segments of several thresholds
     if (tuning().rc_bn == 128)
       return tc_recount_bn<128, tc::stages1<128, EpiRCm>(), EpiRCm>(
-          idx, Ut, Pt, nseg, ncand, seg_start, seg_len, seg_user, seg_self, ths, hist, hist_hi,
-          st, refined, split, self_col, self_pos);
+          idx, Ut, Pt, nseg, ncand, seg_start, seg_len, seg_user, seg_self, thr, ths, hist,
+          hist_hi, st, refined, split, self_col, self_pos);
     return tc_recount_bn<256, tc::stages1<256, EpiRCm>(), EpiRCm>(
-        idx, Ut, Pt, nseg, ncand, seg_start, seg_len, seg_user, seg_self, ths, hist, hist_hi, st,
-        refined, split, self_col, self_pos);
+        idx, Ut, Pt, nseg, ncand, seg_start, seg_len, seg_user, seg_self, thr, ths, hist,
+        hist_hi, st, refined, split, self_col, self_pos);
   }
   if (tuning().rc_bn == 128)
     return tc_recount_bn<128, 6, EpiRC>(idx, Ut, Pt, nseg, ncand, seg_start, seg_len, seg_user,
-                                        seg_self, ths, hist, hist_hi, st, refined, split,
+                                        seg_self, thr, ths, hist, hist_hi, st, refined, split,
                                         nullptr, nullptr);
   return tc_recount_bn<256, 4, EpiRC>(idx, Ut, Pt, nseg, ncand, seg_start, seg_len, seg_user,
-                                      seg_self, ths, hist, hist_hi, st, refined, split, nullptr,
-                                      nullptr);
+                                      seg_self, thr, ths, hist, hist_hi, st, refined, split,
+                                      nullptr, nullptr);
 }
 
 template <class Epi>
-static void set_recount_fields(Epi &e, const int32_t *, const int32_t *, const int32_t *seg_self) {
+static void set_recount_fields(Epi &e, const int32_t *, const int32_t *, const int32_t *seg_self,
+                               const float2 *thr) {
   e.seg_self = seg_self;
+  e.thr = thr;
 }
 template <>
 void set_recount_fields<EpiRCm>(EpiRCm &e, const int32_t *self_col, const int32_t *self_pos,
-                                const int32_t *) {
+                                const int32_t *, const float2 *) {
   e.self_col = self_col;
   e.self_pos = self_pos;
 }
@@ -2036,31 +2091,13 @@ template <int BN, int STAGES, class Epi>
 static rkr_status tc_recount_bn(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt,
                                 int64_t nseg, int64_t ncand, const int64_t *seg_start,
                                 const int32_t *seg_len, const int32_t *seg_user,
-                                const int32_t *seg_self, const double *ths, uint32_t *hist,
-                                uint32_t *hist_hi, cudaStream_t st, int64_t *refined, int split,
+                                const int32_t *seg_self, const float2 *thr, const double *ths,
+                                uint32_t *hist, uint32_t *hist_hi, cudaStream_t st, int64_t *refined, int split,
                                 const int32_t *self_col, const int32_t *self_pos) {
   const int64_t m = Pt.rows;   // all of P, or a prefix of the norm-sorted items
   if (nseg <= 0) return RKR_OK;
   TcSide A;
-  A.rows = nseg;
-  A.d = Ut.d;
-  A.kp = Ut.kp;
-  A.pitch = Ut.pitch;
-  A.owned = false;
-  size_t cnt = (size_t)nseg * A.ld();
-  RKR_CUDA(pool_malloc_async((void **)&A.hi, cnt * 2, st));
-  RKR_CUDA(pool_malloc_async((void **)&A.lo, cnt * 2, st));
-  RKR_CUDA(pool_malloc_async((void **)&A.rb1, sizeof(tc::RowBound) * nseg, st));
-  RKR_CUDA(pool_malloc_async((void **)&A.rb3, sizeof(tc::RowBound) * nseg, st));
-  dim3 blk(32, 8);
-  {
-    const int prof_slot = prof_begin("k_gather_side", st);
-    k_gather_side<<<(unsigned)((nseg + 7) / 8), blk, 0, st>>>(Ut.hi, Ut.lo, Ut.rb1, Ut.rb3, A.kp, A.ld(),
-                                                               seg_user, nseg, A.hi, A.lo, A.rb1,
-                                                               A.rb3);
-    prof_end(prof_slot, st, 0.0);
-  }
-  note_launch();
+  RKR_TRY(tc_gather_side(Ut, seg_user, nseg, split != 0, A, st));
   tc::RowBound *tb = nullptr;
   RKR_TRY(tc_tile_bounds(Pt, BN, split, &tb, st));
   unsigned long long *qcount;
@@ -2083,7 +2120,7 @@ static rkr_status tc_recount_bn(const rkr_index *idx, const TcSide &Ut, const Tc
   e.gacc = tc_gacc(A.kp, split); e.gcan = tc_gcan(idx->d);
   e.seg_start = seg_start; e.seg_len = seg_len; e.ths = ths; e.hist = hist;
   e.hist_hi = hist_hi;
-  set_recount_fields(e, self_col, self_pos, seg_self);
+  set_recount_fields(e, self_col, self_pos, seg_self, thr);
   e.q = PairQueue{qitems, qcount, cap, flags + 1};
   rkr_status s =
       launch_screen<BN, STAGES>(A, Pt, split, row_schedule(nseg, m, BN), e, flags, st);
@@ -2103,9 +2140,9 @@ static rkr_status tc_recount_bn(const rkr_index *idx, const TcSide &Ut, const Tc
   cudaMemcpyAsync(&hq, qcount, sizeof(hq), cudaMemcpyDeviceToHost, st);
   cudaMemcpyAsync(&h64, nfp64, sizeof(h64), cudaMemcpyDeviceToHost, st);
   cudaError_t err = cudaStreamSynchronize(st);
-  for (void *p : {(void *)A.hi, (void *)A.lo, (void *)A.rb1, (void *)A.rb3, (void *)tb,
-                  (void *)qcount, (void *)qitems, (void *)flags, (void *)nfp64})
+  for (void *p : {(void *)tb, (void *)qcount, (void *)qitems, (void *)flags, (void *)nfp64})
     cudaFreeAsync(p, st);
+  tc_gather_free(A, st);
   if (err != cudaSuccess) return cuda_fail(err, "tc_recount");
   RKR_TRY(s);
   if (hf[0]) return fail(RKR_ETIMEOUT, "recount screen wait timed out (%d)", hf[0]);

@@ -108,7 +108,8 @@ rkr_status launch_screen(const TcSide &A, const TcSide &B, int split, const tc::
   // a split product over concatenated operands runs as one pass over K = 3 kp
   const bool cat = split == 1 && tuning().split_cat && A.cat && B.cat && A.cat_role == 1 &&
                    B.cat_role == 2;
-  const __nv_bfloat16 *ah = cat ? A.cat : A.hi, *al = cat ? A.cat : A.lo;
+  // (a side gathered for a single-product screen has no lo part)
+  const __nv_bfloat16 *ah = cat ? A.cat : A.hi, *al = cat ? A.cat : A.lo ? A.lo : A.hi;
   const __nv_bfloat16 *bh = cat ? B.cat : B.hi, *bl = cat ? B.cat : B.lo;
   const int kw = cat ? 3 * A.kp : A.kp;
   const int lda = cat ? tc_pitch(kw) : A.ld(), ldb = cat ? tc_pitch(kw) : B.ld();
