@@ -675,6 +675,30 @@ __global__ void __launch_bounds__(128, 8) k_list_rank(int64_t count, const int32
 // Threads of the per-query filters: a query may have a million candidates.
 constexpr int kFilterThreads = 512;
 
+// Width of a radix key for counts up to `top`: a multiple of 8 bits whose largest
+// value lies above top (it stands for the dropped candidates' ~0, see count_key).
+__host__ __device__ inline int count_bits(uint64_t top) {
+  int bits = 8;
+  while (bits < 32 && (((uint64_t)1 << bits) - 1) <= top) bits += 8;
+  return bits;
+}
+__device__ __forceinline__ uint64_t count_key(uint32_t c, int bits) {
+  return bits < 32 ? min(c, (1u << bits) - 1u) : c;
+}
+// k-th smallest of the counts cc[0 .. cnt) (each at most top, or ~0), walking only
+// the bytes such counts have.
+__device__ __forceinline__ uint64_t block_kth_count(const uint32_t *cc, int64_t cnt, uint64_t k,
+                                                    uint64_t top, uint32_t *hist, uint64_t *bc) {
+  const int bits = count_bits(top);
+  const uint64_t r = block_kth(cnt, k, bits,
+                               [&](int64_t i, uint64_t &key) {
+                                 key = count_key(cc[i], bits);
+                                 return true;
+                               },
+                               hist, bc);
+  return r == ((uint64_t)1 << bits) - 1 ? 0xffffffffull : r;
+}
+
 // Per query: cap = k-th smallest of (exact count, or upper bound for candidates
 // still to be recounted).  A candidate whose lower bound exceeds the cap cannot
 // be among the k smallest ranks: it is dropped from the recount and given the
@@ -682,7 +706,8 @@ constexpr int kFilterThreads = 512;
 __global__ void __launch_bounds__(kFilterThreads)
     k_recount_filter(int qa, const int64_t *__restrict__ qoff, const uint32_t *__restrict__ qcount,
                      const int32_t *__restrict__ kq, uint32_t *__restrict__ ccount,
-                     const uint32_t *__restrict__ clb, int32_t *__restrict__ cu_fb) {
+                     const uint32_t *__restrict__ clb, int32_t *__restrict__ cu_fb,
+                     uint32_t mtop) {
   __shared__ uint32_t hist[256];
   __shared__ uint64_t bc[2];
   const int q = qa + blockIdx.x;
@@ -693,9 +718,7 @@ __global__ void __launch_bounds__(kFilterThreads)
   uint32_t *cc = ccount + base;
   const uint32_t *lb = clb + base;
   int32_t *fb = cu_fb + base;
-  const uint64_t cap = block_kth(cnt, (uint64_t)k, 32,
-                                 [&](int64_t i, uint64_t &key) { key = cc[i]; return true; },
-                                 hist, bc);
+  const uint64_t cap = block_kth_count(cc, cnt, (uint64_t)k, mtop, hist, bc);
   for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x)
     if (fb[i] >= 0 && (uint64_t)lb[i] > cap) {
       fb[i] = -1;
@@ -776,13 +799,21 @@ __global__ void k_prefix_unpark(int64_t n, const int32_t *__restrict__ cu_park,
   if (i < n && cu_park[i] >= 0) cu_fb[i] = cu_park[i];
 }
 
+// Bytes of a user index, in bits.
+static int user_bits(int64_t n) {
+  int bits = 8;
+  while (bits < 32 && ((int64_t)1 << bits) < n) bits += 8;
+  return bits;
+}
+
 // One CTA per query: the k smallest (rank, index) among its candidates.
 __global__ void __launch_bounds__(kSelThreads)
     k_select_exact(int qa, const int64_t *__restrict__ qoff, const uint32_t *__restrict__ qcount,
                    const int32_t *__restrict__ cuid,
                    const uint32_t *__restrict__ ccount, const int32_t *__restrict__ kq,
                    const int64_t *__restrict__ out_off, int32_t *__restrict__ out_users,
-                   int32_t *__restrict__ out_ranks, int *__restrict__ err) {
+                   int32_t *__restrict__ out_ranks, int *__restrict__ err, uint32_t mtop,
+                   int ubits) {
   extern __shared__ unsigned char sbuf[];
   SortEnt *ent = (SortEnt *)sbuf;
   __shared__ uint32_t hist[256];
@@ -798,20 +829,26 @@ __global__ void __launch_bounds__(kSelThreads)
   }
   const int32_t *uid = cuid + base;
   const uint32_t *cc = ccount + base;
-  uint64_t kth = block_kth(cnt, (uint64_t)k, 64,
-                           [&](int64_t i, uint64_t &key) {
-                             key = ((uint64_t)cc[i] << 32) | (uint32_t)uid[i];
-                             return true;
-                           },
-                           hist, bc);
+  // (count, user) packed into the bytes they need: mtop bounds the counts (~0 marks
+  // a dropped candidate), ubits (a multiple of 8) the users
+  const int cbits = count_bits(mtop);
+  auto key_of = [&](int64_t i) {
+    const uint32_t u = uid[i] < 0 ? 0u : (uint32_t)uid[i];   // (dropped: behind every count)
+    return (count_key(cc[i], cbits) << ubits) | u;
+  };
+  const uint64_t kth = block_kth(cnt, (uint64_t)k, cbits + ubits,
+                                 [&](int64_t i, uint64_t &key) {
+                                   key = key_of(i);
+                                   return true;
+                                 },
+                                 hist, bc);
   if (threadIdx.x == 0) gcount = 0;
   __syncthreads();
   for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-    uint64_t key = ((uint64_t)cc[i] << 32) | (uint32_t)uid[i];
-    if (key <= kth) {
+    if (key_of(i) <= kth) {
       int pos = atomicAdd(&gcount, 1);
       if (pos < kMaxK) {
-        ent[pos].k1 = key;
+        ent[pos].k1 = ((uint64_t)cc[i] << 32) | (uint32_t)uid[i];
         ent[pos].k2 = 0;
         ent[pos].idx = (int32_t)i;
       }
@@ -1776,7 +1813,7 @@ static rkr_status grid_prune(const rkr_index *idx, const QueryCommon &qc, int qa
   {
     const int prof_slot = prof_begin("k_recount_filter", st);
     k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount,
-                                                         clb, cu_fb);
+                                                         clb, cu_fb, (uint32_t)idx->m);
     prof_end(prof_slot, st, 0.0);
   }
   note_launch();
@@ -1840,9 +1877,10 @@ static rkr_status prefix_prune(const rkr_index *idx, const QueryCommon &qc, int 
                                recount_users, tuning().rc_single_first ? 0 : 1, 0, ncanon));
   {
     const int prof_slot = prof_begin("k_recount_filter", st);
-    k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount, clb, cu_fb);
+    k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount, clb, cu_fb,
+                                                         (uint32_t)idx->m);
     k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount, clb,
-                                              cu_park);
+                                                         cu_park, (uint32_t)idx->m);
     prof_end(prof_slot, st, 0.0);
   }
   note_launch();
@@ -2349,7 +2387,8 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
       RKR_CUDA(cudaGetLastError());
       {
         const int prof_slot = prof_begin("k_recount_filter", st);
-        k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount, clb, cu_fb);
+        k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount, clb, cu_fb,
+                                                         (uint32_t)idx->m);
         prof_end(prof_slot, st, 0.0);
       }
       note_launch();
@@ -2409,7 +2448,7 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
           {
             const int prof_slot = prof_begin("k_recount_filter", st);
             k_recount_filter<<<qb - qa, kFilterThreads, 0, st>>>(qa, qoff_rel, cursor, qc.kq_d, ccount,
-                                                     clb, cu_fb);
+                                                     clb, cu_fb, (uint32_t)idx->m);
             prof_end(prof_slot, st, 0.0);
           }
           note_launch();
@@ -2464,7 +2503,8 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
     {
       const int prof_slot = prof_begin("k_select_exact", st);
       k_select_exact<<<qb - qa, kSelThreads, sm, st>>>(qa, qoff_rel, cursor, cu, ccount, qc.kq_d,
-                                                       qc.out_off_d, users_d, ranks_d, sel_err);
+                                                       qc.out_off_d, users_d, ranks_d, sel_err,
+                                                       (uint32_t)idx->m, user_bits(idx->n));
       prof_end(prof_slot, st, 0.0);
     }
     note_launch();

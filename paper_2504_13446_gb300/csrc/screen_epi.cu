@@ -815,6 +815,7 @@ struct EpiDeep {
   static const char *name() { return "k_screen<EpiDeep>"; }
   static constexpr int kWarps = 16;
   static constexpr int kBins = kDGrid + 1;
+  static constexpr unsigned kDense = 8;   // marked scores of a lane per chunk
   struct Thread {
     float b, top_lo;     // bound; lower ends above top_lo are above the whole grid
     float bot_hi;        // upper ends below bot_hi are below the whole grid
@@ -869,36 +870,53 @@ struct EpiDeep {
     if (left < 32) mask &= left <= 0 ? 0u : (1u << left) - 1u;
     const BinFP &bf = ts.bf;
     const bool fast = bf.invd32 > 0.0f && bf.err <= 1e6f;   // the row's grid has a step
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) tile[j * 32] = v[16 * h + j];
-    uint32_t mine = h ? mask >> 16 : mask & 0xffffu;
-    while (mine) {
-      const int j = __ffs(mine) - 1;
-      mine &= mine - 1;
-      const float x = tile[j * 32];
-      const float lo = __fsub_rd(x, ts.b), hi = __fadd_ru(x, ts.b);
-      int jl, jh;
-      if (fast) {
-        // bin_interval without branches: the clamps of bin_lo / bin_hi by fminf /
-        // fmaxf (which also send a NaN lower end to 0), a NaN upper end to G
-        float vlo, vhi;
-        bin_coord(bf, lo, hi, vlo, vhi);
-        jl = (int)ceilf(fminf(fmaxf(vlo, 0.0f), (float)kDGrid));
-        const float ch = fminf(floorf(fmaxf(vhi, -1.0f)) + 1.0f, (float)kDGrid);
-        jh = vhi == vhi ? (int)ch : kDGrid;
-      } else {
-        bin_interval(bf, ts.g0, kDGrid, lo, hi, jl, jh);
-      }
-      // certainly above the whole grid: c = G exactly; jh = 0 adds to bin 0, which no
-      // count reads
+    // Adds one score to both histograms.  Certainly above the whole grid: c = G
+    // exactly; jh = 0 adds to bin 0, which no count reads.
+    auto add = [&](const float lo, int jl, int jh, const bool in) {
       const bool top = lo > ts.top_lo;
       jl = top ? kDGrid : jl;
       jh = top ? kDGrid : jh;
-      atomicAdd(&hlo(S, r)[jl * 128], 1u);
-      atomicAdd(&hhi(S, r)[jh * 128], 1u);
+      if (in) {
+        atomicAdd(&hlo(S, r)[jl * 128], 1u);
+        atomicAdd(&hhi(S, r)[jh * 128], 1u);
+      }
+    };
+    auto count_fast = [&](const float x, const bool in) {
+      // bin_interval without branches: the clamps of bin_lo / bin_hi by fminf /
+      // fmaxf (which also send a NaN lower end to 0), a NaN upper end to G
+      const float lo = __fsub_rd(x, ts.b), hi = __fadd_ru(x, ts.b);
+      float vlo, vhi;
+      bin_coord(bf, lo, hi, vlo, vhi);
+      const int jl = (int)ceilf(fminf(fmaxf(vlo, 0.0f), (float)kDGrid));
+      const float ch = fminf(floorf(fmaxf(vhi, -1.0f)) + 1.0f, (float)kDGrid);
+      add(lo, jl, vhi == vhi ? (int)ch : kDGrid, in);
+    };
+    // A lane's marked scores are walked one after another, each a serial chain of a
+    // shared load and the bin arithmetic; where a lane of the warp has many, all 32
+    // columns are taken instead, from registers and independent of each other.
+    if (__reduce_max_sync(__activemask(), (unsigned)__popc(mask)) >= kDense && fast) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) count_fast(v[j], (mask >> j) & 1u);
+      return;
     }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) tile[j * 32] = v[16 * h + j];
+      uint32_t mine = h ? mask >> 16 : mask & 0xffffu;
+      while (mine) {
+        const int j = __ffs(mine) - 1;
+        mine &= mine - 1;
+        const float x = tile[j * 32];
+        if (fast) {
+          count_fast(x, true);
+        } else {
+          const float lo = __fsub_rd(x, ts.b), hi = __fadd_ru(x, ts.b);
+          int jl, jh;
+          bin_interval(bf, ts.g0, kDGrid, lo, hi, jl, jh);
+          add(lo, jl, jh, true);
+        }
+      }
     }
   }
   __device__ void tile_end(char *, int, int, int, int, Thread &) const {}
@@ -1189,7 +1207,7 @@ struct EpiTheta {
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (on[i] && lb[i] <= caps(S)[cl[i]]) emit(qglob(S)[cl[i]], ts.u, x[i]);
+          emit(on[i] && lb[i] <= caps(S)[cl[i]], qglob(S)[cl[i]], ts.u, x[i]);
       }
     }
   }
@@ -1200,9 +1218,17 @@ struct EpiTheta {
     if (bkt >= kFine) bkt = kFine - 1;
     atomicAdd(&fine[(int64_t)q * kFine + bkt], 1u);
   }
-  __device__ void emit(int q, int64_t u, float x) const {
-    uint32_t pos = atomicAdd(&qcursor[q], 1u);
-    int64_t at = qoff[q] + pos;
+  // The whole warp, at one query: the lanes with `take` reserve their slots of the
+  // query's segment together.
+  __device__ void emit(bool take, int q, int64_t u, float x) const {
+    const unsigned act = __ballot_sync(0xffffffffu, take);
+    if (!act) return;
+    const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
+    uint32_t base = 0;
+    if (lane == leader) base = atomicAdd(&qcursor[q], (uint32_t)__popc(act));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (!take) return;
+    const int64_t at = qoff[q] + base + __popc(act & ((1u << lane) - 1u));
     if (at >= qoff[q + 1]) {  // more than the pass-1 count: never written out of the segment
       atomicExch(ovf, 1);
       return;
