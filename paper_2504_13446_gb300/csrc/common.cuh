@@ -78,11 +78,42 @@ struct ProfScope {
 
 // ------------------------------------------------------- canonical scores
 
-// s(a, b): left-to-right FP64 sum of exact float products.
+// FP64 is scarce on this GPU (a dependent FP64 operation takes some 300 cycles and
+// a warp's FP64 instruction about 60 cycles of its SM whatever the active lanes),
+// so hot code decides with FP32 bounds and forms canonical scores only for what
+// those leave open.  Rows are read 16 bytes at a time where both allow it: a
+// thread per pair touches 32 lines per warp and load either way.
+
+__device__ __forceinline__ bool rows_vec4(const float *a, const float *b, int d) {
+  return (d & 3) == 0 && ((((uintptr_t)a) | ((uintptr_t)b)) & 15) == 0;
+}
+
+// Calls f(a[k], b[k]) for k = 0 .. d - 1 in order.
+template <class F>
+__device__ __forceinline__ void for_pairs(const float *__restrict__ a,
+                                          const float *__restrict__ b, int d, F &&f) {
+  if (rows_vec4(a, b, d)) {
+    const float4 *a4 = reinterpret_cast<const float4 *>(a);
+    const float4 *b4 = reinterpret_cast<const float4 *>(b);
+#pragma unroll 2
+    for (int k = 0; k < d >> 2; ++k) {
+      const float4 x = a4[k], y = b4[k];
+      f(x.x, y.x);
+      f(x.y, y.y);
+      f(x.z, y.z);
+      f(x.w, y.w);
+    }
+  } else {
+    for (int k = 0; k < d; ++k) f(a[k], b[k]);
+  }
+}
+
+// s(a, b): left-to-right FP64 sum of exact float products (the product of two
+// floats is exact in FP64, so one FMA rounds exactly like the addition alone).
 __device__ __forceinline__ double canon_dot(const float *__restrict__ a,
                                             const float *__restrict__ b, int d) {
   double acc = 0.0;
-  for (int k = 0; k < d; ++k) acc = __dadd_rn(acc, __dmul_rn((double)a[k], (double)b[k]));
+  for_pairs(a, b, d, [&](float x, float y) { acc = __fma_rn((double)x, (double)y, acc); });
   return acc;
 }
 
@@ -92,20 +123,17 @@ static __device__ __noinline__ double canon_dot_slow(const float *__restrict__ a
   return canon_dot(a, b, d);
 }
 
-// Interval [lo, hi] that holds the canonical score s(a, b).  A compensated FP32
-// dot product (Ogita, Rump and Oishi's Dot2: each product split exactly by an
-// FMA, each addition by an error-free two-sum, the low parts summed apart)
-// satisfies |(p + s) - a.b| <= gamma_d^2 sum|a_k b_k| (gamma_d = d u / (1 - d u),
-// u = 2^-24); the final p + s is formed in FP64 (error <= 2^-53 |p + s|) and the
-// canonical sum differs from a.b by at most gamma'_d sum|a_k b_k| with the FP64
-// unit 2^-53.  Intrinsics keep the compiler from fusing or reordering the steps.
-// A tiny absolute term covers products in the subnormal range.
-__device__ __forceinline__ void dot2_interval(const float *__restrict__ a,
-                                              const float *__restrict__ b, int d, double &lo,
-                                              double &hi) {
+// A compensated FP32 dot product (Ogita, Rump and Oishi's Dot2: each product split
+// exactly by an FMA, each addition by an error-free two-sum, the low parts summed
+// apart): p + s, with |(p + s) - a.b| <= gamma_d^2 sum|a_k b_k| (gamma_d = d u /
+// (1 - d u), u = 2^-24).  The canonical sum differs from a.b by at most gamma'_d
+// sum|a_k b_k| with the FP64 unit 2^-53.  err bounds |(p + s) - s(a, b)| and the
+// rounding of p + s to double, in FP32 rounded up: gamma_d <= g (1 + 2 g) for
+// g = d u <= 1/4, and a tiny absolute term covers products in the subnormal range.
+// Intrinsics keep the compiler from fusing or reordering the steps.
+struct Dot2 {
   float p = 0.0f, s = 0.0f, asum = 0.0f;
-  for (int k = 0; k < d; ++k) {
-    const float x = a[k], y = b[k];
+  __device__ __forceinline__ void add(float x, float y) {
     const float h = __fmul_rn(x, y);
     const float r = __fmaf_rn(x, y, -h);
     const float t = __fadd_rn(p, h);
@@ -115,14 +143,37 @@ __device__ __forceinline__ void dot2_interval(const float *__restrict__ a,
     s = __fadd_rn(s, __fadd_rn(e, r));
     asum = __fadd_ru(asum, fabsf(h));
   }
-  const double res = (double)p + (double)s;
-  const double g = (double)d * 0x1p-24;
-  const double gam = g / (1.0 - g);
-  const double gc = (double)d * 0x1p-53 / (1.0 - (double)d * 0x1p-53);
-  const double E = ((gam * gam + gc) * (double)asum * (1.0 + 0x1p-20) + fabs(res) * 0x1p-52 +
-                    (double)d * 0x1p-140) * (1.0 + 0x1p-20);
+  // roundings: how many additions a term can pass through (d for one chain)
+  __device__ __forceinline__ float err(int roundings) const {
+    const float g = (float)roundings * 0x1p-24f;
+    const float gam = __fmul_ru(g, __fadd_ru(1.0f, 2.0f * g));
+    const float c = __fmaf_ru(gam, gam, __fmul_ru((float)roundings, 0x1.0001p-53f));
+    const float e = __fadd_ru(__fmul_ru(c, asum),
+                              __fmul_ru(__fadd_ru(fabsf(p), fabsf(s)), 0x1p-52f));
+    return __fmul_ru(__fadd_ru(e, (float)roundings * 0x1p-140f), 1.0f + 0x1p-19f);
+  }
+};
+
+// Interval [lo, hi] that holds the canonical score s(a, b).
+__device__ __forceinline__ void dot2_interval(const float *__restrict__ a,
+                                              const float *__restrict__ b, int d, double &lo,
+                                              double &hi) {
+  Dot2 t;
+  for_pairs(a, b, d, [&](float x, float y) { t.add(x, y); });
+  const double res = (double)t.p + (double)t.s, E = (double)t.err(d);
   lo = res - E;
   hi = res + E;
+}
+
+// The same rounded outwards to float, without FP64 operations.
+__device__ __forceinline__ void dot2_interval_f(const float *__restrict__ a,
+                                                const float *__restrict__ b, int d, float &lo,
+                                                float &hi) {
+  Dot2 t;
+  for_pairs(a, b, d, [&](float x, float y) { t.add(x, y); });
+  const float E = t.err(d);
+  lo = __fsub_rd(__fadd_rd(t.p, t.s), E);
+  hi = __fadd_ru(__fadd_ru(t.p, t.s), E);
 }
 
 // Threshold t_{j+1} (0-based i = j): f_min + i * delta, delta = (f_max - f_min) / (tau - 1),
@@ -131,13 +182,24 @@ __device__ __forceinline__ double thr_at(double fmin, double delta, int i) {
   return __dadd_rn(fmin, __dmul_rn((double)i, delta));
 }
 
+// A first guess of #{i : t_i <= theta} for a grid with step delta, from FP32 where
+// the step allows it (the callers' comparisons make it exact).
+__device__ __forceinline__ int grid_guess(double theta, double fmin, double delta, int tau) {
+  const float df = (float)delta;
+  if (df > 1e-30f && df < 1e30f) {
+    const float x = __fdividef((float)(theta - fmin), df);
+    return x < 0.0f ? 0 : (x >= (float)tau ? tau : (int)x + 1);
+  }
+  const double x = (theta - fmin) / delta;
+  return x < 0.0 ? 0 : (x >= (double)tau ? tau : (int)floor(x) + 1);
+}
+
 // j(theta) = #{i in [0, tau) : t_i <= theta}: the 1-based index of the largest
 // threshold not above theta (0 when theta < t_1), Section 4.3 step 1.
 __device__ __forceinline__ int exact_j(double theta, double fmin, double delta, int tau) {
   int g;
   if (delta > 0.0) {
-    double x = (theta - fmin) / delta;
-    g = x < 0.0 ? 0 : (x >= (double)tau ? tau : (int)floor(x) + 1);
+    g = grid_guess(theta, fmin, delta, tau);
   } else {
     g = theta >= fmin ? tau : 0;
   }
@@ -165,8 +227,7 @@ __device__ __forceinline__ double interp_est(double theta, int j, uint32_t nlo, 
 __device__ __forceinline__ int exact_c(double s, double fmin, double delta, int tau) {
   int g;
   if (delta > 0.0) {
-    double x = (s - fmin) / delta;
-    g = x < 0.0 ? 0 : (x >= (double)tau ? tau : (int)floor(x) + 1);
+    g = grid_guess(s, fmin, delta, tau);
   } else {
     g = s > fmin ? tau : 0;
   }
@@ -228,6 +289,41 @@ __device__ __forceinline__ void bin_interval(const BinFP &b, double fmin, int ta
   jlo = bin_lo(vlo, tau);
   jhi = bin_hi(vhi, tau);
 }
+
+// bin_interval with an error that follows the values: the FP32 coordinate
+// (v - f)(1/dx), f = fl(g0), taken with directed roundings, is within
+// e(v) = (|v - f| 2^-21 + |g0| 2^-23) / dx of (v - g0) / dx: the roundings of f, of
+// 1/dx, of the difference and of the product add up to less than
+// |g0| 2^-24 / dx + |v - f| 2^-21.6 / dx.  (1/dx <= invd32 (1 + 2^-22), since invd32
+// is 1/dx rounded to nearest twice, and |g0| <= |f| (1 + 2^-23); both factors are
+// formed in FP32 rounding up.)  Valid for every v, whatever range err was made
+// for; usable() is false for grids without a usable step.
+struct TightBins {
+  float f, inv, e0, e1;
+  bool ok;
+  __device__ __forceinline__ explicit TightBins(const BinFP &b) {
+    f = b.fmin32;
+    inv = b.invd32;
+    ok = b.invd32 > 0.0f && b.err <= 1e6f;
+    const float inv_up = __fmul_ru(b.invd32, 1.0f + 0x1p-22f);
+    e1 = __fmul_ru(inv_up, 0x1p-21f * (1.0f + 0x1p-20f));
+    e0 = __fadd_ru(__fmul_ru(__fmul_ru(fabsf(b.fmin32), (1.0f + 0x1p-23f) * 0x1p-23f), inv_up),
+                   0x1p-30f);
+  }
+  __device__ __forceinline__ bool usable() const { return ok; }
+  // lower bound of #{x_j <= v} (and of #{x_j < v}) over G columns
+  __device__ __forceinline__ int lo(float v, int G) const {
+    const float a = __fsub_rd(v, f);
+    const float e = __fmaf_ru(fmaxf(fabsf(a), fabsf(__fsub_ru(v, f))), e1, e0);
+    return bin_lo(__fsub_rd(__fmul_rd(a, inv), e), G);
+  }
+  // upper bound of the same
+  __device__ __forceinline__ int hi(float v, int G) const {
+    const float a = __fsub_ru(v, f);
+    const float e = __fmaf_ru(fmaxf(fabsf(a), fabsf(__fsub_rd(v, f))), e1, e0);
+    return bin_hi(__fadd_ru(__fmul_ru(a, inv), e), G);
+  }
+};
 
 // FP32 screen bound: |fma-chain(u,x) - s(u,x)| <= cfac * |u| * |x| with
 // cfac = ((d + 4) 2^-24 + d 2^-53 + 2^-40)(1 + 2^-20); nu, nx are FP32 upper

@@ -166,9 +166,9 @@ __global__ void k_resolve_approx(int64_t count, const int32_t *__restrict__ cu,
     bin_interval(bf[u], fmin[u], tau, __fsub_rd(x, b), __fadd_ru(x, b), jlo, jhi);
   }
   if (jlo != jhi) {
-    double tlo, thi;
-    dot2_interval(uu, qq, d, tlo, thi);
-    bin_interval(bf[u], fmin[u], tau, __double2float_rd(tlo), __double2float_ru(thi), jlo, jhi);
+    float tlo, thi;
+    dot2_interval_f(uu, qq, d, tlo, thi);
+    bin_interval(bf[u], fmin[u], tau, tlo, thi, jlo, jhi);
   }
   int j;
   if (jlo == jhi) {
@@ -188,12 +188,23 @@ __global__ void k_resolve_approx(int64_t count, const int32_t *__restrict__ cu,
 struct ApproxCand {
   const int32_t *uid;
   const uint32_t *nlo, *nup;
-  double *th;          // canonical u.q, NaN until formed
+  double *th;          // canonical u.q (NaN: not formed); overwritten by estimates
   const int32_t *j;
   const float *U, *Q;  // rows, for forming u.q on demand
   int d;
   unsigned long long *nfp64;   // canonical products formed (may be null)
 };
+
+// Width of a radix key for counts up to `top`: a multiple of 8 bits whose largest
+// value lies above top (it stands for the dropped candidates' ~0, see count_key).
+__host__ __device__ inline int count_bits(uint64_t top) {
+  int bits = 8;
+  while (bits < 32 && (((uint64_t)1 << bits) - 1) <= top) bits += 8;
+  return bits;
+}
+__device__ __forceinline__ uint64_t count_key(uint32_t c, int bits) {
+  return bits < 32 ? min(c, (1u << bits) - 1u) : c;
+}
 
 constexpr int kSelThreads = 256;
 
@@ -206,7 +217,7 @@ __global__ void __launch_bounds__(kSelThreads)
                     const int64_t *__restrict__ out_off, int32_t *__restrict__ out_users,
                     uint32_t *__restrict__ out_nlo, uint32_t *__restrict__ out_nup,
                     double *__restrict__ out_est, int32_t *__restrict__ out_case,
-                    int32_t *__restrict__ out_nc, int *__restrict__ err) {
+                    int32_t *__restrict__ out_nc, int *__restrict__ err, uint32_t top) {
   extern __shared__ unsigned char sbuf[];
   SortEnt *ent = (SortEnt *)sbuf;                   // kMaxK entries
   __shared__ uint32_t hist[256];
@@ -226,20 +237,22 @@ __global__ void __launch_bounds__(kSelThreads)
   double *th = C.th + base;
   const int32_t *cj = C.j + base;
   const float *qrow = C.Q + (int64_t)q * C.d;
+  // Step-3 estimate from the canonical u.q: some 40 FP64 operations and, where u.q
+  // is not formed yet, a canonical product, so each candidate's is formed once.
   auto est_of = [&](int64_t i) {
     int32_t u = uid[i];
     double t = th[i];
-    if (t != t) {  // not formed yet: the canonical u.q, kept for later calls
+    if (t != t) {  // not formed yet
       t = canon_dot(C.U + (int64_t)u * C.d, qrow, C.d);
-      th[i] = t;
       if (C.nfp64) atomicAdd(C.nfp64, 1ull);
     }
     return interp_est(t, cj[i], nlo[i], nup[i], fmin[u], delta[u], tau, s);
   };
-  // Step 1: k-th smallest lower and upper bound numerators.
-  uint64_t Rlo = block_kth(cnt, (uint64_t)k, 32,
+  // Step 1: k-th smallest lower and upper bound numerators (at most top).
+  const int nbits = count_bits(top);
+  uint64_t Rlo = block_kth(cnt, (uint64_t)k, nbits,
                            [&](int64_t i, uint64_t &key) { key = nlo[i]; return true; }, hist, bc);
-  uint64_t Rup = block_kth(cnt, (uint64_t)k, 32,
+  uint64_t Rup = block_kth(cnt, (uint64_t)k, nbits,
                            [&](int64_t i, uint64_t &key) { key = nup[i]; return true; }, hist, bc);
   const double lhs = c * (double)((uint64_t)s + Rlo);
   const bool caseA = lhs >= (double)((uint64_t)s + Rup);
@@ -284,7 +297,10 @@ __global__ void __launch_bounds__(kSelThreads)
     nc = k;
   } else {
     // U_c = {r_up <= c R_low_k}: fewer than k users, (r_up, r_low, index) order
-    auto in_c = [&](int64_t i) { return (double)((uint64_t)s + nup[i]) <= lhs; };
+    // s + nup <= c (s + R_low_k): integers (below 2^53) against a real, so against
+    // its floor
+    const uint64_t lim = (uint64_t)floor(lhs);
+    auto in_c = [&](int64_t i) { return (uint64_t)s + nup[i] <= lim; };
     if (threadIdx.x == 0) gcount = 0;
     __syncthreads();
     for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
@@ -308,23 +324,39 @@ __global__ void __launch_bounds__(kSelThreads)
       if (out_est) out_est[obase + r] = est_of(i);
     }
     __syncthreads();
-    // Step 3: survivors r_low <= R_up_k outside U_c, smallest (r_hat, index)
+    // Step 3: survivors r_low <= R_up_k outside U_c, smallest (r_hat, index); their
+    // estimates take the place of u.q in th, formed in full warps: the survivors'
+    // indices are gathered in shared memory first where they fit
     auto in_t = [&](int64_t i) { return (uint64_t)nlo[i] <= Rup && !in_c(i); };
     const int need = k - nc;
+    int *todo = (int *)sbuf;
+    constexpr int kTodo = (int)(sizeof(SortEnt) * kMaxK / sizeof(int));
+    if (threadIdx.x == 0) gcount = 0;
+    __syncthreads();
+    for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
+      if (!in_t(i)) continue;
+      const int pos = atomicAdd(&gcount, 1);
+      if (pos < kTodo) todo[pos] = (int)i;
+      else th[i] = est_of(i);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < min(gcount, kTodo); e += blockDim.x)
+      th[todo[e]] = est_of(todo[e]);
+    __syncthreads();
     uint64_t ke = block_kth(cnt, (uint64_t)need, 64,
                             [&](int64_t i, uint64_t &key) {
                               if (!in_t(i)) return false;
-                              key = dkey(est_of(i));
+                              key = dkey(th[i]);
                               return true;
                             },
                             hist, bc);
-    int64_t below = block_count(cnt, [&](int64_t i) { return in_t(i) && dkey(est_of(i)) < ke; },
+    int64_t below = block_count(cnt, [&](int64_t i) { return in_t(i) && dkey(th[i]) < ke; },
                                 &cnt_acc);
     uint64_t ku = ~0ull;
     if (below < need)
       ku = block_kth(cnt, (uint64_t)(need - below), 32,
                      [&](int64_t i, uint64_t &key) {
-                       if (!in_t(i) || dkey(est_of(i)) != ke) return false;
+                       if (!in_t(i) || dkey(th[i]) != ke) return false;
                        key = (uint32_t)uid[i];
                        return true;
                      },
@@ -333,8 +365,7 @@ __global__ void __launch_bounds__(kSelThreads)
     __syncthreads();
     for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
       if (!in_t(i)) continue;
-      double e = est_of(i);
-      uint64_t ek = dkey(e);
+      uint64_t ek = dkey(th[i]);
       if (ek < ke || (ek == ke && (uint64_t)(uint32_t)uid[i] <= ku)) {
         int pos = atomicAdd(&gcount, 1);
         if (pos < kMaxK) {
@@ -520,11 +551,11 @@ __global__ void k_scatter_counts(int64_t nseg, const int64_t *__restrict__ seg_s
 // The deep count grid of an index (dg = 0: none).
 struct DeepGrid {
   int dg;
-  const double *yg0, *ydx;
+  const BinFP *ybin;
   const uint32_t *DLO, *DHI;
 };
 inline DeepGrid deep_grid(const rkr_index *idx) {
-  return DeepGrid{idx->dg, idx->yg0, idx->ydx, idx->DLO, idx->DHI};
+  return DeepGrid{idx->dg, idx->ybin, idx->DLO, idx->DHI};
 }
 
 // Exact ranks from the tail lists.  A candidate (u, q) with u.q >= x_0(u)
@@ -532,7 +563,7 @@ inline DeepGrid deep_grid(const rkr_index *idx) {
 // x_0 is in the list.  Entries are grouped by exact-grid column: whole
 // columns are counted from the column offsets, and the entries of the one or
 // two columns within the screen bound of u.q are settled one by one, by their
-// own bound, an FP32 dot product with its bound, or canonically.  Candidates below x_0 (or with an overflowed list) are
+// own bound, a compensated product, or canonically.  Candidates below x_0 (or with an overflowed list) are
 // passed on, unchanged, in cu_fb for the recount screen; others get -1 there.
 // 64 registers a thread (eight 128-thread blocks per SM): the kernel waits on
 // scattered reads of each candidate's user data and list, so warps in flight matter.
@@ -548,7 +579,8 @@ __global__ void __launch_bounds__(128, 8) k_list_rank(int64_t count, const int32
                             const float *__restrict__ xbmax, const tc::RowBound *__restrict__ rb3,
                             const tc::RowBound *__restrict__ ptile, int pbn, tc::Gacc gacc,
                             float gcan, const double *__restrict__ xg0,
-                            const double *__restrict__ xdx, int GX, const double *__restrict__ ldx,
+                            const BinFP *__restrict__ xbin, int GX,
+                            const double *__restrict__ ldx, const BinFP *__restrict__ lbin,
                             int G, const uint32_t *__restrict__ XLO,
                             const uint32_t *__restrict__ XHI, uint32_t mtop,
                             uint32_t *__restrict__ ccount, uint32_t *__restrict__ clb,
@@ -565,52 +597,73 @@ __global__ void __launch_bounds__(128, 8) k_list_rank(int64_t count, const int32
   }
   const float *uu = U + u * d;
   const float *qq = Q + (int64_t)cq[i] * d;
-  // u.q as an interval [tlo, thi], tightened only where a comparison needs it:
-  // first the candidate's screened score and its bound (no row is read), then
-  // the compensated product, then the canonical value
+  // u.q as an interval, tightened only where a comparison needs it: first the
+  // candidate's screened score and its bound (no row is read), then the
+  // compensated product, then the canonical value.  [flo, fhi] are its ends in
+  // float, enough for every comparison with a screened entry; tlo, thi and theta
+  // hold them in FP64 from the compensated product on.
+  float flo = -INFINITY, fhi = INFINITY;
   double tlo = -INFINITY, thi = INFINITY;
   int state = 1;   // 0: screened interval, 1: compensated, 2: canonical
+  auto compensate = [&]() {
+    dot2_interval(uu, qq, d, tlo, thi);
+    flo = __double2float_rd(tlo);
+    fhi = __double2float_ru(thi);
+    state = 1;
+  };
   const float sx = cx ? cx[i] : __int_as_float(0x7fffffff);
   if (sx == sx) {
     const float b = tc::screen_bound_tc(rb3[u], qrb[cq[i]], gacc, gcan);
-    tlo = (double)__fsub_rd(sx, b);
-    thi = (double)__fadd_ru(sx, b);
+    flo = __fsub_rd(sx, b);
+    fhi = __fadd_ru(sx, b);
     state = 0;
   } else {
-    dot2_interval(uu, qq, d, tlo, thi);
+    compensate();
   }
   double theta = 0.0;
   auto tighten = [&]() {
     if (state == 0) {
-      dot2_interval(uu, qq, d, tlo, thi);
-      state = 1;
+      compensate();
     } else {
       theta = canon_dot(uu, qq, d);
       tlo = thi = theta;
+      flo = __double2float_rd(theta);
+      fhi = __double2float_ru(theta);
       state = 2;
       atomicAdd(&stat[4], 1ull);
     }
   };
   const uint32_t L = xlcnt[u];
-  const double x0 = xg0[u];
-  while (state < 2 && L <= xlcap[u] && tlo < x0 && thi >= x0) tighten();
-  if (L > xlcap[u] || thi < x0) {
-    // bounds from the exact count table at the bins of both ends of u.q
-    int jl = exact_j(tlo, x0, xdx[u], GX), jh = exact_j(thi, x0, xdx[u], GX);
-    const int G2 = deep.dg;
-    const bool below = G2 > 0 && thi < x0;
-    int kl = 0, kh = 0;
-    if (below) {
-      kl = exact_j(tlo, deep.yg0[u], deep.ydx[u], G2);
-      kh = exact_j(thi, deep.yg0[u], deep.ydx[u], G2);
+  const bool full = L > xlcap[u];   // the list overflowed: not usable
+  // u.q against x_0, whose nearest float is the list grid's origin
+  const BinFP lb = lbin[u];
+  bool under = fhi < nextafterf(lb.fmin32, -INFINITY);
+  if (!under && flo < nextafterf(lb.fmin32, INFINITY)) {   // not decided in float
+    const double x0 = xg0[u];
+    if (state == 0) {
+      tlo = (double)flo;
+      thi = (double)fhi;
     }
-    if (state == 0 && (jl != jh || kl != kh)) {   // as tight as the compensated product gives
-      tighten();
-      jl = exact_j(tlo, x0, xdx[u], GX);
-      jh = exact_j(thi, x0, xdx[u], GX);
-      if (below) {
-        kl = exact_j(tlo, deep.yg0[u], deep.ydx[u], G2);
-        kh = exact_j(thi, deep.yg0[u], deep.ydx[u], G2);
+    while (state < 2 && !full && tlo < x0 && thi >= x0) tighten();
+    under = thi < x0;
+  }
+  if (full || under) {
+    // bounds from the exact count table at the bins of both ends of u.q (below x_0:
+    // before its first column)
+    int jl = 0, jh = 0;
+    if (!under) {
+      const TightBins tb(xbin[u]);
+      jl = tb.usable() ? tb.lo(flo, GX) : 0;
+      jh = tb.usable() ? tb.hi(fhi, GX) : GX;
+    }
+    const int G2 = deep.dg;
+    const bool below = G2 > 0 && under;
+    int kl = 0, kh = G2;
+    if (below) {
+      const TightBins tb(deep.ybin[u]);
+      if (tb.usable()) {
+        kl = tb.lo(flo, G2);
+        kh = tb.hi(fhi, G2);
       }
     }
     uint32_t ub = jl >= 1 ? XHI[u * GX + jl - 1] : mtop;
@@ -630,12 +683,21 @@ __global__ void __launch_bounds__(128, 8) k_list_rank(int64_t count, const int32
   // entries are grouped by column c = #{x_j <= v}: x_{c-1} <= v < x_c
   const uint2 *row = xlist + xloff[u];
   const uint16_t *co = xcoff + u * (G + 2);
-  const double B = (double)xbmax[u];
-  const double g0 = xg0[u], dx = ldx[u];
-  // columns c >= chi have v >= x_{c-1} > u.q + B: every entry is above u.q
-  const int chi = exact_j(__dadd_ru(thi, B), g0, dx, G) + 1;
-  // columns c < clo have v < x_c <= u.q - B: no entry is above u.q
-  const int clo = exact_j(__dsub_rd(tlo, B), g0, dx, G);
+  const float B = xbmax[u];
+  // columns c >= chi have v >= x_{c-1} > u.q + B: every entry is above u.q;
+  // columns c < clo have v < x_c <= u.q - B: no entry is above u.q (an upper and a
+  // lower bound of these columns serve as well: the entries between are settled
+  // one by one)
+  int chi, clo;
+  const TightBins tb(lb);
+  if (tb.usable()) {
+    chi = tb.hi(__fadd_ru(fhi, B), G) + 1;
+    clo = tb.lo(__fsub_rd(flo, B), G);
+  } else {
+    const double g0 = xg0[u], dx = ldx[u];
+    chi = exact_j((double)__fadd_ru(fhi, B), g0, dx, G) + 1;
+    clo = exact_j((double)__fsub_rd(flo, B), g0, dx, G);
+  }
   uint32_t above = L - (uint32_t)co[chi];
   const tc::RowBound ru = rb3[u];
   const int32_t self = qself[cq[i]];
@@ -644,8 +706,8 @@ __global__ void __launch_bounds__(128, 8) k_list_rank(int64_t count, const int32
     if ((int32_t)p == self) continue;  // the query's own item: s(u,p) = u.q, not above
     const float v = __uint_as_float(row[e].y);
     const float b = tc::screen_bound_tc(ru, ptile[p / pbn], gacc, gcan);
-    if ((double)__fsub_rd(v, b) > thi) { ++above; continue; }
-    if ((double)__fadd_ru(v, b) <= tlo) continue;
+    if (__fsub_rd(v, b) > fhi) { ++above; continue; }
+    if (__fadd_ru(v, b) <= flo) continue;
     if (state == 0) {   // the screened interval of u.q cannot place it: compensate, look again
       tighten();
       --e;
@@ -675,16 +737,6 @@ __global__ void __launch_bounds__(128, 8) k_list_rank(int64_t count, const int32
 // Threads of the per-query filters: a query may have a million candidates.
 constexpr int kFilterThreads = 512;
 
-// Width of a radix key for counts up to `top`: a multiple of 8 bits whose largest
-// value lies above top (it stands for the dropped candidates' ~0, see count_key).
-__host__ __device__ inline int count_bits(uint64_t top) {
-  int bits = 8;
-  while (bits < 32 && (((uint64_t)1 << bits) - 1) <= top) bits += 8;
-  return bits;
-}
-__device__ __forceinline__ uint64_t count_key(uint32_t c, int bits) {
-  return bits < 32 ? min(c, (1u << bits) - 1u) : c;
-}
 // k-th smallest of the counts cc[0 .. cnt) (each at most top, or ~0), walking only
 // the bytes such counts have.
 __device__ __forceinline__ uint64_t block_kth_count(const uint32_t *cc, int64_t cnt, uint64_t k,
@@ -1636,10 +1688,7 @@ __device__ __forceinline__ void cand_interval(int64_t u, int q, float x,
     lo = __fsub_rd(x, b);
     hi = __fadd_ru(x, b);
   } else {
-    double l, h;
-    dot2_interval(U + u * d, Q + (int64_t)q * d, d, l, h);
-    lo = __double2float_rd(l);
-    hi = __double2float_ru(h);
+    dot2_interval_f(U + u * d, Q + (int64_t)q * d, d, lo, hi);
   }
 }
 
@@ -1703,8 +1752,8 @@ __global__ void k_grid_bound(int64_t cnt, const int32_t *__restrict__ cu_fb,
                              const tc::RowBound *__restrict__ urb,
                              const tc::RowBound *__restrict__ qrb, tc::Gacc gacc, float gcan,
                              const float *__restrict__ U, const float *__restrict__ Q, int d,
-                             const int32_t *__restrict__ uslot, const double *__restrict__ yg0,
-                             const double *__restrict__ ydx, const uint32_t *__restrict__ CLO,
+                             const int32_t *__restrict__ uslot, const BinFP *__restrict__ ybin,
+                             const uint32_t *__restrict__ CLO,
                              const uint32_t *__restrict__ CHI, uint32_t *__restrict__ ccount,
                              uint32_t *__restrict__ clb) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1714,8 +1763,9 @@ __global__ void k_grid_bound(int64_t cnt, const int32_t *__restrict__ cu_fb,
   float lo, hi;
   cand_interval(u, cq[i], cx[i], urb, qrb, gacc, gcan, U, Q, d, lo, hi);
   const int64_t s = uslot[u];
-  const int jl = exact_j((double)lo, yg0[s], ydx[s], kDGrid);
-  const int jh = exact_j((double)hi, yg0[s], ydx[s], kDGrid);
+  const TightBins tb(ybin[s]);
+  if (!tb.usable()) return;   // a grid without a usable step bounds nothing
+  const int jl = tb.lo(lo, kDGrid), jh = tb.hi(hi, kDGrid);
   if (jl >= 1) ccount[i] = min(ccount[i], CHI[s * kDGrid + jl - 1]);
   if (jh < kDGrid) clb[i] = max(clb[i], CLO[s * kDGrid + jh]);
 }
@@ -1807,7 +1857,7 @@ static rkr_status grid_prune(const rkr_index *idx, const QueryCommon &qc, int qa
   tc_gather_free(A, st);
   RKR_TRY(gs);
   k_grid_bound<<<cblocks, 256, 0, st>>>(cnt, cu_fb, cq, cx, idx->Ut.rb3, qc.Qt.rb3, gacc, gcan,
-                                        idx->U, qc.Qd, idx->d, uslot, yg0, ydx, CLO, CHI, ccount,
+                                        idx->U, qc.Qd, idx->d, uslot, ybin, CLO, CHI, ccount,
                                         clb);
   note_launch();
   {
@@ -1992,7 +2042,8 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
       k_select_approx<<<qb - qa, kSelThreads, sm, st>>>(qa, qoff_rel, cursor, C, qc.kq_d, c,
                                                         (uint32_t)idx->s, idx->tau, idx->fmin,
                                                         idx->delta, qc.out_off_d, users_d, nlo_d,
-                                                        nup_d, est_d, case_d, nc_d, sel_err);
+                                                        nup_d, est_d, case_d, nc_d, sel_err,
+                                                        (uint32_t)(idx->m * idx->s));
       prof_end(prof_slot, st, 0.0);
     }
     note_launch();
@@ -2037,7 +2088,7 @@ rkr_status launch_select_approx(int qa, int nblocks, const int64_t *qoff, const 
   k_select_approx<<<nblocks, kSelThreads, sm, st>>>(qa, qoff, qcount, C, kq, c, (uint32_t)idx->s,
                                                    idx->tau, idx->fmin, idx->delta, out_off,
                                                    users_d, nlo_d, nup_d, est_d, case_d, nc_d,
-                                                   err);
+                                                   err, (uint32_t)(idx->m * idx->s));
   prof_end(prof_slot, st, 0.0);
   note_launch();
   RKR_CUDA(cudaGetLastError());
@@ -2377,8 +2428,8 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
         k_list_rank<<<(unsigned)((cnt + 127) / 128), 128, 0, st>>>(
             cnt, cu, cq, cx, qc.Qt.rb3, idx->U, idx->unrm, qc.Qd, idx->Ps, idx->pnrm_s, idx->d,
             idx->xlist, idx->xloff, idx->xlcap, idx->xcoff, idx->xlcnt, idx->xbmax, idx->Ut.rb3, idx->ptile3,
-            idx->ptile_bn, tc_gacc(idx->Ut.kp, 1), tc_gcan(idx->d), idx->xg0, idx->xdx, idx->xg,
-            idx->ldx, kListG,
+            idx->ptile_bn, tc_gacc(idx->Ut.kp, 1), tc_gcan(idx->d), idx->xg0, idx->xbin, idx->xg,
+            idx->ldx, idx->lbin, kListG,
             idx->XLO, idx->XHI, (uint32_t)idx->m, ccount, clb, cu_fb, qself, deep_grid(idx),
             lstat);
         prof_end(prof_slot, st, 0.0);
@@ -2572,8 +2623,8 @@ rkr_status run_rank_pairs(const rkr_index *idx, const QueryCommon &qc, int nq, i
       npairs, cu, cq, nullptr, nullptr, idx->U, idx->unrm, qc.Qd, idx->Ps, idx->pnrm_s, idx->d,
       idx->xlist,
       idx->xloff, idx->xlcap, idx->xcoff, idx->xlcnt, idx->xbmax, idx->Ut.rb3, idx->ptile3,
-      idx->ptile_bn, tc_gacc(idx->Ut.kp, 1), tc_gcan(idx->d), idx->xg0, idx->xdx, idx->xg,
-      idx->ldx, kListG, idx->XLO, idx->XHI, (uint32_t)idx->m, ccount, clb, cu_fb, qself,
+      idx->ptile_bn, tc_gacc(idx->Ut.kp, 1), tc_gcan(idx->d), idx->xg0, idx->xbin, idx->xg,
+      idx->ldx, idx->lbin, kListG, idx->XLO, idx->XHI, (uint32_t)idx->m, ccount, clb, cu_fb, qself,
       deep_grid(idx), lstat);
   note_launch();
   RKR_CUDA(cudaGetLastError());

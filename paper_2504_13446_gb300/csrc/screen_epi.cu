@@ -27,6 +27,12 @@ __device__ __forceinline__ uint64_t dkey_signed(double x) {
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
+// The same for a float.
+__device__ __forceinline__ uint32_t fkey_signed(float x) {
+  const uint32_t b = __float_as_uint(x);
+  return (b >> 31) ? ~b : (b | 0x80000000u);
+}
+
 __device__ __forceinline__ double dkey_inverse(uint64_t k) {
   uint64_t b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
   return __longlong_as_double((long long)b);
@@ -238,23 +244,23 @@ __global__ void k_fb_init(int64_t n, unsigned long long *kmax, unsigned long lon
 }
 
 // Queued items, first pass: per user the largest lower end and the smallest
-// upper end of the compensated intervals holding the canonical scores.
+// upper end of the compensated intervals holding the canonical scores (in float,
+// rounded outwards).
 __global__ void k_fb_bracket(const int2 *__restrict__ items, const unsigned long long *count,
                              unsigned long long cap, const float *__restrict__ U,
                              const float *__restrict__ Ps, int d,
-                             unsigned long long *__restrict__ kmaxlo,
-                             unsigned long long *__restrict__ kminhi,
-                             double2 *__restrict__ ival) {
+                             uint32_t *__restrict__ kmaxlo, uint32_t *__restrict__ kminhi,
+                             float2 *__restrict__ ival) {
   unsigned long long c = *count;
   if (c > cap) c = cap;
   for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < c;
        i += (unsigned long long)gridDim.x * blockDim.x) {
     const int2 it = items[i];
-    double lo, hi;
-    dot2_interval(U + (int64_t)it.x * d, Ps + (int64_t)it.y * d, d, lo, hi);
-    ival[i] = make_double2(lo, hi);
-    atomicMax(&kmaxlo[it.x], (unsigned long long)dkey_signed(lo));
-    atomicMin(&kminhi[it.x], (unsigned long long)dkey_signed(hi));
+    float lo, hi;
+    dot2_interval_f(U + (int64_t)it.x * d, Ps + (int64_t)it.y * d, d, lo, hi);
+    ival[i] = make_float2(lo, hi);
+    atomicMax(&kmaxlo[it.x], fkey_signed(lo));
+    atomicMin(&kminhi[it.x], fkey_signed(hi));
   }
 }
 
@@ -263,9 +269,9 @@ __global__ void k_fb_bracket(const int2 *__restrict__ items, const unsigned long
 __global__ void k_fb_resolve(const int2 *__restrict__ items, const unsigned long long *count,
                              unsigned long long cap, const float *__restrict__ U,
                              const float *__restrict__ Ps, int d,
-                             const unsigned long long *__restrict__ kmaxlo,
-                             const unsigned long long *__restrict__ kminhi,
-                             const double2 *__restrict__ ival, unsigned long long *kmax,
+                             const uint32_t *__restrict__ kmaxlo,
+                             const uint32_t *__restrict__ kminhi,
+                             const float2 *__restrict__ ival, unsigned long long *kmax,
                              unsigned long long *kmin) {
   unsigned long long c = *count;
   if (c > cap) c = cap;
@@ -273,8 +279,8 @@ __global__ void k_fb_resolve(const int2 *__restrict__ items, const unsigned long
        i += (unsigned long long)gridDim.x * blockDim.x) {
     const int2 it = items[i];
     const float *uu = U + (int64_t)it.x * d, *pp = Ps + (int64_t)it.y * d;
-    const double lo = ival[i].x, hi = ival[i].y;
-    const bool maxc = dkey_signed(hi) >= kmaxlo[it.x], minc = dkey_signed(lo) <= kminhi[it.x];
+    const float2 v = ival[i];
+    const bool maxc = fkey_signed(v.y) >= kmaxlo[it.x], minc = fkey_signed(v.x) <= kminhi[it.x];
     if (!maxc && !minc) continue;
     const uint64_t k = dkey_signed(canon_dot(uu, pp, d));
     if (maxc) atomicMax(&kmax[it.x], (unsigned long long)k);
@@ -304,18 +310,19 @@ rkr_status tc_fbounds(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt, 
   const int64_t n = idx->n, m = idx->m;
   tc::RowBound *tb = nullptr;
   RKR_TRY(tc_tile_bounds(Pt, BN, 0, &tb, st));
-  unsigned long long *kmax, *kmin, *kmaxlo, *kminhi, *qcount;
+  unsigned long long *kmax, *kmin, *qcount;
+  uint32_t *kmaxlo, *kminhi;
   int2 *qitems;
   int *flags;  // [0] screen error, [1] overflow, [2] missing extreme
   const unsigned long long cap = std::max<int64_t>(64 * n, 1 << 16);
-  RKR_CUDA(pool_malloc_async(&kmaxlo, sizeof(unsigned long long) * n, st));
-  RKR_CUDA(pool_malloc_async(&kminhi, sizeof(unsigned long long) * n, st));
+  RKR_CUDA(pool_malloc_async(&kmaxlo, sizeof(uint32_t) * n, st));
+  RKR_CUDA(pool_malloc_async(&kminhi, sizeof(uint32_t) * n, st));
   RKR_CUDA(pool_malloc_async(&kmax, sizeof(unsigned long long) * n, st));
   RKR_CUDA(pool_malloc_async(&kmin, sizeof(unsigned long long) * n, st));
   RKR_CUDA(pool_malloc_async(&qcount, sizeof(unsigned long long), st));
   RKR_CUDA(pool_malloc_async(&qitems, sizeof(int2) * cap, st));
-  double2 *ival;
-  RKR_CUDA(pool_malloc_async(&ival, sizeof(double2) * cap, st));
+  float2 *ival;
+  RKR_CUDA(pool_malloc_async(&ival, sizeof(float2) * cap, st));
   RKR_CUDA(pool_malloc_async(&flags, sizeof(int) * 4, st));
   RKR_CUDA(cudaMemsetAsync(qcount, 0, sizeof(unsigned long long), st));
   RKR_CUDA(cudaMemsetAsync(flags, 0, sizeof(int) * 4, st));
@@ -340,8 +347,8 @@ rkr_status tc_fbounds(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt, 
   if (s == RKR_OK) s = launch_screen<BN, 4>(Ut, Pt, 0, sch, a, flags, st);
   cudaFreeAsync(seed, st);
   if (s == RKR_OK) {
-    k_fb_init<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, kmaxlo, kminhi);
-    note_launch();
+    RKR_CUDA(cudaMemsetAsync(kmaxlo, 0, sizeof(uint32_t) * n, st));
+    RKR_CUDA(cudaMemsetAsync(kminhi, 0xff, sizeof(uint32_t) * n, st));
     k_fb_init<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, kmax, kmin);
     note_launch();
     {
@@ -577,26 +584,14 @@ __device__ __forceinline__ void list_group_user(const ListGroupArgs &a, int64_t 
   }
   if (EXT)
     for (uint32_t i = T * kGroupPer + threadIdx.x; i < L; i += T) ext[i - T * kGroupPer] = row[i];
-  // Column c = #{x_j <= v} of the list grid x_j = g0 + j dx.  The FP32 column
-  // coordinate (v - f)(1/dx), f = fl(g0), taken with directed roundings, is
-  // within e(v) = (|v - f| 2^-21 + |g0| 2^-23) / dx of (v - g0) / dx: the
-  // roundings of f, of 1/dx, of the difference and of the product add up to less
-  // than |g0| 2^-24 / dx + |v - f| 2^-21.6 / dx.  Only a coordinate interval that
-  // straddles a column edge is settled in FP64.
-  // (1/dx <= invd32 (1 + 2^-22), since invd32 is 1/dx rounded to nearest twice, and
-  // |g0| <= |f| (1 + 2^-23); both factors are formed in FP32 rounding up)
-  const bool tight = lb.invd32 > 0.0f && lb.err <= 1e6f;
-  const float inv_up = __fmul_ru(lb.invd32, 1.0f + 0x1p-22f);
-  const float e1 = __fmul_ru(inv_up, 0x1p-21f * (1.0f + 0x1p-20f));
-  const float e0 = __fadd_ru(
-      __fmul_ru(__fmul_ru(fabsf(lb.fmin32), (1.0f + 0x1p-23f) * 0x1p-23f), inv_up), 0x1p-30f);
+  // Column c = #{x_j <= v} of the list grid x_j = g0 + j dx: only an FP32 coordinate
+  // interval that straddles a column edge is settled in FP64.
+  const TightBins tb(lb);
   auto list_col = [&](float v) {
     int jlo, jhi;
-    if (tight) {
-      const float alo = __fsub_rd(v, lb.fmin32), ahi = __fsub_ru(v, lb.fmin32);
-      const float e = __fmaf_ru(fmaxf(fabsf(alo), fabsf(ahi)), e1, e0);
-      jlo = bin_lo(__fsub_rd(__fmul_rd(alo, lb.invd32), e), G);
-      jhi = bin_hi(__fadd_ru(__fmul_ru(ahi, lb.invd32), e), G);
+    if (tb.usable()) {
+      jlo = tb.lo(v, G);
+      jhi = tb.hi(v, G);
     } else {
       bin_interval(lb, g0, G, v, v, jlo, jhi);
     }
@@ -1426,8 +1421,8 @@ __global__ void k_table_resolve(const int2 *__restrict__ items,
                                 const unsigned long long *__restrict__ count,
                                 unsigned long long cap, const float *__restrict__ U,
                                 const float *__restrict__ S, int d,
-                                const double *__restrict__ fmin, const double *__restrict__ delta,
-                                int tau, const uint32_t *__restrict__ w, uint32_t *__restrict__ W) {
+                                const BinFP *__restrict__ bf, const double *__restrict__ fmin,
+                                const double *__restrict__ delta, int tau, const uint32_t *__restrict__ w, uint32_t *__restrict__ W) {
   // c(s) = #{t_j < s} is non-decreasing in s: equal at both ends of an interval
   // holding s(u,p) means it is decided
   unsigned long long c = *count;
@@ -1437,15 +1432,16 @@ __global__ void k_table_resolve(const int2 *__restrict__ items,
     const int2 it = items[i];
     const int64_t u = it.x;
     const float *uu = U + u * d, *pp = S + (int64_t)it.y * d;
-    // the compensated interval decides almost every pair; canonical FP64 otherwise
-    double lo, hi;
-    dot2_interval(uu, pp, d, lo, hi);
-    int c;
-    const int clo = exact_c(lo, fmin[u], delta[u], tau), chi = exact_c(hi, fmin[u], delta[u], tau);
-    if (clo == chi) {
-      c = clo;
-    } else {
-      c = exact_c(canon_dot(uu, pp, d), fmin[u], delta[u], tau);
+    // the compensated interval decides almost every pair, nearly always by its FP32
+    // bins; canonical FP64 otherwise
+    float lo, hi;
+    dot2_interval_f(uu, pp, d, lo, hi);
+    int c, chi;
+    bin_interval(bf[u], fmin[u], tau, lo, hi, c, chi);
+    if (c != chi) {
+      c = exact_c((double)lo, fmin[u], delta[u], tau);
+      if (c != exact_c((double)hi, fmin[u], delta[u], tau))
+        c = exact_c(canon_dot(uu, pp, d), fmin[u], delta[u], tau);
     }
     atomicAdd(&W[u * (tau + 1) + c], w[it.y]);
   }
@@ -1536,7 +1532,7 @@ rkr_status tc_rank_table(const rkr_index *idx, const TcSide &Ut, cudaStream_t st
     {
       ProfScope prof("k_table_resolve", st);
       k_table_resolve<<<8 * sm_count(), 256, 0, st>>>(qitems, qcount, cap, idx->U, idx->S, idx->d,
-                                                      idx->fmin, idx->delta, tau, idx->sw, W);
+                                                      idx->binfp, idx->fmin, idx->delta, tau, idx->sw, W);
     }
     note_launch();
     {
@@ -1961,8 +1957,8 @@ struct EpiRCm {
 };
 
 // Exact position of each queued score among its segment's thresholds.  A
-// CUDA-core FP32 dot product with its bound settles most items; the rest are
-// evaluated canonically.
+// CUDA-core FP32 dot product with its bound settles most items, a compensated one
+// nearly all others; what is left is evaluated canonically.
 __global__ void k_rc_refine(const int2 *__restrict__ items, const unsigned long long *count,
                             unsigned long long cap, const int64_t *__restrict__ seg_start,
                             const int32_t *__restrict__ seg_len,
@@ -1981,20 +1977,24 @@ __global__ void k_rc_refine(const int2 *__restrict__ items, const unsigned long 
     const int64_t u = seg_user[it.x];
     const float *uu = U + u * d, *pp = Ps + (int64_t)it.y * d;
     float acc = 0.0f;
-    for (int k = 0; k < d; ++k) acc = fmaf(uu[k], pp[k], acc);
+    for_pairs(uu, pp, d, [&](float x, float y) { acc = fmaf(x, y, acc); });
     float b = screen_bound(cfac, unrm[u], pnrm_s[it.y]);
     double lo = (double)__fsub_rd(acc, b), hi = (double)__fadd_ru(acc, b);
     const double *t = ths + st0;
-    int a0 = 0, a1 = L;
-    while (a0 < a1) { int md = (a0 + a1) >> 1; if (t[md] < lo) a0 = md + 1; else a1 = md; }
-    int pa = a0;
-    a1 = L;
-    while (a0 < a1) { int md = (a0 + a1) >> 1; if (t[md] < hi) a0 = md + 1; else a1 = md; }
-    int pos = pa;
-    if (a0 != pa) {
+    auto below = [&](double x) {   // #{i : t_i < x}
+      int a0 = 0, a1 = L;
+      while (a0 < a1) { int md = (a0 + a1) >> 1; if (t[md] < x) a0 = md + 1; else a1 = md; }
+      return a0;
+    };
+    int pos = below(lo), pe = below(hi);
+    if (pos != pe) {   // the compensated product before the canonical value
+      dot2_interval(uu, pp, d, lo, hi);
+      pos = below(lo);
+      pe = below(hi);
+    }
+    if (pos != pe) {
       atomicAdd(nfp64, 1ull);
-      double s = canon_dot(uu, pp, d);
-      while (pos < a0 && t[pos] < s) ++pos;
+      pos = below(canon_dot(uu, pp, d));
     }
     if (seg_start) atomicAdd(&hist[2 * st0 + pos], 1u);
     else if (pos) atomicAdd(&hist[st0], 1u);

@@ -34,15 +34,38 @@ __device__ uint64_t block_kth(int64_t cnt, uint64_t k, int nbits, F fn, uint32_t
       if (fn(i, key) && (key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      uint64_t acc = 0;
-      int sel = 255;
-      for (int dg = 0; dg < 256; ++dg) {
-        if (acc + hist[dg] >= k) { sel = dg; break; }
-        acc += hist[dg];
+    if (threadIdx.x < 32) {   // eight bins a lane, a scan over the lanes, then the lane's bins
+      const int lane = threadIdx.x;
+      uint32_t h[8], sum = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        h[j] = hist[8 * lane + j];
+        sum += h[j];
       }
-      bc[0] = prefix | ((uint64_t)sel << shift);
-      bc[1] = k - acc;
+      uint64_t incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const unsigned reach = __ballot_sync(0xffffffffu, incl >= k);
+      // (the k-th smallest exists, so some lane reaches k)
+      if (lane == (reach ? __ffs(reach) - 1 : 31)) {
+        uint64_t acc = incl - sum;
+        int sel = 7;
+#pragma unroll
+        for (int j = 7; j >= 0; --j) {   // the first bin whose running count reaches k
+          uint64_t before = acc;
+#pragma unroll
+          for (int i = 0; i < j; ++i) before += h[i];
+          if (before + h[j] >= k) sel = j;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (i < sel) acc += h[i];
+        bc[0] = prefix | ((uint64_t)(8 * lane + sel) << shift);
+        bc[1] = k - acc;
+      }
     }
     __syncthreads();
     prefix = bc[0];
