@@ -78,10 +78,10 @@ struct ProfScope {
 
 // ------------------------------------------------------- canonical scores
 
-// FP64 is scarce on this GPU (a dependent FP64 operation takes some 300 cycles and
-// a warp's FP64 instruction about 60 cycles of its SM whatever the active lanes),
-// so hot code decides with FP32 bounds and forms canonical scores only for what
-// those leave open.  Rows are read 16 bytes at a time where both allow it: a
+// FP64 is scarce on this GPU: a dependent FP64 add or FMA takes 65 cycles, a
+// division 590, and a warp's FP64 instruction holds one of the SM's four FP64 units
+// for 76 cycles whatever its active lanes (measured).  So hot code decides with
+// FP32 bounds and forms canonical scores only for what those leave open.  Rows are read 16 bytes at a time where both allow it: a
 // thread per pair touches 32 lines per warp and load either way.
 
 __device__ __forceinline__ bool rows_vec4(const float *a, const float *b, int d) {

@@ -3,16 +3,17 @@
 // The paper answers each query on its own: u.q for every user and the table
 // lookup of Section 4.3 step 1 (its dominant cost, O(nd) per query), then the
 // k-th smallest bounds, the Case A/B filter and the interpolation.  Per query
-// this runs four launches with no host synchronization between them:
+// this runs three launches with no host synchronization between them:
 //
 //   k_latency_scan     one pass over U (FP32, coalesced): u.q of every user by
-//                      warp-level FP32 products with a rigorous error bound; the
-//                      bin j of Section 4.3 step 1 from that interval (canonical
-//                      FP64 u.q only when the interval straddles a threshold);
-//                      r_low, r_up numerators from the table; a histogram of
-//                      the upper-bound numerators
-//   k_latency_cut      from the histogram, T >= R_up_k (the k-th smallest upper
-//                      bound numerator), the bound of the users that can matter
+//                      FP32 products with a rigorous error bound; the bin j of
+//                      Section 4.3 step 1 from that interval (where it straddles
+//                      a threshold, from a compensated product of the whole warp,
+//                      and canonically only where that straddles one too);
+//                      r_low, r_up numerators from the table; a histogram of the
+//                      upper-bound numerators; the last CTA takes from it
+//                      T >= R_up_k (the k-th smallest upper bound numerator), the
+//                      bound of the users that can matter
 //   k_latency_compact  the users with r_low <= T
 //   k_select_approx    steps 1-3 on those users (query.cu)
 //
@@ -23,6 +24,7 @@
 // for bit.  The scan is bound by HBM: it reads U once (4d bytes per user) and
 // a few bytes of per-user data and table cells.
 #include <math.h>
+#include <stddef.h>
 #include <string.h>
 
 #include <new>
@@ -33,136 +35,228 @@ namespace rkr {
 namespace lat {
 
 constexpr int kLatThreads = 256;
-constexpr int kLatRows = 8;      // rows per warp and sub-batch
-constexpr int kLatSub = 4;       // sub-batches: 32 rows per warp iteration, one per lane
 constexpr int kLatBins = 2048;
 
-// Bound factor of the warp product: every rounding (d FMAs in the lanes' chains,
-// 31 additions of the warp reduction) errs by at most 2^-24 times a partial sum,
+// Bound factor of the scan's products: a term passes at most (d + 31) / 32 * 4
+// FMAs of its lane's chain and three (bulk form: one chain of eight, five)
+// additions of the reduction, each rounding by at most 2^-24 of a partial sum,
 // and every partial sum is at most sum_k |u_k q_k| <= ||u|| ||q||; the canonical
 // FP64 sum differs from the exact value by at most d 2^-53 ||u|| ||q||.
 __host__ __device__ inline float latency_cfac(int d) {
-  const double c = ((double)(d + 36) * 0x1p-24 + (double)d * 0x1p-53 + 0x1p-40) * (1.0 + 0x1p-20);
+  const double c = ((double)((d + 31) / 32 * 4 + 8) * 0x1p-24 + (double)d * 0x1p-53 + 0x1p-40) *
+                   (1.0 + 0x1p-20);
   return (float)c * (1.0f + 0x1p-20f);
 }
 
-// This lane's part of the dot products of kLatRows consecutive rows with q: every
-// load of the batch is issued before the first product, so a warp keeps
-// kLatRows rows in flight (row r0 + rr; rows at or past n contribute 0).
-template <int VEC>
-__device__ __forceinline__ void lane_dots(const float *__restrict__ U, int64_t r0, int64_t n,
-                                          int d, const float *qs, int lane,
-                                          float (&part)[kLatRows]) {
-  if (VEC == 4) {
-    const int dv = d >> 2;
-    float4 a[kLatRows][2];
-#pragma unroll
-    for (int rr = 0; rr < kLatRows; ++rr) {
-      const float4 *r4 = reinterpret_cast<const float4 *>(U + (r0 + rr) * d);
-      const bool ok = r0 + rr < n;
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {  // d <= 256: at most two float4 per lane
-        const int c = lane + 32 * p;
-        a[rr][p] = ok && c < dv ? __ldcs(r4 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-    const float4 *q4 = reinterpret_cast<const float4 *>(qs);
-    const float4 b0 = q4[lane], b1 = q4[lane + 32];   // zero beyond d (qs is padded)
-#pragma unroll
-    for (int rr = 0; rr < kLatRows; ++rr) {
-      float acc = 0.0f;
-      acc = __fmaf_rn(a[rr][0].x, b0.x, acc);
-      acc = __fmaf_rn(a[rr][0].y, b0.y, acc);
-      acc = __fmaf_rn(a[rr][0].z, b0.z, acc);
-      acc = __fmaf_rn(a[rr][0].w, b0.w, acc);
-      acc = __fmaf_rn(a[rr][1].x, b1.x, acc);
-      acc = __fmaf_rn(a[rr][1].y, b1.y, acc);
-      acc = __fmaf_rn(a[rr][1].z, b1.z, acc);
-      acc = __fmaf_rn(a[rr][1].w, b1.w, acc);
-      part[rr] = acc;
-    }
-  } else {
-#pragma unroll
-    for (int rr = 0; rr < kLatRows; ++rr) {
-      const float *row = U + (r0 + rr) * d;
-      const bool ok = r0 + rr < n;
-      float acc = 0.0f;
-#pragma unroll
-      for (int p = 0; p < 8; ++p) {  // d <= 256
-        const int c = lane + 32 * p;
-        if (ok && c < d) acc = __fmaf_rn(__ldcs(row + c), qs[c], acc);
-      }
-      part[rr] = acc;
+// Arguments of the scan kernels.
+struct ScanArgs {
+  const float *U;
+  int64_t n;
+  int d;
+  const float *q, *qn;          // query row and its norm bound
+  const float *unrm;
+  const BinFP *bf;
+  const double *fmin, *delta;
+  const uint32_t *N;
+  int tau;
+  uint32_t top;
+  int shift;
+  uint32_t *nlo, *nup;          // per user
+  int32_t *jout;
+  uint32_t *ghist;              // kLatBins, zero between launches
+  unsigned int *done;           // CTAs that have added their histogram, 0 between launches
+  const int32_t *kq;            // k of the query
+  uint32_t *T, *qcount;         // cut, candidate count (zeroed for the compaction)
+  unsigned long long *nfp64;
+};
+
+// Finish of the warp's users (every lane calls it; lane's user u if live, with its
+// product dot and the bound factors): the bin of u.q, the table's bounds, the
+// histogram.  A lane whose interval straddles a threshold has its row taken again
+// by the whole warp as a compensated product: one lane's canonical product here
+// would hold its SM's FP64 pipe for d dependent steps.
+__device__ __forceinline__ void finish_users(const ScanArgs &a, const float *qs, float cf,
+                                             float qn, int64_t u, bool live, float dot,
+                                             uint32_t *hist, uint32_t &fp64) {
+  const int lane = threadIdx.x & 31;
+  int j = 0, jhi = 0;
+  if (live) {
+    const BinFP bu = a.bf[u];
+    const float b = __fadd_ru(__fmul_ru(__fmul_ru(cf, a.unrm[u]), qn), 1e-30f);
+    const float lo = __fsub_rd(dot, b), hi = __fadd_ru(dot, b);
+    const TightBins tb(bu);
+    if (tb.usable()) {
+      j = tb.lo(lo, a.tau);
+      jhi = tb.hi(hi, a.tau);
+    } else {
+      bin_interval(bu, a.fmin[u], a.tau, lo, hi, j, jhi);
     }
   }
-}
-
-template <int VEC>
-__global__ void __launch_bounds__(kLatThreads)
-    k_latency_scan(const float *__restrict__ U, int64_t n, int d, const float *__restrict__ q,
-                   const float *__restrict__ qn_p, const float *__restrict__ unrm,
-                   const BinFP *__restrict__ bf, const double *__restrict__ fmin,
-                   const double *__restrict__ delta, const uint32_t *__restrict__ N, int tau,
-                   uint32_t top, int shift, uint32_t *__restrict__ nlo,
-                   uint32_t *__restrict__ nup, int32_t *__restrict__ jout,
-                   uint32_t *__restrict__ ghist, unsigned long long *__restrict__ nfp64) {
-  __shared__ __align__(16) float qs[kMaxD];
-  __shared__ uint32_t hist[kLatBins];
-  for (int i = threadIdx.x; i < kMaxD; i += blockDim.x) qs[i] = i < d ? q[i] : 0.0f;
-  for (int i = threadIdx.x; i < kLatBins; i += blockDim.x) hist[i] = 0;
-  __syncthreads();
-  const float qn = *qn_p;
-  const float cf = latency_cfac(d);
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (int64_t)blockIdx.x * (kLatThreads / 32) + (threadIdx.x >> 5);
-  const int64_t nw = (int64_t)gridDim.x * (kLatThreads / 32);
-  constexpr int kPerIter = kLatRows * kLatSub;  // 32 rows: lane r finishes row r0 + r
-  uint32_t fp64 = 0;
-  for (int64_t r0 = gw * kPerIter; r0 < n; r0 += nw * kPerIter) {
-    float mine = 0.0f;
-    // this lane's user: its bound and bin data are loaded while the rows stream in
-    const int64_t u = r0 + lane;
-    const bool live = u < n;
-    const float un = live ? unrm[u] : 0.0f;
-    const BinFP bu = live ? bf[u] : BinFP{0.f, 0.f, 0.f, 0.f};
-    const double fm = live ? fmin[u] : 0.0;
-#pragma unroll 1
-    for (int sb = 0; sb < kLatSub; ++sb) {
-      float part[kLatRows];
-      lane_dots<VEC>(U, r0 + sb * kLatRows, n, d, qs, lane, part);
+  unsigned open = __ballot_sync(0xffffffffu, live && j != jhi);
+  while (open) {
+    const int src = __ffs(open) - 1;
+    open &= open - 1;
+    const int64_t us = __shfl_sync(0xffffffffu, u, src);
+    const float *row = a.U + us * a.d;
+    Dot2 t;
+    for (int k = lane; k < a.d; k += 32) t.add(row[k], qs[k]);
 #pragma unroll
-      for (int rr = 0; rr < kLatRows; ++rr) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-          part[rr] = __fadd_rn(part[rr], __shfl_xor_sync(0xffffffffu, part[rr], o));
-        if (lane == sb * kLatRows + rr) mine = part[rr];
+    for (int o = 16; o > 0; o >>= 1) {
+      const float p2 = __shfl_xor_sync(0xffffffffu, t.p, o);
+      const float s2 = __shfl_xor_sync(0xffffffffu, t.s, o);
+      const float a2 = __shfl_xor_sync(0xffffffffu, t.asum, o);
+      const float sum = __fadd_rn(t.p, p2);
+      const float z = __fsub_rn(sum, t.p);
+      const float e = __fadd_rn(__fsub_rn(t.p, __fsub_rn(sum, z)), __fsub_rn(p2, z));
+      t.p = sum;
+      t.s = __fadd_rn(t.s, __fadd_rn(s2, e));
+      t.asum = __fadd_ru(t.asum, a2);
+    }
+    if (lane == src) {
+      const double res = (double)t.p + (double)t.s, E = (double)t.err(a.d + 8);
+      const double fm = a.fmin[u], dl = a.delta[u];
+      int jl = exact_j(res - E, fm, dl, a.tau);
+      if (jl != exact_j(res + E, fm, dl, a.tau)) {
+        ++fp64;
+        jl = exact_j(canon_dot_slow(row, qs, a.d), fm, dl, a.tau);
       }
+      j = jl;
     }
-    if (!live) continue;
-    const float b = __fadd_ru(__fmul_ru(__fmul_ru(cf, un), qn), 1e-30f);
-    int jlo, jhi;
-    bin_interval(bu, fm, tau, __fsub_rd(mine, b), __fadd_ru(mine, b), jlo, jhi);
-    int j = jlo;
-    if (jlo != jhi) {
-      ++fp64;
-      j = exact_j(canon_dot_slow(U + u * d, qs, d), fm, delta[u], tau);
-    }
-    const uint32_t lo = j < tau ? N[u * tau + j] : 0u;
-    const uint32_t up = j >= 1 ? N[u * tau + j - 1] : top;
-    nlo[u] = lo;
-    nup[u] = up;
-    jout[u] = j;
+  }
+  if (live) {
+    const uint32_t lo = j < a.tau ? a.N[u * a.tau + j] : 0u;
+    const uint32_t up = j >= 1 ? a.N[u * a.tau + j - 1] : a.top;
+    a.nlo[u] = lo;
+    a.nup[u] = up;
+    a.jout[u] = j;
     // lanes with the same bin add once (upper bounds crowd into few bins)
-    const unsigned bin = min(up >> shift, (uint32_t)(kLatBins - 1));
+    const unsigned bin = min(up >> a.shift, (uint32_t)(kLatBins - 1));
     const unsigned peers = __match_any_sync(__activemask(), bin);
     if (lane == __ffs(peers) - 1) atomicAdd(&hist[bin], (uint32_t)__popc(peers));
   }
-  __syncthreads();
-  // this CTA's histogram, stored whole (no atomics across CTAs)
-  uint32_t *mine_h = ghist + (size_t)blockIdx.x * kLatBins;
-  for (int i = threadIdx.x; i < kLatBins; i += blockDim.x) mine_h[i] = hist[i];
+}
+
+// End of a scan CTA: its histogram is added to the query's (most bins are empty),
+// and the last CTA to do so finds T = upper end of the bin holding the k-th
+// smallest upper-bound numerator (so T >= R_up_k), zeroes the query's candidate
+// count and leaves the histogram and the counter at zero for the next launch.
+__device__ __forceinline__ void flush_and_cut(const ScanArgs &a, uint32_t *hist, uint32_t fp64) {
+  __shared__ uint32_t wsum[8];
+  __shared__ int is_last;
   fp64 = __reduce_add_sync(0xffffffffu, fp64);
-  if (lane == 0 && fp64) atomicAdd(nfp64, (unsigned long long)fp64);
+  if ((threadIdx.x & 31) == 0 && fp64) atomicAdd(a.nfp64, (unsigned long long)fp64);
+  __syncthreads();
+  for (int i = threadIdx.x; i < kLatBins; i += blockDim.x)
+    if (hist[i]) atomicAdd(&a.ghist[i], hist[i]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) is_last = atomicAdd(a.done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  constexpr int kPer = kLatBins / 256;
+  const int t = threadIdx.x, lane = t & 31;
+  uint32_t h[kPer], sum = 0, incl = 0;
+  if (t < 256) {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      h[i] = __ldcg(&a.ghist[kPer * t + i]);
+      a.ghist[kPer * t + i] = 0;
+      sum += h[i];
+    }
+    incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    if (lane == 31) wsum[t >> 5] = incl;
+  }
+  __syncthreads();
+  if (t < 256) {
+    for (int w = 0; w < (t >> 5); ++w) incl += wsum[w];
+    const uint32_t k = (uint32_t)*a.kq;
+    uint32_t run = incl - sum;
+    if (run < k && incl >= k) {
+      int bin = kPer * t;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        if (run < k && run + h[i] >= k) bin = kPer * t + i;
+        run += h[i];
+      }
+      const uint64_t hi = ((uint64_t)(bin + 1) << a.shift) - 1;
+      *a.T = bin == kLatBins - 1 || hi > 0xffffffffull ? 0xffffffffu : (uint32_t)hi;
+      *a.qcount = 0;
+    }
+    if (t == 0) *a.done = 0;
+  }
+}
+
+// One pass over U: a warp takes 32 rows per iteration, four at a time with eight
+// lanes each (16-byte loads where VEC = 4: 128 contiguous bytes of a row per load
+// and row; single floats otherwise), so that a product costs three shuffles for
+// four rows, and lane l finishes one of the 32 users.  Bound by HBM: 4 d bytes per
+// user and about 60 more of bounds, table cells and results.  1M users at d = 200:
+// 159 us (5.0 TB/s of the rows alone); with two or four groups of rows in flight
+// per warp 194 and 268 us.
+template <int VEC>
+__global__ void __launch_bounds__(kLatThreads, 4) k_latency_scan(const ScanArgs a) {
+  __shared__ __align__(16) float qs[kMaxD];
+  __shared__ uint32_t hist[kLatBins];
+  for (int i = threadIdx.x; i < kMaxD; i += blockDim.x) qs[i] = i < a.d ? a.q[i] : 0.0f;
+  for (int i = threadIdx.x; i < kLatBins; i += blockDim.x) hist[i] = 0;
+  __syncthreads();
+  const float qn = *a.qn;
+  const float cf = latency_cfac(a.d);
+  const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
+  const int64_t gw = (int64_t)blockIdx.x * (kLatThreads / 32) + (threadIdx.x >> 5);
+  const int64_t nw = (int64_t)gridDim.x * (kLatThreads / 32);
+  [[maybe_unused]] constexpr int kPieces = kMaxD / (8 * VEC);   // per lane and row, at most
+  const int pieces = (a.d + 8 * VEC - 1) / (8 * VEC);
+  uint32_t fp64 = 0;
+  for (int64_t r0 = gw * 32; r0 < a.n; r0 += nw * 32) {
+    float mine = 0.0f;
+#pragma unroll 1
+    for (int sb = 0; sb < 8; ++sb) {
+      const int64_t row = r0 + sb * 4 + grp;
+      const bool ok = row < a.n;
+      float acc = 0.0f;
+      if constexpr (VEC == 4) {
+        const float4 *r4 = reinterpret_cast<const float4 *>(a.U + row * a.d);
+        const float4 *q4 = reinterpret_cast<const float4 *>(qs);
+        const int dv = a.d >> 2;
+        float4 x[kPieces];
+#pragma unroll
+        for (int p = 0; p < kPieces; ++p) {
+          const int c = sub + 8 * p;
+          x[p] = p < pieces && ok && c < dv ? __ldcs(r4 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int p = 0; p < kPieces; ++p) {
+          if (p < pieces) {
+            const float4 y = q4[sub + 8 * p];   // zero beyond d
+            acc = __fmaf_rn(x[p].x, y.x, acc);
+            acc = __fmaf_rn(x[p].y, y.y, acc);
+            acc = __fmaf_rn(x[p].z, y.z, acc);
+            acc = __fmaf_rn(x[p].w, y.w, acc);
+          }
+        }
+      } else {
+        const float *rp = a.U + row * a.d;
+#pragma unroll 8
+        for (int p = 0; p < pieces; ++p) {
+          const int c = sub + 8 * p;
+          if (ok && c < a.d) acc = __fmaf_rn(__ldg(rp + c), qs[c], acc);
+        }
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1)
+        acc = __fadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, o));
+      if (sub == sb) mine = acc;
+    }
+    const int64_t u = r0 + sub * 4 + grp;
+    finish_users(a, qs, cf, qn, u, u < a.n, mine, hist, fp64);
+  }
+  flush_and_cut(a, hist, fp64);
 }
 
 // ------------------------------------------------------------------
@@ -204,14 +298,10 @@ size_t bulk_smem_bytes(int d) {
 }
 
 __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
-    k_latency_scan_bulk(const float *__restrict__ U, int64_t n, int d,
-                        const float *__restrict__ q, const float *__restrict__ qn_p,
-                        const float *__restrict__ unrm, const BinFP *__restrict__ bf,
-                        const double *__restrict__ fmin, const double *__restrict__ delta,
-                        const uint32_t *__restrict__ N, int tau, uint32_t top, int shift,
-                        uint32_t *__restrict__ nlo, uint32_t *__restrict__ nup,
-                        int32_t *__restrict__ jout, uint32_t *__restrict__ ghist,
-                        unsigned long long *__restrict__ nfp64, int *__restrict__ err) {
+    k_latency_scan_bulk(const ScanArgs a, int *__restrict__ err) {
+  const float *U = a.U;
+  const int64_t n = a.n;
+  const int d = a.d;
   extern __shared__ __align__(128) unsigned char bsm[];
   unsigned char *base = (unsigned char *)(((uintptr_t)bsm + 127) & ~(uintptr_t)127);
   const size_t stage_bytes = (size_t)kBulkRows * d * 4;
@@ -221,7 +311,7 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
   float *qs = (float *)(empty + kBulkStages);
   uint32_t *hist = (uint32_t *)(qs + kMaxD);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < kMaxD; i += blockDim.x) qs[i] = i < d ? q[i] : 0.0f;
+  for (int i = threadIdx.x; i < kMaxD; i += blockDim.x) qs[i] = i < d ? a.q[i] : 0.0f;
   for (int i = threadIdx.x; i < kLatBins; i += blockDim.x) hist[i] = 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kBulkStages; ++s) {
@@ -264,7 +354,7 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
     }
   } else {
     // ------------------------------------------------------------ consumers
-    const float qn = *qn_p;
+    const float qn = *a.qn;
     const float cf = latency_cfac(d);
     const float4 *q4 = reinterpret_cast<const float4 *>(qs);
     const float4 b0 = q4[lane], b1 = q4[lane + 32];
@@ -283,18 +373,18 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
         float acc = 0.0f;
         if (u0 + rr < n) {
           if (lane < dv) {
-            const float4 a = r4[lane];
-            acc = __fmaf_rn(a.x, b0.x, acc);
-            acc = __fmaf_rn(a.y, b0.y, acc);
-            acc = __fmaf_rn(a.z, b0.z, acc);
-            acc = __fmaf_rn(a.w, b0.w, acc);
+            const float4 x = r4[lane];
+            acc = __fmaf_rn(x.x, b0.x, acc);
+            acc = __fmaf_rn(x.y, b0.y, acc);
+            acc = __fmaf_rn(x.z, b0.z, acc);
+            acc = __fmaf_rn(x.w, b0.w, acc);
           }
           if (lane + 32 < dv) {
-            const float4 a = r4[lane + 32];
-            acc = __fmaf_rn(a.x, b1.x, acc);
-            acc = __fmaf_rn(a.y, b1.y, acc);
-            acc = __fmaf_rn(a.z, b1.z, acc);
-            acc = __fmaf_rn(a.w, b1.w, acc);
+            const float4 x = r4[lane + 32];
+            acc = __fmaf_rn(x.x, b1.x, acc);
+            acc = __fmaf_rn(x.y, b1.y, acc);
+            acc = __fmaf_rn(x.z, b1.z, acc);
+            acc = __fmaf_rn(x.w, b1.w, acc);
           }
         }
 #pragma unroll
@@ -308,74 +398,15 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bulk_smem(&empty[s]))
                      : "memory");
       const int64_t u = u0 + lane;
-      if (lane < kBulkRowsPerWarp && u < n) {
-        const float b = __fadd_ru(__fmul_ru(__fmul_ru(cf, unrm[u]), qn), 1e-30f);
-        int jlo, jhi;
-        const double fm = fmin[u];
-        bin_interval(bf[u], fm, tau, __fsub_rd(mine, b), __fadd_ru(mine, b), jlo, jhi);
-        int j = jlo;
-        if (jlo != jhi) {
-          ++fp64;
-          j = exact_j(canon_dot_slow(U + u * d, qs, d), fm, delta[u], tau);
-        }
-        const uint32_t lo = j < tau ? N[u * tau + j] : 0u;
-        const uint32_t up = j >= 1 ? N[u * tau + j - 1] : top;
-        nlo[u] = lo;
-        nup[u] = up;
-        jout[u] = j;
-        atomicAdd(&hist[min(up >> shift, (uint32_t)(kLatBins - 1))], 1u);
-      }
+      finish_users(a, qs, cf, qn, u, lane < kBulkRowsPerWarp && u < n, mine, hist, fp64);
     }
     if (failed && lane == 0) atomicExch(err, 2);
   }
-  __syncthreads();
-  uint32_t *mine_h = ghist + (size_t)blockIdx.x * kLatBins;
-  for (int i = threadIdx.x; i < kLatBins; i += blockDim.x) mine_h[i] = hist[i];
-  fp64 = __reduce_add_sync(0xffffffffu, fp64);
-  if (lane == 0 && fp64) atomicAdd(nfp64, (unsigned long long)fp64);
+  flush_and_cut(a, hist, fp64);
 }
 
-// Sum of the scan CTAs' histograms: thread b adds bin b over the `parts` rows.
-__global__ void __launch_bounds__(128)
-    k_latency_hsum(const uint32_t *__restrict__ parts_h, int parts, uint32_t *__restrict__ ghist) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= kLatBins) return;
-  uint32_t acc = 0;
-#pragma unroll 8
-  for (int g = 0; g < parts; ++g) acc += parts_h[(size_t)g * kLatBins + b];
-  ghist[b] = acc;
-}
-
-// T = upper end of the histogram bin holding the k-th smallest upper-bound
-// numerator (so T >= R_up_k); the candidate count of query q is zeroed.
-__global__ void __launch_bounds__(1024)
-    k_latency_cut(uint32_t *__restrict__ ghist, const int32_t *__restrict__ kq, int q, int shift,
-                  uint32_t *__restrict__ T, uint32_t *__restrict__ qcount) {
-  __shared__ uint32_t h[kLatBins];
-  __shared__ uint32_t part[1024];
-  const int t = threadIdx.x;
-  for (int i = t; i < kLatBins; i += blockDim.x) h[i] = ghist[i];
-  __syncthreads();
-  // each thread sums two bins; inclusive scan of the pair sums
-  const uint32_t mine = h[2 * t] + h[2 * t + 1];
-  part[t] = mine;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const uint32_t v = t >= o ? part[t - o] : 0u;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
-  }
-  const uint32_t k = (uint32_t)kq[q];
-  const uint32_t before = part[t] - mine;
-  if (before < k && part[t] >= k) {
-    const int bin = before + h[2 * t] >= k ? 2 * t : 2 * t + 1;
-    const uint64_t hi = ((uint64_t)(bin + 1) << shift) - 1;
-    *T = bin == kLatBins - 1 || hi > 0xffffffffull ? 0xffffffffu : (uint32_t)hi;
-    qcount[q] = 0;
-  }
-}
-
+// Users with r_low <= T, four a thread (their lower bounds in one load), slots by
+// one atomic per warp.
 __global__ void k_latency_compact(int64_t n, const uint32_t *__restrict__ nlo,
                                   const uint32_t *__restrict__ nup, const int32_t *__restrict__ j,
                                   const uint32_t *__restrict__ T, int q,
@@ -383,21 +414,40 @@ __global__ void k_latency_compact(int64_t n, const uint32_t *__restrict__ nlo,
                                   uint32_t *__restrict__ clo, uint32_t *__restrict__ cup,
                                   int32_t *__restrict__ cj, double *__restrict__ cth) {
   const uint32_t t = *T;
-  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    const bool take = nlo[u] <= t;
-    const unsigned act = __ballot_sync(__activemask(), take);
-    if (!take) continue;
-    const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(&qcount[q], (uint32_t)__popc(act));
-    base = __shfl_sync(act, base, leader);
-    const uint32_t pos = base + __popc(act & ((1u << lane) - 1u));
+  const int lane = threadIdx.x & 31;
+  const int64_t u0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4;
+  uint32_t lo[4];
+  if (u0 + 3 < n) {   // nlo is 256-byte aligned
+    const uint4 v = *reinterpret_cast<const uint4 *>(nlo + u0);
+    lo[0] = v.x; lo[1] = v.y; lo[2] = v.z; lo[3] = v.w;
+  } else {
+    for (int e = 0; e < 4; ++e) lo[e] = u0 + e < n ? nlo[u0 + e] : 0u;
+  }
+  int mine = 0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) mine += u0 + e < n && lo[e] <= t;
+  int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += x;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  if (total == 0) return;
+  uint32_t base = 0;
+  if (lane == 0) base = atomicAdd(&qcount[q], (uint32_t)total);
+  base = __shfl_sync(0xffffffffu, base, 0);
+  uint32_t pos = base + (uint32_t)(incl - mine);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int64_t u = u0 + e;
+    if (u >= n || lo[e] > t) continue;
     cu[pos] = (int32_t)u;
-    clo[pos] = nlo[u];
+    clo[pos] = lo[e];
     cup[pos] = nup[u];
     cj[pos] = j[u];
     cth[pos] = __longlong_as_double(0x7ff8000000000000ll);  // u.q formed on demand
+    ++pos;
   }
 }
 
@@ -425,7 +475,7 @@ __global__ void k_candidate_out(const uint32_t *__restrict__ qcount, int q,
 
 // Scratch of the per-query bounds pass.
 struct ScanBufs {
-  uint32_t *nlo, *nup, *parts, *ghist, *T, *qcount;
+  uint32_t *nlo, *nup, *ghist, *T, *qcount;   // ghist: kLatBins, then the CTA counter
   int32_t *jall;
   unsigned long long *nfp64;   // [0] canonical evaluations, [1] select error, [2] scan error
   int grid, shift;
@@ -434,7 +484,7 @@ struct ScanBufs {
   size_t bulk_smem;
 };
 
-rkr_status alloc_scan(const rkr_index *idx, int nq, int ctas_per_sm, DevBuf (&b)[8], ScanBufs &sb,
+rkr_status alloc_scan(const rkr_index *idx, int nq, int ctas_per_sm, DevBuf (&b)[7], ScanBufs &sb,
                       cudaStream_t st) {
   const int64_t n = idx->n;
   sb.top = (uint32_t)(idx->m * idx->s);
@@ -465,11 +515,11 @@ rkr_status alloc_scan(const rkr_index *idx, int nq, int ctas_per_sm, DevBuf (&b)
   RKR_TRY(tmp_alloc(b[0], &sb.nlo, n, st));
   RKR_TRY(tmp_alloc(b[1], &sb.nup, n, st));
   RKR_TRY(tmp_alloc(b[2], &sb.jall, n, st));
-  RKR_TRY(tmp_alloc(b[3], &sb.parts, (size_t)sb.grid * kLatBins, st));
-  RKR_TRY(tmp_alloc(b[4], &sb.ghist, kLatBins, st));
-  RKR_TRY(tmp_alloc(b[5], &sb.T, 1, st));
-  RKR_TRY(tmp_alloc(b[6], &sb.qcount, nq, st));
-  RKR_TRY(tmp_alloc(b[7], &sb.nfp64, 3, st));
+  RKR_TRY(tmp_alloc(b[3], &sb.ghist, kLatBins + 1, st));
+  RKR_TRY(tmp_alloc(b[4], &sb.T, 1, st));
+  RKR_TRY(tmp_alloc(b[5], &sb.qcount, nq, st));
+  RKR_TRY(tmp_alloc(b[6], &sb.nfp64, 3, st));
+  RKR_CUDA(cudaMemsetAsync(sb.ghist, 0, sizeof(uint32_t) * (kLatBins + 1), st));
   RKR_CUDA(cudaMemsetAsync(sb.qcount, 0, sizeof(uint32_t) * nq, st));
   RKR_CUDA(cudaMemsetAsync(sb.nfp64, 0, 3 * sizeof(unsigned long long), st));
   return RKR_OK;
@@ -482,31 +532,20 @@ rkr_status scan_pass(const rkr_index *idx, const QueryCommon &qc, int q, const S
   {
     ProfScope prof("k_latency_scan", st,
                    (double)idx->n * (4.0 * idx->d + 4 + sizeof(BinFP) + 8 + 8 + 12));
+    ScanArgs a;
+    a.U = idx->U; a.n = idx->n; a.d = idx->d; a.q = qrow; a.qn = qc.qnrm + q;
+    a.unrm = idx->unrm; a.bf = idx->binfp; a.fmin = idx->fmin; a.delta = idx->delta;
+    a.N = idx->N; a.tau = idx->tau; a.top = sb.top; a.shift = sb.shift;
+    a.nlo = sb.nlo; a.nup = sb.nup; a.jout = sb.jall;
+    a.ghist = sb.ghist; a.done = sb.ghist + kLatBins; a.kq = qc.kq_d + q;
+    a.T = sb.T; a.qcount = sb.qcount + q; a.nfp64 = sb.nfp64;
     if (sb.bulk)
       k_latency_scan_bulk<<<sb.grid, (kBulkWarps + 1) * 32, sb.bulk_smem, st>>>(
-          idx->U, idx->n, idx->d, qrow, qc.qnrm + q, idx->unrm, qc.bf, idx->fmin, idx->delta,
-          idx->N, idx->tau, sb.top, sb.shift, sb.nlo, sb.nup, sb.jall, sb.parts, sb.nfp64,
-          (int *)(sb.nfp64 + 2));
+          a, (int *)(sb.nfp64 + 2));
     else if (sb.vec4)
-      k_latency_scan<4><<<sb.grid, kLatThreads, 0, st>>>(
-          idx->U, idx->n, idx->d, qrow, qc.qnrm + q, idx->unrm, qc.bf, idx->fmin, idx->delta,
-          idx->N, idx->tau, sb.top, sb.shift, sb.nlo, sb.nup, sb.jall, sb.parts, sb.nfp64);
+      k_latency_scan<4><<<sb.grid, kLatThreads, 0, st>>>(a);
     else
-      k_latency_scan<1><<<sb.grid, kLatThreads, 0, st>>>(
-          idx->U, idx->n, idx->d, qrow, qc.qnrm + q, idx->unrm, qc.bf, idx->fmin, idx->delta,
-          idx->N, idx->tau, sb.top, sb.shift, sb.nlo, sb.nup, sb.jall, sb.parts, sb.nfp64);
-    note_launch();
-  }
-  {
-    const int prof_slot = prof_begin("k_latency_hsum", st);
-    k_latency_hsum<<<kLatBins / 128, 128, 0, st>>>(sb.parts, sb.grid, sb.ghist);
-    prof_end(prof_slot, st, 0.0);
-    note_launch();
-  }
-  {
-    const int prof_slot = prof_begin("k_latency_cut", st);
-    k_latency_cut<<<1, 1024, 0, st>>>(sb.ghist, qc.kq_d, q, sb.shift, sb.T, sb.qcount);
-    prof_end(prof_slot, st, 0.0);
+      k_latency_scan<1><<<sb.grid, kLatThreads, 0, st>>>(a);
     note_launch();
   }
   RKR_CUDA(cudaGetLastError());
@@ -525,7 +564,7 @@ rkr_status run_query_approx_candidates(const rkr_index *idx, const QueryCommon &
                                        double *est_d, cudaStream_t st) {
   const int64_t n = idx->n;
   const int d = idx->d;
-  DevBuf bs[8], b7, b8, b9, b10, b11;
+  DevBuf bs[7], b7, b8, b9, b10, b11;
   ScanBufs sb;
   RKR_TRY(alloc_scan(idx, nq, tuning().latency_ctas_per_sm, bs, sb, st));
   uint32_t *clo, *cup;
@@ -536,7 +575,7 @@ rkr_status run_query_approx_candidates(const rkr_index *idx, const QueryCommon &
   RKR_TRY(tmp_alloc(b9, &cup, n, st));
   RKR_TRY(tmp_alloc(b10, &cj, n, st));
   RKR_TRY(tmp_alloc(b11, &cth, n, st));
-  const int cgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8);
+  const unsigned cgrid = (unsigned)((n + 1023) / 1024);   // four users a thread
   offs_host[0] = 0;
   for (int q = 0; q < nq; ++q) {
     const float *qrow = qc.Qd + (int64_t)q * d;
@@ -575,7 +614,7 @@ rkr_status run_query_approx_single(const rkr_index *idx, const QueryCommon &qc, 
                                    double *est_d, int32_t *case_d, int32_t *nc_d,
                                    rkr_query_stats *stats, cudaStream_t st) {
   const int64_t n = idx->n;
-  DevBuf bs[8], b7, b8, b9, b10, b11;
+  DevBuf bs[7], b7, b8, b9, b10, b11;
   ScanBufs sb;
   RKR_TRY(alloc_scan(idx, nq, tuning().latency_ctas_per_sm, bs, sb, st));
   uint32_t *clo, *cup;
@@ -587,7 +626,7 @@ rkr_status run_query_approx_single(const rkr_index *idx, const QueryCommon &qc, 
   RKR_TRY(tmp_alloc(b10, &cj, n, st));
   RKR_TRY(tmp_alloc(b11, &cth, n, st));
   int *err = (int *)(sb.nfp64 + 1);
-  const int cgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8);
+  const unsigned cgrid = (unsigned)((n + 1023) / 1024);   // four users a thread
   Timer t1(st);
   for (int q = 0; q < nq; ++q) {
     RKR_TRY(scan_pass(idx, qc, q, sb, st));
@@ -629,22 +668,26 @@ struct rkr_session {
   int max_k = 0, d = 0;
   double c = 2.0;
   cudaStream_t st = nullptr;
-  float *q_dev = nullptr, *qn_dev = nullptr;
-  int32_t *k_dev = nullptr;
+  unsigned char *in_dev = nullptr;   // an In
   int64_t *off_dev = nullptr;
-  int32_t *users = nullptr, *ocase = nullptr, *onc = nullptr;
-  uint32_t *onlo = nullptr, *onup = nullptr;
+  // outputs (pinned host memory, max_k entries each) and error words
   double *oest = nullptr;
-  rkr::DevBuf scan_bufs[8], cand_bufs[5], out_bufs[10];
+  int32_t *users = nullptr, *ocase = nullptr, *onc = nullptr, *oerr = nullptr;
+  uint32_t *onlo = nullptr, *onup = nullptr;
+  rkr::DevBuf scan_bufs[7], cand_bufs[5], out_bufs[2];
   rkr::lat::ScanBufs sb;
   uint32_t *clo = nullptr, *cup = nullptr;
   int32_t *cu = nullptr, *cj = nullptr;
   double *cth = nullptr;
-  // pinned host staging: query, k, then the outputs and the two error words
-  float *q_h = nullptr;
-  int32_t *k_h = nullptr;
+  // pinned host memory: the query with its norm bound and k as one block, copied to
+  // in_dev by the graph; the outputs and the two error words, written by the kernels
+  struct In {
+    float q[rkr::kMaxD];
+    float qn;
+    int32_t k;
+  };
+  In *in_h = nullptr;
   unsigned char *out_h = nullptr;
-  size_t out_bytes = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -654,24 +697,24 @@ namespace {
 
 rkr_status session_enqueue(rkr_session *s) {
   QueryCommon qc;
-  qc.Qd = s->q_dev;
-  qc.qnrm = s->qn_dev;
-  qc.kq_d = s->k_dev;
+  qc.Qd = (float *)(s->in_dev + offsetof(rkr_session::In, q));
+  qc.qnrm = (float *)(s->in_dev + offsetof(rkr_session::In, qn));
+  qc.kq_d = (int32_t *)(s->in_dev + offsetof(rkr_session::In, k));
   qc.out_off_d = s->off_dev;
   qc.bf = s->idx->binfp;
   qc.xbf = s->idx->xbin;
-  RKR_TRY(row_norms(s->q_dev, 1, s->d, nullptr, s->qn_dev, s->st));
+  RKR_CUDA(cudaMemcpyAsync(s->in_dev, s->in_h, sizeof(rkr_session::In), cudaMemcpyHostToDevice,
+                           s->st));
   RKR_TRY(scan_pass(s->idx, qc, 0, s->sb, s->st));
   const int64_t n = s->idx->n;
-  const int cgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8);
+  const unsigned cgrid = (unsigned)((n + 1023) / 1024);   // four users a thread
   k_latency_compact<<<cgrid, 256, 0, s->st>>>(n, s->sb.nlo, s->sb.nup, s->sb.jall, s->sb.T, 0,
                                               s->sb.qcount, s->cu, s->clo, s->cup, s->cj,
                                               s->cth);
   note_launch();
   RKR_TRY(launch_select_approx(0, 1, s->off_dev, s->sb.qcount, s->cu, s->clo, s->cup, s->cth,
-                               s->cj, s->q_dev, s->k_dev, s->c, s->off_dev, s->users, s->onlo,
-                               s->onup, s->oest, s->ocase, s->onc, (int *)(s->sb.nfp64 + 1),
-                               s->st, s->idx));
+                               s->cj, qc.Qd, qc.kq_d, s->c, s->off_dev, s->users, s->onlo,
+                               s->onup, s->oest, s->ocase, s->onc, s->oerr, s->st, s->idx));
   return RKR_OK;
 }
 
@@ -679,12 +722,9 @@ void session_release(rkr_session *s) {
   if (!s) return;
   if (s->exec) cudaGraphExecDestroy(s->exec);
   if (s->graph) cudaGraphDestroy(s->graph);
-  if (s->q_h) cudaFreeHost(s->q_h);
-  if (s->k_h) cudaFreeHost(s->k_h);
-  if (s->out_h) cudaFreeHost(s->out_h);
   // device blocks go back to the pool on the session's stream, before it goes
   for (DevBuf *group : {s->scan_bufs, s->cand_bufs, s->out_bufs}) {
-    const int count = group == s->scan_bufs ? 8 : (group == s->cand_bufs ? 5 : 10);
+    const int count = group == s->scan_bufs ? 7 : (group == s->cand_bufs ? 5 : 2);
     for (int i = 0; i < count; ++i)
       if (group[i].p) {
         cudaFreeAsync(group[i].p, group[i].st);
@@ -695,6 +735,8 @@ void session_release(rkr_session *s) {
     cudaStreamSynchronize(s->st);
     cudaStreamDestroy(s->st);
   }
+  if (s->in_h) cudaFreeHost(s->in_h);
+  if (s->out_h) cudaFreeHost(s->out_h);
   delete s;
 }
 
@@ -732,24 +774,23 @@ extern "C" rkr_status rkr_session_create(rkr_index *idx, int32_t max_k, double c
   RKR_TRY(tmp_alloc(s->cand_bufs[2], &s->cup, n, st));
   RKR_TRY(tmp_alloc(s->cand_bufs[3], &s->cj, n, st));
   RKR_TRY(tmp_alloc(s->cand_bufs[4], &s->cth, n, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[0], &s->q_dev, kMaxD, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[1], &s->qn_dev, 1, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[2], &s->k_dev, 1, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[3], &s->off_dev, 2, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[4], &s->users, max_k, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[5], &s->onlo, max_k, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[6], &s->onup, max_k, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[7], &s->oest, max_k, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[8], &s->ocase, 1, st));
-  RKR_TRY(tmp_alloc(s->out_bufs[9], &s->onc, 1, st));
+  RKR_TRY(tmp_alloc(s->out_bufs[0], &s->in_dev, sizeof(rkr_session::In), st));
+  RKR_TRY(tmp_alloc(s->out_bufs[1], &s->off_dev, 2, st));
   RKR_CUDA(cudaMemsetAsync(s->off_dev, 0, 2 * sizeof(int64_t), st));
-  RKR_CUDA(cudaMemsetAsync(s->q_dev, 0, kMaxD * sizeof(float), st));
-  const int32_t one = 1;
-  RKR_CUDA(cudaMemcpyAsync(s->k_dev, &one, sizeof(one), cudaMemcpyHostToDevice, st));
-  s->out_bytes = (size_t)max_k * (4 + 4 + 4 + 8) + 4 + 4 + 8 + 8;
-  RKR_CUDA(cudaMallocHost(&s->q_h, sizeof(float) * kMaxD));
-  RKR_CUDA(cudaMallocHost(&s->k_h, sizeof(int32_t)));
-  RKR_CUDA(cudaMallocHost(&s->out_h, s->out_bytes));
+  const size_t K = (size_t)max_k;
+  const size_t out_bytes = K * (8 + 4 + 4 + 4) + 4 * sizeof(int32_t);
+  RKR_CUDA(cudaMallocHost(&s->in_h, sizeof(rkr_session::In)));
+  memset(s->in_h, 0, sizeof(rkr_session::In));
+  s->in_h->k = 1;
+  RKR_CUDA(cudaMallocHost(&s->out_h, out_bytes));
+  memset(s->out_h, 0, out_bytes);
+  s->oest = (double *)s->out_h;
+  s->users = (int32_t *)(s->out_h + 8 * K);
+  s->onlo = (uint32_t *)(s->out_h + 12 * K);
+  s->onup = (uint32_t *)(s->out_h + 16 * K);
+  s->ocase = (int32_t *)(s->out_h + 20 * K);
+  s->onc = s->ocase + 1;
+  s->oerr = s->ocase + 2;
   // one uncaptured run (sets function attributes, warms the pool), then the capture
   RKR_TRY(session_enqueue(s));
   RKR_CUDA(cudaStreamSynchronize(st));
@@ -779,12 +820,13 @@ extern "C" rkr_status rkr_session_query(rkr_session *s, const float *q, int32_t 
   const bool qdev = cudaPointerGetAttributes(&pa, q) == cudaSuccess &&
                     (pa.type == cudaMemoryTypeDevice || pa.type == cudaMemoryTypeManaged);
   cudaGetLastError();
-  if (qdev) RKR_CUDA(cudaMemcpy(s->q_h, q, sizeof(float) * d, cudaMemcpyDeviceToHost));
-  else memcpy(s->q_h, q, sizeof(float) * d);
+  float *qh = s->in_h->q;
+  if (qdev) RKR_CUDA(cudaMemcpy(qh, q, sizeof(float) * d, cudaMemcpyDeviceToHost));
+  else memcpy(qh, q, sizeof(float) * d);
   double ss = 0.0;
   for (int i = 0; i < d; ++i) {
-    if (!isfinite(s->q_h[i])) return fail(RKR_EINVAL, "q must be finite");
-    ss += (double)s->q_h[i] * (double)s->q_h[i];
+    if (!isfinite(qh[i])) return fail(RKR_EINVAL, "q must be finite");
+    ss += (double)qh[i] * (double)qh[i];
   }
   if (sqrt(ss) * (1.0 + 0x1p-20) > (double)s->idx->pmax) {
     // outside the item norms: the bin bounds of this query need a wider range,
@@ -792,37 +834,35 @@ extern "C" rkr_status rkr_session_query(rkr_session *s, const float *q, int32_t 
     return rkr_query_approx_single(s->idx, q, 1, &k, s->c, out_users, out_nlow, out_nup,
                                    out_est, out_case, out_nc, nullptr, st);
   }
-  *s->k_h = k;
-  RKR_CUDA(cudaMemcpyAsync(s->q_dev, s->q_h, sizeof(float) * d, cudaMemcpyHostToDevice, st));
-  RKR_CUDA(cudaMemcpyAsync(s->k_dev, s->k_h, sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  // FP32 upper bound of ||q||, as row_norms forms it on the device
+  const double nv = sqrt(ss) * (1.0 + 0x1p-40) + 1e-300;
+  float qn = (float)nv;
+  if ((double)qn < nv) qn = nextafterf(qn, INFINITY);
+  s->in_h->qn = qn;
+  s->in_h->k = k;
+  *s->oerr = 0;
   RKR_CUDA(cudaGraphLaunch(s->exec, st));
-  unsigned char *o = s->out_h;
-  const size_t K = (size_t)k;
-  RKR_CUDA(cudaMemcpyAsync(o, s->users, 4 * K, cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaMemcpyAsync(o + 4 * K, s->onlo, 4 * K, cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaMemcpyAsync(o + 8 * K, s->onup, 4 * K, cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaMemcpyAsync(o + 12 * K, s->oest, 8 * K, cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaMemcpyAsync(o + 20 * K, s->ocase, 4, cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaMemcpyAsync(o + 20 * K + 4, s->onc, 4, cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaMemcpyAsync(o + 20 * K + 8, s->sb.nfp64 + 1, 16, cudaMemcpyDeviceToHost, st));
   RKR_CUDA(cudaStreamSynchronize(st));
-  unsigned long long ew[2];
-  memcpy(ew, o + 20 * K + 8, 16);
-  if ((int)ew[1]) return fail(RKR_ETIMEOUT, "latency scan wait timed out (%d)", (int)ew[1]);
-  if ((int)ew[0]) return fail(RKR_EINTERNAL, "fewer than k candidates for the query");
+  unsigned long long scan_err = 0;
+  if (s->sb.bulk)   // only the bulk-staged scan has waits that can run out
+    RKR_CUDA(cudaMemcpy(&scan_err, s->sb.nfp64 + 2, sizeof(scan_err), cudaMemcpyDeviceToHost));
+  if ((int)scan_err) return fail(RKR_ETIMEOUT, "latency scan wait timed out (%d)", (int)scan_err);
+  if (*s->oerr) return fail(RKR_EINTERNAL, "fewer than k candidates for the query");
+  const size_t K = (size_t)k;
   struct Out {
     void *dst;
-    size_t off, bytes;
-  } outs[] = {{out_users, 0, 4 * K},       {out_nlow, 4 * K, 4 * K}, {out_nup, 8 * K, 4 * K},
-              {out_est, 12 * K, 8 * K},    {out_case, 20 * K, 4},    {out_nc, 20 * K + 4, 4}};
+    const void *src;
+    size_t bytes;
+  } outs[] = {{out_users, s->users, 4 * K}, {out_nlow, s->onlo, 4 * K}, {out_nup, s->onup, 4 * K},
+              {out_est, s->oest, 8 * K},    {out_case, s->ocase, 4},    {out_nc, s->onc, 4}};
   for (const Out &x : outs) {
     if (!x.dst) continue;
     cudaPointerAttributes a;
     const bool dev = cudaPointerGetAttributes(&a, x.dst) == cudaSuccess &&
                      (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged);
     cudaGetLastError();
-    if (dev) RKR_CUDA(cudaMemcpy(x.dst, o + x.off, x.bytes, cudaMemcpyHostToDevice));
-    else memcpy(x.dst, o + x.off, x.bytes);
+    if (dev) RKR_CUDA(cudaMemcpy(x.dst, x.src, x.bytes, cudaMemcpyHostToDevice));
+    else memcpy(x.dst, x.src, x.bytes);
   }
   return RKR_OK;
 }

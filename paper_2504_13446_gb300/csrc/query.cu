@@ -206,10 +206,24 @@ __device__ __forceinline__ uint64_t count_key(uint32_t c, int bits) {
   return bits < 32 ? min(c, (1u << bits) - 1u) : c;
 }
 
+// Bytes of a user index, in bits.
+static int user_bits(int64_t n) {
+  int bits = 8;
+  while (bits < 32 && ((int64_t)1 << bits) < n) bits += 8;
+  return bits;
+}
+
+// Threads of the per-query selections: 256 where many queries share the SMs, 1,024
+// where there are fewer queries than SMs (one CTA's walk of its candidates is then
+// the time of the launch).
 constexpr int kSelThreads = 256;
+constexpr int kSelThreadsFew = 1024;
+constexpr int kSelSmall = 512;     // entries sorted beside the survivors (k_select_approx)
+constexpr size_t kSelSmem = sizeof(SortEnt) * (kMaxK + kSelSmall);
 
 // One CTA per query: steps 1-3 of Section 4.3 over the query's candidates.
-__global__ void __launch_bounds__(kSelThreads)
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
     k_select_approx(int qa, const int64_t *__restrict__ qoff, const uint32_t *__restrict__ qcount,
                     ApproxCand C,
                     const int32_t *__restrict__ kq, double c, uint32_t s, int tau,
@@ -217,11 +231,13 @@ __global__ void __launch_bounds__(kSelThreads)
                     const int64_t *__restrict__ out_off, int32_t *__restrict__ out_users,
                     uint32_t *__restrict__ out_nlo, uint32_t *__restrict__ out_nup,
                     double *__restrict__ out_est, int32_t *__restrict__ out_case,
-                    int32_t *__restrict__ out_nc, int *__restrict__ err, uint32_t top) {
+                    int32_t *__restrict__ out_nc, int *__restrict__ err, uint32_t top,
+                    int ubits) {
   extern __shared__ unsigned char sbuf[];
   SortEnt *ent = (SortEnt *)sbuf;                   // kMaxK entries
-  __shared__ uint32_t hist[256];
-  __shared__ uint64_t bc[2];
+  SortEnt *small = ent + kMaxK;                     // kSelSmall entries
+  __shared__ uint32_t hist[512];
+  __shared__ uint64_t bc[4];
   __shared__ unsigned long long cnt_acc;
   __shared__ int gcount;
   const int q = qa + blockIdx.x;
@@ -250,37 +266,51 @@ __global__ void __launch_bounds__(kSelThreads)
   };
   // Step 1: k-th smallest lower and upper bound numerators (at most top).
   const int nbits = count_bits(top);
-  uint64_t Rlo = block_kth(cnt, (uint64_t)k, nbits,
-                           [&](int64_t i, uint64_t &key) { key = nlo[i]; return true; }, hist, bc);
-  uint64_t Rup = block_kth(cnt, (uint64_t)k, nbits,
-                           [&](int64_t i, uint64_t &key) { key = nup[i]; return true; }, hist, bc);
+  uint64_t Rlo, Rup;
+  block_kth_pair(nlo, nup, cnt, (uint64_t)k, nbits, hist, bc, Rlo, Rup);
   const double lhs = c * (double)((uint64_t)s + Rlo);
   const bool caseA = lhs >= (double)((uint64_t)s + Rup);
   const int64_t obase = out_off[q];
   int nc;
   if (caseA) {
-    // k smallest (r_up, r_low, index): all with nup < Rup, then ties by (nlo, index)
-    int64_t below = block_count(cnt, [&](int64_t i) { return (uint64_t)nup[i] < Rup; }, &cnt_acc);
-    uint64_t kth2 = ~0ull;
-    if (below < k)
-      kth2 = block_kth(cnt, (uint64_t)(k - below), 64,
-                       [&](int64_t i, uint64_t &key) {
-                         key = ((uint64_t)nlo[i] << 32) | (uint32_t)uid[i];
-                         return (uint64_t)nup[i] == Rup;
-                       },
-                       hist, bc);
+    // k smallest (r_up, r_low, index).  All with nup <= Rup are gathered; if they are
+    // few, sorting them gives the k first.  Otherwise all with nup < Rup, then of the
+    // ties the smallest (nlo, index).
+    auto put = [&](int pos, int64_t i) {
+      ent[pos].k1 = ((uint64_t)nup[i] << 32) | nlo[i];
+      ent[pos].k2 = (uint32_t)uid[i];
+      ent[pos].idx = (int32_t)i;
+    };
+    constexpr int kSort = 512;   // (sorting 4,096 takes twice the radix passes' time)
     if (threadIdx.x == 0) gcount = 0;
     __syncthreads();
-    for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-      uint64_t a = nup[i];
-      bool take = a < Rup ||
-                  (a == Rup && (((uint64_t)nlo[i] << 32) | (uint32_t)uid[i]) <= kth2);
-      if (take) {
-        int pos = atomicAdd(&gcount, 1);
-        if (pos < kMaxK) {
-          ent[pos].k1 = ((uint64_t)nup[i] << 32) | nlo[i];
-          ent[pos].k2 = (uint32_t)uid[i];
-          ent[pos].idx = (int32_t)i;
+    for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x)
+      if ((uint64_t)nup[i] <= Rup) {
+        const int pos = atomicAdd(&gcount, 1);
+        if (pos < kSort) put(pos, i);
+      }
+    __syncthreads();
+    const int upto = gcount;
+    __syncthreads();
+    if (upto > kSort) {
+      const int64_t below =
+          block_count(cnt, [&](int64_t i) { return (uint64_t)nup[i] < Rup; }, &cnt_acc);
+      uint64_t kth2 = ~0ull;
+      auto tie_key = [&](int64_t i) { return ((uint64_t)nlo[i] << ubits) | (uint32_t)uid[i]; };
+      if (below < k)
+        kth2 = block_kth(cnt, (uint64_t)(k - below), nbits + ubits,
+                         [&](int64_t i, uint64_t &key) {
+                           key = tie_key(i);
+                           return (uint64_t)nup[i] == Rup;
+                         },
+                         hist, bc);
+      if (threadIdx.x == 0) gcount = 0;
+      __syncthreads();
+      for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
+        const uint64_t a = nup[i];
+        if (a < Rup || (a == Rup && tie_key(i) <= kth2)) {
+          const int pos = atomicAdd(&gcount, 1);
+          if (pos < kMaxK) put(pos, i);
         }
       }
     }
@@ -324,25 +354,67 @@ __global__ void __launch_bounds__(kSelThreads)
       if (out_est) out_est[obase + r] = est_of(i);
     }
     __syncthreads();
-    // Step 3: survivors r_low <= R_up_k outside U_c, smallest (r_hat, index); their
-    // estimates take the place of u.q in th, formed in full warps: the survivors'
-    // indices are gathered in shared memory first where they fit
+    // Step 3: survivors r_low <= R_up_k outside U_c, smallest (r_hat, index).  They
+    // are gathered in shared memory first, so that their estimates are formed in
+    // full warps; where they fit, the selection runs there, else over all candidates
+    // with the estimates in the place of u.q in th.
     auto in_t = [&](int64_t i) { return (uint64_t)nlo[i] <= Rup && !in_c(i); };
     const int need = k - nc;
-    int *todo = (int *)sbuf;
-    constexpr int kTodo = (int)(sizeof(SortEnt) * kMaxK / sizeof(int));
     if (threadIdx.x == 0) gcount = 0;
     __syncthreads();
     for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
       if (!in_t(i)) continue;
       const int pos = atomicAdd(&gcount, 1);
-      if (pos < kTodo) todo[pos] = (int)i;
+      if (pos < kMaxK) ent[pos].idx = (int32_t)i;
       else th[i] = est_of(i);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < min(gcount, kTodo); e += blockDim.x)
-      th[todo[e]] = est_of(todo[e]);
+    const int nt = gcount;
+    __syncthreads();   // every thread has the count before it is reset
+    const bool fits = nt <= kMaxK && need <= kSelSmall;
+    for (int e = threadIdx.x; e < min(nt, kMaxK); e += blockDim.x) {
+      const int64_t i = ent[e].idx;
+      const double est = est_of(i);
+      ent[e].k1 = dkey(est);
+      ent[e].k2 = (uint32_t)uid[i];
+      if (!fits) th[i] = est;
+    }
+    if (threadIdx.x == 0) gcount = 0;
     __syncthreads();
+    if (fits) {
+      const uint64_t ke = block_kth(nt, (uint64_t)need, 64,
+                                    [&](int64_t e, uint64_t &key) {
+                                      key = ent[e].k1;
+                                      return true;
+                                    },
+                                    hist, bc);
+      const int64_t below = block_count(nt, [&](int64_t e) { return ent[e].k1 < ke; }, &cnt_acc);
+      uint64_t ku = ~0ull;
+      if (below < need)
+        ku = block_kth(nt, (uint64_t)(need - below), 32,
+                       [&](int64_t e, uint64_t &key) {
+                         key = ent[e].k2;
+                         return ent[e].k1 == ke;
+                       },
+                       hist, bc);
+      for (int e = threadIdx.x; e < nt; e += blockDim.x) {
+        const SortEnt x = ent[e];
+        if (x.k1 < ke || (x.k1 == ke && (uint64_t)x.k2 <= ku)) {
+          const int pos = atomicAdd(&gcount, 1);
+          if (pos < kSelSmall) small[pos] = x;
+        }
+      }
+      __syncthreads();
+      const int got = min(gcount, kSelSmall);
+      block_sort(small, got);
+      for (int r = threadIdx.x; r < got && r < need; r += blockDim.x) {
+        const int64_t i = small[r].idx;
+        out_users[obase + nc + r] = uid[i];
+        if (out_nlo) out_nlo[obase + nc + r] = nlo[i];
+        if (out_nup) out_nup[obase + nc + r] = nup[i];
+        if (out_est) out_est[obase + nc + r] = __longlong_as_double((long long)small[r].k1);
+      }
+    } else {
     uint64_t ke = block_kth(cnt, (uint64_t)need, 64,
                             [&](int64_t i, uint64_t &key) {
                               if (!in_t(i)) return false;
@@ -384,6 +456,7 @@ __global__ void __launch_bounds__(kSelThreads)
       if (out_nlo) out_nlo[obase + nc + r] = nlo[i];
       if (out_nup) out_nup[obase + nc + r] = nup[i];
       if (out_est) out_est[obase + nc + r] = __longlong_as_double((long long)ent[r].k1);
+    }
     }
   }
   if (threadIdx.x == 0) {
@@ -851,15 +924,8 @@ __global__ void k_prefix_unpark(int64_t n, const int32_t *__restrict__ cu_park,
   if (i < n && cu_park[i] >= 0) cu_fb[i] = cu_park[i];
 }
 
-// Bytes of a user index, in bits.
-static int user_bits(int64_t n) {
-  int bits = 8;
-  while (bits < 32 && ((int64_t)1 << bits) < n) bits += 8;
-  return bits;
-}
-
 // One CTA per query: the k smallest (rank, index) among its candidates.
-__global__ void __launch_bounds__(kSelThreads)
+__global__ void __launch_bounds__(kSelThreadsFew)
     k_select_exact(int qa, const int64_t *__restrict__ qoff, const uint32_t *__restrict__ qcount,
                    const int32_t *__restrict__ cuid,
                    const uint32_t *__restrict__ ccount, const int32_t *__restrict__ kq,
@@ -1947,6 +2013,26 @@ static rkr_status prefix_prune(const rkr_index *idx, const QueryCommon &qc, int 
   return RKR_OK;
 }
 
+// Steps 2-3 of queries qa .. qa + nblocks - 1 (one CTA each).
+static rkr_status select_approx(int qa, int nblocks, const int64_t *qoff, const uint32_t *qcount,
+                                const ApproxCand &C, const int32_t *kq, double c,
+                                const int64_t *out_off, int32_t *users_d, uint32_t *nlo_d,
+                                uint32_t *nup_d, double *est_d, int32_t *case_d, int32_t *nc_d,
+                                int *err, cudaStream_t st, const rkr_index *idx) {
+  const bool few = nblocks <= sm_count();
+  auto kern = few ? k_select_approx<kSelThreadsFew> : k_select_approx<kSelThreads>;
+  RKR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem));
+  const int prof_slot = prof_begin("k_select_approx", st);
+  kern<<<nblocks, few ? kSelThreadsFew : kSelThreads, kSelSmem, st>>>(
+      qa, qoff, qcount, C, kq, c, (uint32_t)idx->s, idx->tau, idx->fmin, idx->delta, out_off,
+      users_d, nlo_d, nup_d, est_d, case_d, nc_d, err, (uint32_t)(idx->m * idx->s),
+      user_bits(idx->n));
+  prof_end(prof_slot, st, 0.0);
+  note_launch();
+  RKR_CUDA(cudaGetLastError());
+  return RKR_OK;
+}
+
 rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq, double c,
                             int32_t *users_d, uint32_t *nlo_d, uint32_t *nup_d, double *est_d,
                             int32_t *case_d, int32_t *nc_d, rkr_query_stats *stats,
@@ -2033,21 +2119,10 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
     }
     ms_res += t3.stop();
     Timer t4(st);
-    ApproxCand C{cu, nlo, nup, th, cj, idx->U, qc.Qd, idx->d, nfp64_d};
-    size_t sm = sizeof(SortEnt) * kMaxK;
-    RKR_CUDA(cudaFuncSetAttribute(k_select_approx, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sm));
-    {
-      const int prof_slot = prof_begin("k_select_approx", st);
-      k_select_approx<<<qb - qa, kSelThreads, sm, st>>>(qa, qoff_rel, cursor, C, qc.kq_d, c,
-                                                        (uint32_t)idx->s, idx->tau, idx->fmin,
-                                                        idx->delta, qc.out_off_d, users_d, nlo_d,
-                                                        nup_d, est_d, case_d, nc_d, sel_err,
-                                                        (uint32_t)(idx->m * idx->s));
-      prof_end(prof_slot, st, 0.0);
-    }
-    note_launch();
-    RKR_CUDA(cudaGetLastError());
+    RKR_TRY(select_approx(qa, qb - qa, qoff_rel, cursor,
+                          ApproxCand{cu, nlo, nup, th, cj, idx->U, qc.Qd, idx->d, nfp64_d},
+                          qc.kq_d, c, qc.out_off_d, users_d, nlo_d, nup_d, est_d, case_d, nc_d,
+                          sel_err, st, idx));
     ms_sel += t4.stop();
   }
   RKR_CUDA(cudaStreamSynchronize(st));
@@ -2080,19 +2155,9 @@ rkr_status launch_select_approx(int qa, int nblocks, const int64_t *qoff, const 
                                 int32_t *users_d, uint32_t *nlo_d, uint32_t *nup_d, double *est_d,
                                 int32_t *case_d, int32_t *nc_d, int *err, cudaStream_t st,
                                 const rkr_index *idx) {
-  ApproxCand C{uid, nlo, nup, th, cj, idx->U, Qd, idx->d, nullptr};
-  size_t sm = sizeof(SortEnt) * kMaxK;
-  RKR_CUDA(cudaFuncSetAttribute(k_select_approx, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sm));
-  const int prof_slot = prof_begin("k_select_approx", st);
-  k_select_approx<<<nblocks, kSelThreads, sm, st>>>(qa, qoff, qcount, C, kq, c, (uint32_t)idx->s,
-                                                   idx->tau, idx->fmin, idx->delta, out_off,
-                                                   users_d, nlo_d, nup_d, est_d, case_d, nc_d,
-                                                   err, (uint32_t)(idx->m * idx->s));
-  prof_end(prof_slot, st, 0.0);
-  note_launch();
-  RKR_CUDA(cudaGetLastError());
-  return RKR_OK;
+  return select_approx(qa, nblocks, qoff, qcount,
+                       ApproxCand{uid, nlo, nup, th, cj, idx->U, Qd, idx->d, nullptr}, kq, c,
+                       out_off, users_d, nlo_d, nup_d, est_d, case_d, nc_d, err, st, idx);
 }
 
 struct LearnedPrune {
@@ -2553,7 +2618,7 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
                                   (int)sm));
     {
       const int prof_slot = prof_begin("k_select_exact", st);
-      k_select_exact<<<qb - qa, kSelThreads, sm, st>>>(qa, qoff_rel, cursor, cu, ccount, qc.kq_d,
+      k_select_exact<<<qb - qa, qb - qa <= sm_count() ? kSelThreadsFew : kSelThreads, sm, st>>>(qa, qoff_rel, cursor, cu, ccount, qc.kq_d,
                                                        qc.out_off_d, users_d, ranks_d, sel_err,
                                                        (uint32_t)idx->m, user_bits(idx->n));
       prof_end(prof_slot, st, 0.0);
