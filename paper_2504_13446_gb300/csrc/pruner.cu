@@ -100,12 +100,18 @@ __global__ void k_mlp_weights(int F, int H, int Fp, int Hp, const float *__restr
 // Dense epilogue of a tensor-core product D (M x N): v = acc + bias[col] +
 // tcol[row] * wcol[col] (each term optional); zout / fout get v (FP32), hout
 // gets relu(v) or v in BF16, houtT the same transposed (houtT[col * ldt + row]).
+// A thread holds 32 columns of one row: row-major outputs go through a shared
+// 32 x 32 tile per warp (padded by one), so that a warp writes 32 consecutive
+// columns of a row; the transposed one is written from registers, 32 consecutive
+// rows of a column.  In a K-sliced product fout holds one M x ldf block per slice.
 struct EpiDense {
   static const char *name() { return "k_screen<EpiDense>"; }
+  static constexpr int kWarps = 8;
   struct Thread {
     int64_t row;
+    int slice;
   };
-  static constexpr size_t kSmem = 0;
+  static constexpr size_t kSmem = sizeof(float) * kWarps * 32 * 33;
   int64_t M, N;
   int bn;
   const float *bias, *tcol, *wcol;
@@ -118,33 +124,62 @@ struct EpiDense {
   int64_t ldh;
   __nv_bfloat16 *houtT;
   int64_t ldt;
-  __device__ void unit_begin(char *, const tc::Unit &, int, Thread &) const {}
+  __device__ void unit_begin(char *, const tc::Unit &u, int, Thread &ts) const {
+    ts.slice = u.slice;
+  }
   __device__ void tile_begin(char *, int rb, int, int r, int, Thread &ts) const {
     ts.row = (int64_t)rb * tc::BM + r;
   }
-  __device__ void chunk(char *, int, int ct, int, int col, uint32_t, const float (&v)[32],
+  __device__ void chunk(char *S, int, int ct, int, int col, uint32_t, const float (&v)[32],
                         Thread &ts) const {
-    if (ts.row >= M) return;
-    const int64_t c0 = (int64_t)ct * bn + col;
-    const float tr = tcol ? tcol[ts.row] : 0.0f;
+    const int lane = threadIdx.x & 31;
+    float *tile = (float *)S + ((threadIdx.x >> 5) - 2) * 32 * 33;
+    const int64_t c0 = (int64_t)ct * bn + col, row0 = ts.row - lane;
+    const bool live = ts.row < M;
+    const float tr = tcol && live ? tcol[ts.row] : 0.0f;
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
       const int64_t c = c0 + j;
+      float x = v[j];
       if (c < N) {
-        float x = v[j];
         if (bias) x += bias[c];
         if (tcol) x = fmaf(tr, wcol[c], x);
-        if (zout) zout[ts.row * ldz + c] = x;
-        if (fout) fout[ts.row * ldf + c] = x;
-        const __nv_bfloat16 h = __float2bfloat16_rn(relu ? fmaxf(x, 0.0f) : x);
-        if (hout) hout[ts.row * ldh + c] = h;
-        if (houtT) houtT[c * ldt + ts.row] = h;
+        if (houtT && live)
+          houtT[c * ldt + ts.row] = __float2bfloat16_rn(relu ? fmaxf(x, 0.0f) : x);
+      }
+      tile[lane * 33 + j] = x;
+    }
+    if (!zout && !fout && !hout) return;
+    __syncwarp();
+    const int64_t c = c0 + lane;   // this lane's column of every row below
+    float *f = fout ? fout + (int64_t)ts.slice * M * ldf : nullptr;
+    if (c < N) {
+#pragma unroll 4
+      for (int i = 0; i < 32; ++i) {
+        const int64_t row = row0 + i;
+        if (row >= M) break;
+        const float x = tile[i * 33 + lane];
+        if (zout) zout[row * ldz + c] = x;
+        if (f) f[row * ldf + c] = x;
+        if (hout) hout[row * ldh + c] = __float2bfloat16_rn(relu ? fmaxf(x, 0.0f) : x);
       }
     }
+    __syncwarp();   // the tile is reused by the next chunk
   }
   __device__ void tile_end(char *, int, int, int, int, Thread &) const {}
   __device__ void unit_end(char *, const tc::Unit &, int, Thread &) const {}
 };
+
+// Sum of the K slices' products, in slice order: out[i] = sum_s part[s * count + i].
+__global__ void k_sum_slices(int64_t count, int slices, const float *__restrict__ part,
+                             float *__restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  float acc = 0.0f;
+#pragma unroll 8
+  for (int s = 0; s < slices; ++s) acc += part[(int64_t)s * count + i];
+  out[i] = acc;
+}
 
 // D = A B^T on the tensor cores: A rows of K = kp BF16 values (pitch kp), B
 // likewise; the epilogue gets D's (row, column) entries.
@@ -165,7 +200,30 @@ rkr_status dense(const __nv_bfloat16 *A, int64_t M, const __nv_bfloat16 *B, int6
   e.M = M;
   e.N = N;
   e.bn = BN;
-  return launch_screen<BN, 4>(a, b, 0, row_schedule(M, N, BN), e, err, st);
+  tc::Schedule sch = row_schedule(M, N, BN);
+  const int nk = (kp + tc::KCH - 1) / tc::KCH;
+  if (e.fout && !e.zout && !e.hout && !e.houtT && nk >= 64 && sch.nrb * sch.nct * 8 <= sm_count()) {
+    // Few tiles and a long K (the weight gradients: K is the batch): one CTA per tile
+    // would walk all of K alone.  K is cut so that the tiles' slices fill the SMs (at
+    // least 8 chunks each), the slices are summed afterwards.
+    const int tiles = sch.nrb * sch.nct;
+    const int want = std::min(sm_count() / tiles, nk / 8);
+    sch.mode = 2;
+    sch.kparts = (nk + want - 1) / want;
+    sch.parts = (nk + sch.kparts - 1) / sch.kparts;
+    sch.nunits = tiles * sch.parts;
+    float *out = e.fout, *part = nullptr;
+    const int64_t count = M * e.ldf;   // (columns past N, if any, are not read back)
+    DevBuf bp;
+    RKR_TRY(tmp_alloc(bp, &part, (size_t)count * sch.parts, st));
+    e.fout = part;
+    RKR_TRY((launch_screen<BN, 4>(a, b, 0, sch, e, err, st)));
+    k_sum_slices<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(count, sch.parts, part, out);
+    note_launch();
+    RKR_CUDA(cudaGetLastError());
+    return RKR_OK;
+  }
+  return launch_screen<BN, 4>(a, b, 0, sch, e, err, st);
 }
 
 EpiDense dense_epi() {
@@ -264,40 +322,42 @@ __global__ void k_mlp_dz1(int64_t B, int64_t cap, int H, const float *__restrict
   d1T[c * cap + r] = __float2bfloat16_rn(v);
 }
 
-// out[n] = sum_r f(D[r, n]) * rowscale[r]: f = relu when asked, rowscale = 1 when null.
-__global__ void k_colsum(int64_t B, int H, const float *__restrict__ D, int relu,
-                         const float *__restrict__ rowscale, float *__restrict__ out) {
-  const int n = blockIdx.x;
+// Column sums of D (B x H), out[n] = sum_r f(D[r, n]) * rowscale[r] (f = relu when
+// asked, rowscale = 1 when null; D null sums rowscale itself): part[s][n] of row
+// slice s by block (32 columns, slice s), a warp reading 32 consecutive columns of a
+// row, then k_sum_slices over the slices.
+constexpr int kColSlices = 64;
+__global__ void __launch_bounds__(256)
+    k_colsum(int64_t B, int H, const float *__restrict__ D, int relu,
+             const float *__restrict__ rowscale, float *__restrict__ part) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int n = blockIdx.x * 32 + lane;
+  const int64_t r0 = B * blockIdx.y / kColSlices, r1 = B * (blockIdx.y + 1) / kColSlices;
   float acc = 0.0f;
-  for (int64_t r = threadIdx.x; r < B; r += blockDim.x) {
-    float v = D[r * H + n];
-    if (relu) v = fmaxf(v, 0.0f);
-    acc += v * (rowscale ? rowscale[r] : 1.0f);
+  if (n < H) {
+#pragma unroll 4
+    for (int64_t r = r0 + w; r < r1; r += 8) {
+      float v = D ? D[r * H + n] : 1.0f;
+      if (relu) v = fmaxf(v, 0.0f);
+      acc += v * (rowscale ? rowscale[r] : 1.0f);
+    }
   }
-  __shared__ float red[256];
-  red[threadIdx.x] = acc;
+  __shared__ float red[8][33];
+  red[w][lane] = acc;
   __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
+  if (w == 0 && n < H) {
+    for (int i = 1; i < 8; ++i) acc += red[i][lane];
+    part[(int64_t)blockIdx.y * H + n] = acc;
   }
-  if (threadIdx.x == 0) out[n] = red[0];
 }
 
-// Gradients of the constrained parameters from those of the effective weights;
-// db3 = sum dy.
-__global__ void k_mlp_chain(int H, const float *__restrict__ p, Off o, float *__restrict__ g,
-                            const float *__restrict__ dy, int64_t B) {
+// Gradients of the constrained parameters from those of the effective weights.
+__global__ void k_mlp_chain(int H, const float *__restrict__ p, Off o, float *__restrict__ g) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < (int64_t)H * H) g[o.V2 + i] *= sigmoidf(p[o.V2 + i]);
   if (i < H) {
     g[o.A + i] *= -sigmoidf(p[o.A + i]);
     g[o.v3 + i] *= sigmoidf(p[o.v3 + i]);
-  }
-  if (i == 0) {
-    float s = 0.0f;
-    for (int64_t r = 0; r < B; ++r) s += dy[r];
-    g[o.b3] = s;
   }
 }
 
@@ -405,15 +465,24 @@ rkr_status backward_batch(rkr_pruner *pr, int64_t B, cudaStream_t st) {
   const Off o(F, H);
   const int64_t cap = pr->cap;
   const unsigned nb = (unsigned)((cap * H + 255) / 256);
-  // dw3 = h2^T dy (the chain rule to v3 follows)
-  k_colsum<<<H, 256, 0, st>>>(B, H, pr->z2, 1, pr->dy, pr->g + o.v3);
-  note_launch();
+  DevBuf bpart;
+  float *part;
+  RKR_TRY(tmp_alloc(bpart, &part, (size_t)kColSlices * H, st));
+  auto colsum = [&](int cols, const float *D, int relu, const float *scale, float *out) {
+    k_colsum<<<dim3((unsigned)((cols + 31) / 32), kColSlices), 256, 0, st>>>(B, cols, D, relu,
+                                                                             scale, part);
+    note_launch();
+    k_sum_slices<<<(unsigned)((cols + 255) / 256), 256, 0, st>>>(cols, kColSlices, part, out);
+    note_launch();
+  };
+  // dw3 = h2^T dy (the chain rule to v3 follows), db3 = sum dy
+  colsum(H, pr->z2, 1, pr->dy, pr->g + o.v3);
+  colsum(1, nullptr, 0, pr->dy, pr->g + o.b3);
   // dz2 = dy w3^T * (z2 > 0); db2 = column sums
   k_mlp_dz2<<<nb, 256, 0, st>>>(B, cap, H, pr->Hp, pr->dy, pr->w3, pr->z2, pr->d2, pr->d2b,
                                 pr->d2T);
   note_launch();
-  k_colsum<<<H, 256, 0, st>>>(B, H, pr->d2, 0, nullptr, pr->g + o.b2);
-  note_launch();
+  colsum(H, pr->d2, 0, nullptr, pr->g + o.b2);
   // dW2 = dz2^T h1 (H x H): K = the batch
   EpiDense ew2 = dense_epi();
   ew2.fout = pr->g + o.V2;
@@ -427,18 +496,16 @@ rkr_status backward_batch(rkr_pruner *pr, int64_t B, cudaStream_t st) {
   k_mlp_dz1<<<nb, 256, 0, st>>>(B, cap, H, pr->z1, pr->d1, pr->d1T);
   note_launch();
   // db1 = column sums; d(wt) = dz1^T t
-  k_colsum<<<H, 256, 0, st>>>(B, H, pr->d1, 0, nullptr, pr->g + o.b1);
-  note_launch();
-  k_colsum<<<H, 256, 0, st>>>(B, H, pr->d1, 0, pr->tb, pr->g + o.A);
-  note_launch();
+  colsum(H, pr->d1, 0, nullptr, pr->g + o.b1);
+  colsum(H, pr->d1, 0, pr->tb, pr->g + o.A);
   // dW1 = dz1^T X (H x F): K = the batch
   EpiDense ew1 = dense_epi();
   ew1.fout = pr->g + o.W1;
   ew1.ldf = F;
   RKR_TRY(dense(pr->d1T, H, pr->XbT, F, (int)cap, ew1, pr->err, st));
-  // constrained parameters and db3
+  // constrained parameters
   const int64_t cnt = std::max<int64_t>((int64_t)H * H, 1);
-  k_mlp_chain<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(H, pr->p, o, pr->g, pr->dy, B);
+  k_mlp_chain<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(H, pr->p, o, pr->g);
   note_launch();
   return RKR_OK;
 }

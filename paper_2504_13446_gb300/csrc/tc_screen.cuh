@@ -28,21 +28,30 @@ namespace tc {
 
 struct Unit {
   int rb0, rb1, ct0, ct1;
+  int slice = 0;    // K mode: the K slice
 };
 
 // How units are formed: ROW = one row block each; COL = one column tile and
-// one of `parts` slices of the row blocks.
+// one of `parts` slices of the row blocks; K = one tile and one of `parts` slices
+// of K, `kparts` chunks each (products with few tiles and a long K, single-CTA
+// kernel and one segment only; the epilogue keeps the slices apart).
 struct Schedule {
-  int mode;       // 0 ROW, 1 COL
+  int mode;       // 0 ROW, 1 COL, 2 K
   int nrb, nct;   // row blocks, column tiles
-  int parts;      // COL: row-block slices per column tile
+  int parts;      // COL: row-block slices per column tile; K: slices of K
   int nunits;
+  int kparts = 0; // K: chunks per slice
 };
 
 __device__ __forceinline__ Unit unit_of(const Schedule &s, int i) {
   Unit u;
   if (s.mode == 0) {
     u.rb0 = i; u.rb1 = i + 1; u.ct0 = 0; u.ct1 = s.nct;
+  } else if (s.mode == 2) {
+    const int tile = i / s.parts;
+    u.slice = i - tile * s.parts;
+    u.rb0 = tile / s.nct; u.rb1 = u.rb0 + 1;
+    u.ct0 = tile - u.rb0 * s.nct; u.ct1 = u.ct0 + 1;
   } else {
     int ct = i / s.parts, part = i - ct * s.parts;
     u.ct0 = ct; u.ct1 = ct + 1;
@@ -237,10 +246,12 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
       const int kstep = op.fp8 ? 2 * KCH : KCH;  // elements of 128 bytes
       for (int ui = blockIdx.x; ui < sch.nunits && !failed; ui += gridDim.x) {
         Unit u = unit_of(sch, ui);
+        const int k0 = u.slice * sch.kparts;   // first chunk (K mode), the slice's chunks
+        const int uk = sch.mode == 2 ? min(sch.kparts, nk - k0) : nk;
         for (int rb = u.rb0; rb < u.rb1 && !failed; ++rb)
           for (int ct = u.ct0; ct < u.ct1 && !failed; ++ct) {
             ChunkWalk w;
-            for (int kc = 0; kc < nk; ++kc, ++it) {
+            for (int kc = 0; kc < uk; ++kc, ++it) {
               const uint32_t s = ring.s;
               if (!mbar_wait(&empty[s], ring.ph ^ 1, kWaitLimit, true)) { failed = true; break; }
               unsigned char *sa = stages + (size_t)s * L::kStage;
@@ -248,7 +259,7 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
               mbar_expect_tx(&full[s], L::kStage);
               // split order: hi.lo, lo.hi, then hi.hi (small terms first)
               const bool alo = op.split && w.g == 1, blo = op.split && w.g == 0;
-              const int kx = w.c * kstep;
+              const int kx = (k0 + w.c) * kstep;
               tma_load_2d(sa, alo ? &mAl : &mAh, kx, rb * BM, &full[s]);
               tma_load_2d(sb, blo ? &mBl : &mBh, kx, ct * BN, &full[s]);
               w.next(op.kchunks);
@@ -272,6 +283,7 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
     uint32_t t = 0;
     for (int ui = blockIdx.x; ui < sch.nunits && !failed; ui += gridDim.x) {
       Unit u = unit_of(sch, ui);
+      const int uk = sch.mode == 2 ? min(sch.kparts, nk - u.slice * sch.kparts) : nk;
       for (int rb = u.rb0; rb < u.rb1 && !failed; ++rb)
         for (int ct = u.ct0; ct < u.ct1 && !failed; ++ct, ++t) {
           const int b = t & 1;
@@ -280,7 +292,7 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
           tc_fence_after();
           const uint32_t dt = tmem + (uint32_t)(b * BN);
           failed = !mma_tile<STAGES, L::kStage, L::kA>(
-              op, nk, full, desc0, ring, ready,
+              op, uk, full, desc0, ring, ready,
               [&](uint64_t da, uint64_t db, uint32_t acc) {
                 if (op.fp8) umma_e4m3(dt, da, db, idesc, acc);
                 else umma_bf16(dt, da, db, idesc, acc);
