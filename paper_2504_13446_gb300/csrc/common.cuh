@@ -154,6 +154,48 @@ struct Dot2 {
   }
 };
 
+// Rigorous FP32 upper bounds of Euclidean norms.  Squares of scaled values (a power
+// of two brings the row's largest magnitude near 1) are summed as in Dot2; all terms
+// are non-negative, so the sum is within 2^-31 (relative, up to 512 terms) of the
+// exact one, up to 2^-140 of underflow.
+struct SquareSum {
+  float p = 0.0f, s = 0.0f;
+  __device__ __forceinline__ void two_sum(float h, float low) {
+    const float t = __fadd_rn(p, h);
+    const float z = __fsub_rn(t, p);
+    const float e = __fadd_rn(__fsub_rn(p, __fsub_rn(t, z)), __fsub_rn(h, z));
+    p = t;
+    s = __fadd_rn(s, __fadd_rn(e, low));
+  }
+  __device__ __forceinline__ void add(float x) {
+    const float h = __fmul_rn(x, x);
+    two_sum(h, __fmaf_rn(x, x, -h));
+  }
+  // over the 32 lanes of a warp
+  __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float p2 = __shfl_xor_sync(0xffffffffu, p, o);
+      const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
+      two_sum(p2, s2);
+    }
+  }
+  // upper bound of sqrt(sum) * unscale
+  __device__ __forceinline__ float norm_up(float unscale) const {
+    const float t = __fadd_ru(__fmul_ru(__fadd_ru(p, fabsf(s)), 1.0f + 0x1p-23f), 0x1p-140f);
+    return __fadd_ru(__fmul_ru(__fsqrt_ru(t), unscale), 1e-45f);
+  }
+};
+
+// Power of two that brings mx (a row's largest magnitude) near 1, and its inverse;
+// both are normal floats for every mx.
+__device__ __forceinline__ void row_scale(float mx, float &scale, float &unscale) {
+  int e = (int)(__float_as_uint(mx) >> 23) - 127;   // exponent of mx (-127: zero or subnormal)
+  e = max(-126, min(e, 126));
+  scale = __uint_as_float((uint32_t)(127 - e) << 23);
+  unscale = __uint_as_float((uint32_t)(127 + e) << 23);
+}
+
 // Interval [lo, hi] that holds the canonical score s(a, b).
 __device__ __forceinline__ void dot2_interval(const float *__restrict__ a,
                                               const float *__restrict__ b, int d, double &lo,

@@ -14,40 +14,76 @@ namespace rkr {
 
 // ---------------------------------------------------------------- staging
 
-// hi = bf16(x), lo = bf16(x - hi) (x - hi and x - hi - lo are exact in FP32),
-// zero padding up to kp, and the bound terms of single and split products
-// (FP64 sums, square roots rounded up to FP32).
-__global__ void k_stage_bf16(const float *__restrict__ X, int64_t rows, int d, int kp, int ld,
-                             __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
-                             tc::RowBound *__restrict__ rb1, tc::RowBound *__restrict__ rb3) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// hi = bf16(x), lo = bf16(x - hi) (x - hi, x - hi - lo and hi + lo are exact in
+// FP32), zero padding up to kp, and the bound terms of single and split products.
+// A warp per row, two neighbouring columns a lane (rows are written 128 bytes at a
+// time); the norms are sums of squares in compensated FP32 (SquareSum), not FP64,
+// of which this GPU does a hundredth: 1M rows of d = 200 took 4.6 ms in FP64 with a
+// thread per row.
+__global__ void __launch_bounds__(256)
+    k_stage_bf16(const float *__restrict__ X, int64_t rows, int d, int kp, int ld,
+                 __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
+                 tc::RowBound *__restrict__ rb1, tc::RowBound *__restrict__ rb3) {
+  const int64_t i = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
   if (i >= rows) return;
+  const int lane = threadIdx.x & 31;
   const float *x = X + i * d;
-  double sx = 0, sh = 0, sl = 0, se1 = 0, se3 = 0, sc = 0;
-  for (int k = 0; k < kp; ++k) {
-    float v = k < d ? x[k] : 0.0f;
-    __nv_bfloat16 h = __float2bfloat16_rn(v);
-    float hf = __bfloat162float(h);
-    float r1 = v - hf;
-    __nv_bfloat16 l = __float2bfloat16_rn(r1);
-    float lf = __bfloat162float(l);
-    float r3 = r1 - lf;
-    hi[i * ld + k] = h;
-    lo[i * ld + k] = l;
-    sx += (double)v * v;
-    sh += (double)hf * hf;
-    sl += (double)lf * lf;
-    se1 += (double)r1 * r1;
-    se3 += (double)r3 * r3;
-    double c = (double)hf + (double)lf;
-    sc += c * c;
+  constexpr int kPieces = kMaxD / 64;   // column pairs per lane, at most
+  float v[kPieces][2];
+  float mx = 0.0f;
+#pragma unroll
+  for (int p = 0; p < kPieces; ++p) {
+    const int c = 64 * p + 2 * lane;
+    v[p][0] = c < d ? x[c] : 0.0f;
+    v[p][1] = c + 1 < d ? x[c + 1] : 0.0f;
+    mx = fmaxf(mx, fmaxf(fabsf(v[p][0]), fabsf(v[p][1])));
   }
-  auto up = [](double s) { return __double2float_ru(sqrt(s) * (1.0 + 0x1p-40) + 1e-300); };
-  tc::RowBound a, b;
-  a.a0 = up(se1); a.a1 = up(sh); a.a2 = up(sx); a.a3 = 0.0f; a.a4 = up(sh);
-  b.a0 = up(se3); b.a1 = up(sc); b.a2 = up(sx); b.a3 = up(sl); b.a4 = up(sh);
-  rb1[i] = a;
-  rb3[i] = b;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  float scale, unscale;
+  row_scale(mx, scale, unscale);
+  SquareSum sx, sh, sl, se1, se3, sc;
+#pragma unroll
+  for (int p = 0; p < kPieces; ++p) {
+    const int c = 64 * p + 2 * lane;
+    if (c >= kp) break;
+    __nv_bfloat162 h2, l2;
+    __nv_bfloat16 *hp = &h2.x, *lp = &l2.x;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float w = v[p][e];
+      const __nv_bfloat16 h = __float2bfloat16_rn(w);
+      const float hf = __bfloat162float(h);
+      const float r1 = w - hf;
+      const __nv_bfloat16 l = __float2bfloat16_rn(r1);
+      const float lf = __bfloat162float(l);
+      hp[e] = h;
+      lp[e] = l;
+      sx.add(w * scale);
+      sh.add(hf * scale);
+      sl.add(lf * scale);
+      se1.add(r1 * scale);
+      se3.add((r1 - lf) * scale);
+      sc.add((hf + lf) * scale);
+    }
+    *reinterpret_cast<__nv_bfloat162 *>(hi + i * ld + c) = h2;
+    *reinterpret_cast<__nv_bfloat162 *>(lo + i * ld + c) = l2;
+  }
+  sx.warp_sum();
+  sh.warp_sum();
+  sl.warp_sum();
+  se1.warp_sum();
+  se3.warp_sum();
+  sc.warp_sum();
+  if (lane == 0) {
+    tc::RowBound a, b;
+    a.a0 = se1.norm_up(unscale); a.a1 = sh.norm_up(unscale); a.a2 = sx.norm_up(unscale);
+    a.a3 = 0.0f; a.a4 = a.a1;
+    b.a0 = se3.norm_up(unscale); b.a1 = sc.norm_up(unscale); b.a2 = a.a2;
+    b.a3 = sl.norm_up(unscale); b.a4 = a.a1;
+    rb1[i] = a;
+    rb3[i] = b;
+  }
 }
 
 rkr_status tc_stage(const float *X, int64_t rows, int d, TcSide &out, cudaStream_t st) {
@@ -70,7 +106,7 @@ rkr_status tc_stage(const float *X, int64_t rows, int d, TcSide &out, cudaStream
   RKR_TRY(alloc((void **)&out.rb3, sizeof(tc::RowBound) * std::max<int64_t>(rows, 1)));
   out.owned = true;
   if (rows > 0) {
-    k_stage_bf16<<<(unsigned)((rows + 127) / 128), 128, 0, st>>>(X, rows, d, out.kp, out.ld(),
+    k_stage_bf16<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(X, rows, d, out.kp, out.ld(),
                                                                  out.hi, out.lo, out.rb1, out.rb3);
     note_launch();
     RKR_CUDA(cudaGetLastError());
@@ -540,10 +576,10 @@ extern "C" rkr_status rkr_screen_scores_static(const float *U, int64_t n, const 
   // the error word is the only scratch that must start at zero; everything else
   // is written in full before it is read
   RKR_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-  k_stage_bf16<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(U, n, d, kp, kp, A.hi, A.lo, A.rb1,
+  k_stage_bf16<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(U, n, d, kp, kp, A.hi, A.lo, A.rb1,
                                                             A.rb3);
   note_launch();
-  k_stage_bf16<<<(unsigned)((mx + 127) / 128), 128, 0, st>>>(X, mx, d, kp, kp, B.hi, B.lo, B.rb1,
+  k_stage_bf16<<<(unsigned)((mx + 7) / 8), 256, 0, st>>>(X, mx, d, kp, kp, B.hi, B.lo, B.rb1,
                                                              B.rb3);
   note_launch();
   k_tile_bounds<<<(unsigned)((ntiles + 127) / 128), 128, 0, st>>>(split ? B.rb3 : B.rb1, mx, BN,

@@ -1447,26 +1447,28 @@ __global__ void k_table_resolve(const int2 *__restrict__ items,
   }
 }
 
-// N[u][j] = sum_{c > j} W[u][c], j < tau: one warp per user.
-__global__ void k_table_suffix(int64_t n, int tau, const uint32_t *__restrict__ W,
-                               uint32_t *__restrict__ N) {
-  const int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+// N[u][j] = sum_{c > j} W[u][c], j < tau: one warp per user, 32 neighbouring columns
+// at a time from the right (loads and stores of whole lines), each with a suffix
+// scan over the lanes.
+__global__ void __launch_bounds__(256)
+    k_table_suffix(int64_t n, int tau, const uint32_t *__restrict__ W, uint32_t *__restrict__ N) {
+  const int64_t u = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
   if (u >= n) return;
-  const uint32_t *Wu = W + u * (tau + 1);
-  const int chunk = (tau + 1 + 31) / 32;
-  const int c0 = lane * chunk, c1 = min(tau + 1, c0 + chunk);
-  uint32_t part = 0;
-  for (int c = c0; c < c1; ++c) part += Wu[c];
-  uint32_t incl = part;  // inclusive suffix over lanes >= lane
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t x = __shfl_down_sync(0xffffffffu, incl, o);
-    if (lane + o < 32) incl += x;
-  }
-  uint32_t run = incl - part;
-  for (int c = c1 - 1; c >= c0; --c) {
-    run += Wu[c];
-    if (c >= 1) N[u * tau + (c - 1)] = run;
+  const int lane = threadIdx.x & 31;
+  const uint32_t *Wu = W + u * (tau + 1) + 1;   // column c = j + 1 belongs to N[j]
+  uint32_t *Nu = N + u * tau;
+  uint32_t run = 0;
+#pragma unroll 2
+  for (int j0 = (tau - 1) / 32 * 32; j0 >= 0; j0 -= 32) {
+    const int j = j0 + lane;
+    uint32_t incl = j < tau ? Wu[j] : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_down_sync(0xffffffffu, incl, o);
+      if (lane + o < 32) incl += x;
+    }
+    if (j < tau) Nu[j] = run + incl;
+    run += __shfl_sync(0xffffffffu, incl, 0);
   }
 }
 
@@ -1537,7 +1539,7 @@ rkr_status tc_rank_table(const rkr_index *idx, const TcSide &Ut, cudaStream_t st
     note_launch();
     {
       ProfScope prof("k_table_suffix", st);
-      k_table_suffix<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n, tau, W, idx->N);
+      k_table_suffix<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(n, tau, W, idx->N);
     }
     note_launch();
   }
