@@ -182,6 +182,82 @@ struct InView {
   }
 };
 
+// The output arrays of one call.  Device arrays are written in place.  Host arrays
+// whose sizes together are small share one device block, copied back in one
+// transfer (each transfer to pageable memory costs a host round trip); larger ones
+// have a device buffer and a copy each.
+struct OutSet {
+  struct Item {
+    void *user;
+    size_t bytes, off;
+    void *dev, *own;
+  };
+  static constexpr size_t kShared = (size_t)256 << 10;
+  std::vector<Item> items;
+  cudaStream_t st;
+  void *block = nullptr;
+  size_t shared = 0;
+  explicit OutSet(cudaStream_t s) : st(s) {}
+  // every array (null: not wanted) first, then alloc()
+  void add(void *p, size_t bytes) { items.push_back(Item{p, bytes, 0, nullptr, nullptr}); }
+  rkr_status alloc() {
+    size_t host = 0;
+    for (Item &x : items) {
+      if (!x.user) continue;
+      if (is_device(x.user)) x.dev = x.user;
+      else host += (x.bytes + 15) & ~(size_t)15;
+    }
+    auto get = [&](void **p, size_t bytes) -> rkr_status {
+      if (pool_malloc_async(p, bytes ? bytes : 1, st) == cudaSuccess) return RKR_OK;
+      cudaGetLastError();
+      *p = nullptr;
+      return fail(RKR_ENOMEM, "device allocation of %zu bytes failed", bytes);
+    };
+    if (host == 0) return RKR_OK;
+    if (host <= kShared) {
+      RKR_TRY(get(&block, host));
+      for (Item &x : items) {
+        if (!x.user || x.dev) continue;
+        x.off = shared;
+        x.dev = (char *)block + shared;
+        shared += (x.bytes + 15) & ~(size_t)15;
+      }
+      return RKR_OK;
+    }
+    for (Item &x : items) {
+      if (!x.user || x.dev) continue;
+      RKR_TRY(get(&x.own, x.bytes));
+      x.dev = x.own;
+    }
+    return RKR_OK;
+  }
+  template <class T>
+  T *dev(int i) const {
+    return (T *)items[i].dev;
+  }
+  // Copies what belongs to the host and waits for the stream.
+  rkr_status finish() {
+    if (block && shared) {
+      std::vector<char> h(shared);
+      RKR_CUDA(cudaMemcpyAsync(h.data(), block, shared, cudaMemcpyDeviceToHost, st));
+      RKR_CUDA(cudaStreamSynchronize(st));
+      for (const Item &x : items)
+        if (x.user && x.dev != x.user && x.bytes) memcpy(x.user, h.data() + x.off, x.bytes);
+      return RKR_OK;
+    }
+    for (const Item &x : items)
+      if (x.own && x.bytes)
+        RKR_CUDA(cudaMemcpyAsync(x.user, x.own, x.bytes, cudaMemcpyDeviceToHost, st));
+    RKR_CUDA(cudaStreamSynchronize(st));
+    return RKR_OK;
+  }
+  ~OutSet() {
+    if (block) cudaFreeAsync(block, st);
+    for (const Item &x : items)
+      if (x.own) cudaFreeAsync(x.own, st);
+  }
+};
+
 // An output array: written in place if device memory, else through a device
 // buffer copied back by finish().
 struct OutView {
@@ -422,8 +498,7 @@ struct QueryStage {
     if (xbf_own) cudaFreeAsync(xbf_own, st);
     if (member) cudaFreeAsync(member, st);
     if (soff) cudaFreeAsync(soff, st);
-    cudaStreamSynchronize(st);
-    tc_free(Qt);
+    tc_free_async(Qt, st);   // staged on this stream: freed in its order
   }
 };
 
@@ -508,15 +583,13 @@ static rkr_status stage_queries(rkr_index *idx, const float *Q, int nq, const in
   RKR_TRY(qs.vq.init(Q, sizeof(float) * (size_t)nq * d, st));
   RKR_TRY(qs.vk.init(k, sizeof(int32_t) * nq, st));
   int ok = 0;
-  RKR_TRY(all_finite((const float *)qs.vq.dev, (int64_t)nq * d, &ok, st));
-  if (!ok) return fail(RKR_EINVAL, "Q must be finite");
+  float qmax = 0.0f;
   RKR_CUDA(pool_malloc_async(&qs.qnrm, sizeof(float) * nq, st));
+  RKR_TRY(query_norms((const float *)qs.vq.dev, nq, d, qs.qnrm, &ok, &qmax, st));
+  if (!ok) return fail(RKR_EINVAL, "Q must be finite");
   RKR_CUDA(pool_malloc_async(&qs.off_d, sizeof(int64_t) * (nq + 1), st));
   RKR_CUDA(cudaMemcpyAsync(qs.off_d, off.data(), sizeof(int64_t) * (nq + 1),
                            cudaMemcpyHostToDevice, st));
-  RKR_TRY(row_norms((const float *)qs.vq.dev, nq, d, nullptr, qs.qnrm, st));
-  float qmax = 0.0f;
-  RKR_TRY(max_float(qs.qnrm, nq, &qmax, st));
   qc.Qd = (float *)qs.vq.dev;
   qc.qnrm = qs.qnrm;
   qc.kq_d = (int32_t *)qs.vk.dev;
@@ -556,15 +629,13 @@ static rkr_status query_exact_impl(rkr_index *idx, const float *Q, int32_t nq, c
   if (subsets) RKR_TRY(stage_subsets(idx, nq, kh, subset_offs, subset_users, st, qs, qc));
   if (words >= 0) RKR_TRY(stage_bitmaps(idx, nq, kh, member, words, st, qs, qc));
   RKR_TRY(stage_queries(idx, Q, nq, k, off, st, qs, qc));
-  OutView ou, orr;
+  OutSet out(st);
   size_t tot = (size_t)off[nq];
-  RKR_TRY(ou.init(out_users, sizeof(int32_t) * tot, st));
-  RKR_TRY(orr.init(out_ranks, sizeof(int32_t) * tot, st));
-  RKR_TRY(run_query_exact(idx, qc, nq, (int32_t *)ou.dev, (int32_t *)orr.dev, stats, st));
-  RKR_TRY(ou.finish());
-  RKR_TRY(orr.finish());
-  RKR_CUDA(cudaStreamSynchronize(st));
-  return RKR_OK;
+  out.add(out_users, sizeof(int32_t) * tot);
+  out.add(out_ranks, sizeof(int32_t) * tot);
+  RKR_TRY(out.alloc());
+  RKR_TRY(run_query_exact(idx, qc, nq, out.dev<int32_t>(0), out.dev<int32_t>(1), stats, st));
+  return out.finish();
 }
 
 static rkr_status query_approx_impl(rkr_index *idx, const float *Q, int32_t nq,
@@ -587,29 +658,18 @@ static rkr_status query_approx_impl(rkr_index *idx, const float *Q, int32_t nq,
   if (words >= 0) RKR_TRY(stage_bitmaps(idx, nq, kh, member, words, st, qs, qc));
   RKR_TRY(stage_queries(idx, Q, nq, k, off, st, qs, qc));
   size_t tot = (size_t)off[nq];
-  OutView ou, olo, oup, oes, oca, onc;
-  RKR_TRY(ou.init(out_users, sizeof(int32_t) * tot, st));
-  RKR_TRY(olo.init(out_nlow, sizeof(uint32_t) * tot, st));
-  RKR_TRY(oup.init(out_nup, sizeof(uint32_t) * tot, st));
-  RKR_TRY(oes.init(out_est, sizeof(double) * tot, st));
-  RKR_TRY(oca.init(out_case, sizeof(int32_t) * nq, st));
-  RKR_TRY(onc.init(out_nc, sizeof(int32_t) * nq, st));
-  if (single)
-    RKR_TRY(run_query_approx_single(idx, qc, nq, c, (int32_t *)ou.dev, (uint32_t *)olo.dev,
-                                    (uint32_t *)oup.dev, (double *)oes.dev, (int32_t *)oca.dev,
-                                    (int32_t *)onc.dev, stats, st));
-  else
-    RKR_TRY(run_query_approx(idx, qc, nq, c, (int32_t *)ou.dev, (uint32_t *)olo.dev,
-                             (uint32_t *)oup.dev, (double *)oes.dev, (int32_t *)oca.dev,
-                             (int32_t *)onc.dev, stats, st));
-  RKR_TRY(ou.finish());
-  RKR_TRY(olo.finish());
-  RKR_TRY(oup.finish());
-  RKR_TRY(oes.finish());
-  RKR_TRY(oca.finish());
-  RKR_TRY(onc.finish());
-  RKR_CUDA(cudaStreamSynchronize(st));
-  return RKR_OK;
+  OutSet out(st);
+  out.add(out_users, sizeof(int32_t) * tot);
+  out.add(out_nlow, sizeof(uint32_t) * tot);
+  out.add(out_nup, sizeof(uint32_t) * tot);
+  out.add(out_est, sizeof(double) * tot);
+  out.add(out_case, sizeof(int32_t) * nq);
+  out.add(out_nc, sizeof(int32_t) * nq);
+  RKR_TRY(out.alloc());
+  auto run = single ? run_query_approx_single : run_query_approx;
+  RKR_TRY(run(idx, qc, nq, c, out.dev<int32_t>(0), out.dev<uint32_t>(1), out.dev<uint32_t>(2),
+              out.dev<double>(3), out.dev<int32_t>(4), out.dev<int32_t>(5), stats, st));
+  return out.finish();
 }
 
 rkr_status rkr_query_exact(rkr_index *idx, const float *Q, int32_t nq, const int32_t *k,

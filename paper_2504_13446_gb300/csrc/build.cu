@@ -86,6 +86,61 @@ rkr_status row_norms(const float *X, int64_t rows, int d, double *nrm64, float *
   return RKR_OK;
 }
 
+// Queries: the norm bound of each row as above, whether every value is finite
+// (out[0] stays 0) and the largest bound (out[1], float bits), in one launch.
+__global__ void __launch_bounds__(256)
+    k_query_norms(const float *__restrict__ X, int64_t rows, int d, float *__restrict__ nrm32,
+                  unsigned *__restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
+  if (i >= rows) return;
+  const int lane = threadIdx.x & 31;
+  const float *x = X + i * d;
+  constexpr int kPieces = kMaxD / 32;
+  float v[kPieces], mx = 0.0f;
+  bool bad = false;
+#pragma unroll
+  for (int p = 0; p < kPieces; ++p) {
+    const int c = lane + 32 * p;
+    v[p] = c < d ? x[c] : 0.0f;
+    bad |= !isfinite(v[p]);
+    mx = fmaxf(mx, fabsf(v[p]));
+  }
+  bad = __any_sync(0xffffffffu, bad);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  float scale, unscale;
+  row_scale(mx, scale, unscale);
+  SquareSum s;
+#pragma unroll
+  for (int p = 0; p < kPieces; ++p)
+    if (32 * p < d) s.add(v[p] * scale);
+  s.warp_sum();
+  if (lane == 0) {
+    const float nv = s.norm_up(unscale);
+    nrm32[i] = nv;
+    if (bad) atomicOr(&out[0], 1u);
+    else atomicMax(&out[1], __float_as_uint(nv));   // nv >= 0
+  }
+}
+
+rkr_status query_norms(const float *Q, int64_t rows, int d, float *nrm32, int *ok_host,
+                       float *max_host, cudaStream_t st) {
+  DevBuf b;
+  unsigned *out, h[2] = {0, 0};
+  RKR_TRY(tmp_alloc(b, &out, 2, st));
+  RKR_CUDA(cudaMemsetAsync(out, 0, sizeof(h), st));
+  const int prof_slot = prof_begin("k_query_norms", st);
+  k_query_norms<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(Q, rows, d, nrm32, out);
+  prof_end(prof_slot, st, 0.0);
+  note_launch();
+  RKR_CUDA(cudaGetLastError());
+  RKR_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, st));
+  RKR_CUDA(cudaStreamSynchronize(st));
+  *ok_host = h[0] == 0;
+  *max_host = u32_float(h[1]);
+  return RKR_OK;
+}
+
 __global__ void k_max_float(const float *__restrict__ x, int64_t count, unsigned *out) {
   float m = 0.0f;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
@@ -558,11 +613,11 @@ static uint64_t splitmix64(uint64_t &x) {
 // ----------------------------------------------------------------- build
 
 template <class T>
-static rkr_status dalloc(T **p, size_t count) {
-  // index arrays: from the library pool, usable on every stream once this returns
+static rkr_status dalloc(T **p, size_t count, cudaStream_t st) {
+  // index arrays: from the library pool in the order of the build's stream, which the
+  // build synchronizes before it returns (from then on every stream may use them)
   if (count == 0) count = 1;
-  cudaError_t e = pool_malloc_async(p, count * sizeof(T), (cudaStream_t)0);
-  if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)0);
+  cudaError_t e = pool_malloc_async(p, count * sizeof(T), st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -594,28 +649,28 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
   RKR_CUDA(cudaEventRecord(ev[0], st));
 
   // users: own copy + norm bounds
-  RKR_TRY(dalloc(&idx->U, (size_t)n * d));
+  RKR_TRY(dalloc(&idx->U, (size_t)n * d, st));
   RKR_CUDA(cudaMemcpyAsync(idx->U, U_dev, sizeof(float) * n * d, cudaMemcpyDeviceToDevice, st));
-  RKR_TRY(dalloc(&idx->unrm, n));
+  RKR_TRY(dalloc(&idx->unrm, n, st));
   RKR_TRY(row_norms(idx->U, n, d, nullptr, idx->unrm, st));
 
   // items: FP64 norms, sort by (descending norm, index)
   float *pn32 = nullptr;
-  RKR_TRY(dalloc(&idx->pnorm, m));
-  RKR_TRY(dalloc(&pn32, m));
+  RKR_TRY(dalloc(&idx->pnorm, m, st));
+  RKR_TRY(dalloc(&pn32, m, st));
   RKR_TRY(row_norms(P_dev, m, d, idx->pnorm, pn32, st));
   int64_t Np2 = 1;
   while (Np2 < m) Np2 <<= 1;
   uint64_t *keys = nullptr;
   int32_t *vals = nullptr;
-  RKR_TRY(dalloc(&keys, Np2));
-  RKR_TRY(dalloc(&vals, Np2));
+  RKR_TRY(dalloc(&keys, Np2, st));
+  RKR_TRY(dalloc(&vals, Np2, st));
   k_norm_keys<<<(unsigned)((Np2 + bs - 1) / bs), bs, 0, st>>>(idx->pnorm, m, Np2, keys, vals); note_launch();
   RKR_TRY(sort_pairs(keys, vals, Np2, st));
-  RKR_TRY(dalloc(&idx->perm, m));
+  RKR_TRY(dalloc(&idx->perm, m, st));
   RKR_CUDA(cudaMemcpyAsync(idx->perm, vals, sizeof(int32_t) * m, cudaMemcpyDeviceToDevice, st));
-  RKR_TRY(dalloc(&idx->Ps, (size_t)m * d));
-  RKR_TRY(dalloc(&idx->pnrm_s, m));
+  RKR_TRY(dalloc(&idx->Ps, (size_t)m * d, st));
+  RKR_TRY(dalloc(&idx->pnrm_s, m, st));
   {
     const int prof_slot = prof_begin("k_gather_sorted", st);
     k_gather_sorted<<<(unsigned)((m + 127) / 128), 128, 0, st>>>(P_dev, idx->perm, pn32, m, d,
@@ -631,8 +686,8 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
   RKR_TRY(tc_make_cat(idx->Pt, 2, st));
   // hash table of the sorted item rows (a query equal to an item ties with it exactly)
   idx->phn = Np2;
-  RKR_TRY(dalloc(&idx->phk, Np2));
-  RKR_TRY(dalloc(&idx->phv, Np2));
+  RKR_TRY(dalloc(&idx->phk, Np2, st));
+  RKR_TRY(dalloc(&idx->phv, Np2, st));
   RKR_TRY(row_hashes(idx->Ps, m, d, Np2, idx->phk, idx->phv, st));
   RKR_TRY(sort_pairs(idx->phk, idx->phv, Np2, st));
   cudaFreeAsync(keys, st);
@@ -696,15 +751,15 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
   }
   idx->nsamp = (int)spos.size();
   int64_t *spos_d = nullptr;
-  RKR_TRY(dalloc(&spos_d, spos.size()));
-  RKR_TRY(dalloc(&idx->sw, sw.size()));
+  RKR_TRY(dalloc(&spos_d, spos.size(), st));
+  RKR_TRY(dalloc(&idx->sw, sw.size(), st));
   RKR_CUDA(cudaMemcpyAsync(spos_d, spos.data(), sizeof(int64_t) * spos.size(),
                            cudaMemcpyHostToDevice, st));
   RKR_CUDA(cudaMemcpyAsync(idx->sw, sw.data(), sizeof(uint32_t) * sw.size(),
                            cudaMemcpyHostToDevice, st));
-  RKR_TRY(dalloc(&idx->S, (size_t)idx->nsamp * d));
-  RKR_TRY(dalloc(&idx->snrm, idx->nsamp));
-  RKR_TRY(dalloc(&idx->samp_items, idx->nsamp));
+  RKR_TRY(dalloc(&idx->S, (size_t)idx->nsamp * d, st));
+  RKR_TRY(dalloc(&idx->snrm, idx->nsamp, st));
+  RKR_TRY(dalloc(&idx->samp_items, idx->nsamp, st));
   k_gather_samples<<<(idx->nsamp + 127) / 128, 128, 0, st>>>(idx->Ps, idx->pnrm_s, idx->perm, d,
                                                              spos_d, idx->sw, idx->nsamp, idx->S,
                                                              idx->snrm, idx->samp_items); note_launch();
@@ -715,10 +770,10 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
 
   RKR_CUDA(cudaEventRecord(ev[2], st));
   // f_min / f_max and bins
-  RKR_TRY(dalloc(&idx->fmin, n));
-  RKR_TRY(dalloc(&idx->fmax, n));
-  RKR_TRY(dalloc(&idx->delta, n));
-  RKR_TRY(dalloc(&idx->binfp, n));
+  RKR_TRY(dalloc(&idx->fmin, n, st));
+  RKR_TRY(dalloc(&idx->fmax, n, st));
+  RKR_TRY(dalloc(&idx->delta, n, st));
+  RKR_TRY(dalloc(&idx->binfp, n, st));
   bool fb_done = false;
   if (idx->fbounds == 0) {
     rkr_status fs = tc_fbounds(idx, idx->Ut, idx->Pt, idx->fmin, idx->fmax, st);
@@ -756,7 +811,7 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
 
   RKR_CUDA(cudaEventRecord(ev[3], st));
   // sampled rank table
-  RKR_TRY(dalloc(&idx->N, (size_t)n * tau));
+  RKR_TRY(dalloc(&idx->N, (size_t)n * tau, st));
   bool table_done = false;
   RKR_TRY(tc_rank_table(idx, idx->Ut, st, &table_done));
   if (!table_done) {
@@ -778,8 +833,8 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
   }
   RKR_CUDA(cudaEventRecord(ev[4], st));
   idx->nlev_a = levels_for((uint64_t)m);
-  RKR_TRY(dalloc(&idx->JU, (size_t)n * kMaxLevels));
-  RKR_TRY(dalloc(&idx->JL, (size_t)n * kMaxLevels));
+  RKR_TRY(dalloc(&idx->JU, (size_t)n * kMaxLevels, st));
+  RKR_TRY(dalloc(&idx->JL, (size_t)n * kMaxLevels, st));
   k_levels<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(n, tau, idx->N, idx->N,
                                                         (uint32_t)(m * s), (uint32_t)s,
                                                         idx->nlev_a, idx->JU, idx->JL); note_launch();
@@ -789,20 +844,20 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
   // exact count table
   if (idx->has_exact) {
     idx->xg = kXGrid;
-    RKR_TRY(dalloc(&idx->xfloor, n));
-    RKR_TRY(dalloc(&idx->xg0, n));
-    RKR_TRY(dalloc(&idx->xdx, n));
-    RKR_TRY(dalloc(&idx->xbin, n));
-    RKR_TRY(dalloc(&idx->XLO, (size_t)n * kXGrid));
-    RKR_TRY(dalloc(&idx->XHI, (size_t)n * kXGrid));
-    RKR_TRY(dalloc(&idx->xlcnt, n));
-    RKR_TRY(dalloc(&idx->xcoff, (size_t)n * (kListG + 2)));
-    RKR_TRY(dalloc(&idx->ldx, n));
-    RKR_TRY(dalloc(&idx->lbin, n));
-    RKR_TRY(dalloc(&idx->xbmax, n));
-    RKR_TRY(dalloc(&idx->ptile3, (size_t)((m + 255) / 256)));
-    RKR_TRY(dalloc(&idx->xlcap, n));
-    RKR_TRY(dalloc(&idx->xloff, n + 1));
+    RKR_TRY(dalloc(&idx->xfloor, n, st));
+    RKR_TRY(dalloc(&idx->xg0, n, st));
+    RKR_TRY(dalloc(&idx->xdx, n, st));
+    RKR_TRY(dalloc(&idx->xbin, n, st));
+    RKR_TRY(dalloc(&idx->XLO, (size_t)n * kXGrid, st));
+    RKR_TRY(dalloc(&idx->XHI, (size_t)n * kXGrid, st));
+    RKR_TRY(dalloc(&idx->xlcnt, n, st));
+    RKR_TRY(dalloc(&idx->xcoff, (size_t)n * (kListG + 2), st));
+    RKR_TRY(dalloc(&idx->ldx, n, st));
+    RKR_TRY(dalloc(&idx->lbin, n, st));
+    RKR_TRY(dalloc(&idx->xbmax, n, st));
+    RKR_TRY(dalloc(&idx->ptile3, (size_t)((m + 255) / 256), st));
+    RKR_TRY(dalloc(&idx->xlcap, n, st));
+    RKR_TRY(dalloc(&idx->xloff, n + 1, st));
     k_floor_cols<<<(unsigned)((n + bs - 1) / bs), bs, 0, st>>>(n, tau, idx->N, (uint32_t)s,
                                                                (uint64_t)idx->floor_rank,
                                                                idx->xfloor); note_launch();
@@ -817,7 +872,7 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
                                cudaMemcpyDeviceToHost, st));
       RKR_CUDA(cudaStreamSynchronize(st));
       for (int64_t u = 0; u < n; ++u) off[u + 1] = off[u] + cap[u];
-      RKR_TRY(dalloc(&idx->xlist, (size_t)std::max<int64_t>(off[n], 1)));
+      RKR_TRY(dalloc(&idx->xlist, (size_t)std::max<int64_t>(off[n], 1), st));
       RKR_CUDA(cudaMemcpyAsync(idx->xloff, off.data(), sizeof(int64_t) * (n + 1),
                                cudaMemcpyHostToDevice, st));
       RKR_CUDA(cudaStreamSynchronize(st));
@@ -827,11 +882,11 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
       // deep count grid from the sampled table's threshold of estimated count
       // m / 8 up to x_0
       idx->dg = kDGrid;
-      RKR_TRY(dalloc(&idx->yg0, n));
-      RKR_TRY(dalloc(&idx->ydx, n));
-      RKR_TRY(dalloc(&idx->ybin, n));
-      RKR_TRY(dalloc(&idx->DLO, (size_t)n * kDGrid));
-      RKR_TRY(dalloc(&idx->DHI, (size_t)n * kDGrid));
+      RKR_TRY(dalloc(&idx->yg0, n, st));
+      RKR_TRY(dalloc(&idx->ydx, n, st));
+      RKR_TRY(dalloc(&idx->ybin, n, st));
+      RKR_TRY(dalloc(&idx->DLO, (size_t)n * kDGrid, st));
+      RKR_TRY(dalloc(&idx->DHI, (size_t)n * kDGrid, st));
       DevBuf bcol, btop, bbot;
       int32_t *col;
       float *ytop, *ybot;
@@ -850,8 +905,8 @@ rkr_status build_index(rkr_index *idx, const float *U_dev, const float *P_dev,
       RKR_TRY(tc_deep_table(idx, idx->Ut, idx->Pt, ytop, ybot, st));
     }
     idx->nlev_x = levels_for((uint64_t)m);
-    RKR_TRY(dalloc(&idx->XJU, (size_t)n * kMaxLevels));
-    RKR_TRY(dalloc(&idx->XJL, (size_t)n * kMaxLevels));
+    RKR_TRY(dalloc(&idx->XJU, (size_t)n * kMaxLevels, st));
+    RKR_TRY(dalloc(&idx->XJL, (size_t)n * kMaxLevels, st));
     k_levels<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(n, kXGrid, idx->XHI, idx->XLO,
                                                           (uint32_t)m, 1u, idx->nlev_x, idx->XJU,
                                                           idx->XJL); note_launch();

@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "rkr.h"
 
 namespace rkr {
@@ -428,25 +430,43 @@ inline rkr_status tmp_alloc(DevBuf &b, T **out, size_t count, cudaStream_t st) {
   return RKR_OK;
 }
 
-struct Timer {
-  cudaEvent_t a = nullptr, b = nullptr;
+// Device times of stretches of one call: events recorded as the stretches begin and
+// end, read once by finish() after the call's own synchronization (no waiting in
+// between).
+struct SpanClock {
+  struct Span {
+    cudaEvent_t a, b;
+    double *acc;   // milliseconds are added here
+  };
   cudaStream_t st;
-  explicit Timer(cudaStream_t s) : st(s) {
-    cudaEventCreate(&a);
-    cudaEventCreate(&b);
-    cudaEventRecord(a, st);
+  std::vector<Span> spans;
+  explicit SpanClock(cudaStream_t s) : st(s) {}
+  int begin(double *acc) {
+    Span x{nullptr, nullptr, acc};
+    if (cudaEventCreate(&x.a) != cudaSuccess || cudaEventCreate(&x.b) != cudaSuccess)
+      cudaGetLastError();
+    spans.push_back(x);
+    if (x.a) cudaEventRecord(x.a, st);
+    return (int)spans.size() - 1;
   }
-  double stop() {
-    cudaEventRecord(b, st);
-    cudaEventSynchronize(b);
-    float ms = 0.0f;
-    cudaEventElapsedTime(&ms, a, b);
-    return ms;
+  void end(int i) {
+    if (spans[i].b) cudaEventRecord(spans[i].b, st);
   }
-  ~Timer() {
-    cudaEventDestroy(a);
-    cudaEventDestroy(b);
+  void finish() {   // the stream has been synchronized
+    for (Span &x : spans) {
+      float ms = 0.0f;
+      if (x.a && x.b && cudaEventElapsedTime(&ms, x.a, x.b) == cudaSuccess) *x.acc += ms;
+      else cudaGetLastError();
+    }
   }
+  ~SpanClock() {
+    for (Span &x : spans) {
+      if (x.a) cudaEventDestroy(x.a);
+      if (x.b) cudaEventDestroy(x.b);
+    }
+  }
+  SpanClock(const SpanClock &) = delete;
+  SpanClock &operator=(const SpanClock &) = delete;
 };
 
 // Order-preserving key of a non-negative double.

@@ -217,6 +217,11 @@ rkr_status query_self(const rkr_index *idx, const float *Q, int nq, int32_t *qse
 rkr_status row_norms(const float *X, int64_t rows, int d, double *nrm64, float *nrm32,
                      cudaStream_t st);
 
+// Norm bounds of a query batch, whether it is finite and the largest bound (one host
+// round trip).
+rkr_status query_norms(const float *Q, int64_t rows, int d, float *nrm32, int *ok_host,
+                       float *max_host, cudaStream_t st);
+
 // Largest element of a float array (device -> host), used for norm bounds.
 rkr_status max_float(const float *x, int64_t count, float *out_host, cudaStream_t st);
 

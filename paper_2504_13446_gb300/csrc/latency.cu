@@ -627,7 +627,9 @@ rkr_status run_query_approx_single(const rkr_index *idx, const QueryCommon &qc, 
   RKR_TRY(tmp_alloc(b11, &cth, n, st));
   int *err = (int *)(sb.nfp64 + 1);
   const unsigned cgrid = (unsigned)((n + 1023) / 1024);   // four users a thread
-  Timer t1(st);
+  double ms = 0.0;
+  SpanClock clk(st);
+  const int t1 = clk.begin(&ms);
   for (int q = 0; q < nq; ++q) {
     RKR_TRY(scan_pass(idx, qc, q, sb, st));
     {
@@ -642,10 +644,11 @@ rkr_status run_query_approx_single(const rkr_index *idx, const QueryCommon &qc, 
                                  nc_d, err, st, idx));
   }
   RKR_CUDA(cudaGetLastError());
-  const double ms = t1.stop();
+  clk.end(t1);
   unsigned long long h[3] = {0, 0, 0};
   RKR_CUDA(cudaMemcpyAsync(h, sb.nfp64, sizeof(h), cudaMemcpyDeviceToHost, st));
   RKR_CUDA(cudaStreamSynchronize(st));
+  clk.finish();
   if ((int)h[2]) return fail(RKR_ETIMEOUT, "latency scan wait timed out (%d)", (int)h[2]);
   if ((int)h[1]) return fail(RKR_EINTERNAL, "fewer than k candidates for a query");
   if (stats) {

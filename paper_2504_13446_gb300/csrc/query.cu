@@ -1141,16 +1141,20 @@ static rkr_status skim_queries(const rkr_index *idx, const QueryCommon &qc, int 
     return true;
   };
   if (!try_alloc(plan.blu, &L.u, ent) || !try_alloc(plan.blq, &L.q, ent) ||
-      !try_alloc(plan.blx, &L.x, ent) || !try_alloc(plan.blc, &L.cnt, regions) ||
+      !try_alloc(plan.blx, &L.x, ent) || !try_alloc(plan.blc, &L.cnt, regions + 1) ||
       !try_alloc(plan.bjj, &plan.jj, ent) || !try_alloc(plan.blv, &plan.lv, ent))
     return RKR_OK;
   RKR_CUDA(cudaMemsetAsync(L.cnt, 0, sizeof(uint32_t) * regions, st));
   RKR_TRY(tc_skim(idx, idx->Ut, qc.Qt, plan.xs, L, flag, st));
-  std::vector<uint32_t> cnt(regions);
-  RKR_CUDA(cudaMemcpyAsync(cnt.data(), L.cnt, sizeof(uint32_t) * regions, cudaMemcpyDeviceToHost,
-                           st));
+  std::vector<uint32_t> cnt(regions + 1);
+  // (the screen's error word stands behind the counts: one transfer)
+  RKR_CUDA(cudaMemcpyAsync(L.cnt + regions, flag, sizeof(int), cudaMemcpyDeviceToDevice, st));
+  RKR_CUDA(cudaMemcpyAsync(cnt.data(), L.cnt, sizeof(uint32_t) * (regions + 1),
+                           cudaMemcpyDeviceToHost, st));
   RKR_CUDA(cudaStreamSynchronize(st));
-  RKR_TRY(check_flag(flag, "skim screen", st));
+  if (cnt[regions]) return fail(RKR_ETIMEOUT, "skim screen: screen kernel wait timed out (%d)",
+                                (int)cnt[regions]);
+  cnt.resize(regions);
   uint32_t mx = 0;
   for (uint32_t c : cnt) {
     if ((int64_t)c > L.rcap) return RKR_OK;  // overflow: not listed
@@ -1211,6 +1215,10 @@ static ThetaArgs theta_args(const Grid &g, int qa, const QueryCommon &qc) {
   a.scale = g.scale;
   return a;
 }
+
+// Bytes of the plan's per-query results: int64 candidate counts, int32 levels, then
+// the screens' error word.
+static size_t plan_bytes(int nq) { return (sizeof(int64_t) + sizeof(int32_t)) * nq + sizeof(int); }
 
 // Passes 1 and 3: per-query cutoff level, refined cap, and candidate-count bounds.
 static rkr_status screen_plan(const rkr_index *idx, const QueryCommon &qc, int nq,
@@ -1333,23 +1341,66 @@ static rkr_status screen_plan(const rkr_index *idx, const QueryCommon &qc, int n
                                                   cap_d);
   note_launch();
   RKR_CUDA(cudaGetLastError());
-  RKR_TRY(check_flag(flag, "theta passes 1 and 3", st));
+  // candidate counts, cutoff levels and the error word lie behind one another
   plan.ncand.resize(nq);
   plan.lstar.resize(nq);
-  RKR_CUDA(cudaMemcpyAsync(plan.ncand.data(), ncand_d, sizeof(int64_t) * nq,
-                           cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaMemcpyAsync(plan.lstar.data(), lstar_d, sizeof(int32_t) * nq,
-                           cudaMemcpyDeviceToHost, st));
+  std::vector<char> h(plan_bytes(nq));
+  RKR_CUDA(cudaMemcpyAsync((char *)ncand_d + h.size() - sizeof(int), flag, sizeof(int),
+                           cudaMemcpyDeviceToDevice, st));
+  RKR_CUDA(cudaMemcpyAsync(h.data(), ncand_d, h.size(), cudaMemcpyDeviceToHost, st));
   RKR_CUDA(cudaStreamSynchronize(st));
+  memcpy(plan.ncand.data(), h.data(), sizeof(int64_t) * nq);
+  memcpy(plan.lstar.data(), h.data() + sizeof(int64_t) * nq, sizeof(int32_t) * nq);
+  int err = 0;
+  memcpy(&err, h.data() + h.size() - sizeof(int), sizeof(int));
+  if (err) return fail(RKR_ETIMEOUT, "theta passes 1 and 3: screen kernel wait timed out (%d)", err);
   return RKR_OK;
 }
 
-// Pass 2: candidates of queries [qa, qb) appended to per-query segments.
+// Error words and counters of one query call on the device, read once at its end
+// (zeroed at its start).  Every write of a failed screen stays within its buffers.
+struct CallWords {
+  int screen_err, overflow, select_err, pad;
+  unsigned long long nfp64, candidates, ties[2];
+};
+static rkr_status words_alloc(DevBuf &b, CallWords **w, cudaStream_t st) {
+  RKR_TRY(tmp_alloc(b, w, 1, st));
+  RKR_CUDA(cudaMemsetAsync(*w, 0, sizeof(CallWords), st));
+  return RKR_OK;
+}
+// Reads them (waiting for the stream) and turns errors into a status.
+static rkr_status words_check(const CallWords *w, CallWords &h, cudaStream_t st) {
+  RKR_CUDA(cudaMemcpyAsync(&h, w, sizeof(h), cudaMemcpyDeviceToHost, st));
+  RKR_CUDA(cudaStreamSynchronize(st));
+  if (h.screen_err)
+    return fail(RKR_ETIMEOUT, "theta pass 2: screen kernel wait timed out (%d)", h.screen_err);
+  if (h.overflow) return fail(RKR_EINTERNAL, "candidate segment overflow in theta pass 2");
+  if (h.select_err) return fail(RKR_EINTERNAL, "fewer than k candidates for a query");
+  return RKR_OK;
+}
+
+// Sums the candidates of queries [qa, qb).  A cursor that ran past its segment
+// (reported as overflow) goes back to the segment's end: what follows reads no further.
+__global__ void k_close_segments(int qa, int qb, const int64_t *__restrict__ qoff,
+                                 uint32_t *__restrict__ cursor,
+                                 unsigned long long *__restrict__ sum) {
+  unsigned long long s = 0;
+  for (int q = qa + blockIdx.x * blockDim.x + threadIdx.x; q < qb; q += gridDim.x * blockDim.x) {
+    const int64_t room = qoff[q + 1] - qoff[q];
+    if ((int64_t)cursor[q] > room) cursor[q] = (uint32_t)room;
+    s += cursor[q];
+  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0 && s) atomicAdd(sum, s);
+}
+
+// Pass 2: candidates of queries [qa, qb) appended to per-query segments.  Nothing is
+// waited for: errors stand in *words.
 static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, int qa, int qb,
                                   const Grid &g, const Plan &plan, const int32_t *lstar_d,
                                   const uint32_t *cap_d, const int64_t *qoff_d, uint32_t *cursor_d,
                                   int32_t *cand_u, int32_t *cand_q, float *cand_x,
-                                  cudaStream_t st) {
+                                  CallWords *words, cudaStream_t st) {
   TcSide sub = qc.Qt;
   sub.owned = false;
   sub.rows = qb - qa;
@@ -1357,13 +1408,10 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
   sub.lo = qc.Qt.lo + (size_t)qa * qc.Qt.ld();
   sub.rb1 = qc.Qt.rb1 + qa;
   sub.rb3 = qc.Qt.rb3 + qa;
-  DevBuf bf;
-  int *flag;
-  RKR_TRY(tmp_alloc(bf, &flag, 2, st));
-  RKR_CUDA(cudaMemsetAsync(flag, 0, 2 * sizeof(int), st));
+  int *flag = &words->screen_err;
   ThetaArgs a = theta_args(g, qa, qc);
   a.nq_all = qc.Qt.rows;
-  a.ovf = flag + 1;
+  a.ovf = &words->overflow;
   a.lstar = lstar_d;
   a.cap = cap_d;
   a.qoff = qoff_d;
@@ -1379,7 +1427,8 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
         const int prof_slot = prof_begin("k_list_emit", st);
         k_list_emit<<<list_grid(plan), 256, 0, st>>>(plan.list, plan.jj, plan.lv, qa, qb, lstar_d,
                                                      plan.lskip, cap_d, g.tlo, g.tau, qoff_d,
-                                                     cursor_d, cand_u, cand_q, cand_x, flag + 1);
+                                                     cursor_d, cand_u, cand_q, cand_x,
+                                                     &words->overflow);
         prof_end(prof_slot, st, 0.0);
       }
       note_launch();
@@ -1405,10 +1454,10 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
     ad.lskip = 1 << 30;
     RKR_TRY(tc_theta_pass(2, idx, idx->Ut, ds, ad, kThetaSplit, flag, st));
   }
-  RKR_TRY(check_flag(flag, "theta pass 2", st));
-  int ovf = 0;
-  RKR_CUDA(cudaMemcpy(&ovf, flag + 1, sizeof(int), cudaMemcpyDeviceToHost));
-  if (ovf) return fail(RKR_EINTERNAL, "candidate segment overflow in theta pass 2");
+  k_close_segments<<<std::min((qb - qa + 255) / 256, 64), 256, 0, st>>>(qa, qb, qoff_d, cursor_d,
+                                                                        &words->candidates);
+  note_launch();
+  RKR_CUDA(cudaGetLastError());
   return RKR_OK;
 }
 
@@ -2037,27 +2086,25 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
                             int32_t *users_d, uint32_t *nlo_d, uint32_t *nup_d, double *est_d,
                             int32_t *case_d, int32_t *nc_d, rkr_query_stats *stats,
                             cudaStream_t st) {
-  DevBuf bl, bn, bcap;
+  DevBuf bn, bcap;
   int32_t *lstar_d;
   int64_t *ncand_d;
   uint32_t *cap_d;
-  RKR_TRY(tmp_alloc(bl, &lstar_d, nq, st));
-  RKR_TRY(tmp_alloc(bn, &ncand_d, nq, st));
+  RKR_TRY(tmp_alloc(bn, (char **)&ncand_d, plan_bytes(nq), st));
+  lstar_d = (int32_t *)(ncand_d + nq);
   RKR_TRY(tmp_alloc(bcap, &cap_d, nq, st));
-  DevBuf bse, bnf;
-  int *sel_err;
-  unsigned long long *nfp64_d;
-  RKR_TRY(tmp_alloc(bse, &sel_err, 1, st));
-  RKR_CUDA(cudaMemsetAsync(sel_err, 0, sizeof(int), st));
-  RKR_TRY(tmp_alloc(bnf, &nfp64_d, 1, st));
-  RKR_CUDA(cudaMemsetAsync(nfp64_d, 0, sizeof(unsigned long long), st));
+  DevBuf bw;
+  CallWords *words;
+  RKR_TRY(words_alloc(bw, &words, st));
+  unsigned long long *nfp64_d = &words->nfp64;
   Plan plan;
-  Timer t1(st);
+  double ms_theta = 0.0, ms_res = 0.0, ms_sel = 0.0;
+  SpanClock clk(st);
+  const int t1 = clk.begin(&ms_theta);
   const Grid grid{qc.bf,  idx->fmin, idx->tau, idx->JU, idx->JL, idx->nlev_a,
                   idx->N, idx->N,    (uint32_t)(idx->m * idx->s), (uint32_t)idx->s};
   RKR_TRY(screen_plan(idx, qc, nq, grid, st, lstar_d, cap_d, ncand_d, plan));
-  double ms_theta = t1.stop(), ms_res = 0.0, ms_sel = 0.0;
-  int64_t total = 0;
+  clk.end(t1);
   int wide = 0;
   for (int q = 0; q < nq; ++q) wide += plan.lstar[q] >= idx->nlev_a - 1;
   std::vector<int64_t> qoff(nq + 1, 0);
@@ -2093,18 +2140,11 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
                              cudaMemcpyHostToDevice, st));
     RKR_CUDA(cudaMemsetAsync(cursor, 0, sizeof(uint32_t) * nq, st));
     RKR_CUDA(cudaMemsetAsync(cu, 0xff, sizeof(int32_t) * std::max<int64_t>(cnt, 1), st));
-    Timer t2(st);
+    const int t2 = clk.begin(&ms_theta);
     RKR_TRY(emit_candidates(idx, qc, qa, qb, grid, plan, lstar_d, cap_d, qoff_rel, cursor, cu, cq,
-                            cx, st));
-    ms_theta += t2.stop();
-    {
-      std::vector<uint32_t> hc(nq);
-      RKR_CUDA(cudaMemcpyAsync(hc.data(), cursor, sizeof(uint32_t) * nq, cudaMemcpyDeviceToHost,
-                               st));
-      RKR_CUDA(cudaStreamSynchronize(st));
-      for (int q = qa; q < qb; ++q) total += hc[q];
-    }
-    Timer t3(st);
+                            cx, words, st));
+    clk.end(t2);
+    const int t3 = clk.begin(&ms_res);
     if (cnt > 0) {
       {
         const int prof_slot = prof_begin("k_resolve_approx", st);
@@ -2117,27 +2157,21 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
       }
       RKR_CUDA(cudaGetLastError());
     }
-    ms_res += t3.stop();
-    Timer t4(st);
+    clk.end(t3);
+    const int t4 = clk.begin(&ms_sel);
     RKR_TRY(select_approx(qa, qb - qa, qoff_rel, cursor,
                           ApproxCand{cu, nlo, nup, th, cj, idx->U, qc.Qd, idx->d, nfp64_d},
                           qc.kq_d, c, qc.out_off_d, users_d, nlo_d, nup_d, est_d, case_d, nc_d,
-                          sel_err, st, idx));
-    ms_sel += t4.stop();
+                          &words->select_err, st, idx));
+    clk.end(t4);
   }
-  RKR_CUDA(cudaStreamSynchronize(st));
-  {
-    int h = 0;
-    RKR_CUDA(cudaMemcpy(&h, sel_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (h) return fail(RKR_EINTERNAL, "fewer than k candidates for a query");
-  }
+  CallWords hw;
+  RKR_TRY(words_check(words, hw, st));
+  clk.finish();
   if (stats) {
     stats->pairs = idx->n * (int64_t)nq;
-    stats->candidates = total;
-    unsigned long long nf = 0;
-    RKR_CUDA(cudaMemcpyAsync(&nf, nfp64_d, sizeof(nf), cudaMemcpyDeviceToHost, st));
-    RKR_CUDA(cudaStreamSynchronize(st));
-    stats->fp64_dots = (int64_t)nf;
+    stats->candidates = (int64_t)hw.candidates;
+    stats->fp64_dots = (int64_t)hw.nfp64;
     stats->near_ties = 0;
     stats->wide_queries = wide;
     stats->deep_queries = (int32_t)plan.deep.size();
@@ -2411,23 +2445,20 @@ static rkr_status learned_cut(const rkr_index *idx, const QueryCommon &qc, const
 static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, int nq,
                                    const LearnedPrune *lp, int32_t *users_d, int32_t *ranks_d,
                                    rkr_query_stats *stats, cudaStream_t st) {
-  DevBuf bl, bn, bt, bcap;
+  DevBuf bn, bcap;
   int32_t *lstar_d;
   int64_t *ncand_d;
   uint32_t *cap_d;
-  unsigned long long *ties_d;
-  RKR_TRY(tmp_alloc(bl, &lstar_d, nq, st));
-  RKR_TRY(tmp_alloc(bn, &ncand_d, nq, st));
+  RKR_TRY(tmp_alloc(bn, (char **)&ncand_d, plan_bytes(nq), st));
+  lstar_d = (int32_t *)(ncand_d + nq);
   RKR_TRY(tmp_alloc(bcap, &cap_d, nq, st));
-  DevBuf bse;
-  int *sel_err;
-  RKR_TRY(tmp_alloc(bse, &sel_err, 1, st));
-  RKR_CUDA(cudaMemsetAsync(sel_err, 0, sizeof(int), st));
-  RKR_TRY(tmp_alloc(bt, &ties_d, 2, st));
-  RKR_CUDA(cudaMemsetAsync(ties_d, 0, 2 * sizeof(unsigned long long), st));
+  DevBuf bw;
+  CallWords *words;
+  RKR_TRY(words_alloc(bw, &words, st));
+  unsigned long long *ties_d = words->ties;
   DevBuf bls;
   unsigned long long *lstat;
-  RKR_TRY(tmp_alloc(bls, &lstat, 5, st));
+  RKR_TRY(tmp_alloc(bls, &lstat, 6, st));   // [5]: candidates still to be recounted
   DevBuf bqs;
   int32_t *qself;
   RKR_TRY(tmp_alloc(bqs, &qself, nq, st));
@@ -2438,12 +2469,13 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
   int64_t prefix_rows = 0, prefix_pruned = 0, canon_rows = 0, canon_theta = 0;
   unsigned long long lstat_host_fb = 0;
   Plan plan;
-  Timer t1(st);
+  double ms_theta = 0.0, ms_res = 0.0, ms_sel = 0.0;
+  SpanClock clk(st);
+  const int t1 = clk.begin(&ms_theta);
   const Grid grid{qc.xbf,   idx->xg0, idx->xg,       idx->XJU, idx->XJL, idx->nlev_x,
                   idx->XHI, idx->XLO, (uint32_t)idx->m, 1u};
   RKR_TRY(screen_plan(idx, qc, nq, grid, st, lstar_d, cap_d, ncand_d, plan));
-  double ms_theta = t1.stop(), ms_res = 0.0, ms_sel = 0.0;
-  int64_t total = 0;
+  clk.end(t1);
   int wide = 0;
   for (int q = 0; q < nq; ++q) wide += plan.lstar[q] >= idx->nlev_x - 1;
   std::vector<int64_t> qoff(nq + 1, 0);
@@ -2469,25 +2501,18 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
                              cudaMemcpyHostToDevice, st));
     RKR_CUDA(cudaMemsetAsync(cursor, 0, sizeof(uint32_t) * nq, st));
     RKR_CUDA(cudaMemsetAsync(cu, 0xff, sizeof(int32_t) * std::max<int64_t>(cnt, 1), st));
-    Timer t2(st);
+    const int t2 = clk.begin(&ms_theta);
     RKR_TRY(emit_candidates(idx, qc, qa, qb, grid, plan, lstar_d, cap_d, qoff_rel, cursor, cu, cq,
-                            cx, st));
-    ms_theta += t2.stop();
-    {
-      std::vector<uint32_t> hc(nq);
-      RKR_CUDA(cudaMemcpyAsync(hc.data(), cursor, sizeof(uint32_t) * nq, cudaMemcpyDeviceToHost,
-                               st));
-      RKR_CUDA(cudaStreamSynchronize(st));
-      for (int q = qa; q < qb; ++q) total += hc[q];
-    }
-    Timer t3(st);
+                            cx, words, st));
+    clk.end(t2);
+    const int t3 = clk.begin(&ms_res);
     if (cnt > 0) {
       DevBuf bfb, blb;
       int32_t *cu_fb;
       uint32_t *clb;
       RKR_TRY(tmp_alloc(bfb, &cu_fb, cnt, st));
       RKR_TRY(tmp_alloc(blb, &clb, cnt, st));
-      RKR_CUDA(cudaMemsetAsync(lstat, 0, 5 * sizeof(unsigned long long), st));
+      RKR_CUDA(cudaMemsetAsync(lstat, 0, 6 * sizeof(unsigned long long), st));
       {
         const int prof_slot = prof_begin("k_list_rank", st);
         k_list_rank<<<(unsigned)((cnt + 127) / 128), 128, 0, st>>>(
@@ -2509,21 +2534,15 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
       }
       note_launch();
       RKR_CUDA(cudaGetLastError());
-      {  // candidates that still need the recount
-        DevBuf bn2;
-        unsigned long long *nfb;
-        RKR_TRY(tmp_alloc(bn2, &nfb, 1, st));
-        RKR_CUDA(cudaMemsetAsync(nfb, 0, sizeof(unsigned long long), st));
-        k_count_valid<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(cnt, cu_fb, nfb);
-        note_launch();
-        RKR_CUDA(cudaMemcpyAsync(&lstat_host_fb, nfb, sizeof(unsigned long long),
-                                 cudaMemcpyDeviceToHost, st));
-        RKR_CUDA(cudaStreamSynchronize(st));
-      }
-      unsigned long long ls[5] = {0, 0, 0, 0, 0};
+      // candidates that still need the recount, with the rank statistics
+      k_count_valid<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(cnt, cu_fb, lstat + 5);
+      note_launch();
+      RKR_CUDA(cudaGetLastError());
+      unsigned long long ls[6] = {0, 0, 0, 0, 0, 0};
       RKR_CUDA(cudaMemcpyAsync(ls, lstat, sizeof(ls), cudaMemcpyDeviceToHost, st));
-      canon_theta += (int64_t)ls[4];
       RKR_CUDA(cudaStreamSynchronize(st));
+      canon_theta += (int64_t)ls[4];
+      lstat_host_fb = ls[5];
       err_ratio = std::max(err_ratio, (double)u32_float((uint32_t)ls[2]));
       err_rel = std::max(err_rel, (double)u32_float((uint32_t)ls[3]));
       DevBuf bcut;
@@ -2611,37 +2630,34 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
         if (hrev > 0) RKR_TRY(recount_open_candidates(hrev));
       }
     }
-    ms_res += t3.stop();
-    Timer t4(st);
+    clk.end(t3);
+    const int t4 = clk.begin(&ms_sel);
     size_t sm = sizeof(SortEnt) * kMaxK;
     RKR_CUDA(cudaFuncSetAttribute(k_select_exact, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)sm));
     {
       const int prof_slot = prof_begin("k_select_exact", st);
       k_select_exact<<<qb - qa, qb - qa <= sm_count() ? kSelThreadsFew : kSelThreads, sm, st>>>(qa, qoff_rel, cursor, cu, ccount, qc.kq_d,
-                                                       qc.out_off_d, users_d, ranks_d, sel_err,
+                                                       qc.out_off_d, users_d, ranks_d,
+                                                       &words->select_err,
                                                        (uint32_t)idx->m, user_bits(idx->n));
       prof_end(prof_slot, st, 0.0);
     }
     note_launch();
     RKR_CUDA(cudaGetLastError());
-    ms_sel += t4.stop();
+    clk.end(t4);
   }
-  unsigned long long tiesv[2] = {0, 0};
-  RKR_CUDA(cudaMemcpyAsync(tiesv, ties_d, sizeof(tiesv), cudaMemcpyDeviceToHost, st));
-  RKR_CUDA(cudaStreamSynchronize(st));
-  {
-    int h = 0;
-    RKR_CUDA(cudaMemcpy(&h, sel_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (h) return fail(RKR_EINTERNAL, "fewer than k candidates for a query");
-  }
+  CallWords hw;
+  RKR_TRY(words_check(words, hw, st));
+  clk.finish();
+  const int64_t total = (int64_t)hw.candidates;
   if (stats) {
     stats->pairs = idx->n * (int64_t)nq;
     stats->candidates = total;
     // canonical u.q of list-ranked candidates that needed it, of every recounted
     // row, the near-tie items of the recount and the list entries next to u.q
-    stats->fp64_dots = canon_theta + canon_rows + (int64_t)tiesv[1] + list_fp64;
-    stats->near_ties = (int64_t)tiesv[0];
+    stats->fp64_dots = canon_theta + canon_rows + (int64_t)hw.ties[1] + list_fp64;
+    stats->near_ties = (int64_t)hw.ties[0];
     stats->recounted = fallback;
     stats->recount_users = recount_users;
     stats->recount_open = recount_open;

@@ -162,6 +162,15 @@ void tc_free(TcSide &s) {
   s.cat_role = 0;
 }
 
+void tc_free_async(TcSide &s, cudaStream_t st) {
+  if (!s.owned) return;
+  for (void *p : {(void *)s.hi, (void *)s.lo, (void *)s.rb1, (void *)s.rb3, (void *)s.cat})
+    if (p) cudaFreeAsync(p, st);
+  s.hi = s.lo = s.cat = nullptr;
+  s.rb1 = s.rb3 = nullptr;
+  s.cat_role = 0;
+}
+
 __global__ void k_tile_bounds(const tc::RowBound *__restrict__ rb, int64_t rows, int bn,
                               int ntiles, tc::RowBound *__restrict__ out) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;

@@ -46,6 +46,8 @@ inline int split_chunks_cat(int kp) { return (3 * kp + 63) / 64; }
 // from hi and lo (allocates); nothing is built when it would save no stage.
 rkr_status tc_make_cat(TcSide &s, int role, cudaStream_t st);
 void tc_free(TcSide &s);
+// The same for a side staged and used on `st` alone: no synchronization.
+void tc_free_async(TcSide &s, cudaStream_t st);
 
 // Per column-tile maxima of the bound terms of a side used as B with tiles of bn rows.
 rkr_status tc_tile_bounds(const TcSide &b, int bn, int split, tc::RowBound **out,
