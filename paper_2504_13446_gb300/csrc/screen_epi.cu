@@ -57,6 +57,7 @@ __device__ __forceinline__ uint32_t bitmask32(F &&pred) {
   return (m0 | m1) | (m2 | m3);
 }
 
+template <bool INTERLEAVE>
 struct TilePrefetch {
   tc::RowBound next;
   int nct;   // the column tile `next` holds
@@ -67,9 +68,10 @@ struct TilePrefetch {
   __device__ __forceinline__ tc::RowBound take(const tc::RowBound *tileb, int ct, int64_t ncols,
                                                int bn) {
     const tc::RowBound cur = ct == nct ? next : tileb[ct];
-    if ((int64_t)(ct + 1) * bn < ncols) {
-      nct = ct + 1;
-      next = tileb[ct + 1];
+    const int after = tc::tile_after<INTERLEAVE>(ct, (int)((ncols + bn - 1) / bn));
+    if (after >= 0 && (int64_t)after * bn < ncols) {
+      nct = after;
+      next = tileb[after];
     }
     return cur;
   }
@@ -119,7 +121,7 @@ struct EpiFb {
     float b, mxlo, mnhi;
     int64_t row;
     tc::RowBound ru;     // the row's bound terms
-    TilePrefetch tp;     // the bound terms of the next column tile
+    TilePrefetch<false> tp;     // the bound terms of the next column tile
   };
   static constexpr size_t kSmem = 0;
   int64_t nrows, ncols;
@@ -405,13 +407,14 @@ __global__ void k_xgrid(int64_t n, const double *__restrict__ fmin,
 struct EpiXT {
   static const char *name() { return "k_screen<EpiXT>"; }
   static constexpr int kWarps = 8;   // 98 ms at 1M x 100k x 200 (16 warps: 102)
+  static constexpr bool kInterleave = true;   // 98.3 -> 93.1 ms
   struct Thread {
     float skip, b, g0;
     int64_t row;
     int64_t off;
     uint32_t cap;
     tc::RowBound ru;     // the row's bound terms
-    TilePrefetch tp;     // the bound terms of the next column tile
+    TilePrefetch<kInterleave> tp;     // the bound terms of the next column tile
   };
   // list cursors of the block's 128 rows, then a 32 x 32 staging tile per warp
   // stored [column][lane] (a lane's lookups hit its own bank)
@@ -818,7 +821,7 @@ struct EpiDeep {
     BinFP bf;
     double g0;
     tc::RowBound ru;
-    TilePrefetch tp;
+    TilePrefetch<false> tp;
   };
   static constexpr size_t kHist = sizeof(uint32_t) * 128 * kBins;   // one of Hlo, Hhi
   static constexpr size_t kStageOff = 2 * kHist;
@@ -1706,7 +1709,7 @@ struct EpiRC {
     int64_t self;                // item tying exactly with u.q (never above), or -1
     uint32_t clo, chi;           // items certainly / possibly above u.q
     tc::RowBound ru;             // the row's bound terms
-    TilePrefetch tp;             // the bound terms of the next column tile
+    TilePrefetch<false> tp;             // the bound terms of the next column tile
   };
   static constexpr size_t kSmem = 0;
   int64_t nseg, ncols;
@@ -1817,7 +1820,7 @@ struct EpiRCm {
     int scur, send;      // cursor over the segment's self columns
     int64_t snext;       // next self column, or INT64_MAX
     tc::RowBound ru;     // the row's bound terms
-    TilePrefetch tp;     // the bound terms of the next column tile
+    TilePrefetch<false> tp;     // the bound terms of the next column tile
   };
   // Per row the thresholds (rounded down; +inf beyond L, so that a search over
   // all kL slots needs no bound) and the pos_lo and pos_hi histograms.  Every

@@ -124,7 +124,8 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
       Ring<STAGES> ring;
       for (int p = pair0; p < npairs && !failed; p += npair_ctas) {
         const int rb = 2 * p + rank;    // may be one past the last row block
-        for (int ct = 0; ct < sch.nct && !failed; ++ct) {
+        for (int i = 0; i < sch.nct && !failed; ++i) {
+          const int ct = tile_at<EpiInterleave<Epi>::value>(i, 0, sch.nct);
           ChunkWalk w;
           for (int kc = 0; kc < nk; ++kc, ++it) {
             const uint32_t s = ring.s;
@@ -199,7 +200,8 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
       u.rb0 = rb; u.rb1 = rb + 1; u.ct0 = 0; u.ct1 = sch.nct;
       if (real) epi.unit_begin(escratch, u, et, ts);
       epi_sync<EW>();
-      for (int ct = 0; ct < sch.nct; ++ct, ++t) {
+      for (int i = 0; i < sch.nct; ++i, ++t) {
+        const int ct = tile_at<EpiInterleave<Epi>::value>(i, 0, sch.nct);
         const int b = t & 1;
         const uint32_t aph = (t >> 1) & 1;
         if (!failed && !mbar_wait_warp(&acc_full[b], aph, op.epi_wait)) failed = true;
@@ -399,7 +401,8 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
       Ring<STAGES> ring;
       for (int p = pair0; p < npairs && !failed; p += npair_ctas) {
         const int rb = 2 * p + rank;    // may be one past the last row block
-        for (int ct = 0; ct < sch.nct && !failed; ++ct) {
+        for (int i = 0; i < sch.nct && !failed; ++i) {
+          const int ct = tile_at<EpiInterleave<Epi>::value>(i, 0, sch.nct);
           ChunkWalk w;
           for (int kc = 0; kc < nk; ++kc, ++it) {
             const uint32_t s = ring.s;
@@ -477,7 +480,8 @@ __global__ void __launch_bounds__(screen_threads<Epi>(), 1)
       u.rb0 = rb; u.rb1 = rb + 1; u.ct0 = 0; u.ct1 = sch.nct;
       if (real) epi.unit_begin(escratch, u, et, ts);
       epi_sync<EW>();
-      for (int ct = 0; ct < sch.nct; ++ct, ++t) {
+      for (int i = 0; i < sch.nct; ++i, ++t) {
+        const int ct = tile_at<EpiInterleave<Epi>::value>(i, 0, sch.nct);
         const int b = t & 1;
         const uint32_t aph = (t >> 1) & 1;
         if (!failed && !mbar_wait_warp(&acc_full[b], aph, op.epi_wait)) failed = true;
