@@ -119,6 +119,17 @@ __device__ __forceinline__ double canon_dot(const float *__restrict__ a,
   return acc;
 }
 
+// (double)x of a finite float by integer operations: the conversion instruction
+// runs on the FP64 units, four per SM.
+__device__ __forceinline__ double exact_double(float x) {
+  const bool sub = fabsf(x) < 0x1p-126f;               // a subnormal, scaled to a normal
+  const uint32_t b = __float_as_uint(sub ? __fmul_rn(x, 0x1p64f) : x);
+  const uint32_t mag = b & 0x7fffffffu;
+  const uint32_t bias = sub ? (896u - 64u) << 20 : 896u << 20;
+  const uint32_t hi = mag ? (mag >> 3) + bias : 0u;
+  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(b << 29));
+}
+
 // Out-of-line copy for rarely taken paths inside unrolled loops.
 static __device__ __noinline__ double canon_dot_slow(const float *__restrict__ a,
                                                      const float *__restrict__ b, int d) {

@@ -201,7 +201,7 @@ __device__ __forceinline__ void flush_and_cut(const ScanArgs &a, uint32_t *hist,
 template <int VEC>
 __global__ void __launch_bounds__(kLatThreads, 4) k_latency_scan(const ScanArgs a) {
   __shared__ __align__(16) float qs[kMaxD];
-  __shared__ uint32_t hist[kLatBins];
+  __shared__ __align__(16) uint32_t hist[kLatBins];
   for (int i = threadIdx.x; i < kMaxD; i += blockDim.x) qs[i] = i < a.d ? a.q[i] : 0.0f;
   for (int i = threadIdx.x; i < kLatBins; i += blockDim.x) hist[i] = 0;
   __syncthreads();

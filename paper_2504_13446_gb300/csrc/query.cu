@@ -220,6 +220,20 @@ constexpr int kSelThreads = 256;
 constexpr int kSelThreadsFew = 1024;
 constexpr int kSelSmall = 512;     // entries sorted beside the survivors (k_select_approx)
 constexpr size_t kSelSmem = sizeof(SortEnt) * (kMaxK + kSelSmall);
+// Rows staged at a time for the canonical products of k_select_approx with 1,024
+// threads, behind the query as doubles.
+constexpr int kSelRows = 128;
+static size_t select_smem(bool few, int d) {
+  return kSelSmem + (few ? sizeof(double) * d + sizeof(float) * kSelRows * (d | 1) : 0);
+}
+
+// Entries a selection may leave to the sort: 64, which its short form places at once,
+// or as many as the bitonic form sorts for k.
+__device__ __forceinline__ uint32_t sort_room(int k) {
+  uint32_t r = 64;
+  while (r < (uint32_t)k) r <<= 1;
+  return r;
+}
 
 // One CTA per query: steps 1-3 of Section 4.3 over the query's candidates.
 template <int THREADS>
@@ -236,7 +250,7 @@ __global__ void __launch_bounds__(THREADS)
   extern __shared__ unsigned char sbuf[];
   SortEnt *ent = (SortEnt *)sbuf;                   // kMaxK entries
   SortEnt *small = ent + kMaxK;                     // kSelSmall entries
-  __shared__ uint32_t hist[512];
+  __shared__ __align__(16) uint32_t hist[512];
   __shared__ uint64_t bc[4];
   __shared__ unsigned long long cnt_acc;
   __shared__ int gcount;
@@ -264,12 +278,64 @@ __global__ void __launch_bounds__(THREADS)
     }
     return interp_est(t, cj[i], nlo[i], nup[i], fmin[u], delta[u], tau, s);
   };
+  // Canonical products of the users of e[0, count) that have none yet, where few
+  // queries leave the SM to this one: their rows are staged in shared memory by the
+  // whole block (one round trip to memory for 128 of them), then a lane per row adds
+  // its products in order, with operands converted by integer operations.  A lane
+  // reading its own row from memory took 245 cycles a dimension for 32 users, this 90.
+  auto form_dots = [&](const SortEnt *e, int count) {
+    if constexpr (THREADS == kSelThreadsFew) {
+      double *qd = (double *)(small + kSelSmall);
+      float *tile = (float *)(qd + C.d);
+      const int d = C.d, ld = d | 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+      for (int c0 = threadIdx.x; c0 < d; c0 += THREADS) qd[c0] = exact_double(qrow[c0]);
+      for (int b = 0; b < count; b += kSelRows) {
+        const int nr = min(kSelRows, count - b);
+        __syncthreads();
+        for (int r = warp; r < nr; r += THREADS / 32) {
+          const int64_t i = e[b + r].idx;
+          const double t = th[i];
+          if (t == t) continue;
+          const float *row = C.U + (int64_t)uid[i] * d;
+          float v[kMaxD / 32];
+#pragma unroll
+          for (int p = 0; p < kMaxD / 32; ++p) v[p] = lane + 32 * p < d ? row[lane + 32 * p] : 0.0f;
+#pragma unroll
+          for (int p = 0; p < kMaxD / 32; ++p)
+            if (lane + 32 * p < d) tile[r * ld + lane + 32 * p] = v[p];
+        }
+        __syncthreads();
+        if (threadIdx.x < nr) {
+          const int64_t i = e[b + threadIdx.x].idx;
+          const double t = th[i];
+          if (t != t) {
+            const float *x = tile + threadIdx.x * ld;
+            double acc = 0.0;
+#pragma unroll 8
+            for (int c0 = 0; c0 < d; ++c0) acc = __fma_rn(exact_double(x[c0]), qd[c0], acc);
+            th[i] = acc;
+            if (C.nfp64) atomicAdd(C.nfp64, 1ull);
+          }
+        }
+      }
+      __syncthreads();
+    }
+  };
   // Step 1: k-th smallest lower and upper bound numerators (at most top).
   const int nbits = count_bits(top);
   uint64_t Rlo, Rup;
   block_kth_pair(nlo, nup, cnt, (uint64_t)k, nbits, hist, bc, Rlo, Rup);
-  const double lhs = c * (double)((uint64_t)s + Rlo);
-  const bool caseA = lhs >= (double)((uint64_t)s + Rup);
+  // c R_low_k against R_up_k, by one thread: an FP64 instruction of every warp of the
+  // block takes eight times as long
+  if (threadIdx.x == 0) {
+    const double lhs = c * (double)((uint64_t)s + Rlo);
+    bc[0] = lhs >= (double)((uint64_t)s + Rup);
+    bc[1] = (uint64_t)floor(lhs);
+  }
+  __syncthreads();
+  const bool caseA = bc[0] != 0;
+  const uint64_t lim = bc[1];
+  __syncthreads();   // bc is the selections' from here on
   const int64_t obase = out_off[q];
   int nc;
   if (caseA) {
@@ -281,34 +347,41 @@ __global__ void __launch_bounds__(THREADS)
       ent[pos].k2 = (uint32_t)uid[i];
       ent[pos].idx = (int32_t)i;
     };
-    constexpr int kSort = 512;   // (sorting 4,096 takes twice the radix passes' time)
-    if (threadIdx.x == 0) gcount = 0;
+    const uint32_t room = sort_room(k);
+    if (threadIdx.x == 0) {
+      gcount = 0;
+      cnt_acc = 0;
+    }
     __syncthreads();
-    for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x)
-      if ((uint64_t)nup[i] <= Rup) {
+    for (int64_t i0 = 0; i0 < cnt; i0 += blockDim.x) {   // whole warps
+      const int64_t i = i0 + threadIdx.x;
+      const uint64_t v = i < cnt ? nup[i] : ~0ull;
+      if (v <= Rup) {
         const int pos = atomicAdd(&gcount, 1);
-        if (pos < kSort) put(pos, i);
+        if (pos < (int)room) put(pos, i);
       }
+      const unsigned less = __ballot_sync(0xffffffffu, v < Rup);
+      if ((threadIdx.x & 31) == 0 && less) atomicAdd(&cnt_acc, (unsigned long long)__popc(less));
+    }
     __syncthreads();
     const int upto = gcount;
+    const int64_t below = (int64_t)cnt_acc;
     __syncthreads();
-    if (upto > kSort) {
-      const int64_t below =
-          block_count(cnt, [&](int64_t i) { return (uint64_t)nup[i] < Rup; }, &cnt_acc);
-      uint64_t kth2 = ~0ull;
+    if (upto > (int)room) {
+      // (below < k: Rup is the k-th; the keys are distinct, so at most `room` remain)
       auto tie_key = [&](int64_t i) { return ((uint64_t)nlo[i] << ubits) | (uint32_t)uid[i]; };
-      if (below < k)
-        kth2 = block_kth(cnt, (uint64_t)(k - below), nbits + ubits,
-                         [&](int64_t i, uint64_t &key) {
-                           key = tie_key(i);
-                           return (uint64_t)nup[i] == Rup;
-                         },
-                         hist, bc);
+      uint32_t ties;
+      const uint64_t last = block_kth_cut(cnt, (uint64_t)(k - below), nbits + ubits,
+                                          [&](int64_t i, uint64_t &key) {
+                                            key = tie_key(i);
+                                            return (uint64_t)nup[i] == Rup;
+                                          },
+                                          hist, bc, room - (uint32_t)below, ties);
       if (threadIdx.x == 0) gcount = 0;
       __syncthreads();
       for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
         const uint64_t a = nup[i];
-        if (a < Rup || (a == Rup && tie_key(i) <= kth2)) {
+        if (a < Rup || (a == Rup && tie_key(i) <= last)) {
           const int pos = atomicAdd(&gcount, 1);
           if (pos < kMaxK) put(pos, i);
         }
@@ -317,6 +390,7 @@ __global__ void __launch_bounds__(THREADS)
     __syncthreads();
     int got = min(gcount, kMaxK);
     block_sort(ent, got);
+    if (out_est) form_dots(ent, min(got, k));
     for (int r = threadIdx.x; r < got && r < k; r += blockDim.x) {
       int64_t i = ent[r].idx;
       out_users[obase + r] = uid[i];
@@ -329,7 +403,6 @@ __global__ void __launch_bounds__(THREADS)
     // U_c = {r_up <= c R_low_k}: fewer than k users, (r_up, r_low, index) order
     // s + nup <= c (s + R_low_k): integers (below 2^53) against a real, so against
     // its floor
-    const uint64_t lim = (uint64_t)floor(lhs);
     auto in_c = [&](int64_t i) { return (uint64_t)s + nup[i] <= lim; };
     if (threadIdx.x == 0) gcount = 0;
     __syncthreads();
@@ -346,6 +419,7 @@ __global__ void __launch_bounds__(THREADS)
     __syncthreads();
     nc = min(gcount, kMaxK);
     block_sort(ent, nc);
+    if (out_est) form_dots(ent, nc);
     for (int r = threadIdx.x; r < nc; r += blockDim.x) {
       int64_t i = ent[r].idx;
       out_users[obase + r] = uid[i];
@@ -372,6 +446,7 @@ __global__ void __launch_bounds__(THREADS)
     const int nt = gcount;
     __syncthreads();   // every thread has the count before it is reset
     const bool fits = nt <= kMaxK && need <= kSelSmall;
+    form_dots(ent, min(nt, kMaxK));
     for (int e = threadIdx.x; e < min(nt, kMaxK); e += blockDim.x) {
       const int64_t i = ent[e].idx;
       const double est = est_of(i);
@@ -382,21 +457,28 @@ __global__ void __launch_bounds__(THREADS)
     if (threadIdx.x == 0) gcount = 0;
     __syncthreads();
     if (fits) {
-      const uint64_t ke = block_kth(nt, (uint64_t)need, 64,
-                                    [&](int64_t e, uint64_t &key) {
-                                      key = ent[e].k1;
-                                      return true;
-                                    },
-                                    hist, bc);
-      const int64_t below = block_count(nt, [&](int64_t e) { return ent[e].k1 < ke; }, &cnt_acc);
-      uint64_t ku = ~0ull;
-      if (below < need)
+      // those up to the need-th estimate, or a little past it, go to the sort; only
+      // estimates that tie beyond its room are told apart by their users
+      const uint32_t room = sort_room(need);
+      uint64_t ke = ~0ull, ku = ~0ull;
+      uint32_t upto = (uint32_t)nt;
+      if (upto > room)
+        ke = block_kth_cut(nt, (uint64_t)need, 64,
+                           [&](int64_t e, uint64_t &key) {
+                             key = ent[e].k1;
+                             return true;
+                           },
+                           hist, bc, room, upto);
+      if (upto > room) {
+        const int64_t below =
+            block_count(nt, [&](int64_t e) { return ent[e].k1 < ke; }, &cnt_acc);
         ku = block_kth(nt, (uint64_t)(need - below), 32,
                        [&](int64_t e, uint64_t &key) {
                          key = ent[e].k2;
                          return ent[e].k1 == ke;
                        },
                        hist, bc);
+      }
       for (int e = threadIdx.x; e < nt; e += blockDim.x) {
         const SortEnt x = ent[e];
         if (x.k1 < ke || (x.k1 == ke && (uint64_t)x.k2 <= ku)) {
@@ -833,7 +915,7 @@ __global__ void __launch_bounds__(kFilterThreads)
                      const int32_t *__restrict__ kq, uint32_t *__restrict__ ccount,
                      const uint32_t *__restrict__ clb, int32_t *__restrict__ cu_fb,
                      uint32_t mtop) {
-  __shared__ uint32_t hist[256];
+  __shared__ __align__(16) uint32_t hist[256];
   __shared__ uint64_t bc[2];
   const int q = qa + blockIdx.x;
   const int64_t base = qoff[q] - qoff[qa];
@@ -890,7 +972,7 @@ __global__ void __launch_bounds__(kFilterThreads)
                   const uint32_t *__restrict__ hi1, const uint32_t *__restrict__ lo1,
                   uint32_t *__restrict__ clb, int32_t *__restrict__ cu_fb,
                   int32_t *__restrict__ cu_park) {
-  __shared__ uint32_t hist[256];
+  __shared__ __align__(16) uint32_t hist[256];
   __shared__ uint64_t bc[2];
   __shared__ unsigned long long acc;
   const int q = qa + blockIdx.x;
@@ -934,7 +1016,7 @@ __global__ void __launch_bounds__(kSelThreadsFew)
                    int ubits) {
   extern __shared__ unsigned char sbuf[];
   SortEnt *ent = (SortEnt *)sbuf;
-  __shared__ uint32_t hist[256];
+  __shared__ __align__(16) uint32_t hist[256];
   __shared__ uint64_t bc[2];
   __shared__ int gcount;
   const int q = qa + blockIdx.x;
@@ -954,16 +1036,17 @@ __global__ void __launch_bounds__(kSelThreadsFew)
     const uint32_t u = uid[i] < 0 ? 0u : (uint32_t)uid[i];   // (dropped: behind every count)
     return (count_key(cc[i], cbits) << ubits) | u;
   };
-  const uint64_t kth = block_kth(cnt, (uint64_t)k, cbits + ubits,
-                                 [&](int64_t i, uint64_t &key) {
-                                   key = key_of(i);
-                                   return true;
-                                 },
-                                 hist, bc);
+  uint32_t upto;
+  const uint64_t last = block_kth_cut(cnt, (uint64_t)k, cbits + ubits,
+                                      [&](int64_t i, uint64_t &key) {
+                                        key = key_of(i);
+                                        return true;
+                                      },
+                                      hist, bc, sort_room(k), upto);
   if (threadIdx.x == 0) gcount = 0;
   __syncthreads();
   for (int64_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-    if (key_of(i) <= kth) {
+    if (key_of(i) <= last) {
       int pos = atomicAdd(&gcount, 1);
       if (pos < kMaxK) {
         ent[pos].k1 = ((uint64_t)cc[i] << 32) | (uint32_t)uid[i];
@@ -2070,9 +2153,11 @@ static rkr_status select_approx(int qa, int nblocks, const int64_t *qoff, const 
                                 int *err, cudaStream_t st, const rkr_index *idx) {
   const bool few = nblocks <= sm_count();
   auto kern = few ? k_select_approx<kSelThreadsFew> : k_select_approx<kSelThreads>;
-  RKR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem));
+  const size_t sm = select_smem(few, idx->d);
+  RKR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)select_smem(few, kMaxD)));
   const int prof_slot = prof_begin("k_select_approx", st);
-  kern<<<nblocks, few ? kSelThreadsFew : kSelThreads, kSelSmem, st>>>(
+  kern<<<nblocks, few ? kSelThreadsFew : kSelThreads, sm, st>>>(
       qa, qoff, qcount, C, kq, c, (uint32_t)idx->s, idx->tau, idx->fmin, idx->delta, out_off,
       users_d, nlo_d, nup_d, est_d, case_d, nc_d, err, (uint32_t)(idx->m * idx->s),
       user_bits(idx->n));
@@ -2214,7 +2299,7 @@ __global__ void __launch_bounds__(kFilterThreads)
                   int32_t *__restrict__ fb_all, int32_t *__restrict__ cu_all,
                   uint32_t *__restrict__ ccount, int32_t *__restrict__ cutu_all,
                   int64_t n_users, unsigned long long *__restrict__ ncut) {
-  __shared__ uint32_t hist[256];
+  __shared__ __align__(16) uint32_t hist[256];
   __shared__ uint64_t bc[2];
   __shared__ unsigned long long acc;
   const int q = qa + blockIdx.x;
@@ -2264,7 +2349,7 @@ __global__ void __launch_bounds__(256)
                      const uint32_t *__restrict__ ccount, const uint32_t *__restrict__ clb,
                      int32_t *__restrict__ fb_all, int32_t *__restrict__ cu_all,
                      int32_t *__restrict__ cutu_all, unsigned long long *__restrict__ nrev) {
-  __shared__ uint32_t hist[256];
+  __shared__ __align__(16) uint32_t hist[256];
   __shared__ uint64_t bc[2];
   __shared__ unsigned long long acc;
   const int q = qa + blockIdx.x;
