@@ -175,8 +175,8 @@ rkr_status rkr_query_approx(rkr_index *idx, const float *Q, int32_t nq, const in
 /*
  * rkr_session_*: a serving form of rkr_query_approx_single for one query per call
  * (not in the paper).  rkr_session_create keeps device buffers for one query and
- * captures the query's launches (query norm, the scan of U fused with the bounds
- * lookup, the cut, the compaction, steps 2-3) in a CUDA graph on a stream of its
+ * captures the query's launches (the scan of U fused with the bounds lookup
+ * and the cut, the compaction, steps 2-3) in a CUDA graph on a stream of its
  * own, for this index, k <= max_k and this c.  rkr_session_query copies q (d
  * floats, host or device) in, replays the graph and copies the outputs back:
  * out_users, out_nlow, out_nup, out_est (k entries each), *out_case, *out_nc, as
@@ -220,7 +220,7 @@ rkr_status rkr_query_approx_bitmap(rkr_index *idx, const float *Q, int32_t nq, c
  * every user (FP32 warp products with a rigorous bound; canonical FP64 only where
  * the bound straddles a threshold) fused with the bounds lookup of Section 4.3
  * step 1, then steps 2-3 run on the users whose lower bound is at most an upper
- * estimate of R_up_k (every user the steps can return is among them).  Four
+ * estimate of R_up_k (every user the steps can return is among them).  Three
  * kernel launches per query, no host synchronization until the call returns.
  * The pass is bound by HBM bandwidth: about 4d + 48 bytes per user per query.
  * Temporaries: about 37 bytes per user, reused by every query of the call.

@@ -664,8 +664,8 @@ rkr_status run_query_approx_single(const rkr_index *idx, const QueryCommon &qc, 
 
 // ------------------------------------------------------------------ session
 // A serving form of the one-at-a-time path: persistent device buffers for one
-// query and a CUDA graph of its launches (query norm, scan, histogram sum, cut,
-// compaction, steps 2-3), captured once at creation and replayed per query.
+// query and a CUDA graph of its launches (scan with the cut, compaction, steps 2-3),
+// captured once at creation and replayed per query.
 struct rkr_session {
   rkr_index *idx = nullptr;
   int max_k = 0, d = 0;

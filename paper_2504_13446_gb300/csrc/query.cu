@@ -282,7 +282,8 @@ __global__ void __launch_bounds__(THREADS)
   // queries leave the SM to this one: their rows are staged in shared memory by the
   // whole block (one round trip to memory for 128 of them), then a lane per row adds
   // its products in order, with operands converted by integer operations.  A lane
-  // reading its own row from memory took 245 cycles a dimension for 32 users, this 90.
+  // reading its own row from memory took 245 cycles a dimension for 32 users, this 115 to 145
+  // (an FP64 instruction alone takes 76).
   auto form_dots = [&](const SortEnt *e, int count) {
     if constexpr (THREADS == kSelThreadsFew) {
       double *qd = (double *)(small + kSelSmall);

@@ -178,7 +178,7 @@ __device__ __forceinline__ bool ent_less(const SortEnt &a, const SortEnt &b) {
 
 // Sort of e[0 .. count) in shared memory.  Few entries (count^2 <= 16 threads' worth,
 // so 64 with 256 threads, 128 with 1,024): every entry's place is counted by 4 to 32
-// threads (64 entries: 0.5 us; 21 bitonic steps in one warp 3 us).  More: bitonic; e
+// threads (10 entries: 0.5 us; 21 bitonic steps in one warp 3 us).  More: bitonic; e
 // must have room for the next power of two, the tail is padded with maximal keys.
 __device__ void block_sort(SortEnt *e, int count) {
   __syncthreads();
