@@ -49,13 +49,13 @@ __device__ __forceinline__ void warp_digit(const uint32_t *hist, uint32_t k, int
 // (fn returns false for elements that do not take part).  MSB-first radix
 // select on 8-bit digits over an nbits-wide key.  Every thread of the block must
 // call it with the same arguments; the k-th smallest must exist.
-// A thread evaluates four keys before it adds any to the histogram, so that
+// A thread evaluates AHEAD keys before it adds any to the histogram, so that
 // their loads are in flight together: one CTA may have to walk a million keys.
 //
 // The search ends early once at most `limit` keys lie at or below the bin that holds
 // the k-th: their number is left in total and the bin's last key is returned (so
 // limit 0 searches for the k-th itself).
-template <class F>
+template <int AHEAD = 4, class F>
 __device__ uint64_t block_kth_cut(int64_t cnt, uint64_t k, int nbits, F fn, uint32_t *hist,
                                   uint64_t *bc, uint32_t limit, uint32_t &total) {
   uint64_t prefix = 0, mask = 0;
@@ -66,13 +66,13 @@ __device__ uint64_t block_kth_cut(int64_t cnt, uint64_t k, int nbits, F fn, uint
   __syncthreads();
   for (int shift = nbits - 8; shift >= 0; shift -= 8) {
     int64_t i = threadIdx.x;
-    for (; i + 3 * T < cnt; i += 4 * T) {
-      uint64_t key[4];
-      bool in[4];
+    for (; i + (AHEAD - 1) * T < cnt; i += AHEAD * T) {
+      uint64_t key[AHEAD];
+      bool in[AHEAD];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) in[j] = fn(i + j * T, key[j]);
+      for (int j = 0; j < AHEAD; ++j) in[j] = fn(i + j * T, key[j]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < AHEAD; ++j)
         if (in[j] && (key[j] & mask) == prefix) atomicAdd(&hist[(key[j] >> shift) & 255u], 1u);
     }
     for (; i < cnt; i += T) {
@@ -94,11 +94,11 @@ __device__ uint64_t block_kth_cut(int64_t cnt, uint64_t k, int nbits, F fn, uint
   return (prefix | ~mask) & (~0ull >> (64 - nbits));
 }
 
-template <class F>
+template <int AHEAD = 4, class F>
 __device__ uint64_t block_kth(int64_t cnt, uint64_t k, int nbits, F fn, uint32_t *hist,
                               uint64_t *bc) {
   uint32_t total;
-  return block_kth_cut(cnt, k, nbits, fn, hist, bc, 0u, total);
+  return block_kth_cut<AHEAD>(cnt, k, nbits, fn, hist, bc, 0u, total);
 }
 
 // The k-th smallest of two arrays of 32-bit keys (at most nbits wide) in the same
