@@ -568,8 +568,9 @@ uint64_t rkr_device_allocations(void);
 /* Test hook (not in the paper): the number of try_wait rounds after which the
  * epilogue warps of the tensor-core screens give up waiting for an accumulator
  * tile; the kernel then records the timeout, lets the MMAs and loads already
- * issued finish, and the call returns RKR_ETIMEOUT.  0 gives up at the first
- * wait; a negative value restores the default (2^22 rounds).  Process-wide;
+ * issued finish, and the call returns RKR_ETIMEOUT.  The consumer warps of the
+ * bulk-staged scan (tuning latency_bulk) give up after as many rounds.  0 gives up
+ * at the first wait; a negative value restores the default (2^22 rounds).  Process-wide;
  * takes effect for launches that start after the call.  RKR_EINVAL above 2^32 - 1. */
 rkr_status rkr_set_wait_limit(int64_t rounds);
 

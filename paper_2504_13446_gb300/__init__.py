@@ -263,7 +263,8 @@ def device_allocations() -> int:
 
 
 def rkr_set_wait_limit(rounds: int) -> None:
-    """Test hook: try_wait rounds of the screens' epilogue wait (negative = default)."""
+    """Test hook: try_wait rounds of the screens' epilogue wait and of the bulk-staged
+    scan's stage wait (negative = default)."""
     _check(load().rkr_set_wait_limit(int(rounds)))
 
 

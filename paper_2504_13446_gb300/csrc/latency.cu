@@ -68,6 +68,7 @@ struct ScanArgs {
   const int32_t *kq;            // k of the query
   uint32_t *T, *qcount;         // cut, candidate count (zeroed for the compaction)
   unsigned long long *nfp64;
+  uint32_t wait;                // rounds a consumer warp of the bulk form waits for a stage
 };
 
 // Finish of the warp's users (every lane calls it; lane's user u if live, with its
@@ -265,8 +266,8 @@ __global__ void __launch_bounds__(kLatThreads, 4) k_latency_scan(const ScanArgs 
 // streams chunks into a ring of kBulkStages shared-memory stages; warps
 // 0..kBulkWarps-1 each take kBulkRows / kBulkWarps rows of a stage, free the
 // stage as soon as their products are formed, then finish their users.  One CTA
-// per SM; every wait is bounded (a timeout sets *err and ends the CTA after the
-// copies it issued have landed).
+// per SM; every wait is bounded.  A timeout sets *err; whichever side gave up, the
+// producer waits for the copies it issued before the CTA ends.
 constexpr int kBulkWarps = 8;
 constexpr int kBulkRows = 64;
 constexpr int kBulkStages = 3;
@@ -277,9 +278,10 @@ __device__ __forceinline__ uint32_t bulk_smem(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-__device__ __forceinline__ bool bulk_wait(uint64_t *bar, uint32_t parity) {
+__device__ __forceinline__ bool bulk_wait(uint64_t *bar, uint32_t parity,
+                                          uint32_t limit = kBulkWait) {
   const uint32_t addr = bulk_smem(bar);
-  for (uint32_t i = 0; i < kBulkWait; ++i) {
+  for (uint32_t i = 0; i < limit; ++i) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
@@ -345,12 +347,11 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
             "r"(bulk_smem(&full[s]))
             : "memory");
       }
-      if (failed) {
-        atomicExch(err, 1);
-        // the copies already issued land before the CTA can exit
-        for (uint32_t j = (it > kBulkStages ? it - kBulkStages : 0); j < it; ++j)
-          bulk_wait(&full[j % kBulkStages], (j / kBulkStages) & 1);
-      }
+      if (failed) atomicExch(err, 1);
+      // the copies issued land before the CTA can exit (a consumer that gave up did
+      // not wait for them)
+      for (uint32_t j = (it > kBulkStages ? it - kBulkStages : 0); j < it; ++j)
+        bulk_wait(&full[j % kBulkStages], (j / kBulkStages) & 1);
     }
   } else {
     // ------------------------------------------------------------ consumers
@@ -362,7 +363,11 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
     uint32_t it = 0;
     for (int64_t ch = blockIdx.x; ch < nch; ch += gridDim.x, ++it) {
       const int s = it % kBulkStages;
-      if (!bulk_wait(&full[s], (it / kBulkStages) & 1)) { failed = true; break; }
+      // (one answer for the warp: its lanes meet in shuffles below)
+      if (!__all_sync(0xffffffffu, bulk_wait(&full[s], (it / kBulkStages) & 1, a.wait))) {
+        failed = true;
+        break;
+      }
       const float *st = (const float *)(stages + s * stage_bytes);
       const int64_t u0 = ch * kBulkRows + warp * kBulkRowsPerWarp;
       float mine = 0.0f;
@@ -539,6 +544,7 @@ rkr_status scan_pass(const rkr_index *idx, const QueryCommon &qc, int q, const S
     a.nlo = sb.nlo; a.nup = sb.nup; a.jout = sb.jall;
     a.ghist = sb.ghist; a.done = sb.ghist + kLatBins; a.kq = qc.kq_d + q;
     a.T = sb.T; a.qcount = sb.qcount + q; a.nfp64 = sb.nfp64;
+    a.wait = epi_wait_limit();
     if (sb.bulk)
       k_latency_scan_bulk<<<sb.grid, (kBulkWarps + 1) * 32, sb.bulk_smem, st>>>(
           a, (int *)(sb.nfp64 + 2));
