@@ -69,6 +69,7 @@ struct ScanArgs {
   uint32_t *T, *qcount;         // cut, candidate count (zeroed for the compaction)
   unsigned long long *nfp64;
   uint32_t wait;                // rounds a consumer warp of the bulk form waits for a stage
+  const uint32_t *wait_p;       // the same read on the device (a captured launch), or null
 };
 
 // Finish of the warp's users (every lane calls it; lane's user u if live, with its
@@ -140,7 +141,9 @@ __device__ __forceinline__ void finish_users(const ScanArgs &a, const float *qs,
 // End of a scan CTA: its histogram is added to the query's (most bins are empty),
 // and the last CTA to do so finds T = upper end of the bin holding the k-th
 // smallest upper-bound numerator (so T >= R_up_k), zeroes the query's candidate
-// count and leaves the histogram and the counter at zero for the next launch.
+// count and leaves the histogram and the counter at zero for the next launch.  A scan
+// that timed out may have counted fewer than k users: T is then 0.  Either way the
+// compaction starts from a count of zero, so it stays within its n slots.
 __device__ __forceinline__ void flush_and_cut(const ScanArgs &a, uint32_t *hist, uint32_t fp64) {
   __shared__ uint32_t wsum[8];
   __shared__ int is_last;
@@ -172,6 +175,11 @@ __device__ __forceinline__ void flush_and_cut(const ScanArgs &a, uint32_t *hist,
     }
     if (lane == 31) wsum[t >> 5] = incl;
   }
+  if (t == 0) {
+    *a.T = 0;
+    *a.qcount = 0;
+    *a.done = 0;
+  }
   __syncthreads();
   if (t < 256) {
     for (int w = 0; w < (t >> 5); ++w) incl += wsum[w];
@@ -186,9 +194,7 @@ __device__ __forceinline__ void flush_and_cut(const ScanArgs &a, uint32_t *hist,
       }
       const uint64_t hi = ((uint64_t)(bin + 1) << a.shift) - 1;
       *a.T = bin == kLatBins - 1 || hi > 0xffffffffull ? 0xffffffffu : (uint32_t)hi;
-      *a.qcount = 0;
     }
-    if (t == 0) *a.done = 0;
   }
 }
 
@@ -356,6 +362,7 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
   } else {
     // ------------------------------------------------------------ consumers
     const float qn = *a.qn;
+    const uint32_t limit = a.wait_p ? *a.wait_p : a.wait;
     const float cf = latency_cfac(d);
     const float4 *q4 = reinterpret_cast<const float4 *>(qs);
     const float4 b0 = q4[lane], b1 = q4[lane + 32];
@@ -364,7 +371,7 @@ __global__ void __launch_bounds__((kBulkWarps + 1) * 32, 1)
     for (int64_t ch = blockIdx.x; ch < nch; ch += gridDim.x, ++it) {
       const int s = it % kBulkStages;
       // (one answer for the warp: its lanes meet in shuffles below)
-      if (!__all_sync(0xffffffffu, bulk_wait(&full[s], (it / kBulkStages) & 1, a.wait))) {
+      if (!__all_sync(0xffffffffu, bulk_wait(&full[s], (it / kBulkStages) & 1, limit))) {
         failed = true;
         break;
       }
@@ -483,6 +490,8 @@ struct ScanBufs {
   uint32_t *nlo, *nup, *ghist, *T, *qcount;   // ghist: kLatBins, then the CTA counter
   int32_t *jall;
   unsigned long long *nfp64;   // [0] canonical evaluations, [1] select error, [2] scan error
+  int *err;                    // the scan's error word (nfp64[2] unless replaced)
+  const uint32_t *wait_p;      // see ScanArgs
   int grid, shift;
   uint32_t top;
   bool vec4, bulk;
@@ -524,6 +533,8 @@ rkr_status alloc_scan(const rkr_index *idx, int nq, int ctas_per_sm, DevBuf (&b)
   RKR_TRY(tmp_alloc(b[4], &sb.T, 1, st));
   RKR_TRY(tmp_alloc(b[5], &sb.qcount, nq, st));
   RKR_TRY(tmp_alloc(b[6], &sb.nfp64, 3, st));
+  sb.err = (int *)(sb.nfp64 + 2);
+  sb.wait_p = nullptr;
   RKR_CUDA(cudaMemsetAsync(sb.ghist, 0, sizeof(uint32_t) * (kLatBins + 1), st));
   RKR_CUDA(cudaMemsetAsync(sb.qcount, 0, sizeof(uint32_t) * nq, st));
   RKR_CUDA(cudaMemsetAsync(sb.nfp64, 0, 3 * sizeof(unsigned long long), st));
@@ -545,9 +556,10 @@ rkr_status scan_pass(const rkr_index *idx, const QueryCommon &qc, int q, const S
     a.ghist = sb.ghist; a.done = sb.ghist + kLatBins; a.kq = qc.kq_d + q;
     a.T = sb.T; a.qcount = sb.qcount + q; a.nfp64 = sb.nfp64;
     a.wait = epi_wait_limit();
+    a.wait_p = sb.wait_p;
     if (sb.bulk)
       k_latency_scan_bulk<<<sb.grid, (kBulkWarps + 1) * 32, sb.bulk_smem, st>>>(
-          a, (int *)(sb.nfp64 + 2));
+          a, sb.err);
     else if (sb.vec4)
       k_latency_scan<4><<<sb.grid, kLatThreads, 0, st>>>(a);
     else
@@ -681,7 +693,8 @@ struct rkr_session {
   int64_t *off_dev = nullptr;
   // outputs (pinned host memory, max_k entries each) and error words
   double *oest = nullptr;
-  int32_t *users = nullptr, *ocase = nullptr, *onc = nullptr, *oerr = nullptr;
+  int32_t *users = nullptr, *ocase = nullptr, *onc = nullptr;
+  int32_t *oerr = nullptr;   // [0] selection, [1] scan
   uint32_t *onlo = nullptr, *onup = nullptr;
   rkr::DevBuf scan_bufs[7], cand_bufs[5], out_bufs[2];
   rkr::lat::ScanBufs sb;
@@ -694,6 +707,7 @@ struct rkr_session {
     float q[rkr::kMaxD];
     float qn;
     int32_t k;
+    uint32_t wait;   // stage wait limit of the bulk-staged scan
   };
   In *in_h = nullptr;
   unsigned char *out_h = nullptr;
@@ -791,6 +805,7 @@ extern "C" rkr_status rkr_session_create(rkr_index *idx, int32_t max_k, double c
   RKR_CUDA(cudaMallocHost(&s->in_h, sizeof(rkr_session::In)));
   memset(s->in_h, 0, sizeof(rkr_session::In));
   s->in_h->k = 1;
+  s->in_h->wait = epi_wait_limit();
   RKR_CUDA(cudaMallocHost(&s->out_h, out_bytes));
   memset(s->out_h, 0, out_bytes);
   s->oest = (double *)s->out_h;
@@ -800,6 +815,8 @@ extern "C" rkr_status rkr_session_create(rkr_index *idx, int32_t max_k, double c
   s->ocase = (int32_t *)(s->out_h + 20 * K);
   s->onc = s->ocase + 1;
   s->oerr = s->ocase + 2;
+  s->sb.err = s->oerr + 1;
+  s->sb.wait_p = (const uint32_t *)(s->in_dev + offsetof(rkr_session::In, wait));
   // one uncaptured run (sets function attributes, warms the pool), then the capture
   RKR_TRY(session_enqueue(s));
   RKR_CUDA(cudaStreamSynchronize(st));
@@ -849,14 +866,12 @@ extern "C" rkr_status rkr_session_query(rkr_session *s, const float *q, int32_t 
   if ((double)qn < nv) qn = nextafterf(qn, INFINITY);
   s->in_h->qn = qn;
   s->in_h->k = k;
-  *s->oerr = 0;
+  s->in_h->wait = epi_wait_limit();
+  s->oerr[0] = s->oerr[1] = 0;
   RKR_CUDA(cudaGraphLaunch(s->exec, st));
   RKR_CUDA(cudaStreamSynchronize(st));
-  unsigned long long scan_err = 0;
-  if (s->sb.bulk)   // only the bulk-staged scan has waits that can run out
-    RKR_CUDA(cudaMemcpy(&scan_err, s->sb.nfp64 + 2, sizeof(scan_err), cudaMemcpyDeviceToHost));
-  if ((int)scan_err) return fail(RKR_ETIMEOUT, "latency scan wait timed out (%d)", (int)scan_err);
-  if (*s->oerr) return fail(RKR_EINTERNAL, "fewer than k candidates for the query");
+  if (s->oerr[1]) return fail(RKR_ETIMEOUT, "latency scan wait timed out (%d)", s->oerr[1]);
+  if (s->oerr[0]) return fail(RKR_EINTERNAL, "fewer than k candidates for the query");
   const size_t K = (size_t)k;
   struct Out {
     void *dst;

@@ -49,3 +49,22 @@ def test_calls_report_the_timeout_and_recover(bulk):
             got = idx.query_approx(w.Q, w.k, 2.0, single=True)
             for key in KEYS:
                 assert (got[key] == want[key]).all(), key
+
+
+def test_session_survives_a_timeout(bulk):
+    # the counts of a replay that timed out carry over to no later one, and neither
+    # does its error
+    w, idx = _index()
+    with idx, rkr.Session(idx, max_k=int(w.k.max())) as sess:
+        want = [sess.query(w.Q[q], int(w.k[q])) for q in range(len(w.Q))]
+        for _ in range(3):
+            rkr.rkr_set_wait_limit(0)
+            for q in range(len(w.Q)):
+                with pytest.raises(rkr.RKRError) as e:
+                    sess.query(w.Q[q], int(w.k[q]))
+                assert e.value.status == ETIMEOUT
+            rkr.rkr_set_wait_limit(-1)
+            for q in range(len(w.Q)):
+                got = sess.query(w.Q[q], int(w.k[q]))
+                for key in KEYS:
+                    assert (got[key] == want[q][key]).all(), (q, key)
