@@ -1894,8 +1894,9 @@ static rkr_status count_valid(const int32_t *v, int64_t n, unsigned long long *o
 }
 
 // Interval [lo, hi] of a candidate's u.q in float: from its screened score, or from
-// the compensated product of its rows.
-__device__ __forceinline__ void cand_interval(int64_t u, int q, float x,
+// the compensated product of its rows.  False when an end is not finite (products of
+// the rows beyond the range of float): such a candidate takes no part in the grid.
+__device__ __forceinline__ bool cand_interval(int64_t u, int q, float x,
                                               const tc::RowBound *__restrict__ urb,
                                               const tc::RowBound *__restrict__ qrb, tc::Gacc gacc,
                                               float gcan, const float *__restrict__ U,
@@ -1908,6 +1909,7 @@ __device__ __forceinline__ void cand_interval(int64_t u, int q, float x,
   } else {
     dot2_interval_f(U + u * d, Q + (int64_t)q * d, d, lo, hi);
   }
+  return lo > -INFINITY && hi < INFINITY;   // (a NaN end fails both)
 }
 
 // Order-preserving 32-bit key of a float, and its inverse.
@@ -1919,7 +1921,8 @@ __device__ __forceinline__ float key_float(uint32_t k) {
   return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k);
 }
 
-// Range of the open candidates' u.q per user, as keys (kmin starts at ~0, kmax at 0).
+// Range of the open candidates' u.q per user, as keys (kmin starts at ~0, the key of
+// no finite value, kmax at 0).
 __global__ void k_open_range(int64_t cnt, const int32_t *__restrict__ cu_fb,
                              const int32_t *__restrict__ cq, const float *__restrict__ cx,
                              const tc::RowBound *__restrict__ urb,
@@ -1931,7 +1934,7 @@ __global__ void k_open_range(int64_t cnt, const int32_t *__restrict__ cu_fb,
   const int64_t u = cu_fb[i];
   if (u < 0) return;
   float lo, hi;
-  cand_interval(u, cq[i], cx[i], urb, qrb, gacc, gcan, U, Q, d, lo, hi);
+  if (!cand_interval(u, cq[i], cx[i], urb, qrb, gacc, gcan, U, Q, d, lo, hi)) return;
   const uint32_t a = float_key(lo), b = float_key(hi);
   if (a < kmin[u]) atomicMin(&kmin[u], a);
   if (b > kmax[u]) atomicMax(&kmax[u], b);
@@ -1979,8 +1982,8 @@ __global__ void k_grid_bound(int64_t cnt, const int32_t *__restrict__ cu_fb,
   const int64_t u = cu_fb[i];
   if (u < 0) return;
   float lo, hi;
-  cand_interval(u, cq[i], cx[i], urb, qrb, gacc, gcan, U, Q, d, lo, hi);
-  const int64_t s = uslot[u];
+  if (!cand_interval(u, cq[i], cx[i], urb, qrb, gacc, gcan, U, Q, d, lo, hi)) return;
+  const int64_t s = uslot[u];   // set: k_open_range saw this finite interval
   const TightBins tb(ybin[s]);
   if (!tb.usable()) return;   // a grid without a usable step bounds nothing
   const int jl = tb.lo(lo, kDGrid), jh = tb.hi(hi, kDGrid);

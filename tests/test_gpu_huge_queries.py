@@ -1,0 +1,42 @@
+"""Queries whose products with a user exceed the range of float: FP32 scores and
+compensated products are then infinite or NaN, the canonical FP64 score is not."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+rkr = pytest.importorskip("paper_2504_13446_gb300")
+
+
+def test_count_grid_leaves_out_scores_beyond_float():
+    # Half of the users lie in the first two coordinates, where the queries are huge
+    # and of opposite signs (FP32: inf - inf) and every item is alike, so that their
+    # tail lists overflow and they stay open to the recount with no finite interval
+    # of u.q.  The other users see ordinary queries.
+    n, m, d, nq = 6000, 1500, 24, 64
+    rng = np.random.default_rng(8)
+    U = synth.workloads.gaussian_rows(rng, n, d, 0.7)
+    U[:, :2] = 0
+    U[::2] = 0
+    U[::2, :2] = np.float32(30)
+    P = synth.workloads.gaussian_rows(rng, m, d, 0.7)
+    P[:, :2] = np.float32(0.01)
+    Q = (synth.workloads.gaussian_rows(rng, nq, d, 0.5) * np.float32(0.2)).astype(np.float32)
+    Q[:, 0] = np.float32(1e38)
+    Q[:, 1] = -Q[:, 0]
+    step = np.where(np.arange(nq) % 2 == 0, np.float32(2e38), np.float32(0))
+    Q[:, 1] = np.nextafter(Q[:, 1], -step).astype(np.float32)
+    k = rng.integers(1, 40, nq).astype(np.int32)
+    with rkr.Index(U, P, tau=32, omega=4, s=20, floor_rank=max(2, m // 32)) as idx:
+        rkr.rkr_profile_start()
+        try:
+            users, ranks, off, _ = idx.query_exact(Q, k)
+        finally:
+            report = rkr.rkr_profile_stop()
+    assert "k_screen<EpiDeep>" in report, "the count grid was not built"
+    for q, (wu, wr) in enumerate(oracle.exact_query(U, P, Q, k)):
+        assert np.array_equal(users[off[q]:off[q + 1]], wu), q
+        assert np.array_equal(ranks[off[q]:off[q + 1]], wr), q
