@@ -117,8 +117,10 @@ __device__ __forceinline__ void finish_users(const ScanArgs &a, const float *qs,
     if (lane == src) {
       const double res = (double)t.p + (double)t.s, E = (double)t.err(a.d + 8);
       const double fm = a.fmin[u], dl = a.delta[u];
-      int jl = exact_j(res - E, fm, dl, a.tau);
-      if (jl != exact_j(res + E, fm, dl, a.tau)) {
+      const double tlo = res - E, thi = res + E;
+      int jl = exact_j(tlo, fm, dl, a.tau);
+      // (NaN ends, of products beyond the range of float, decide nothing)
+      if (!(tlo <= thi) || jl != exact_j(thi, fm, dl, a.tau)) {
         ++fp64;
         jl = exact_j(canon_dot_slow(row, qs, a.d), fm, dl, a.tau);
       }

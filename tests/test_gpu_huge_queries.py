@@ -40,3 +40,32 @@ def test_count_grid_leaves_out_scores_beyond_float():
     for q, (wu, wr) in enumerate(oracle.exact_query(U, P, Q, k)):
         assert np.array_equal(users[off[q]:off[q + 1]], wu), q
         assert np.array_equal(ranks[off[q]:off[q + 1]], wr), q
+
+
+@pytest.mark.parametrize("d,bulk", [(24, 0), (24, 1), (37, 0)])
+def test_one_at_a_time_scores_beyond_float(d, bulk):
+    rng = np.random.default_rng(d)
+    n, m, nq, tau, omega, s = 3000, 700, 6, 40, 3, 20
+    U = synth.workloads.gaussian_rows(rng, n, d, 0.7)
+    U *= np.float32(30)
+    P = synth.workloads.gaussian_rows(rng, m, d, 0.7)
+    Q = synth.workloads.gaussian_rows(rng, nq, d, 0.5)
+    Q = (Q / np.linalg.norm(Q, axis=1, keepdims=True) * 2e38).astype(np.float32)
+    Q[0] = P[5]
+    k = np.array([5, 1, 60, 700, 33, 2500], np.int32)
+    pos = synth.sample_positions(1, oracle.bucket_sizes(m, omega), s)
+    ora = oracle.build_index(U, P, tau, omega, s, pos, fbounds="exact")
+    was = rkr.rkr_tuning_get()
+    try:
+        rkr.rkr_tuning_set(**{**was, "latency_bulk": bulk})
+        with rkr.Index(U, P, tau=tau, omega=omega, s=s, sample_pos=pos,
+                       exact_table=False) as idx:
+            got = idx.query_approx(Q, k, 2.0, single=True)
+    finally:
+        rkr.rkr_tuning_set(**was)
+    off = got["offsets"]
+    for q, w in enumerate(oracle.approx_query(ora, U, Q, k, 2.0)):
+        sl = slice(off[q], off[q + 1])
+        assert got["case"][q] == w["case"] and got["nc"][q] == w["nc"], q
+        for a in ("users", "n_low", "n_up", "est"):
+            assert np.array_equal(got[a][sl], w[a]), (q, a)
