@@ -32,24 +32,21 @@ __global__ void k_row_norms(const float *__restrict__ X, int64_t rows, int d,
   double nv = sqrt(ss);
   if (nrm64) nrm64[i] = nv;
   // upper bound of the exact norm: the canonical sum is within d 2^-53 (relative)
-  if (nrm32) nrm32[i] = __double2float_ru(nv * (1.0 + 0x1p-40) + 1e-300);
+  if (nrm32) nrm32[i] = norm_up64(nv);
 }
 
-// The FP32 upper bounds alone: a warp per row, compensated FP32 (no FP64 values are
-// wanted: users and queries).
-__global__ void __launch_bounds__(256)
-    k_row_norm_bounds(const float *__restrict__ X, int64_t rows, int d,
-                      float *__restrict__ nrm32) {
-  const int64_t i = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
-  if (i >= rows) return;
+// The FP32 upper bound of one row's norm by a warp (every lane gets it), with the
+// bits that k_row_norms gives; *bad tells a row that is not finite.
+__device__ __forceinline__ float warp_norm_bound(const float *__restrict__ x, int d, bool *bad) {
   const int lane = threadIdx.x & 31;
-  const float *x = X + i * d;
   constexpr int kPieces = kMaxD / 32;
   float v[kPieces], mx = 0.0f;
+  bool nonfinite = false;
 #pragma unroll
   for (int p = 0; p < kPieces; ++p) {
     const int c = lane + 32 * p;
     v[p] = c < d ? x[c] : 0.0f;
+    nonfinite |= !isfinite(v[p]);
     mx = fmaxf(mx, fabsf(v[p]));
   }
 #pragma unroll
@@ -61,7 +58,22 @@ __global__ void __launch_bounds__(256)
   for (int p = 0; p < kPieces; ++p)
     if (32 * p < d) s.add(v[p] * scale);
   s.warp_sum();
-  if (lane == 0) nrm32[i] = s.norm_up(unscale);
+  *bad = __any_sync(0xffffffffu, nonfinite);
+  float up;
+  if (!s.norm_up(unscale, up) && lane == 0 && !*bad)
+    up = mx > 0.0f ? norm_up64(sqrt(canon_dot(x, x, d))) : 1e-45f;
+  return __shfl_sync(0xffffffffu, up, 0);
+}
+
+// The FP32 upper bounds alone: a warp per row (no FP64 values are wanted: users).
+__global__ void __launch_bounds__(256)
+    k_row_norm_bounds(const float *__restrict__ X, int64_t rows, int d,
+                      float *__restrict__ nrm32) {
+  const int64_t i = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
+  if (i >= rows) return;
+  bool bad;
+  const float up = warp_norm_bound(X + i * d, d, &bad);
+  if ((threadIdx.x & 31) == 0) nrm32[i] = up;
 }
 
 rkr_status row_norms(const float *X, int64_t rows, int d, double *nrm64, float *nrm32,
@@ -93,33 +105,12 @@ __global__ void __launch_bounds__(256)
                   unsigned *__restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
   if (i >= rows) return;
-  const int lane = threadIdx.x & 31;
-  const float *x = X + i * d;
-  constexpr int kPieces = kMaxD / 32;
-  float v[kPieces], mx = 0.0f;
-  bool bad = false;
-#pragma unroll
-  for (int p = 0; p < kPieces; ++p) {
-    const int c = lane + 32 * p;
-    v[p] = c < d ? x[c] : 0.0f;
-    bad |= !isfinite(v[p]);
-    mx = fmaxf(mx, fabsf(v[p]));
-  }
-  bad = __any_sync(0xffffffffu, bad);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  float scale, unscale;
-  row_scale(mx, scale, unscale);
-  SquareSum s;
-#pragma unroll
-  for (int p = 0; p < kPieces; ++p)
-    if (32 * p < d) s.add(v[p] * scale);
-  s.warp_sum();
-  if (lane == 0) {
-    const float nv = s.norm_up(unscale);
-    nrm32[i] = nv;
+  bool bad;
+  const float up = warp_norm_bound(X + i * d, d, &bad);
+  if ((threadIdx.x & 31) == 0) {
+    nrm32[i] = up;
     if (bad) atomicOr(&out[0], 1u);
-    else atomicMax(&out[1], __float_as_uint(nv));   // nv >= 0
+    else atomicMax(&out[1], __float_as_uint(up));   // up >= 0
   }
 }
 

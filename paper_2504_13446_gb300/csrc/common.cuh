@@ -167,10 +167,18 @@ struct Dot2 {
   }
 };
 
-// Rigorous FP32 upper bounds of Euclidean norms.  Squares of scaled values (a power
-// of two brings the row's largest magnitude near 1) are summed as in Dot2; all terms
-// are non-negative, so the sum is within 2^-31 (relative, up to 512 terms) of the
-// exact one, up to 2^-140 of underflow.
+// FP32 upper bound of a Euclidean norm from its FP64 value (the square root of a sum
+// of exact squares, up to 2^-44 off): the one definition of these bounds.
+__device__ __forceinline__ float norm_up64(double nv) {
+  return __double2float_ru(nv * (1.0 + 0x1p-40) + 1e-300);
+}
+
+// The same bound, bit for bit, from compensated FP32 sums (all but some 2^-14 of the
+// rows need no FP64 operation).  Squares of scaled values (a power of two brings the
+// row's largest magnitude near 1) are summed as in Dot2; all terms are non-negative
+// and one passes at most 8 + 5 additions here (a lane's eight, five of the warp), so
+// that with u = 2^-24 the low parts stay within 14 u of p and the sum p + s within
+// 233 u^2 < 2^-40 (relative) of the exact one.
 struct SquareSum {
   float p = 0.0f, s = 0.0f;
   __device__ __forceinline__ void two_sum(float h, float low) {
@@ -193,10 +201,29 @@ struct SquareSum {
       two_sum(p2, s2);
     }
   }
-  // upper bound of sqrt(sum) * unscale
-  __device__ __forceinline__ float norm_up(float unscale) const {
-    const float t = __fadd_ru(__fmul_ru(__fadd_ru(p, fabsf(s)), 1.0f + 0x1p-23f), 0x1p-140f);
-    return __fadd_ru(__fmul_ru(__fsqrt_ru(t), unscale), 1e-45f);
+  // norm_up64 of sqrt(sum) * unscale; false when these bits do not decide it (also for
+  // sums so small that underflow, 2^-140 in all, could matter).  With
+  // A = p + s the FP64 form rounds up a T with A < T^2 < A (1 + 2^-38) (its factor
+  // 1 + 2^-40 against the 2^-40 above and 2^-44 of its own), so it gives the smallest
+  // float r with r^2 > A, unless r^2 lies within A (1 + 2^-38).  A = t + l exactly, and
+  // r^2 - t is exact or, a neighbour further off, right in sign and to 2^-24.
+  __device__ __forceinline__ bool norm_up(float unscale, float &out) const {
+    const float t = __fadd_rn(p, s), l = __fsub_rn(s, __fsub_rn(t, p));
+    out = 0.0f;
+    if (!(t >= 0x1p-90f)) return false;
+    auto over = [&](float r) { return __fsub_rn(__fmaf_rn(r, r, -t), l); };
+    const uint32_t r0 = __float_as_uint(__fsqrt_rn(t));
+    float r = 0.0f, d = 0.0f;
+#pragma unroll
+    for (int i = 2; i >= -2; --i) {   // sqrt(A) is within an ulp of the root of t
+      const float x = __uint_as_float(r0 + i), e = over(x);
+      if (e > 0.0f) {
+        r = x;
+        d = e;
+      }
+    }
+    out = __fmul_ru(r, unscale);
+    return d > __fmul_ru(t, 0x1p-37f);
   }
 };
 

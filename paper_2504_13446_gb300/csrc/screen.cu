@@ -17,9 +17,9 @@ namespace rkr {
 // hi = bf16(x), lo = bf16(x - hi) (x - hi, x - hi - lo and hi + lo are exact in
 // FP32), zero padding up to kp, and the bound terms of single and split products.
 // A warp per row, two neighbouring columns a lane (rows are written 128 bytes at a
-// time); the norms are sums of squares in compensated FP32 (SquareSum), not FP64,
-// of which this GPU does a hundredth: 1M rows of d = 200 took 4.6 ms in FP64 with a
-// thread per row.
+// time); the norms are sums of squares in compensated FP32 (SquareSum), in FP64 (of
+// which this GPU does a hundredth) only where their bits do not decide: 1M rows of
+// d = 200 took 4.6 ms in FP64 with a thread per row.
 __global__ void __launch_bounds__(256)
     k_stage_bf16(const float *__restrict__ X, int64_t rows, int d, int kp, int ld,
                  __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
@@ -75,12 +75,36 @@ __global__ void __launch_bounds__(256)
   se1.warp_sum();
   se3.warp_sum();
   sc.warp_sum();
+  // lane 0's sums decide for the warp; part(x, h, l) is the term of a value and its parts
+  auto bound = [&](const SquareSum &q, auto &&part) {
+    float up;
+    if (__shfl_sync(0xffffffffu, q.norm_up(unscale, up), 0)) return up;
+    double acc = 0.0;
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < 2 * kPieces; ++i) {
+      const float x = v[i >> 1][i & 1];
+      const float h = __bfloat162float(__float2bfloat16_rn(x));
+      const float t = part(x, h, __bfloat162float(__float2bfloat16_rn(x - h)));
+      if (t != 0.0f) {   // (rows whose values are their own hi parts have no others)
+        acc = fma((double)t, (double)t, acc);
+        any = true;
+      }
+    }
+    if (!__any_sync(0xffffffffu, any)) return 1e-45f;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return norm_up64(sqrt(acc));
+  };
+  tc::RowBound a, b;
+  a.a0 = bound(se1, [](float x, float h, float) { return x - h; });
+  a.a1 = bound(sh, [](float, float h, float) { return h; });
+  a.a2 = bound(sx, [](float x, float, float) { return x; });
+  b.a0 = bound(se3, [](float x, float h, float l) { return x - h - l; });
+  b.a1 = bound(sc, [](float, float h, float l) { return h + l; });
+  b.a3 = bound(sl, [](float, float, float l) { return l; });
   if (lane == 0) {
-    tc::RowBound a, b;
-    a.a0 = se1.norm_up(unscale); a.a1 = sh.norm_up(unscale); a.a2 = sx.norm_up(unscale);
     a.a3 = 0.0f; a.a4 = a.a1;
-    b.a0 = se3.norm_up(unscale); b.a1 = sc.norm_up(unscale); b.a2 = a.a2;
-    b.a3 = sl.norm_up(unscale); b.a4 = a.a1;
+    b.a2 = a.a2; b.a4 = a.a1;
     rb1[i] = a;
     rb3[i] = b;
   }
