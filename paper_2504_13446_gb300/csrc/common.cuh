@@ -236,7 +236,8 @@ __device__ __forceinline__ void row_scale(float mx, float &scale, float &unscale
   unscale = __uint_as_float((uint32_t)(127 + e) << 23);
 }
 
-// Interval [lo, hi] that holds the canonical score s(a, b).
+// Interval [lo, hi] that holds the canonical score s(a, b); everything when a product
+// or a sum of the rows leaves the range of float (the ends are then NaN).
 __device__ __forceinline__ void dot2_interval(const float *__restrict__ a,
                                               const float *__restrict__ b, int d, double &lo,
                                               double &hi) {
@@ -245,6 +246,10 @@ __device__ __forceinline__ void dot2_interval(const float *__restrict__ a,
   const double res = (double)t.p + (double)t.s, E = (double)t.err(d);
   lo = res - E;
   hi = res + E;
+  if (!(lo <= hi)) {
+    lo = -INFINITY;
+    hi = INFINITY;
+  }
 }
 
 // The same rounded outwards to float, without FP64 operations.
@@ -256,6 +261,10 @@ __device__ __forceinline__ void dot2_interval_f(const float *__restrict__ a,
   const float E = t.err(d);
   lo = __fsub_rd(__fadd_rd(t.p, t.s), E);
   hi = __fadd_ru(__fadd_ru(t.p, t.s), E);
+  if (!(lo <= hi)) {
+    lo = -INFINITY;
+    hi = INFINITY;
+  }
 }
 
 // Threshold t_{j+1} (0-based i = j): f_min + i * delta, delta = (f_max - f_min) / (tau - 1),
@@ -265,15 +274,16 @@ __device__ __forceinline__ double thr_at(double fmin, double delta, int i) {
 }
 
 // A first guess of #{i : t_i <= theta} for a grid with step delta, from FP32 where
-// the step allows it (the callers' comparisons make it exact).
+// the step allows it (the callers' comparisons make it exact).  Always in [0, tau]:
+// 0 for a NaN, which no comparison moves.
 __device__ __forceinline__ int grid_guess(double theta, double fmin, double delta, int tau) {
   const float df = (float)delta;
   if (df > 1e-30f && df < 1e30f) {
     const float x = __fdividef((float)(theta - fmin), df);
-    return x < 0.0f ? 0 : (x >= (float)tau ? tau : (int)x + 1);
+    return !(x >= 0.0f) ? 0 : (x >= (float)tau ? tau : (int)x + 1);
   }
   const double x = (theta - fmin) / delta;
-  return x < 0.0 ? 0 : (x >= (double)tau ? tau : (int)floor(x) + 1);
+  return !(x >= 0.0) ? 0 : (x >= (double)tau ? tau : (int)floor(x) + 1);
 }
 
 // j(theta) = #{i in [0, tau) : t_i <= theta}: the 1-based index of the largest
@@ -362,7 +372,7 @@ __device__ __forceinline__ void bin_interval(const BinFP &b, double fmin, int ta
                                              float xhi, int &jlo, int &jhi) {
   if (b.invd32 < 0.0f) {  // delta == 0: all thresholds equal f_min
     jlo = ((double)xlo > fmin) ? tau : 0;
-    jhi = ((double)xhi >= fmin) ? tau : 0;
+    jhi = ((double)xhi < fmin) ? 0 : tau;   // (NaN: undecided)
     return;
   }
   if (b.err > 1e6f) { jlo = 0; jhi = tau; return; }

@@ -772,6 +772,10 @@ __global__ void __launch_bounds__(128, 8) k_list_rank(int64_t count, const int32
     const float b = tc::screen_bound_tc(rb3[u], qrb[cq[i]], gacc, gcan);
     flo = __fsub_rd(sx, b);
     fhi = __fadd_ru(sx, b);
+    if (!(flo <= fhi)) {   // an infinite score within an infinite bound
+      flo = -INFINITY;
+      fhi = INFINITY;
+    }
     state = 0;
   } else {
     compensate();
@@ -1608,7 +1612,7 @@ __global__ void k_scatter_back(int64_t n, const int32_t *__restrict__ oi,
 // exactly with it.  With cx (the screened scores of all candidates, by their index
 // ci) and no_theta, a row whose candidate has a screened score takes the interval
 // [score - bound, score + bound] holding u.q as its threshold, so no row of U or Q
-// is read; the others take the canonical u.q rounded both ways (ths, when wanted,
+// is read (unless the score and its bound are infinite); the others take the canonical u.q rounded both ways (ths, when wanted,
 // gets the value itself).  ncanon counts the canonical products.
 __global__ void k_row_thresholds(int64_t count, const int32_t *__restrict__ cu,
                                  const int32_t *__restrict__ cq, const int32_t *__restrict__ ci,
@@ -1625,9 +1629,13 @@ __global__ void k_row_thresholds(int64_t count, const int32_t *__restrict__ cu,
     const int q = cq[i];
     rself[i] = qself[q];
     const float x = cx ? cx[ci[i]] : __int_as_float(0x7fffffff);
+    float2 t2 = make_float2(x, x);
     if (x == x) {
       const float b = tc::screen_bound_tc(urb[u], qrb[q], gacc, gcan);
-      thr[i] = make_float2(__fsub_rd(x, b), __fadd_ru(x, b));
+      t2 = make_float2(__fsub_rd(x, b), __fadd_ru(x, b));
+    }
+    if (t2.x <= t2.y) {
+      thr[i] = t2;
     } else {
       const double t = canon_dot(U + u * d, Q + (int64_t)q * d, d);
       thr[i] = make_float2(__double2float_rd(t), __double2float_ru(t));

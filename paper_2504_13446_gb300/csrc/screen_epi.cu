@@ -77,6 +77,14 @@ struct TilePrefetch {
   }
 };
 
+// Screened scores at most this are skipped: xs less the tile's bound.  NaN, which
+// skips nothing, where that is -inf (no skip score, or products that may leave the
+// range of float: a score of -inf then says nothing about u.q).
+__device__ __forceinline__ float skip_below(float xs, float b) {
+  const float x = __fsub_rd(xs, b);
+  return x > -INFINITY ? x : __int_as_float(0x7fffffff);
+}
+
 // Queue of (row, column) pairs with a capacity; overflow raises a flag.
 struct PairQueue {
   int2 *items;
@@ -1115,7 +1123,7 @@ struct EpiTheta {
       ts.rb = ts.prb;
       ts.bf = ts.pbf;
       ts.fm = ts.pfm;
-      ts.xsb = __fsub_rd(ts.pxs, ts.b);
+      ts.xsb = skip_below(ts.pxs, ts.b);
     }
     tc::epi_sync<kWarps>();
     // prefetch the next row block of this unit while this tile is processed
@@ -1596,7 +1604,7 @@ struct EpiSkim {
     }
     if (ts.u < nrows) {
       ts.b = tc::screen_bound_tc(ts.prb, tileb[ct], gacc, gcan);
-      ts.xsb = __fsub_rd(ts.pxs, ts.b);
+      ts.xsb = skip_below(ts.pxs, ts.b);
     }
   }
   __device__ void chunk(char *S, int, int ct, int, int col, uint32_t, const float (&v)[32],
@@ -1992,7 +2000,7 @@ __global__ void k_rc_refine(const int2 *__restrict__ items, const unsigned long 
       return a0;
     };
     int pos = below(lo), pe = below(hi);
-    if (pos != pe) {   // the compensated product before the canonical value
+    if (pos != pe || !(lo <= hi)) {   // the compensated product before the canonical value
       dot2_interval(uu, pp, d, lo, hi);
       pos = below(lo);
       pe = below(hi);
