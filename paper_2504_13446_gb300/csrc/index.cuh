@@ -135,7 +135,7 @@ struct ThetaArgs {
   const int64_t *qoff;          // pass 2
   uint32_t *qcursor;
   int32_t *cand_u, *cand_q;
-  float *cand_x;                // pass 2: screened score of each candidate
+  float *cand_x;                // pass 2: screened score of each candidate, or null
   int nq_all;                   // queries of the whole batch (pass 1 histogram pitch)
   const float *xs;              // per-user skip scores (null: every pair is screened)
   const int32_t *qmap;          // global query of each column (null: qa + column)

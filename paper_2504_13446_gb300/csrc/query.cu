@@ -1502,12 +1502,13 @@ __global__ void k_close_segments(int qa, int qb, const int64_t *__restrict__ qof
 }
 
 // Pass 2: candidates of queries [qa, qb) appended to per-query segments.  Nothing is
-// waited for: errors stand in *words.
+// waited for: errors stand in *words.  cand_x gets the screened scores of listed
+// candidates and, with screen_x, those of the screen's own candidates too.
 static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, int qa, int qb,
                                   const Grid &g, const Plan &plan, const int32_t *lstar_d,
                                   const uint32_t *cap_d, const int64_t *qoff_d, uint32_t *cursor_d,
                                   int32_t *cand_u, int32_t *cand_q, float *cand_x,
-                                  CallWords *words, cudaStream_t st) {
+                                  bool screen_x, CallWords *words, cudaStream_t st) {
   TcSide sub = qc.Qt;
   sub.owned = false;
   sub.rows = qb - qa;
@@ -1525,7 +1526,7 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
   a.qcursor = cursor_d;
   a.cand_u = cand_u;
   a.cand_q = cand_q;
-  a.cand_x = cand_x;
+  a.cand_x = screen_x ? cand_x : nullptr;
   a.xs = plan.xs;
   a.lskip = plan.lskip;
   if (plan.listed) {
@@ -2258,7 +2259,7 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
     RKR_CUDA(cudaMemsetAsync(cu, 0xff, sizeof(int32_t) * std::max<int64_t>(cnt, 1), st));
     const int t2 = clk.begin(&ms_theta);
     RKR_TRY(emit_candidates(idx, qc, qa, qb, grid, plan, lstar_d, cap_d, qoff_rel, cursor, cu, cq,
-                            cx, words, st));
+                            cx, true, words, st));
     clk.end(t2);
     const int t3 = clk.begin(&ms_res);
     if (cnt > 0) {
@@ -2617,9 +2618,10 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
                              cudaMemcpyHostToDevice, st));
     RKR_CUDA(cudaMemsetAsync(cursor, 0, sizeof(uint32_t) * nq, st));
     RKR_CUDA(cudaMemsetAsync(cu, 0xff, sizeof(int32_t) * std::max<int64_t>(cnt, 1), st));
+    // (the learned cut takes t of a screen's own candidates from their rows)
     const int t2 = clk.begin(&ms_theta);
     RKR_TRY(emit_candidates(idx, qc, qa, qb, grid, plan, lstar_d, cap_d, qoff_rel, cursor, cu, cq,
-                            cx, words, st));
+                            cx, !lp, words, st));
     clk.end(t2);
     const int t3 = clk.begin(&ms_res);
     if (cnt > 0) {

@@ -1038,7 +1038,7 @@ struct EpiTheta {
   const int64_t *qoff;
   uint32_t *qcursor;
   int32_t *cand_u, *cand_q;
-  float *cand_x;                // PASS 2: the candidate's screened score
+  float *cand_x;                // PASS 2: the candidate's screened score (null: not wanted)
   int *ovf;                     // PASS 2: set when a query's segment would overflow
   const float *xs;              // per user: pairs scoring <= xs[u] - b are skipped (or null)
   const uint32_t *member;       // per-query user subsets (bitmaps), or null
@@ -1241,7 +1241,7 @@ struct EpiTheta {
     }
     cand_u[at] = (int32_t)u;
     cand_q[at] = q;
-    cand_x[at] = x;
+    if (cand_x) cand_x[at] = x;
   }
   __device__ void tile_end(char *, int, int, int, int, Thread &) const {}
   __device__ void unit_end(char *S, const tc::Unit &u, int et, Thread &) const {
