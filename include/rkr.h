@@ -574,6 +574,12 @@ uint64_t rkr_device_allocations(void);
  * takes effect for launches that start after the call.  RKR_EINVAL above 2^32 - 1. */
 rkr_status rkr_set_wait_limit(int64_t rounds);
 
+/* Test hook (not in the paper): of the calling thread's next pool allocations, the
+ * one after `after` others fails as if the device had no memory left, once.  The call
+ * it belongs to returns RKR_ENOMEM, or goes on where it can do without.  A negative
+ * value takes the fault back. */
+rkr_status rkr_set_alloc_fault(int64_t after);
+
 /* Release an index (NULL is allowed). */
 void rkr_index_free(rkr_index *idx);
 

@@ -30,7 +30,7 @@ __all__ = ["RKRError", "Index", "QueryStats", "load", "rkr_build", "rkr_query_ex
            "rkr_screen_scores", "rkr_screen_scores_static",
            "rkr_profile_start", "rkr_profile_stop", "Pruner", "rkr_rank_pairs",
            "rkr_pair_features", "rkr_query_exact_learned", "rkr_release_cached_memory",
-           "rkr_set_wait_limit", "device_allocations", "version", "EXPORTS", "Tuning",
+           "rkr_set_wait_limit", "rkr_set_alloc_fault", "device_allocations", "version", "EXPORTS", "Tuning",
            "rkr_tuning_get", "rkr_tuning_set", "rkr_autotune", "Session"]
 
 _lock = threading.Lock()
@@ -200,6 +200,8 @@ def load() -> ctypes.CDLL:
         lib.rkr_device_allocations.argtypes = []
         lib.rkr_set_wait_limit.restype = I32
         lib.rkr_set_wait_limit.argtypes = [I64]
+        lib.rkr_set_alloc_fault.restype = I32
+        lib.rkr_set_alloc_fault.argtypes = [I64]
         lib.rkr_last_error.restype = ctypes.c_char_p
         lib.rkr_version.restype = ctypes.c_char_p
         _lib = lib
@@ -266,6 +268,12 @@ def rkr_set_wait_limit(rounds: int) -> None:
     """Test hook: try_wait rounds of the screens' epilogue wait and of the bulk-staged
     scan's stage wait (negative = default)."""
     _check(load().rkr_set_wait_limit(int(rounds)))
+
+
+def rkr_set_alloc_fault(after: int) -> None:
+    """Test hook: the calling thread's pool allocation after `after` more fails, once
+    (negative = none)."""
+    _check(load().rkr_set_alloc_fault(int(after)))
 
 
 def version() -> str:
@@ -470,7 +478,7 @@ def rkr_query_approx_candidates(index, Q, k, *, user_offset: int = 0, capacity=N
     pq, kq = _ptr(Q, np.float32)
     cap = int(capacity) if capacity is not None else int(max(1024, 16 * kk.sum()))
     while True:
-        offs = np.empty(nq + 1, np.int64)
+        offs = np.zeros(nq + 1, np.int64)   # (a call that fails early leaves them)
         out = dict(users=np.empty(cap, np.int32), n_low=np.empty(cap, np.uint32),
                    n_up=np.empty(cap, np.uint32), est=np.empty(cap, np.float64))
         st = lib.rkr_query_approx_candidates(

@@ -26,6 +26,14 @@ void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 static std::atomic<uint64_t> g_allocs{0};
 void note_alloc() { g_allocs.fetch_add(1, std::memory_order_relaxed); }
 
+// Allocations the calling thread has left before one fails (rkr_set_alloc_fault);
+// negative = none does.
+static thread_local int64_t g_alloc_fault = -1;
+bool alloc_fault() {
+  if (g_alloc_fault < 0) return false;
+  return g_alloc_fault-- == 0;
+}
+
 static std::atomic<uint64_t> g_index_serial{0};
 uint64_t next_index_serial() { return g_index_serial.fetch_add(1, std::memory_order_relaxed) + 1; }
 
@@ -354,6 +362,11 @@ rkr_status rkr_set_wait_limit(int64_t rounds) {
   return RKR_OK;
 }
 
+rkr_status rkr_set_alloc_fault(int64_t after) {
+  g_alloc_fault = after < 0 ? -1 : after;
+  return RKR_OK;
+}
+
 rkr_status rkr_index_timings(const rkr_index *idx, double *out, int32_t count) {
   if (!idx || !out || count < 0) return fail(RKR_EINVAL, "null argument");
   for (int i = 0; i < count; ++i) out[i] = i < (int)(sizeof(idx->build_ms) / sizeof(double)) ? idx->build_ms[i] : 0.0;
@@ -482,6 +495,9 @@ static rkr_status query_prologue(rkr_index *idx, const float *Q, int32_t nq, con
   return RKR_OK;
 }
 
+// What a query call stages on its stream.  A call that ends before it has waited for
+// the stream (settled) waits here: the caller's arrays are no longer in use when it
+// returns, whatever it returns.
 struct QueryStage {
   InView vq, vk, vsu;
   uint32_t *member = nullptr;
@@ -490,8 +506,11 @@ struct QueryStage {
   int64_t *off_d = nullptr;
   BinFP *bf_own = nullptr, *xbf_own = nullptr;
   TcSide Qt;
-  cudaStream_t st = nullptr;
+  cudaStream_t st;
+  bool settled = false;
+  explicit QueryStage(cudaStream_t s) : st(s) {}
   ~QueryStage() {
+    if (!settled) cudaStreamSynchronize(st);
     if (qnrm) cudaFreeAsync(qnrm, st);
     if (off_d) cudaFreeAsync(off_d, st);
     if (bf_own) cudaFreeAsync(bf_own, st);
@@ -578,7 +597,6 @@ static rkr_status stage_bitmaps(rkr_index *idx, int32_t nq, const std::vector<in
 static rkr_status stage_queries(rkr_index *idx, const float *Q, int nq, const int32_t *k,
                                 const std::vector<int64_t> &off, cudaStream_t st,
                                 QueryStage &qs, QueryCommon &qc) {
-  qs.st = st;
   const int d = idx->d;
   RKR_TRY(qs.vq.init(Q, sizeof(float) * (size_t)nq * d, st));
   RKR_TRY(qs.vk.init(k, sizeof(int32_t) * nq, st));
@@ -624,7 +642,7 @@ static rkr_status query_exact_impl(rkr_index *idx, const float *Q, int32_t nq, c
   std::vector<int64_t> off;
   RKR_TRY(query_prologue(idx, Q, nq, k, st, kh, off));
   if (!idx->has_exact) return fail(RKR_EINVAL, "index was built without exact_table");
-  QueryStage qs;
+  QueryStage qs(st);
   QueryCommon qc;
   if (subsets) RKR_TRY(stage_subsets(idx, nq, kh, subset_offs, subset_users, st, qs, qc));
   if (words >= 0) RKR_TRY(stage_bitmaps(idx, nq, kh, member, words, st, qs, qc));
@@ -635,7 +653,9 @@ static rkr_status query_exact_impl(rkr_index *idx, const float *Q, int32_t nq, c
   out.add(out_ranks, sizeof(int32_t) * tot);
   RKR_TRY(out.alloc());
   RKR_TRY(run_query_exact(idx, qc, nq, out.dev<int32_t>(0), out.dev<int32_t>(1), stats, st));
-  return out.finish();
+  RKR_TRY(out.finish());
+  qs.settled = true;
+  return RKR_OK;
 }
 
 static rkr_status query_approx_impl(rkr_index *idx, const float *Q, int32_t nq,
@@ -652,7 +672,7 @@ static rkr_status query_approx_impl(rkr_index *idx, const float *Q, int32_t nq,
   std::vector<int32_t> kh;
   std::vector<int64_t> off;
   RKR_TRY(query_prologue(idx, Q, nq, k, st, kh, off));
-  QueryStage qs;
+  QueryStage qs(st);
   QueryCommon qc;
   if (subsets) RKR_TRY(stage_subsets(idx, nq, kh, subset_offs, subset_users, st, qs, qc));
   if (words >= 0) RKR_TRY(stage_bitmaps(idx, nq, kh, member, words, st, qs, qc));
@@ -669,7 +689,9 @@ static rkr_status query_approx_impl(rkr_index *idx, const float *Q, int32_t nq,
   auto run = single ? run_query_approx_single : run_query_approx;
   RKR_TRY(run(idx, qc, nq, c, out.dev<int32_t>(0), out.dev<uint32_t>(1), out.dev<uint32_t>(2),
               out.dev<double>(3), out.dev<int32_t>(4), out.dev<int32_t>(5), stats, st));
-  return out.finish();
+  RKR_TRY(out.finish());
+  qs.settled = true;
+  return RKR_OK;
 }
 
 rkr_status rkr_query_exact(rkr_index *idx, const float *Q, int32_t nq, const int32_t *k,
@@ -734,7 +756,7 @@ rkr_status rkr_query_approx_candidates(rkr_index *idx, const float *Q, int32_t n
   std::vector<int32_t> kh;
   std::vector<int64_t> off;
   RKR_TRY(query_prologue(idx, Q, nq, k, st, kh, off));
-  QueryStage qs;
+  QueryStage qs(st);
   QueryCommon qc;
   RKR_TRY(stage_queries(idx, Q, nq, k, off, st, qs, qc));
   const size_t cap = (size_t)capacity;
@@ -767,6 +789,7 @@ rkr_status rkr_query_approx_candidates(rkr_index *idx, const float *Q, int32_t n
   RKR_TRY(oup.finish());
   RKR_TRY(oes.finish());
   RKR_CUDA(cudaStreamSynchronize(st));
+  qs.settled = true;
   return RKR_OK;
 }
 
@@ -792,7 +815,7 @@ rkr_status rkr_rank_pairs(rkr_index *idx, const float *Q, int32_t nq, int64_t np
   std::vector<int32_t> kh(nq, 1);
   std::vector<int64_t> off(nq + 1, 0);
   for (int q = 0; q < nq; ++q) off[q + 1] = q + 1;
-  QueryStage qs;
+  QueryStage qs(st);
   QueryCommon qc;
   RKR_TRY(stage_queries(idx, Q, nq, kh.data(), off, st, qs, qc));
   if (npairs == 0) return RKR_OK;
@@ -809,6 +832,7 @@ rkr_status rkr_rank_pairs(rkr_index *idx, const float *Q, int32_t nq, int64_t np
                          (int32_t *)orr.dev, st));
   RKR_TRY(orr.finish());
   RKR_CUDA(cudaStreamSynchronize(st));
+  qs.settled = true;
   return RKR_OK;
 }
 
@@ -872,7 +896,7 @@ rkr_status rkr_query_exact_learned(rkr_index *idx, rkr_pruner *pr, const float *
   for (int q = 0; q < nq; ++q)
     if (keeph[q] < kh[q])
       return fail(RKR_EINVAL, "keep[%d] = %d must be at least k[%d] = %d", q, keeph[q], q, kh[q]);
-  QueryStage qs;
+  QueryStage qs(st);
   QueryCommon qc;
   RKR_TRY(stage_queries(idx, Q, nq, k, off, st, qs, qc));
   InView vr;
@@ -908,6 +932,7 @@ rkr_status rkr_query_exact_learned(rkr_index *idx, rkr_pruner *pr, const float *
   RKR_TRY(ou.finish());
   RKR_TRY(orr.finish());
   RKR_CUDA(cudaStreamSynchronize(st));
+  qs.settled = true;
   return RKR_OK;
 }
 

@@ -26,9 +26,13 @@ cudaMemPool_t lib_pool();
 // Count of device allocations the library has requested (rkr_device_allocations).
 void note_alloc();
 
+// Whether this allocation is the one that rkr_set_alloc_fault made the calling thread fail.
+bool alloc_fault();
+
 template <class T>
 inline cudaError_t pool_malloc_async(T **p, size_t bytes, cudaStream_t st) {
   note_alloc();
+  if (alloc_fault()) return cudaErrorMemoryAllocation;
   return cudaMallocFromPoolAsync((void **)p, bytes, lib_pool(), st);
 }
 
@@ -462,6 +466,20 @@ struct DevBuf {
   ~DevBuf() {
     if (p) cudaFreeAsync(p, st);
   }
+};
+
+// Waits for a stream when a call ends before it has done so itself (settled): on an
+// error, kernels and copies that use the caller's arrays or the call's own host
+// vectors may still be queued.  Declared after those vectors.
+struct StreamGuard {
+  cudaStream_t st;
+  bool settled = false;
+  explicit StreamGuard(cudaStream_t s) : st(s) {}
+  ~StreamGuard() {
+    if (!settled) cudaStreamSynchronize(st);
+  }
+  StreamGuard(const StreamGuard &) = delete;
+  StreamGuard &operator=(const StreamGuard &) = delete;
 };
 
 template <class T>

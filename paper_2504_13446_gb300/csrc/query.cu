@@ -2229,6 +2229,8 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
   DevBuf bo;
   int64_t *qoff_d;
   RKR_TRY(tmp_alloc(bo, &qoff_d, nq + 1, st));
+  std::vector<std::vector<int64_t>> rels;   // per chunk, copied from until the call settles
+  StreamGuard guard(st);
   RKR_CUDA(cudaMemcpyAsync(qoff_d, qoff.data(), sizeof(int64_t) * (nq + 1),
                            cudaMemcpyHostToDevice, st));
   for (auto ch : chunk_queries(plan.ncand, candidate_budget())) {
@@ -2251,7 +2253,8 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
     RKR_TRY(tmp_alloc(b7, &nup, cnt, st));
     RKR_TRY(tmp_alloc(b8, &qoff_rel, nq + 1, st));
     // offsets relative to the chunk start, so candidate arrays hold only this chunk
-    std::vector<int64_t> rel(nq + 1, 0);
+    rels.emplace_back(nq + 1, 0);
+    std::vector<int64_t> &rel = rels.back();
     for (int q = 0; q <= nq; ++q) rel[q] = qoff[q] - qoff[qa];
     RKR_CUDA(cudaMemcpyAsync(qoff_rel, rel.data(), sizeof(int64_t) * (nq + 1),
                              cudaMemcpyHostToDevice, st));
@@ -2284,6 +2287,7 @@ rkr_status run_query_approx(const rkr_index *idx, const QueryCommon &qc, int nq,
   }
   CallWords hw;
   RKR_TRY(words_check(words, hw, st));
+  guard.settled = true;
   clk.finish();
   if (stats) {
     stats->pairs = idx->n * (int64_t)nq;
@@ -2597,6 +2601,8 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
   for (int q = 0; q < nq; ++q) wide += plan.lstar[q] >= idx->nlev_x - 1;
   std::vector<int64_t> qoff(nq + 1, 0);
   for (int q = 0; q < nq; ++q) qoff[q + 1] = qoff[q] + plan.ncand[q];
+  std::vector<std::vector<int64_t>> rels;   // per chunk, copied from until the call settles
+  StreamGuard guard(st);
   for (auto ch : chunk_queries(plan.ncand, candidate_budget())) {
     int qa = ch.first, qb = ch.second;
     int64_t cnt = qoff[qb] - qoff[qa];
@@ -2612,7 +2618,8 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
     RKR_TRY(tmp_alloc(b3, &cursor, nq, st));
     RKR_TRY(tmp_alloc(b4, &ccount, cnt, st));
     RKR_TRY(tmp_alloc(b8, &qoff_rel, nq + 1, st));
-    std::vector<int64_t> rel(nq + 1, 0);
+    rels.emplace_back(nq + 1, 0);
+    std::vector<int64_t> &rel = rels.back();
     for (int q = 0; q <= nq; ++q) rel[q] = qoff[q] - qoff[qa];
     RKR_CUDA(cudaMemcpyAsync(qoff_rel, rel.data(), sizeof(int64_t) * (nq + 1),
                              cudaMemcpyHostToDevice, st));
@@ -2767,6 +2774,7 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
   }
   CallWords hw;
   RKR_TRY(words_check(words, hw, st));
+  guard.settled = true;
   clk.finish();
   const int64_t total = (int64_t)hw.candidates;
   if (stats) {
