@@ -2586,7 +2586,9 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
   RKR_TRY(query_self(idx, qc.Qd, nq, qself, st));
   int64_t fallback = 0, list_fp64 = 0, cut_total = 0;
   double err_ratio = 0.0, err_rel = 0.0;
-  int64_t recount_users = 0, recount_open = 0, recount_split = 0, revived = 0;
+  int64_t recount_users = 0;   // counted for the caller's statistics alone
+  int64_t *const count_users = stats ? &recount_users : nullptr;
+  int64_t recount_open = 0, recount_split = 0, revived = 0;
   int64_t prefix_rows = 0, prefix_pruned = 0, canon_rows = 0, canon_theta = 0;
   unsigned long long lstat_host_fb = 0;
   Plan plan;
@@ -2702,7 +2704,7 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
         for (int pass = tuning().rc_single_first ? 0 : 1; pass < 2 && h2 > 0; ++pass) {
           const bool first = pass == 0 || !tuning().rc_single_first;
           RKR_TRY(recount_candidates(idx, qc, cnt, cu_fb, cq, cx, qself, ccount, clb, nullptr,
-                                     st, first ? &recount_users : nullptr, pass == 0 ? 0 : 1, 0,
+                                     st, first ? count_users : nullptr, pass == 0 ? 0 : 1, 0,
                                      &canon_rows));
           if (pass == 1) recount_split += (int64_t)h2;
           {
@@ -2735,7 +2737,7 @@ static rkr_status query_exact_core(const rkr_index *idx, const QueryCommon &qc, 
                            &lstat_host_fb, st));
       if (!lp && tuning().rc_prefix > 0 && lstat_host_fb >= (unsigned long long)prefix_min_rows(1))
         RKR_TRY(prefix_prune(idx, qc, qa, qb, cnt, qoff_rel, cursor, cq, cx, qself, ccount, clb, cu_fb,
-                             &recount_users, &lstat_host_fb, &prefix_rows, &prefix_pruned,
+                             count_users, &lstat_host_fb, &prefix_rows, &prefix_pruned,
                              &canon_rows, st));
       if (lstat_host_fb > 0) RKR_TRY(recount_open_candidates(lstat_host_fb));
       if (lp && lp->certify && cut_total > 0) {
