@@ -12,7 +12,10 @@ namespace rkr {
 
 // Row pitch (elements) of a staged operand of `width` bf16 columns.  A TMA box
 // reads 128 bytes of each row: with a pitch that is no multiple of 128 bytes
-// almost every such piece straddles two cache lines.
+// almost every such piece straddles two cache lines.  Rows of 48, 80 and 144 columns
+// grow by a third to three fifths for it (operands, under 1 % of an index with its
+// lists): list screen of 400k x 50k at d = 40 14.5 -> 14.4 ms, 72 14.7 -> 14.4,
+// 136 16.4 -> 15.9, 200 20.4 -> 18.5; the screens of U x Q up to 6 % faster.
 inline int tc_pitch(int width) {
   return width == 16 || width == 32 ? width : (width + tc::KCH - 1) / tc::KCH * tc::KCH;
 }
