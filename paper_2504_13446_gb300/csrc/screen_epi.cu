@@ -412,10 +412,11 @@ __global__ void k_xgrid(int64_t n, const double *__restrict__ fmin,
 // XLO[j] = #{clo > j} <= #{p : s(u,p) > x_j} <= #{chi > j} = XHI[j].
 // Histograms are 16-bit pairs packed in 32-bit words; a row whose tail holds
 // more than 65535 items gets the trivial bounds 0 and m instead.
+template <bool INTERLEAVE>
 struct EpiXT {
   static const char *name() { return "k_screen<EpiXT>"; }
   static constexpr int kWarps = 8;   // 98 ms at 1M x 100k x 200 (16 warps: 102)
-  static constexpr bool kInterleave = true;   // 98.3 -> 93.1 ms
+  static constexpr bool kInterleave = INTERLEAVE;   // see kInterleaveChunks
   struct Thread {
     float skip, b, g0;
     int64_t row;
@@ -769,10 +770,33 @@ rkr_status tc_sort_lists(rkr_index *idx, const tc::RowBound *tb, int bn, cudaStr
   return RKR_OK;
 }
 
+// The list screen takes its tiles from both ends in turn where a tile has at least
+// this many K chunks.  With fewer, a light tile's MMAs are shorter than any tile's
+// epilogue and hide nothing, and the norm order is the better one.  400k x 50k, norm
+// order -> both ends: d = 32 (2 chunks) 13.2 -> 13.8 ms, 64 (3) 13.6 -> 14.3, 88 (5)
+// 14.6 -> 14.9, 104 (6) 15.3 -> 15.3, 120 (6) 15.3 -> 15.4, 136 (7) 16.3 -> 15.9,
+// 168 (9) 18.2 -> 17.3, 200 (10) 19.4 -> 18.5, 256 (12) 21.3 -> 20.5.
+constexpr int kInterleaveChunks = 7;
+
+template <bool INTERLEAVE>
+static rkr_status list_screen(const rkr_index *idx, const TcSide &Ut, const TcSide &Pt,
+                              const float *g0f, const tc::RowBound *tb, int *flags,
+                              cudaStream_t st) {
+  constexpr int BN = 256;
+  using Epi = EpiXT<INTERLEAVE>;
+  Epi e;
+  e.nrows = idx->n; e.ncols = idx->m; e.bn = BN; e.rowb = Ut.rb3; e.tileb = tb;
+  e.gacc = tc_gacc(Ut.kp, 1); e.gcan = tc_gcan(idx->d);
+  e.g0f = g0f;
+  e.list = idx->xlist; e.loff = idx->xloff; e.lcapv = idx->xlcap; e.lcnt = idx->xlcnt;
+  static_assert(tc::screen_smem_bytes<BN, 4, Epi>() <= 232448, "exact-table smem");
+  return launch_screen<BN, 4>(Ut, Pt, 1, row_schedule(idx->n, idx->m, BN), e, flags, st);
+}
+
 rkr_status tc_exact_table(rkr_index *idx, const TcSide &Ut, const TcSide &Pt, cudaStream_t st,
                           int64_t *) {
   constexpr int BN = 256;
-  const int64_t n = idx->n, m = idx->m;
+  const int64_t n = idx->n;
   tc::RowBound *tb = nullptr;
   RKR_TRY(tc_tile_bounds(Pt, BN, 1, &tb, st));
   float *g0f;
@@ -785,13 +809,9 @@ rkr_status tc_exact_table(rkr_index *idx, const TcSide &Ut, const TcSide &Pt, cu
   note_launch();
 
   RKR_TRY(make_binfp_grid(idx, idx->xg0, idx->fmax, kXG, idx->pmax, idx->xdx, idx->xbin, st));
-  EpiXT e;
-  e.nrows = n; e.ncols = m; e.bn = BN; e.rowb = Ut.rb3; e.tileb = tb;
-  e.gacc = tc_gacc(Ut.kp, 1); e.gcan = tc_gcan(idx->d);
-  e.g0f = g0f;
-  e.list = idx->xlist; e.loff = idx->xloff; e.lcapv = idx->xlcap; e.lcnt = idx->xlcnt;
-  static_assert(tc::screen_smem_bytes<BN, 4, EpiXT>() <= 232448, "exact-table smem");
-  rkr_status s = launch_screen<BN, 4>(Ut, Pt, 1, row_schedule(n, m, BN), e, flags, st);
+  auto screen = split_chunks_cat(Ut.kp) >= kInterleaveChunks ? list_screen<true>
+                                                             : list_screen<false>;
+  rkr_status s = screen(idx, Ut, Pt, g0f, tb, flags, st);
   if (s == RKR_OK) s = tc_sort_lists(idx, tb, BN, st);
   int hf[2] = {0, 0};
   cudaMemcpyAsync(hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, st);

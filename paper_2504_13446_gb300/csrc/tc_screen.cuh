@@ -80,8 +80,8 @@ __device__ __forceinline__ int tile_after(int ct, int nct) {
 // Whether a screen takes its column tiles from both ends in turn: where the item
 // side is sorted by norm, the epilogue's work falls from the first tile to the last,
 // and a heavy tile's epilogue then overlaps a light tile's MMAs.  Taken where it
-// pays: the list screen 98.3 -> 93.1 ms (1M x 100k x 200); the extremes 30.1 -> 32.5
-// (they want the large norms first), the counting screens 3 to 9 % slower.
+// pays: the list screen of long rows, 98.3 -> 93.1 ms (1M x 100k x 200); the extremes
+// 30.1 -> 32.5 (they want the large norms first), the counting screens 3 to 9 % slower.
 template <class Epi, class = void>
 struct EpiInterleave {
   static constexpr bool value = false;
