@@ -217,8 +217,8 @@ rkr_status rkr_query_approx_bitmap(rkr_index *idx, const float *Q, int32_t nq, c
  * rkr_query_approx_single: rkr_query_approx answered one query at a time (latency
  * mode), as the paper runs its queries (Section 5: each query on its own).  Same
  * arguments and outputs, bit for bit.  Per query: one pass over U computes u.q for
- * every user (FP32 warp products with a rigorous bound; canonical FP64 only where
- * the bound straddles a threshold) fused with the bounds lookup of Section 4.3
+ * every user (FP32 products with a rigorous bound; where that straddles a threshold a
+ * compensated one, and canonical FP64 only where both do) fused with the bounds lookup of Section 4.3
  * step 1, then steps 2-3 run on the users whose lower bound is at most an upper
  * estimate of R_up_k (every user the steps can return is among them).  Three
  * kernel launches per query, no host synchronization until the call returns.

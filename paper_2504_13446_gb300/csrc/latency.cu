@@ -857,8 +857,8 @@ extern "C" rkr_status rkr_session_query(rkr_session *s, const float *q, int32_t 
     ss += (double)qh[i] * (double)qh[i];
   }
   if (sqrt(ss) * (1.0 + 0x1p-20) > (double)s->idx->pmax) {
-    // outside the item norms: the bin bounds of this query need a wider range,
-    // which the captured launches do not cover
+    // outside the item norms: the general call, whose bounds need no assumption about
+    // the query's norm (the scan itself makes none: see TightBins)
     return rkr_query_approx_single(s->idx, q, 1, &k, s->c, out_users, out_nlow, out_nup,
                                    out_est, out_case, out_nc, nullptr, st);
   }

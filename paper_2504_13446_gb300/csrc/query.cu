@@ -1587,10 +1587,8 @@ static std::vector<std::pair<int, int>> chunk_queries(const std::vector<int64_t>
 
 static int64_t candidate_budget() { return (int64_t)1 << tuning().cand_budget_log2; }
 
-
-
-// Exact ranks of `cnt` candidates (cu, cq): canonical u.q, sort by (user, u.q),
-// one grouped pass over P per user.  ccount[i] = #{p : s(u_i, p) > u_i.q_i}.
+// The valid candidates (cu >= 0) one behind another, each with its index in oi; their
+// order is that of the atomic cursor.
 __global__ void k_compact(int64_t n, const int32_t *__restrict__ cu, const int32_t *__restrict__ cq,
                           unsigned long long *__restrict__ cursor, int32_t *__restrict__ ou,
                           int32_t *__restrict__ oq, int32_t *__restrict__ oi) {
@@ -1611,10 +1609,10 @@ __global__ void k_scatter_back(int64_t n, const int32_t *__restrict__ oi,
 
 // Rows of a recount with one threshold each: the row's threshold and the item tying
 // exactly with it.  With cx (the screened scores of all candidates, by their index
-// ci) and no_theta, a row whose candidate has a screened score takes the interval
-// [score - bound, score + bound] holding u.q as its threshold, so no row of U or Q
-// is read (unless the score and its bound are infinite); the others take the canonical u.q rounded both ways (ths, when wanted,
-// gets the value itself).  ncanon counts the canonical products.
+// ci) a row whose candidate has a screened score takes the interval [score - bound,
+// score + bound] holding u.q as its threshold, so no row of U or Q is read (unless the
+// score and its bound are infinite).  The others take the canonical u.q rounded both
+// ways (ths, when wanted, gets the value itself).  ncanon counts the canonical products.
 __global__ void k_row_thresholds(int64_t count, const int32_t *__restrict__ cu,
                                  const int32_t *__restrict__ cq, const int32_t *__restrict__ ci,
                                  const float *__restrict__ cx, const tc::RowBound *__restrict__ urb,

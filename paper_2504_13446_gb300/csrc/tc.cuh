@@ -9,7 +9,8 @@
 //
 // Warp roles (one CTA per SM, persistent):
 //   warp 0      TMA producer (one lane)
-//   warp 1      TMEM allocation and MMA issue (one lane)
+//   warp 1      TMEM allocation and MMA issue (the warp walks the loop converged, one
+//               elected lane issues)
 //   warps 2..   epilogue, 8 or 16 warps (epi_warps): warp w reads TMEM lanes
 //               32*(w%4) .. +31 and column group (w-2)/4, so each accumulator
 //               row (user) is handled by two or four threads
