@@ -123,7 +123,9 @@ struct PairQueue {
 // thread at near-final extremes, so few items are queued.
 struct EpiFb {
   static const char *name() { return "k_screen<EpiFb>"; }
-  static constexpr int kWarps = 8;   // 30.0 ms at 1M x 100k x 200 (16 warps: 31.2)
+  // 30.0 ms at 1M x 100k x 200 (16 warps: 31.2); 400k x 50k: d = 32 5.3 (4.6), 72 5.4
+  // (4.7), 200 6.1 (6.4)
+  static constexpr int kWarps = 8;
   static constexpr int kGroups = kWarps / 4;   // threads of a row
   struct Thread {
     float b, mxlo, mnhi;
@@ -415,7 +417,9 @@ __global__ void k_xgrid(int64_t n, const double *__restrict__ fmin,
 template <bool INTERLEAVE>
 struct EpiXT {
   static const char *name() { return "k_screen<EpiXT>"; }
-  static constexpr int kWarps = 8;   // 98 ms at 1M x 100k x 200 (16 warps: 102)
+  // 98 ms at 1M x 100k x 200 (16 warps: 102); 400k x 50k: d = 32 13.2 (13.0), 72 14.0
+  // (13.7), 200 18.5 (19.5)
+  static constexpr int kWarps = 8;
   static constexpr bool kInterleave = INTERLEAVE;   // see kInterleaveChunks
   struct Thread {
     float skip, b, g0;
