@@ -1514,6 +1514,7 @@ static rkr_status emit_candidates(const rkr_index *idx, const QueryCommon &qc, i
   sub.rows = qb - qa;
   sub.hi = qc.Qt.hi + (size_t)qa * qc.Qt.ld();
   sub.lo = qc.Qt.lo + (size_t)qa * qc.Qt.ld();
+  if (qc.Qt.cat) sub.cat = qc.Qt.cat + (size_t)qa * tc_pitch(3 * qc.Qt.kp);
   sub.rb1 = qc.Qt.rb1 + qa;
   sub.rb3 = qc.Qt.rb3 + qa;
   int *flag = &words->screen_err;
